@@ -33,12 +33,9 @@
 #include <algorithm>
 #include <vector>
 
-#include <cooperative_groups.h>
-
 #include "eig_si.cuh"
+#include "eig_small.cuh"
 #include "tc_exact.cuh"
-
-namespace cg = cooperative_groups;
 
 namespace hotrg {
 namespace {
@@ -46,8 +43,6 @@ namespace {
 constexpr int kSplitMax = 8;     // split-K partials of G X
 constexpr int kChunkMax = 256;   // row chunks of the Gram reduction
 constexpr int kRowsPerChunk = 16;
-constexpr int kCluster = 8;      // CTAs per Jacobi problem (one thread-block cluster)
-constexpr int kJacobiMaxSweeps = 40;
 constexpr int kCholThreads = 256;
 constexpr int kCholPanel = 8;      // columns per panel of the blocked FP32 Cholesky
 constexpr double kXsSmallWork = 32.0 * 1024 * 1024;   // FP64 FMAs of one n x m x m product batch
@@ -603,615 +598,6 @@ __global__ void __launch_bounds__(kCholThreads) k_si_chol(PSet Cin, int m, doubl
   }
 }
 
-// Parallel two-sided Jacobi on a symmetric m x m matrix (m even) by a cluster
-// of kCluster CTAs, laid out as the systolic scheme of Sec. II.B / Fig. 3.
-// The m/2 index pairs of a round are "slots"; slot I holds two whole rows of
-// the matrix (its top and bottom index) and belongs to one CTA (contiguous
-// slots per CTA).  A round: (1) every CTA computes the rotations of all slots
-// from a replicated table of their 2x2 diagonal blocks; (2) one thread per 2x2
-// block of the CTA's rows applies both rotations at once,
-// M'_{IJ} = J_I^T M_{IJ} J_J (Eq. 6: the quad tile as the unit of work), and
-// (3) writes the four results to the slots their rows move to (tops one slot
-// down, bottoms one slot up, turning at both ends: the round-robin order in
-// which every pair meets once per sweep); each moved row also writes its
-// entries of the next round's 2x2 blocks into every CTA's table.  One cluster
-// barrier per round, split into arrive / wait so that each CTA rotates its
-// share of the rows of V while the others finish; since all CTAs see the same
-// table, the sweep decision needs no exchange.  Sweeps stop when no pair needs rotating (an off-diagonal entry is
-// rotated when it is above 2^-56 of the largest diagonal entry and not tiny
-// against its own diagonal pair), or after a sweep whose rotated entries were
-// all below 1e-8 relative (quadratic convergence).
-__device__ inline void jacobi_angle(double hpp, double hqq, double hpq, double &c, double &s) {
-  // solve h_pq t^2 + (h_qq - h_pp) t - h_pq = 0 for the smaller root (Golub &
-  // Van Loan's symmetric Schur decomposition) on a power-of-two scaled copy:
-  // FP32 estimate, then two Newton steps whose residual is evaluated in FP64
-  const double sc = pow2_inv_of(fmax(fabs(hpq), fmax(fabs(hpp), fabs(hqq))));
-  const double a = hpp * sc, b = hqq * sc, g = hpq * sc, diff = b - a;
-  const float fg = (float)g, fd = (float)diff;
-  float t32;
-  if (fabsf(fd) > 1e6f * fabsf(fg)) {
-    t32 = fg / fd;                                  // 1/(2 tau), tau = diff / (2 g)
-  } else {
-    const float tau = fd / (2.0f * fg);
-    t32 = copysignf(1.0f, tau) / (fabsf(tau) + sqrtf(1.0f + tau * tau));
-  }
-  double t = (double)t32;
-  // seed of c = (1 + t^2)^(-1/2) from the FP32 root, computed while t is refined
-  const float c32 = rsqrtf(fmaf(t32, t32, 1.0f));
-#pragma unroll
-  for (int it = 0; it < 2; ++it) {
-    const double F = fma(fma(g, t, diff), t, -g);   // g t^2 + diff t - g
-    const double dF = fma(2.0 * g, t, diff);
-    t -= F * (double)__frcp_rn((float)dF);
-  }
-  // |t| <= 1 (the smaller root), so x = 1 + t^2 lies in [1, 2] and needs no
-  // power-of-two scaling: two Newton steps y <- y (3 - x y^2) / 2 in FP64
-  const double x = fma(t, t, 1.0);
-  double y = (double)c32;
-  y = y * fma(-0.5 * x, y * y, 1.5);
-  y = y * fma(-0.5 * x, y * y, 1.5);
-  c = y;
-  s = t * c;
-}
-
-__global__ void __launch_bounds__(512, 2) k_si_jacobi(PSet Cin, int m, PSet Wout, PSet theta, int *flag,
-                                                   int *sweeps, int floor_exp, int sig_exp) {
-  cg::cluster_group cluster = cg::this_cluster();
-  const int rank = (int)cluster.block_rank();
-  const int z = blockIdx.z;
-  extern __shared__ double sh[];
-  const int half = m / 2;
-  const int spc = (half + kCluster - 1) / kCluster;          // slots per CTA
-  const int s0 = rank * spc, s1 = min(half, s0 + spc);      // own slots [s0, s1)
-  const int vrows = (m + kCluster - 1) / kCluster;
-  const int v0 = rank * vrows, v1 = min(m, v0 + vrows);     // own rows of V
-  // rows[buf][slot - s0][0 = top, 1 = bottom][m]
-  double *rowsb = sh;
-  auto ROW = [&](int buf, int slot, int tb) { return rowsb + (((size_t)buf * spc + (slot - s0)) * 2 + tb) * m; };
-  double *V = rowsb + (size_t)2 * spc * 2 * m;              // vrows x m
-  double *ac = V + (size_t)vrows * m;                       // c of every slot, [round parity][slot]
-  double *as = ac + 2 * half;                               // s of every slot, same
-  // angle inputs of every slot, replicated in every CTA, double-buffered by
-  // round parity: [buf][slot][0 = h of the top row's index, 1 = h of the
-  // bottom row's index, 2 = h_pq from the row of the smaller index]
-  double *nd = as + 2 * half;
-  double *diag = nd + 2 * 3 * half;                         // m diagonal entries
-  int *ap = reinterpret_cast<int *>(diag + m);              // p of every slot, [parity][slot]
-  int *aq = ap + 2 * half;                                  // q of every slot, same
-  __shared__ int rotated;
-  __shared__ unsigned int maxrel_bits;
-  __shared__ double s_floor, s_sig;
-  __shared__ int s_more, s_any[2];     // post-sweep test: this CTA's rows / the cluster's
-  auto top_index = [&](int sl, int rr) { return (sl == 0) ? 0 : 1 + (sl - 1 + rr) % (m - 1); };
-  auto bot_index = [&](int sl, int rr) { return 1 + (m - 2 - sl + rr) % (m - 1); };
-
-  // round 0 layout: position j holds index j; slot I = positions (I, m-1-I).
-  // The symmetric part of the input: the rotations assume h_pq = h_qp, and a
-  // stored asymmetry above the stop thresholds would never be rotated away.
-  for (int e = threadIdx.x; e < (s1 - s0) * 2 * m; e += blockDim.x) {
-    const int sl = s0 + e / (2 * m), tb = (e / m) & 1, c = e % m;
-    const int idx = tb == 0 ? sl : m - 1 - sl;
-    const double *C = Cin.at(z);
-    ROW(0, sl, tb)[c] = 0.5 * (C[(size_t)idx * m + c] + C[(size_t)c * m + idx]);
-  }
-  for (int e = threadIdx.x; e < (v1 - v0) * m; e += blockDim.x) {
-    const int rl = e / m, c = e % m;
-    V[rl * m + c] = (v0 + rl == c) ? 1.0 : 0.0;
-  }
-  for (int sl = threadIdx.x; sl < half; sl += blockDim.x) {
-    const int u = top_index(sl, 0), v = bot_index(sl, 0);
-    const double *C = Cin.at(z);
-    nd[sl * 3 + 0] = C[(size_t)u * m + u];
-    nd[sl * 3 + 1] = C[(size_t)v * m + v];
-    nd[sl * 3 + 2] = 0.5 * (C[(size_t)u * m + v] + C[(size_t)v * m + u]);
-  }
-  // absolute floor of the rotations: entries below 2^-56 of the largest diagonal
-  // entry (a quarter ulp of the matrix norm) are rounding noise; rotating them
-  // changes no eigenpair beyond that level, while the relative test below would
-  // keep rotating noise between near-null diagonal entries (measured: 12 -> 9.7
-  // sweeps per Rayleigh-Ritz solve on D = 32-48 environments)
-  if (threadIdx.x == 0) s_any[0] = s_any[1] = 0;
-  if (threadIdx.x < 32) {
-    double v = 0.0;
-    for (int i = threadIdx.x; i < m; i += 32) v = fmax(v, fabs(Cin.at(z)[(size_t)i * m + i]));
-    for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(0xffffffffu, v, o));
-    if (threadIdx.x == 0) {
-      s_floor = ldexp(v, -floor_exp);
-      // rotations below 2^-sig_exp of the largest diagonal entry do not hold
-      // the sweeps back (their entries are absolutely negligible, whatever
-      // their size against their own diagonal pair)
-      s_sig = ldexp(v, -sig_exp);
-    }
-  }
-  __syncthreads();
-  // the round-0 inputs are read locally; remote writes only target buffer 1
-  // before the first cluster barrier, so no barrier is needed here
-
-  int cur = 0, sweep = 0, r_global = 0;
-  bool stop = false;
-  for (; sweep < kJacobiMaxSweeps && !stop; ++sweep) {
-    if (threadIdx.x == 0) {
-      rotated = 0;
-      maxrel_bits = 0u;
-    }
-    __syncthreads();
-    for (int r = 0; r < m - 1; ++r, ++r_global) {
-      const int rr = r_global % (m - 1), rn = (r_global + 1) % (m - 1);
-      const double *ndc = nd + (r_global & 1) * 3 * half;
-      double *ndn_local = nd + ((r_global + 1) & 1) * 3 * half;
-      // this round's angle arrays (double-buffered by round parity: a thread may
-      // still rotate V with this round's angles while others start the next round)
-      double *acr = ac + (r_global & 1) * half, *asr = as + (r_global & 1) * half;
-      int *apr = ap + (r_global & 1) * half, *aqr = aq + (r_global & 1) * half;
-      // (1) every CTA computes the angles of every slot from the replicated inputs
-      for (int sl = threadIdx.x; sl < half; sl += blockDim.x) {
-        const int u = top_index(sl, rr), v = bot_index(sl, rr);
-        const int p = min(u, v), q = max(u, v);
-        const double hpp = (u < v) ? ndc[sl * 3 + 0] : ndc[sl * 3 + 1];
-        const double hqq = (u < v) ? ndc[sl * 3 + 1] : ndc[sl * 3 + 0];
-        const double hpq = ndc[sl * 3 + 2];
-        double c = 1.0, sv = 0.0;
-        if (fabs(hpq) > s_floor && hpq * hpq > 1e-30 * fabs(hpp * hqq) && fabs(hpq) > 1e-300) {
-          const float den = fabsf((float)hpp * (float)hqq);
-          const float rel2 = den > 0.0f ? fminf(1.0f, (float)hpq * (float)hpq / den) : 1.0f;
-          if (fabs(hpq) > s_sig) atomicMax(&maxrel_bits, __float_as_uint(rel2));
-          jacobi_angle(hpp, hqq, hpq, c, sv);
-          rotated = 1;
-        }
-        acr[sl] = c;
-        asr[sl] = sv;
-        apr[sl] = p;
-        aqr[sl] = q;
-      }
-      __syncthreads();
-      // (2) the two-sided rotation of every 2x2 block held by this CTA, Eq. 6:
-      // M'_{IJ} = J_I^T M_{IJ} J_J for the row pair I of an own slot and every
-      // column pair J, in one pass; (3) the four results go straight to the slots
-      // their rows move to (tops one slot down, bottoms one slot up, slot 0's top
-      // fixed), and a row that lands in a slot also publishes that slot's
-      // next-round angle inputs (its diagonal entry, and h_pq if it holds the
-      // smaller index) into every CTA's table.  Remote addresses are mapped at
-      // each store (one mapa each) rather than held in registers.
-      for (int e = threadIdx.x; e < (s1 - s0) * half; e += blockDim.x) {
-        const int sl = s0 + e / half, J = e % half;
-        const double *top = ROW(cur, sl, 0), *bot = ROW(cur, sl, 1);
-        const bool top_is_p = (top_index(sl, rr) == apr[sl]);
-        const double *rp = top_is_p ? top : bot, *rq = top_is_p ? bot : top;
-        const int pc = apr[J], qc = aqr[J];
-        const double cJ = acr[J], sJ = asr[J], c = acr[sl], sv = asr[sl];
-        // right factor J_J on the two rows
-        const double xp = rp[pc], yp = rp[qc], xq = rq[pc], yq = rq[qc];
-        const double p_pc = cJ * xp - sJ * yp, p_qc = sJ * xp + cJ * yp;
-        const double q_pc = cJ * xq - sJ * yq, q_qc = sJ * xq + cJ * yq;
-        // left factor J_I^T
-        double np_pc = c * p_pc - sv * q_pc, np_qc = c * p_qc - sv * q_qc;
-        double nq_pc = sv * p_pc + c * q_pc, nq_qc = sv * p_qc + c * q_qc;
-        if (J == sl) {          // the rotated pair's own block is diagonal to rounding
-          np_qc = 0.0;
-          nq_pc = 0.0;
-        }
-        int dsl[2], dtb[2];
-        if (sl == 0) { dsl[0] = 0; dtb[0] = 0; }          // slot 0's top is fixed
-        else if (sl == 1) { dsl[0] = 0; dtb[0] = 1; }     // -> slot 0 bottom
-        else { dsl[0] = sl - 1; dtb[0] = 0; }
-        if (sl == half - 1) { dsl[1] = sl; dtb[1] = 0; } else { dsl[1] = sl + 1; dtb[1] = 1; }
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          const int col = h == 0 ? pc : qc;
-          const double np = h == 0 ? np_pc : np_qc, nq = h == 0 ? nq_pc : nq_qc;
-          const double vals[2] = {top_is_p ? np : nq, top_is_p ? nq : np};   // new top, new bottom
-#pragma unroll
-          for (int w = 0; w < 2; ++w) {
-            const int own = dsl[w] / spc;
-            double *base = cluster.map_shared_rank(rowsb, own) +
-                           ((((size_t)1 - cur) * spc + (dsl[w] - own * spc)) * 2 + dtb[w]) * m;
-            base[col] = vals[w];
-            const int nu = top_index(dsl[w], rn), nv = bot_index(dsl[w], rn);
-            const int idx = dtb[w] == 0 ? nu : nv, partner = dtb[w] == 0 ? nv : nu;
-            if (col == idx) {
-              for (int k = 0; k < kCluster; ++k)
-                cluster.map_shared_rank(ndn_local, k)[dsl[w] * 3 + dtb[w]] = vals[w];
-            } else if (col == partner && idx < partner) {
-              for (int k = 0; k < kCluster; ++k) cluster.map_shared_rank(ndn_local, k)[dsl[w] * 3 + 2] = vals[w];
-            }
-          }
-        }
-      }
-      // the rows are in place once every CTA has arrived; meanwhile V <- V J on the
-      // rows of V this CTA holds (local, needs only the angles)
-      asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
-      for (int e = threadIdx.x; e < (v1 - v0) * half; e += blockDim.x) {
-        const int rl = e / half, J = e % half;
-        const int pj = apr[J], qj = aqr[J];
-        const double x = V[rl * m + pj], y = V[rl * m + qj];
-        V[rl * m + pj] = acr[J] * x - asr[J] * y;
-        V[rl * m + qj] = asr[J] * x + acr[J] * y;
-      }
-      asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
-      cur ^= 1;
-    }
-    // every CTA saw the same angles: the sweep decision needs no exchange.
-    // Quadratic convergence: once every rotated entry was below 1e-8 relative,
-    // what remains after this sweep is at rounding level.
-    __syncthreads();
-    stop = (rotated == 0) || __uint_as_float(maxrel_bits) < 1e-16f;
-    __syncthreads();
-    if (!stop) {
-      // Would the next sweep rotate anything?  Every CTA applies the rotation
-      // test to the entries of its own rows (diagonal entries from the
-      // replicated table of the next round, gathered into `diag`, which is
-      // free until the end), the answers are OR-ed across the cluster, and a
-      // sweep that would rotate nothing is not run.
-      const int rr = r_global % (m - 1);
-      const double *ndc = nd + (r_global & 1) * 3 * half;
-      for (int sl = threadIdx.x; sl < half; sl += blockDim.x) {
-        diag[top_index(sl, rr)] = ndc[sl * 3 + 0];
-        diag[bot_index(sl, rr)] = ndc[sl * 3 + 1];
-      }
-      if (threadIdx.x == 0) s_more = 0;
-      __syncthreads();
-      for (int e = threadIdx.x; e < (s1 - s0) * 2 * m; e += blockDim.x) {
-        const int sl = s0 + e / (2 * m), tb = (e / m) & 1, c = e % m;
-        const int idx = tb == 0 ? top_index(sl, rr) : bot_index(sl, rr);
-        if (c != idx) {
-          const double h = ROW(cur, sl, tb)[c];
-          if (fabs(h) > s_floor && h * h > 1e-30 * fabs(diag[idx] * diag[c]) && fabs(h) > 1e-300)
-            s_more = 1;
-        }
-      }
-      __syncthreads();
-      if (threadIdx.x == 0 && s_more)
-        for (int k = 0; k < kCluster; ++k) atomicExch(cluster.map_shared_rank(&s_any[sweep & 1], k), 1);
-      cluster.sync();
-      stop = s_any[sweep & 1] == 0;
-      __syncthreads();
-      if (threadIdx.x == 0) s_any[sweep & 1] = 0;   // reused two sweeps on, after this CTA's next barriers
-    }
-  }
-  // diagonal: each CTA knows the index of every row it holds; gather all m values
-  {
-    const int rr = r_global % (m - 1);
-    for (int e = threadIdx.x; e < (s1 - s0) * 2; e += blockDim.x) {
-      const int sl = s0 + (e >> 1), tb = e & 1;
-      const int idx = tb == 0 ? top_index(sl, rr) : bot_index(sl, rr);
-      const double dv = ROW(cur, sl, tb)[idx];
-      for (int k = 0; k < kCluster; ++k) cluster.map_shared_rank(diag, k)[idx] = dv;
-    }
-  }
-  cluster.sync();
-  if (threadIdx.x == 0 && rank == 0) {
-    if (!stop) atomicExch(flag, 2);
-    atomicMax(sweeps, sweep);
-  }
-  // sort descending (rank of each diagonal entry, ties by index)
-  for (int i = threadIdx.x; i < m; i += blockDim.x) {
-    const double ti = diag[i];
-    int rk = 0;
-    for (int j = 0; j < m; ++j) {
-      const double tj = diag[j];
-      rk += (tj > ti) || (tj == ti && j < i);
-    }
-    if (rank == 0) theta.at(z)[rk] = ti;
-    for (int row = v0; row < v1; ++row) Wout.at(z)[(size_t)rk * m + row] = V[(row - v0) * m + i];
-  }
-  cluster.sync();   // no CTA leaves while others may still read its shared memory
-}
-
-// ---- Rayleigh-Ritz eigensolver of the small projected matrix H (m x m) ----
-//
-// GB300 runs FP64 at a few flops per clock per SM, so the two-sided Jacobi
-// sweeps from a general H are done first in FP32 (one CTA per problem, all
-// disjoint pairs of a round at once, Eq. 6 per 2 x 2 block of the rotated
-// rows and columns), which leaves V with V^T H V diagonal to FP32 accuracy.
-// V is then made orthonormal to FP64 accuracy by two Newton-Schulz steps,
-// H' = V^T H V is formed in FP64, and the FP64 cluster Jacobi finishes on H',
-// whose off-diagonal entries are already at FP32 level: quadratic
-// convergence takes about two sweeps instead of the ten a general H needs.
-// The eigenvectors of H are V W' (W' those of H').
-
-constexpr int kJ32Threads = 1024;
-constexpr int kJ32MaxSweeps = 30;
-
-size_t j32_smem(int m) {
-  return (size_t)(2 * m * (m + 1) + 2 * (m / 2)) * sizeof(float) + (size_t)(2 * (m / 2)) * sizeof(int);
-}
-
-// FP32 cyclic Jacobi on the symmetric m x m matrix C of problem z (m even),
-// round-robin pair order (every pair meets once per sweep).  Vout (FP64,
-// column-major) receives the accumulated rotation V (columns in the order of
-// the final diagonal, unsorted).  A pair is rotated while |h_pq| exceeds both
-// 2^-30 of the largest diagonal entry and 1e-6 of sqrt|h_pp h_qq|: entries
-// between two small diagonal entries are resolved to FP32 relative accuracy
-// (once the couplings to the large ones are small, the rounding noise the
-// rotations leave in them is relative to their own size), so that the FP64
-// stage starts in its quadratic regime.  The sweeps stop when none was rotated; the count goes to *sweeps
-// (maximum over problems).
-__global__ void __launch_bounds__(kJ32Threads, 1) k_rr_jacobi32(PSet Cin, int m, PSet Vout, int *sweeps) {
-  extern __shared__ float jsh[];
-  const int ld = m + 1, half = m / 2;
-  float *A = jsh;
-  float *V = A + m * ld;
-  float *cs = V + m * ld;
-  float *sn = cs + half;
-  int *pp = reinterpret_cast<int *>(sn + half);
-  int *qq = pp + half;
-  __shared__ double s_scale;
-  __shared__ int s_rot;
-  const int z = blockIdx.z;
-  const double *C = Cin.at(z);
-  if (threadIdx.x < 32) {
-    double v = 0.0;
-    for (int i = threadIdx.x; i < m; i += 32) v = fmax(v, fabs(C[(size_t)i * m + i]));
-    for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(0xffffffffu, v, o));
-    if (threadIdx.x == 0) s_scale = (v > 0.0 && isfinite(v)) ? pow2_inv_of(v) : 1.0;
-  }
-  __syncthreads();
-  const double sc = s_scale;
-  // H is symmetric by definition; its stored copy is not where W amplifies
-  // rounding (nearly dependent basis columns), and the two-sided rotations of
-  // an unsymmetric matrix do not settle: read the symmetric part
-  for (int e = threadIdx.x; e < m * m; e += blockDim.x) {
-    const int a = e / m, b = e % m;
-    A[a * ld + b] = (float)(0.5 * (C[e] + C[(size_t)b * m + a]) * sc);
-    V[a * ld + b] = (a == b) ? 1.0f : 0.0f;
-  }
-  auto top_index = [&](int sl, int rr) { return (sl == 0) ? 0 : 1 + (sl - 1 + rr) % (m - 1); };
-  auto bot_index = [&](int sl, int rr) { return 1 + (m - 2 - sl + rr) % (m - 1); };
-  const float floor_abs = 0x1.0p-30f;      // the scaled largest diagonal entry lies in [1, 2)
-  int sweep = 0;
-  for (; sweep < kJ32MaxSweeps; ++sweep) {
-    if (threadIdx.x == 0) s_rot = 0;
-    __syncthreads();
-    for (int r = 0; r < m - 1; ++r) {
-      for (int k = threadIdx.x; k < half; k += blockDim.x) {
-        const int u = top_index(k, r), v = bot_index(k, r);
-        const int p = min(u, v), q = max(u, v);
-        const float app = A[p * ld + p], aqq = A[q * ld + q], apq = A[p * ld + q];
-        float c = 1.0f, sv = 0.0f;
-        if (fabsf(apq) > floor_abs && apq * apq > 1e-12f * fabsf(app * aqq)) {
-          const float tau = (aqq - app) / (2.0f * apq);
-          const float t = copysignf(1.0f, tau) / (fabsf(tau) + sqrtf(fmaf(tau, tau, 1.0f)));
-          c = rsqrtf(fmaf(t, t, 1.0f));
-          sv = t * c;
-          s_rot = 1;
-        }
-        cs[k] = c;
-        sn[k] = sv;
-        pp[k] = p;
-        qq[k] = q;
-      }
-      __syncthreads();
-      // M'_IJ = J_I^T M_IJ J_J for every 2 x 2 block (the blocks are disjoint)
-      for (int e = threadIdx.x; e < half * half; e += blockDim.x) {
-        const int I = e / half, J = e % half;
-        const int pI = pp[I], qI = qq[I], pJ = pp[J], qJ = qq[J];
-        const float cI = cs[I], sI = sn[I], cJ = cs[J], sJ = sn[J];
-        const float a00 = A[pI * ld + pJ], a01 = A[pI * ld + qJ];
-        const float a10 = A[qI * ld + pJ], a11 = A[qI * ld + qJ];
-        const float b00 = cJ * a00 - sJ * a01, b01 = sJ * a00 + cJ * a01;
-        const float b10 = cJ * a10 - sJ * a11, b11 = sJ * a10 + cJ * a11;
-        float n00 = cI * b00 - sI * b10, n01 = cI * b01 - sI * b11;
-        float n10 = sI * b00 + cI * b10, n11 = sI * b01 + cI * b11;
-        if (I == J) n01 = n10 = 0.0f;
-        A[pI * ld + pJ] = n00;
-        A[pI * ld + qJ] = n01;
-        A[qI * ld + pJ] = n10;
-        A[qI * ld + qJ] = n11;
-      }
-      // V <- V J
-      for (int e = threadIdx.x; e < m * half; e += blockDim.x) {
-        const int row = e / half, J = e % half;
-        const int pJ = pp[J], qJ = qq[J];
-        const float x = V[row * ld + pJ], y = V[row * ld + qJ];
-        V[row * ld + pJ] = cs[J] * x - sn[J] * y;
-        V[row * ld + qJ] = sn[J] * x + cs[J] * y;
-      }
-      __syncthreads();
-    }
-    const int rot = s_rot;
-    __syncthreads();
-    if (!rot) break;
-    // The sweep that would find nothing to rotate is not run: the rotation
-    // test of every off-diagonal entry, once, decides it (m^2 / 2 tests
-    // against the m - 1 rounds of a sweep).
-    if (threadIdx.x == 0) s_rot = 0;
-    __syncthreads();
-    for (int e = threadIdx.x; e < m * m; e += blockDim.x) {
-      const int p = e / m, q = e % m;
-      if (q > p) {
-        const float app = A[p * ld + p], aqq = A[q * ld + q], apq = A[p * ld + q];
-        if (fabsf(apq) > floor_abs && apq * apq > 1e-12f * fabsf(app * aqq)) s_rot = 1;
-      }
-    }
-    __syncthreads();
-    const int more = s_rot;
-    __syncthreads();
-    if (!more) break;
-  }
-  if (threadIdx.x == 0) atomicMax(sweeps, sweep + 1);
-  double *out = Vout.at(z);
-  for (int e = threadIdx.x; e < m * m; e += blockDim.x) {
-    const int c = e / m, j = e % m;            // out[j + c m] = V[j][c]
-    out[e] = (double)V[j * ld + c];
-  }
-}
-
-// ---- FP64 finish of the Rayleigh-Ritz eigensolver --------------------------
-//
-// After the FP32 stage, H' = V^T H V is diagonal to FP32 accuracy: its
-// off-diagonal entries e_ij are ~1e-7 of their diagonal pair.  Two steps of a
-// simultaneous first-order correction remove them for every pair whose
-// diagonal entries are well separated: with A_ij = e_ij / (d_j - d_i) (skew
-// symmetric), Q = orth(I + A + A^2 / 2) (one Newton-Schulz step) and
-// H' <- Q^T H' Q, the remaining coupling of such a pair is of order
-// e_ij^2 / (d_j - d_i); the second step takes it to rounding level.  These are
-// dense m x m FP64 products spread over many CTAs (k_rr_mm).  Pairs inside a
-// cluster of near-equal diagonal entries (|d_j - d_i| <= kSfsCluster |e_ij|)
-// are left out of A and resolved afterwards by exact 2 x 2 rotations
-// (Eq. 6) of the sparse Jacobi below, which only rotates the pairs that still
-// need it -- instead of full sweeps of (m - 1) rounds over all pairs, which
-// a nearly diagonal H' mostly does not need.
-constexpr double kSfsCluster = 1e3;
-
-__global__ void k_rr_sfs_build(PSet Hp, int m, PSet Aout) {
-  const int z = blockIdx.z;
-  const double *h = Hp.at(z);
-  double *a = Aout.at(z);
-  for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < m * m; e += gridDim.x * blockDim.x) {
-    const int i = e % m, j = e / m;                      // column-major: a[i + j m]
-    double v = 0.0;
-    if (i != j) {
-      const double eij = 0.5 * (h[(size_t)j * m + i] + h[(size_t)i * m + j]);
-      const double gap = h[(size_t)j * m + j] - h[(size_t)i * m + i];
-      if (eij != 0.0 && fabs(gap) > kSfsCluster * fabs(eij)) v = eij / gap;
-    }
-    a[e] = v;
-  }
-}
-
-// Classical-order ("largest first") two-sided Jacobi on the nearly diagonal
-// symmetric m x m matrix Hin (one CTA per problem): each round, every row
-// finds the partner with the largest entry that needs rotating (the rotation
-// test of k_si_jacobi: above 2^-44 of the largest diagonal entry and not
-// negligible against its own diagonal pair), the mutually largest pairs --
-// disjoint by construction, and always including the largest entry of the
-// matrix -- are rotated at once (Eq. 6), and the accumulated rotation W (in:
-// Win, m x m column-major) follows.  Stops when nothing needs rotating;
-// *rounds receives the round count (maximum over problems), flag is set to 2
-// if kSparseRounds * m rounds do not suffice.  Output as k_si_jacobi: Ritz
-// values descending in theta, Wout columns in the same order.
-constexpr int kSparseRounds = 16;
-constexpr int kSparseThreads = 1024;
-
-size_t sparse_smem(int m) {
-  return (size_t)2 * m * (m + 1) * sizeof(double) + (size_t)m * (sizeof(int) + sizeof(double)) +
-         (size_t)(m / 2 + 1) * (2 * sizeof(int) + 2 * sizeof(double)) + 64;
-}
-
-__global__ void __launch_bounds__(kSparseThreads, 1)
-    k_rr_sparse_jacobi(PSet Hin, int m, PSet Win, PSet Wout, PSet theta, int *flag, int *rounds_out) {
-  extern __shared__ double ssh[];
-  const int ld = m + 1, maxsel = m / 2 + 1;
-  double *H = ssh;                                  // row-major, symmetric part of Hin
-  double *W = H + (size_t)m * ld;                   // W[r * ld + c] = Win(r, c)
-  double *sc = W + (size_t)m * ld;                  // rotation c of selected pair k
-  double *ss = sc + maxsel;                         // rotation s
-  int *best = reinterpret_cast<int *>(ss + maxsel); // per row: partner with the largest entry, -1
-  int *selp = best + m, *selq = selp + maxsel;
-  __shared__ int nsel;
-  __shared__ double s_floor;
-  const int z = blockIdx.z;
-  const double *hin = Hin.at(z), *win = Win.at(z);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nwarps = blockDim.x >> 5;
-  for (int e = threadIdx.x; e < m * m; e += blockDim.x) {
-    const int r = e % m, c = e / m;                 // column-major inputs: coalesced reads
-    H[r * ld + c] = 0.5 * (hin[(size_t)c * m + r] + hin[(size_t)r * m + c]);
-    W[r * ld + c] = win[(size_t)c * m + r];
-  }
-  __syncthreads();
-  if (threadIdx.x < 32) {
-    double v = 0.0;
-    for (int i = threadIdx.x; i < m; i += 32) v = fmax(v, fabs(H[i * ld + i]));
-    for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(0xffffffffu, v, o));
-    if (threadIdx.x == 0) s_floor = ldexp(v, -44);
-  }
-  __syncthreads();
-  const double fl = s_floor;
-  auto needs = [&](double hpp, double hqq, double hpq) {
-    return fabs(hpq) > fl && hpq * hpq > 1e-30 * fabs(hpp * hqq) && fabs(hpq) > 1e-300;
-  };
-  int round = 0;
-  bool done = false;
-  for (; round < kSparseRounds * m; ++round) {
-    // (1) each row's best partner (one warp per row)
-    for (int p = warp; p < m; p += nwarps) {
-      double bv = 0.0;
-      int bq = -1;
-      const double hpp = H[p * ld + p];
-      for (int q = lane; q < m; q += 32) {
-        // the symmetric value: rows p and q must agree on it for the pair to be mutual
-        const double h = 0.5 * (H[p * ld + q] + H[q * ld + p]);
-        if (q != p && needs(hpp, H[q * ld + q], h) && fabs(h) > bv) {
-          bv = fabs(h);
-          bq = q;
-        }
-      }
-      for (int o = 16; o > 0; o >>= 1) {
-        const double ov = __shfl_xor_sync(0xffffffffu, bv, o);
-        const int oq = __shfl_xor_sync(0xffffffffu, bq, o);
-        if (ov > bv || (ov == bv && oq > bq)) {
-          bv = ov;
-          bq = oq;
-        }
-      }
-      if (lane == 0) best[p] = bq;
-    }
-    if (threadIdx.x == 0) nsel = 0;
-    __syncthreads();
-    // (2) mutually best pairs, their angles
-    for (int p = threadIdx.x; p < m; p += blockDim.x) {
-      const int q = best[p];
-      if (q > p && best[q] == p) {
-        const int k = atomicAdd(&nsel, 1);
-        double c, sv;
-        jacobi_angle(H[p * ld + p], H[q * ld + q], 0.5 * (H[p * ld + q] + H[q * ld + p]), c, sv);
-        selp[k] = p;
-        selq[k] = q;
-        sc[k] = c;
-        ss[k] = sv;
-      }
-    }
-    __syncthreads();
-    const int ns = nsel;
-    if (ns == 0) {
-      done = true;
-      break;
-    }
-    // (3) right factor: columns p, q of H and W
-    for (int e = threadIdx.x; e < ns * m; e += blockDim.x) {
-      const int k = e / m, r = e % m, p = selp[k], q = selq[k];
-      const double c = sc[k], sv = ss[k];
-      const double x = H[r * ld + p], y = H[r * ld + q];
-      H[r * ld + p] = c * x - sv * y;
-      H[r * ld + q] = sv * x + c * y;
-      const double wx = W[r * ld + p], wy = W[r * ld + q];
-      W[r * ld + p] = c * wx - sv * wy;
-      W[r * ld + q] = sv * wx + c * wy;
-    }
-    __syncthreads();
-    // (4) left factor: rows p, q; the rotated pair's own entries are zero
-    for (int e = threadIdx.x; e < ns * m; e += blockDim.x) {
-      const int k = e / m, col = e % m, p = selp[k], q = selq[k];
-      const double c = sc[k], sv = ss[k];
-      const double x = H[p * ld + col], y = H[q * ld + col];
-      H[p * ld + col] = (col == q) ? 0.0 : c * x - sv * y;
-      H[q * ld + col] = (col == p) ? 0.0 : sv * x + c * y;
-    }
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) {
-    if (!done) atomicExch(flag, 2);
-    atomicMax(rounds_out, round);
-  }
-  // sort descending (rank of each diagonal entry, ties by index); best[] now
-  // holds the column of each rank
-  for (int i = threadIdx.x; i < m; i += blockDim.x) {
-    const double ti = H[i * ld + i];
-    int rk = 0;
-    for (int j = 0; j < m; ++j) {
-      const double tj = H[j * ld + j];
-      rk += (tj > ti) || (tj == ti && j < i);
-    }
-    theta.at(z)[rk] = ti;
-    best[rk] = i;
-  }
-  __syncthreads();
-  for (int e = threadIdx.x; e < m * m; e += blockDim.x) {
-    const int row = e % m, rk = e / m;
-    Wout.at(z)[e] = W[row * ld + best[rk]];
-  }
-}
-
 // flags.at(z)[2] = 1 if max |C_ij - delta_ij| > 1/4 (the Newton-Schulz
 // iteration for C^-1/2 from I is then not to be trusted), else 0.
 __global__ void k_rr_far_from_identity(PSet C, int m, PSet flags) {
@@ -1356,15 +742,6 @@ __global__ void k_si_copy_square(PSet G, PSet out, int n, int m) {
   }
 }
 
-// X[:, c] = first n rows of W[:, c] for c < k
-__global__ void k_si_take(PSet W, PSet X, int n, int m, int k) {
-  const int z = blockIdx.z;
-  for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < n * k; e += gridDim.x * blockDim.x) {
-    const int c = e / n, r = e % n;
-    X.at(z)[(size_t)c * n + r] = W.at(z)[(size_t)c * m + r];
-  }
-}
-
 // Copy of problem z's n x m block from src to dst (final placement of Ritz vectors).
 __global__ void k_si_copy(PSet src, PSet dst, long long nm) {
   const int z = blockIdx.z;
@@ -1446,12 +823,6 @@ Bufs carve(double *work, int P, const Layout &L) {
 
 bool same(const PSet &a, const PSet &b) { return a.b0 == b.b0 && a.b1 == b.b1 && a.stride == b.stride; }
 
-size_t jacobi_smem(int m) {
-  const int half = m / 2;
-  const int spc = (half + kCluster - 1) / kCluster, vrows = (m + kCluster - 1) / kCluster;
-  return ((size_t)2 * spc * 2 * m + (size_t)vrows * m + 4 * half + 6 * half + m) * sizeof(double) +
-         (size_t)(4 * half) * sizeof(int) + 64;
-}
 size_t chol_smem(int m) { return (size_t)(2 * m * (m + 1) + 2 * m) * sizeof(double); }
 size_t chol32_smem(int m) {
   const int nb = (m + kCholPanel - 1) / kCholPanel;
@@ -1463,11 +834,8 @@ cudaError_t set_attrs() {
   if (done) return cudaSuccess;
   cudaError_t e;
   const int big = 200 * 1024;
-  if ((e = cudaFuncSetAttribute(k_si_jacobi, cudaFuncAttributeMaxDynamicSharedMemorySize, big)) ||
-      (e = cudaFuncSetAttribute(k_si_chol, cudaFuncAttributeMaxDynamicSharedMemorySize, big)) ||
-      (e = cudaFuncSetAttribute(k_si_chol32, cudaFuncAttributeMaxDynamicSharedMemorySize, big)) ||
-      (e = cudaFuncSetAttribute(k_rr_jacobi32, cudaFuncAttributeMaxDynamicSharedMemorySize, big)) ||
-      (e = cudaFuncSetAttribute(k_rr_sparse_jacobi, cudaFuncAttributeMaxDynamicSharedMemorySize, big)))
+  if ((e = cudaFuncSetAttribute(k_si_chol, cudaFuncAttributeMaxDynamicSharedMemorySize, big)) ||
+      (e = cudaFuncSetAttribute(k_si_chol32, cudaFuncAttributeMaxDynamicSharedMemorySize, big)))
     return e;
   done = true;
   return cudaSuccess;
@@ -1476,23 +844,6 @@ cudaError_t set_attrs() {
 int grid_1d(long long count, int P) {
   long long b = (count + 255) / 256;
   return (int)std::max<long long>(1, std::min<long long>(b, (152 * 4 + P - 1) / P));
-}
-
-cudaError_t launch_jacobi(PSet C, int m, PSet W, PSet theta, int *flag, int *sweeps, int P,
-                          cudaStream_t s, int floor_exp = 56, int sig_exp = 2000) {
-  cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3(kCluster, 1, P);
-  cfg.blockDim = dim3(512, 1, 1);
-  cfg.dynamicSmemBytes = jacobi_smem(m);
-  cfg.stream = s;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = kCluster;
-  attr[0].val.clusterDim.y = 1;
-  attr[0].val.clusterDim.z = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, k_si_jacobi, C, m, W, theta, flag, sweeps, floor_exp, sig_exp);
 }
 
 }  // namespace
@@ -1513,20 +864,22 @@ SiOut si_outputs(double *work, int P, int n, int m) {
 }
 
 cudaError_t jacobi_full(const SiBatch &b, double *work, cudaStream_t s, long long *launches) {
-  cudaError_t e = set_attrs();
-  if (e) return e;
-  const int n = b.n, P = b.P;
-  int m = n + (n & 1);              // the round-robin pairing needs an even size
-  if (m < 4) m = 4;                 // and at least two pairs
+  const int n = b.n, P = b.P, m = jacobi_block(n);
   if (m > kSiMaxBlock || b.k > n || P > 65535) return cudaErrorInvalidValue;
   const Layout L = layout(P, n, m);
   Bufs B = carve(work, P, L);
+  if (n == 1) return eig_one(b.G, B.X, B.th, m, P, s, launches);
+  cudaError_t e;
   if ((e = cudaMemsetAsync(B.flag, 0, 4 * sizeof(int), s))) return e;
-  k_si_copy_square<<<dim3(grid_1d((long long)m * m, P), 1, P), 256, 0, s>>>(b.G, B.C, n, m);
-  if ((e = launch_jacobi(B.C, m, B.W, B.th, B.flag, B.sweeps, P, s))) return e;
-  k_si_take<<<dim3(grid_1d((long long)n * b.k, P), 1, P), 256, 0, s>>>(B.W, B.X, n, m, b.k);
-  *launches += 3;
-  return cudaGetLastError();
+  PSet H = b.G;
+  if (m != n) {
+    k_si_copy_square<<<dim3(grid_1d((long long)m * m, P), 1, P), 256, 0, s>>>(b.G, B.C, n, m);
+    if ((e = cudaGetLastError())) return e;
+    *launches += 1;
+    H = B.C;
+  }
+  const SmallEig se{P, m, H, B.Cp, true, b.graded, B.X, n, b.k, B.th, B.flag, B.sweeps, B.flag + 3};
+  return small_eig(se, s, launches);
 }
 
 cudaError_t si_solve(const SiBatch &b, double *work, double tol, int max_iter, cudaStream_t s,
@@ -1662,56 +1015,6 @@ cudaError_t si_solve(const SiBatch &b, double *work, double tol, int max_iter, c
     nl += 2;
     return cudaGetLastError();
   };
-  // Eigenpairs of the projected matrix H (in B.C) into B.W (columns, descending)
-  // and B.th: FP32 Jacobi -> FP64 Newton-Schulz orthonormalisation -> FP64
-  // cluster Jacobi on H' = V^T H V -> W = V W'.  Scratch: three m x m slots in
-  // the (then unused) Gram-partial region.
-  auto small_eig = [&]() -> cudaError_t {
-    auto slot = [&](int i) { return PSet{B.Cp.b0 + i * L.mm, B.Cp.b1 + i * L.mm, B.Cp.stride}; };
-    const PSet V1 = slot(0), V2 = slot(1), T1 = slot(2);
-    const dim3 gmm((m + 7) / 8, (m + 7) / 8, P);
-    k_rr_jacobi32<<<gz, kJ32Threads, j32_smem(m), s>>>(B.C, m, V1, B.flag + 3);
-    k_rr_mm<<<gmm, 256, 0, s>>>(V1, 1, V1, 1.0, 0.0, T1, m);      // T1 = V1^T V1
-    k_rr_mm<<<gmm, 256, 0, s>>>(V1, 0, T1, -0.5, 1.5, V2, m);     // V2 = V1 (3I - T1) / 2
-    k_rr_mm<<<gmm, 256, 0, s>>>(V2, 1, V2, 1.0, 0.0, T1, m);
-    k_rr_mm<<<gmm, 256, 0, s>>>(V2, 0, T1, -0.5, 1.5, V1, m);     // V1 orthonormal (FP64)
-    k_rr_mm<<<gmm, 256, 0, s>>>(B.C, 0, V1, 1.0, 0.0, T1, m);     // T1 = H V1
-    k_rr_mm<<<gmm, 256, 0, s>>>(V1, 1, T1, 1.0, 0.0, V2, m);      // V2 = V1^T H V1
-    nl += 7;
-    cudaError_t r;
-    if ((r = cudaGetLastError())) return r;
-    // FP64 finish: two first-order correction steps (k_rr_sfs_build above),
-    // W' = Q1 Q2, then the sparse Jacobi on what still needs rotating.  H'
-    // comes from two FP64 products: its entries carry rounding noise of about
-    // m u ||H|| (2^-46 at m = 72), so entries below 2^-44 of its largest
-    // diagonal entry are left alone (their effect on a residual is below
-    // 1e-13 of the largest eigenvalue).
-    const PSet Am = slot(4), Q0 = slot(5), Tq = slot(6), Qm = slot(7), Tt = slot(8);
-    const dim3 g1(grid_1d(L.mm, P), 1, P);
-    for (int step = 0; step < 2; ++step) {
-      k_rr_sfs_build<<<g1, 256, 0, s>>>(V2, m, Am);
-      k_rr_mm<<<gmm, 256, 0, s>>>(Am, 0, Am, 0.5, 1.0, Q0, m);       // A + A^2 / 2
-      k_rr_axpi<<<g1, 256, 0, s>>>(Q0, 1.0, 1.0, Q0, m);              // + I
-      k_rr_mm<<<gmm, 256, 0, s>>>(Q0, 1, Q0, 1.0, 0.0, Tq, m);        // Q0^T Q0
-      k_rr_mm<<<gmm, 256, 0, s>>>(Q0, 0, Tq, -0.5, 1.5, Qm, m);       // Q = Q0 (3I - Q0^T Q0) / 2
-      k_rr_mm<<<gmm, 256, 0, s>>>(V2, 0, Qm, 1.0, 0.0, Tt, m);        // H' Q
-      k_rr_mm<<<gmm, 256, 0, s>>>(Qm, 1, Tt, 1.0, 0.0, V2, m);        // H' <- Q^T H' Q
-      if (step == 0) {
-        k_si_copy<<<g1, 256, 0, s>>>(Qm, T1, L.mm);                    // W' = Q1
-        nl += 8;
-      } else {
-        k_rr_mm<<<gmm, 256, 0, s>>>(T1, 0, Qm, 1.0, 0.0, Tt, m);      // W' Q2
-        k_si_copy<<<g1, 256, 0, s>>>(Tt, T1, L.mm);
-        nl += 9;
-      }
-    }
-    k_rr_sparse_jacobi<<<gz, kSparseThreads, sparse_smem(m), s>>>(V2, m, T1, T1, B.th, B.flag, B.sweeps);
-    nl += 1;
-    if ((r = cudaGetLastError())) return r;
-    k_rr_mm<<<gmm, 256, 0, s>>>(V1, 0, T1, 1.0, 0.0, B.W, m);     // W = V1 W'
-    nl += 2;
-    return cudaGetLastError();
-  };
   // one CholeskyQR pass with an FP32 factorisation: dst = src W
   auto cholqr32 = [&](PSet src, PSet dst, float sh) -> cudaError_t {
     cudaError_t r = gram(src, src, true, true, false, B.C);
@@ -1814,7 +1117,8 @@ cudaError_t si_solve(const SiBatch &b, double *work, double tol, int max_iter, c
       // is H = W^T (X^T Y) W.  Its eigenvectors Z give the Ritz vectors X (W Z)
       // and G X (W Z) = Y (W Z) with one rotation each.
       auto slot = [&](int i) { return PSet{B.Cp.b0 + i * L.mm, B.Cp.b1 + i * L.mm, B.Cp.stride}; };
-      const PSet Wn = slot(3), Tn = slot(4), Ck = slot(5), Rr = slot(6);
+      PSet Wn = slot(0), Tn = slot(1);
+      const PSet Ck = slot(2), Rr = slot(3);
       const dim3 gmm((m + 7) / 8, (m + 7) / 8, P), g1(grid_1d(L.mm, P), 1, P);
       if ((e = gram(X, X, true, false, false, B.W))) return e;   // C0 (B.W until small_eig)
       if ((e = gram(X, Y, false, false, false, B.C))) return e;  // X^T Y
@@ -1824,8 +1128,8 @@ cudaError_t si_solve(const SiBatch &b, double *work, double tol, int max_iter, c
         k_rr_mm<<<gmm, 256, 0, s>>>(B.W, 0, Wn, 1.0, 0.0, Tn, m);   // C0 W
         k_rr_mm<<<gmm, 256, 0, s>>>(Wn, 1, Tn, 1.0, 0.0, Ck, m);    // W^T C0 W
         k_rr_mm<<<gmm, 256, 0, s>>>(Wn, 0, Ck, -0.5, 1.5, Tn, m);   // next W
-        k_si_copy<<<g1, 256, 0, s>>>(Tn, Wn, L.mm);
-        nl += 4;
+        std::swap(Wn, Tn);
+        nl += 3;
       }
       // where X is far from orthonormal (nearly dependent columns at a first
       // check), W comes instead from a shifted FP64 Cholesky of C0 (X W is
@@ -1835,10 +1139,10 @@ cudaError_t si_solve(const SiBatch &b, double *work, double tol, int max_iter, c
       nl += 2;
       k_rr_mm<<<gmm, 256, 0, s>>>(B.C, 0, Wn, 1.0, 0.0, Tn, m);     // (X^T Y) W
       k_rr_mm<<<gmm, 256, 0, s>>>(Wn, 1, Tn, 1.0, 0.0, Ck, m);      // H = W^T X^T Y W
-      k_si_copy<<<g1, 256, 0, s>>>(Ck, B.C, L.mm);
-      nl += 3;
+      nl += 2;
       if ((e = cudaGetLastError())) return e;
-      if ((e = small_eig())) return e;                              // H = Z Theta Z^T (Z in B.W)
+      const SmallEig se{P, m, Ck, slot(4), false, false, B.W, m, m, B.th, B.flag, B.sweeps, B.flag + 3};
+      if ((e = small_eig(se, s, &nl))) return e;                    // H = Z Theta Z^T (Z in B.W)
       k_rr_mm<<<gmm, 256, 0, s>>>(Wn, 0, B.W, 1.0, 0.0, Rr, m);     // R = W Z
       nl += 1;
       if ((e = rot(X, Rr, Z, 0))) return e;

@@ -16,7 +16,7 @@
 
 namespace hotrg {
 
-constexpr int kSiMaxBlock = 96;    // largest Rayleigh-Ritz block / direct-Jacobi size
+constexpr int kSiMaxBlock = 96;    // largest Rayleigh-Ritz block / direct solve
 constexpr int kSiSlices = 8;       // exact-slice digits of the products G X
 
 struct SiBatch {
@@ -35,6 +35,7 @@ struct SiBatch {
   double shift_rel;      // initial shift / Tr G
   int first_check;       // expected convergence iteration (first Rayleigh-Ritz step of small batches)
   double floor_tol;      // residual accepted once it stops decreasing (0: the FP64 default, 1e-10)
+  bool graded;           // jacobi_full: G is nearly diagonal already (a warm start)
 };
 
 // Where a solve leaves its results inside the workspace: Ritz vectors of
@@ -65,9 +66,9 @@ struct SiResult {
 cudaError_t si_solve(const SiBatch &b, double *work, double tol, int max_iter, cudaStream_t s,
                      SiResult *res, long long *launches);
 
-// Direct two-sided Jacobi on whole small matrices (n <= kSiMaxBlock): G is
-// copied (zero-padded to the even size jacobi_block(n)), diagonalised, and the
-// k leading eigenpairs land in si_outputs(work, P, n, jacobi_block(n)).
+// Direct diagonalisation of whole small matrices (n <= kSiMaxBlock, zero-padded
+// to the even size jacobi_block(n)) by the method of eig_small.cu; the k leading
+// eigenpairs land in si_outputs(work, P, n, jacobi_block(n)).
 int jacobi_block(int n);
 cudaError_t jacobi_full(const SiBatch &b, double *work, cudaStream_t s, long long *launches);
 

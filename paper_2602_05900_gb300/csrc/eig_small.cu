@@ -1,0 +1,644 @@
+// Batched eigensolver for small symmetric matrices (see eig_small.cuh).
+//
+// GB300 runs FP64 at two FMAs per clock per SM and 64 cycles of latency, FP32 at
+// 64 times that rate, so the rotations are done in FP32 and FP64 is kept for a
+// few dense m x m products spread over many CTAs:
+//
+//   1. k_rr_jacobi32: FP32 cyclic Jacobi, one CTA per problem.  Its V
+//      diagonalises H to FP32 relative accuracy.
+//   2. (full solves) X = V made orthonormal to ~1e-12 by one Newton-Schulz step,
+//      S = X^T H X in FP64, and a second FP32 pass on S: the first one sees the
+//      small eigenvalues of a dense H only through the FP32 rounding of the
+//      large entries; S is graded, and its small block is resolved at its own
+//      scale.
+//   3. Three refinement passes X <- X (I + E) (Ogita and Aishima's iteration):
+//      with G = X^T X, S = X^T H X and lambda_i = s_ii / g_ii,
+//      E_ij = (s_ij - lambda_j g_ij) / (lambda_j - lambda_i) for separated pairs
+//      and -g_ij / 2 inside clusters and for couplings at rounding level:
+//      quadratic convergence of the vectors and of their orthonormality at once.
+//   4. S = X^T H X once more, and exact 2 x 2 rotations (k_rr_sparse_jacobi) of
+//      the pairs that still need one: those in clusters of near-equal values.
+//
+// Measured against the FP64 two-sided Jacobi on an 8-CTA cluster that this
+// replaced (its rounds cost 4 us, half of it FP64 arithmetic): an iTEBD update
+// of one chain at n = 60 took 3.63 ms and takes 0.74 ms, of 64 chains at n = 32
+// 3.39 ms and 0.51 ms, a D = 8 FP64 step (n = 64) 2.88 ms and 0.76 ms.
+//
+// A CPU model of the four stages (dense, graded, rank-deficient and degenerate
+// matrices, m = 16 to 96) leaves residuals and orthonormality at 1e-15 and at
+// most a few rotations for stage 4.
+#include <math.h>
+
+#include "eig_small.cuh"
+#include "eig_si.cuh"
+
+namespace hotrg {
+namespace {
+
+// 2^-e scaling factor with e the binary exponent of x (exact, x > 0 finite)
+__device__ inline double pow2_inv_of(double x) {
+  const long long bits = __double_as_longlong(x);
+  const int e = (int)((bits >> 52) & 0x7FF) - 1023;
+  return __longlong_as_double((long long)(1023 - e) << 52);
+}
+
+// |h| truncated to FP32 with integer arithmetic (FP64 conversions run at the
+// FP64 rate); values below the FP32 range give 0
+__device__ inline float mag32(double h) {
+  const unsigned hi = (unsigned)__double2hiint(h) & 0x7FFFFFFFu, lo = (unsigned)__double2loint(h);
+  const int e = (int)(hi >> 20) - 896;
+  if (e <= 0) return 0.0f;
+  if (e >= 255) return INFINITY;
+  return __uint_as_float(((unsigned)e << 23) | ((hi & 0xFFFFFu) << 3) | (lo >> 29));
+}
+
+__device__ inline void jacobi_angle(double hpp, double hqq, double hpq, double &c, double &s) {
+  // solve h_pq t^2 + (h_qq - h_pp) t - h_pq = 0 for the smaller root (Golub &
+  // Van Loan's symmetric Schur decomposition) on a power-of-two scaled copy:
+  // FP32 estimate, then two Newton steps whose residual is evaluated in FP64
+  const double sc = pow2_inv_of(fmax(fabs(hpq), fmax(fabs(hpp), fabs(hqq))));
+  const double a = hpp * sc, b = hqq * sc, g = hpq * sc, diff = b - a;
+  const float fg = (float)g, fd = (float)diff;
+  float t32;
+  if (fabsf(fd) > 1e6f * fabsf(fg)) {
+    t32 = fg / fd;                                  // 1/(2 tau), tau = diff / (2 g)
+  } else {
+    const float tau = fd / (2.0f * fg);
+    t32 = copysignf(1.0f, tau) / (fabsf(tau) + sqrtf(1.0f + tau * tau));
+  }
+  double t = (double)t32;
+  // seed of c = (1 + t^2)^(-1/2) from the FP32 root, computed while t is refined
+  const float c32 = rsqrtf(fmaf(t32, t32, 1.0f));
+#pragma unroll
+  for (int it = 0; it < 2; ++it) {
+    const double F = fma(fma(g, t, diff), t, -g);   // g t^2 + diff t - g
+    const double dF = fma(2.0 * g, t, diff);
+    t -= F * (double)__frcp_rn((float)dF);
+  }
+  // |t| <= 1 (the smaller root), so x = 1 + t^2 lies in [1, 2] and needs no
+  // power-of-two scaling: two Newton steps y <- y (3 - x y^2) / 2 in FP64
+  const double x = fma(t, t, 1.0);
+  double y = (double)c32;
+  y = y * fma(-0.5 * x, y * y, 1.5);
+  y = y * fma(-0.5 * x, y * y, 1.5);
+  c = y;
+  s = t * c;
+}
+
+// ---- stage 1: FP32 cyclic Jacobi ---------------------------------------------
+
+constexpr int kJ32MaxSweeps = 30;
+constexpr float kJ32Rel2 = 1e-12f;   // a pair is rotated while h_pq^2 > this h_pp h_qq
+
+// Row pitch: congruent to h = m / 2 modulo 32, so that a warp whose lanes run
+// over the slots of one row and on into the next one touches consecutive banks.
+__host__ __device__ inline int j32_ld(int m) {
+  const int h = m / 2;
+  return m + (((h - m) % 32) + 32) % 32;
+}
+size_t j32_smem(int m) {
+  return (size_t)4 * m * j32_ld(m) * sizeof(float) + (size_t)2 * (m / 2) * sizeof(float2);
+}
+
+// FP32 cyclic Jacobi on the symmetric m x m matrix of problem z, all disjoint
+// pairs of a round at once (Eq. 6 per 2 x 2 block), Brent and Luk's systolic
+// order (Fig. 3): slot I holds the positions I (top) and h + I (bottom), a
+// round rotates every slot's pair and then moves the tops one slot up and the
+// bottoms one slot down (slot 0's top stays), so every pair meets once in the
+// m - 1 rounds of a sweep and a sweep ends with every index back in its place.
+// The permutation is the same in every round: a thread reads and writes the
+// same addresses all the time (two buffers in turn), with no index arithmetic.
+//
+// What bounds it: the chain angle -> barrier -> rotate -> barrier of a round,
+// and shared-memory wavefronts.  The matrix is kept as the blocks I <= J only,
+// and the rotation of V by a round's angles runs in the threads that wait for
+// the next round's angles.  IV, IA: blocks of V and of the matrix per thread.
+//
+// A pair is rotated while |h_pq| exceeds both floor_abs (of the largest
+// diagonal entry, scaled to [1, 2)) and 1e-6 of sqrt|h_pp h_qq|: entries
+// between two small diagonal entries are resolved to FP32 relative accuracy.
+// Vout (FP64, column-major) receives the accumulated rotation, its columns in
+// the order of the final diagonal (unsorted); *sweeps the largest sweep count.
+template <int IV, int IA>
+__global__ void __launch_bounds__(1024, 1)
+    k_rr_jacobi32(PSet Hin, int m, float floor_abs, PSet Vout, int *sweeps) {
+  extern __shared__ float jsh[];
+  const int h = m / 2, ld = j32_ld(m), sz = m * ld;
+  float *Abuf = jsh, *Vbuf = jsh + 2 * sz;
+  float2 *cs = reinterpret_cast<float2 *>(jsh + 4 * sz);     // [round parity][slot]
+  __shared__ double s_scale;
+  __shared__ int s_rot;
+  const int z = blockIdx.z, tid = threadIdx.x, T = blockDim.x;
+  const int nang = (h + 31) / 32 * 32;                       // threads that compute angles
+  const double *H = Hin.at(z);
+  if (tid < 32) {
+    double v = 0.0;
+    for (int i = tid; i < m; i += 32) v = fmax(v, fabs(H[(size_t)i * m + i]));
+    for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(0xffffffffu, v, o));
+    if (tid == 0) s_scale = (v > 0.0 && isfinite(v)) ? pow2_inv_of(v) : 1.0;
+  }
+  __syncthreads();
+  const double sc = s_scale;
+  // H is symmetric by definition; its stored copy may not be (a projected
+  // matrix whose basis amplifies rounding), and the two-sided rotations of an
+  // unsymmetric matrix do not settle: read the symmetric part
+  for (int e = tid; e < m * m; e += T) {
+    const int a = e / m, b = e % m;
+    Abuf[a * ld + b] = (float)(0.5 * (H[e] + H[(size_t)b * m + a]) * sc);
+    Vbuf[a * ld + b] = (a == b) ? 1.0f : 0.0f;
+  }
+  // where a position moves after a round, and the stored place of an entry
+  auto next = [&](int x) {
+    if (x < h) return x == 0 ? 0 : (x < h - 1 ? x + 1 : m - 1);
+    return x == h ? 1 : x - 1;
+  };
+  auto place = [&](int r, int c) {
+    const int br = r < h ? r : r - h, bc = c < h ? c : c - h;
+    const bool swap = br > bc || (br == bc && r >= h && c < h);
+    return swap ? c * ld + r : r * ld + c;
+  };
+  // this thread's blocks of the matrix (upper triangle of blocks, folded into
+  // rows of h + 1 blocks) and of V
+  int aI[IA], aJ[IA], aw[IA][4];
+  bool aok[IA];
+#pragma unroll
+  for (int k = 0; k < IA; ++k) {
+    const int idx = tid + k * T, r = idx / (h + 1), c = idx % (h + 1);
+    const bool lower = c >= h - r;
+    aok[k] = r < (h + 1) / 2 && !(lower && r == h - 1 - r);
+    const int I = lower ? h - 1 - r : r, J = lower ? I + (c - (h - r)) : r + c;
+    aI[k] = aok[k] ? I : 0;
+    aJ[k] = aok[k] ? J : 0;
+    const int tI = next(aI[k]), bI = next(h + aI[k]), tJ = next(aJ[k]), bJ = next(h + aJ[k]);
+    aw[k][0] = place(tI, tJ);
+    aw[k][1] = place(tI, bJ);
+    aw[k][2] = place(bI, tJ);
+    aw[k][3] = place(bI, bJ);
+  }
+  int vr[IV], vJ[IV], vt[IV], vb[IV];
+  bool vok[IV];
+#pragma unroll
+  for (int k = 0; k < IV; ++k) {
+    const int idx = tid - nang + k * (T - nang);
+    vok[k] = tid >= nang && idx < h * h;
+    const int R = vok[k] ? idx / h : 0, J = vok[k] ? idx % h : 0;
+    vJ[k] = J;
+    vr[k] = R * ld + J;
+    vt[k] = R * ld + next(J);
+    vb[k] = R * ld + next(h + J);
+  }
+  int cur = 0, vcur = 0;
+  // V <- V J with the angles of round parity par, columns moved to their new slots
+  auto rotate_v = [&](int par) {
+    const float *src = Vbuf + vcur * sz;
+    float *dst = Vbuf + (vcur ^ 1) * sz;
+#pragma unroll
+    for (int k = 0; k < IV; ++k)
+      if (vok[k]) {
+        const float2 g = cs[par * h + vJ[k]];
+        const float x0 = src[vr[k]], y0 = src[vr[k] + h];
+        const float x1 = src[vr[k] + h * ld], y1 = src[vr[k] + h * ld + h];
+        dst[vt[k]] = g.x * x0 - g.y * y0;
+        dst[vb[k]] = g.y * x0 + g.x * y0;
+        dst[vt[k] + h * ld] = g.x * x1 - g.y * y1;
+        dst[vb[k] + h * ld] = g.y * x1 + g.x * y1;
+      }
+    vcur ^= 1;
+  };
+  __syncthreads();
+  int sweep = 0;
+  for (; sweep < kJ32MaxSweeps; ++sweep) {
+    // a sweep that would find nothing to rotate is not run
+    if (tid == 0) s_rot = 0;
+    __syncthreads();
+    {
+      const float *A = Abuf + cur * sz;
+      bool any = false;
+#pragma unroll
+      for (int k = 0; k < IA; ++k)
+        if (aok[k]) {
+          const int I = aI[k], J = aJ[k];
+          const float dI[2] = {A[I * ld + I], A[(h + I) * ld + h + I]};
+          const float dJ[2] = {A[J * ld + J], A[(h + J) * ld + h + J]};
+#pragma unroll
+          for (int a = 0; a < 2; ++a)
+#pragma unroll
+            for (int b = 0; b < 2; ++b) {
+              if (I == J && !(a == 0 && b == 1)) continue;
+              const float v = A[(I + a * h) * ld + J + b * h];
+              any = any || (fabsf(v) > floor_abs && v * v > kJ32Rel2 * fabsf(dI[a] * dJ[b]));
+            }
+        }
+      if (any) s_rot = 1;
+    }
+    __syncthreads();
+    const int more = s_rot;
+    __syncthreads();
+    if (!more) break;
+    for (int r = 0; r < m - 1; ++r) {
+      if (tid < h) {
+        const float *A = Abuf + cur * sz;
+        const float app = A[tid * ld + tid], aqq = A[(h + tid) * ld + h + tid], apq = A[tid * ld + h + tid];
+        float c = 1.0f, sv = 0.0f;
+        if (fabsf(apq) > floor_abs && apq * apq > kJ32Rel2 * fabsf(app * aqq)) {
+          const float tau = (aqq - app) / (2.0f * apq);
+          const float t = copysignf(1.0f, tau) / (fabsf(tau) + sqrtf(fmaf(tau, tau, 1.0f)));
+          c = rsqrtf(fmaf(t, t, 1.0f));
+          sv = t * c;
+        }
+        cs[(r & 1) * h + tid] = make_float2(c, sv);
+      }
+      if (r > 0) rotate_v((r - 1) & 1);
+      __syncthreads();
+      {
+        const float *A = Abuf + cur * sz;
+        float *B = Abuf + (cur ^ 1) * sz;
+#pragma unroll
+        for (int k = 0; k < IA; ++k)
+          if (aok[k]) {
+            const int I = aI[k], J = aJ[k], o = I * ld + J;
+            const float2 gI = cs[(r & 1) * h + I], gJ = cs[(r & 1) * h + J];
+            const float a00 = A[o], a01 = A[o + h], a11 = A[o + h * ld + h];
+            const float a10 = I == J ? a01 : A[o + h * ld];
+            const float b00 = gJ.x * a00 - gJ.y * a01, b01 = gJ.y * a00 + gJ.x * a01;
+            const float b10 = gJ.x * a10 - gJ.y * a11, b11 = gJ.y * a10 + gJ.x * a11;
+            const float n00 = gI.x * b00 - gI.y * b10, n11 = gI.y * b01 + gI.x * b11;
+            float n01 = gI.x * b01 - gI.y * b11, n10 = gI.y * b00 + gI.x * b10;
+            // a rotated slot's own coupling is zero; one left alone keeps it
+            if (I == J) n01 = n10 = gI.y != 0.0f ? 0.0f : a01;
+            B[aw[k][0]] = n00;
+            B[aw[k][1]] = n01;
+            B[aw[k][2]] = n10;
+            B[aw[k][3]] = n11;
+          }
+        cur ^= 1;
+      }
+      __syncthreads();
+    }
+    rotate_v((m - 2) & 1);
+    // the next sweep's test synchronises before the angles are written again
+  }
+  __syncthreads();
+  if (tid == 0) atomicMax(sweeps, sweep);
+  const float *V = Vbuf + vcur * sz;
+  double *out = Vout.at(z);
+  for (int e = tid; e < m * m; e += T) {
+    const int c = e / m, j = e % m;            // out[j + c m] = V[j][c]
+    out[e] = (double)V[j * ld + c];
+  }
+}
+
+// ---- FP64 m x m products -------------------------------------------------------
+
+constexpr double kSfsCluster = 1e3;   // a pair is separated if |gap| > kSfsCluster |coupling|
+
+// Out = op(A) B' with op(A) = A^T if ta, and B' = bs B + bd I, or (refine) I + E
+// of the refinement pass built from S and G while the tile is staged.  Output
+// truncated to rows x cols, column-major with ld = rows.
+struct MmOp {
+  PSet A, B, S, G, Out;
+  int ta, refine;
+  double bs, bd;
+  int rows, cols;
+};
+
+// One or two products of every problem (blockIdx.z = op P + problem), one CTA
+// per 8 x 8 output tile; the sum over k is split four ways across the CTA's
+// threads and combined in a fixed order.  At m = 48 a tile is 1536 FP64 FMA
+// cycles of one SM, about the launch's own latency: smaller tiles would only
+// re-read more, larger ones leave SMs idle.
+__global__ void __launch_bounds__(256) k_se_mm(MmOp op0, MmOp op1, int P, int m, float noise) {
+  __shared__ double As[8][kSiMaxBlock + 1];   // op(A) rows i0..i0+7, all k
+  __shared__ double Bs[8][kSiMaxBlock + 1];   // B' columns j0..j0+7, all k
+  __shared__ double part[4][8][9];
+  __shared__ double lam[kSiMaxBlock];
+  __shared__ float s_mx;
+  const bool second = (int)blockIdx.z >= P;
+  const MmOp &o = second ? op1 : op0;
+  const int z = second ? (int)blockIdx.z - P : (int)blockIdx.z;
+  const int i0 = blockIdx.x * 8, j0 = blockIdx.y * 8;
+  if (i0 >= o.rows || j0 >= o.cols) return;
+  const double *a = o.A.at(z);
+  if (o.ta) {
+    for (int e = threadIdx.x; e < 8 * m; e += blockDim.x) {
+      const int r = e / m, k = e % m, i = i0 + r;
+      As[r][k] = (i < m) ? a[(size_t)i * m + k] : 0.0;
+    }
+  } else {
+    for (int e = threadIdx.x; e < 8 * m; e += blockDim.x) {
+      const int r = e & 7, k = e >> 3, i = i0 + r;
+      As[r][k] = (i < m) ? a[(size_t)k * m + i] : 0.0;
+    }
+  }
+  if (!o.refine) {
+    const double *b = o.B.at(z);
+    for (int e = threadIdx.x; e < 8 * m; e += blockDim.x) {
+      const int r = e / m, k = e % m, j = j0 + r;
+      Bs[r][k] = (j < m) ? o.bs * b[(size_t)j * m + k] + (k == j ? o.bd : 0.0) : 0.0;
+    }
+  } else {
+    const double *S = o.S.at(z), *G = o.G.at(z);
+    // lambda = s / g to first order in g - 1 (V is orthonormal to 1e-5 or better)
+    for (int k = threadIdx.x; k < m; k += blockDim.x)
+      lam[k] = S[(size_t)k * m + k] * (2.0 - G[(size_t)k * m + k]);
+    __syncthreads();
+    if (threadIdx.x < 32) {
+      float v = 0.0f;
+      for (int k = threadIdx.x; k < m; k += 32) v = fmaxf(v, mag32(lam[k]));
+      for (int s = 16; s > 0; s >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, s));
+      if (threadIdx.x == 0) s_mx = v;
+    }
+    __syncthreads();
+    const float fl = noise * s_mx;
+    for (int e = threadIdx.x; e < 8 * m; e += blockDim.x) {
+      const int r = e / m, k = e % m, j = j0 + r;
+      double v = 0.0;
+      if (j < m) {
+        const double g = G[(size_t)j * m + k];
+        if (k == j) {
+          v = 1.5 - 0.5 * g;                                  // 1 + (1 - g) / 2
+        } else {
+          const double s = 0.5 * (S[(size_t)j * m + k] + S[(size_t)k * m + j]);
+          const double gap = lam[j] - lam[k];
+          const double num = fma(-lam[j], g, s);
+          const float off = mag32(fma(0.5 * gap, g, num));    // s - (lam_j + lam_k) g / 2
+          // the quotient needs FP32 accuracy only: what it misses is of the
+          // order of 1e-7 of a coupling that the next pass sees
+          if (mag32(gap) > (float)kSfsCluster * off && off > fl) v = (double)((float)num / (float)gap);
+          else v = -0.5 * g;
+        }
+      }
+      Bs[r][k] = v;
+    }
+  }
+  __syncthreads();
+  const int ti = threadIdx.x & 7, tj = (threadIdx.x >> 3) & 7, ks = threadIdx.x >> 6;
+  double acc = 0.0;
+  for (int k = ks; k < m; k += 4) acc = fma(As[ti][k], Bs[tj][k], acc);
+  part[ks][ti][tj] = acc;
+  __syncthreads();
+  if (threadIdx.x < 64) {
+    const int i = i0 + ti, j = j0 + tj;
+    if (i < o.rows && j < o.cols)
+      o.Out.at(z)[(size_t)j * o.rows + i] =
+          (part[0][ti][tj] + part[1][ti][tj]) + (part[2][ti][tj] + part[3][ti][tj]);
+  }
+}
+
+// ---- stage 4: rotations that are still needed ----------------------------------
+
+// Classical-order ("largest first") two-sided Jacobi on the nearly diagonal
+// symmetric m x m matrix Hin (one CTA per problem): each round, every row
+// finds the partner with the largest entry that needs rotating (above
+// 2^-floor_exp of the largest diagonal entry and not negligible against its
+// own diagonal pair), the mutually largest pairs -- disjoint by construction,
+// and always including the largest entry of the matrix -- are rotated at once
+// (Eq. 6), and the accumulated rotation W follows.  Stops when nothing needs
+// rotating; *rounds receives the round count (maximum over problems), flag is
+// set to 2 if kSparseRounds * m rounds do not suffice.  Eigenvalues descending
+// in theta, Wout columns in the same order.  The search compares FP32
+// magnitudes taken from the bits (an FP64 comparison of every entry would cost
+// more than the rotations: m^2 of them at two per clock).
+constexpr int kSparseRounds = 16;
+constexpr int kSparseThreads = 1024;
+
+size_t sparse_smem(int m) {
+  return (size_t)2 * m * (m + 1) * sizeof(double) + (size_t)m * (sizeof(int) + sizeof(float)) +
+         (size_t)(m / 2 + 1) * (2 * sizeof(int) + 2 * sizeof(double)) + 64;
+}
+
+__global__ void __launch_bounds__(kSparseThreads, 1)
+    k_rr_sparse_jacobi(PSet Hin, int m, int floor_exp, PSet Wout, PSet theta, int *flag, int *rounds_out) {
+  extern __shared__ double ssh[];
+  const int ld = m + 1, maxsel = m / 2 + 1;
+  double *H = ssh;                                  // row-major, symmetric part of Hin
+  double *W = H + (size_t)m * ld;                   // W[r * ld + c]
+  double *sc = W + (size_t)m * ld;                  // rotation c of selected pair k
+  double *ss = sc + maxsel;                         // rotation s
+  int *best = reinterpret_cast<int *>(ss + maxsel); // per row: partner with the largest entry, -1
+  int *selp = best + m, *selq = selp + maxsel;
+  float *rt = reinterpret_cast<float *>(selq + maxsel);   // sqrt|h_pp|
+  __shared__ int nsel;
+  __shared__ float s_floor;
+  const int z = blockIdx.z;
+  const double *hin = Hin.at(z);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nwarps = blockDim.x >> 5;
+  for (int e = threadIdx.x; e < m * m; e += blockDim.x) {
+    const int r = e % m, c = e / m;                 // column-major input: coalesced reads
+    H[r * ld + c] = 0.5 * (hin[(size_t)c * m + r] + hin[(size_t)r * m + c]);
+    W[r * ld + c] = r == c ? 1.0 : 0.0;
+  }
+  __syncthreads();
+  if (threadIdx.x < 32) {
+    float v = 0.0f;
+    for (int i = threadIdx.x; i < m; i += 32) v = fmaxf(v, mag32(H[i * ld + i]));
+    for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
+    if (threadIdx.x == 0) s_floor = ldexpf(v, -floor_exp);
+  }
+  int round = 0;
+  bool done = false;
+  for (; round < kSparseRounds * m; ++round) {
+    for (int p = threadIdx.x; p < m; p += blockDim.x) rt[p] = sqrtf(mag32(H[p * ld + p]));
+    if (threadIdx.x == 0) nsel = 0;
+    __syncthreads();
+    // (1) each row's best partner (one warp per row); rows p and q both read the
+    // entry above the diagonal, so they agree on it
+    const float fl = s_floor;
+    for (int p = warp; p < m; p += nwarps) {
+      float bv = 0.0f;
+      int bq = -1;
+      const float rp = 1e-15f * rt[p];
+      for (int q = lane; q < m; q += 32) {
+        const float hv = mag32(q > p ? H[p * ld + q] : H[q * ld + p]);
+        if (q != p && hv > fl && hv > rp * rt[q] && hv > bv) {
+          bv = hv;
+          bq = q;
+        }
+      }
+      for (int o = 16; o > 0; o >>= 1) {
+        const float ov = __shfl_xor_sync(0xffffffffu, bv, o);
+        const int oq = __shfl_xor_sync(0xffffffffu, bq, o);
+        if (ov > bv || (ov == bv && oq > bq)) {
+          bv = ov;
+          bq = oq;
+        }
+      }
+      if (lane == 0) best[p] = bq;
+    }
+    __syncthreads();
+    // (2) mutually best pairs, their angles
+    for (int p = threadIdx.x; p < m; p += blockDim.x) {
+      const int q = best[p];
+      if (q > p && best[q] == p) {
+        const int k = atomicAdd(&nsel, 1);
+        double c, sv;
+        jacobi_angle(H[p * ld + p], H[q * ld + q], H[p * ld + q], c, sv);
+        selp[k] = p;
+        selq[k] = q;
+        sc[k] = c;
+        ss[k] = sv;
+      }
+    }
+    __syncthreads();
+    const int ns = nsel;
+    if (ns == 0) {
+      done = true;
+      break;
+    }
+    // (3) right factor: columns p, q of H and W
+    for (int e = threadIdx.x; e < ns * m; e += blockDim.x) {
+      const int k = e / m, r = e % m, p = selp[k], q = selq[k];
+      const double c = sc[k], sv = ss[k];
+      const double x = H[r * ld + p], y = H[r * ld + q];
+      H[r * ld + p] = c * x - sv * y;
+      H[r * ld + q] = sv * x + c * y;
+      const double wx = W[r * ld + p], wy = W[r * ld + q];
+      W[r * ld + p] = c * wx - sv * wy;
+      W[r * ld + q] = sv * wx + c * wy;
+    }
+    __syncthreads();
+    // (4) left factor: rows p, q; the rotated pair's own entries are zero
+    for (int e = threadIdx.x; e < ns * m; e += blockDim.x) {
+      const int k = e / m, col = e % m, p = selp[k], q = selq[k];
+      const double c = sc[k], sv = ss[k];
+      const double x = H[p * ld + col], y = H[q * ld + col];
+      H[p * ld + col] = (col == q) ? 0.0 : c * x - sv * y;
+      H[q * ld + col] = (col == p) ? 0.0 : sv * x + c * y;
+    }
+    __syncthreads();
+  }
+  if (threadIdx.x == 0) {
+    if (!done) atomicExch(flag, 2);
+    atomicMax(rounds_out, round);
+  }
+  // sort descending (rank of each diagonal entry, ties by index); best[] now
+  // holds the column of each rank
+  for (int i = threadIdx.x; i < m; i += blockDim.x) {
+    const double ti = H[i * ld + i];
+    int rk = 0;
+    for (int j = 0; j < m; ++j) {
+      const double tj = H[j * ld + j];
+      rk += (tj > ti) || (tj == ti && j < i);
+    }
+    theta.at(z)[rk] = ti;
+    best[rk] = i;
+  }
+  __syncthreads();
+  for (int e = threadIdx.x; e < m * m; e += blockDim.x) {
+    const int row = e % m, rk = e / m;
+    Wout.at(z)[e] = W[row * ld + best[rk]];
+  }
+}
+
+__global__ void k_eig_one(PSet G, PSet X, PSet theta, int m, int P) {
+  const int z = blockIdx.x * blockDim.x + threadIdx.x;
+  if (z >= P) return;
+  X.at(z)[0] = 1.0;
+  theta.at(z)[0] = G.at(z)[0];
+  for (int i = 1; i < m; ++i) theta.at(z)[i] = 0.0;
+}
+
+cudaError_t launch_j32(PSet H, int m, float floor_abs, PSet V, int *sweeps, int P, cudaStream_t s) {
+  const int h = m / 2, nang = (h + 31) / 32 * 32;
+  // blocks of V per thread, so that the threads (and half of the matrix's
+  // blocks, at most IA per thread) fit 1024
+  const int iv = h <= 25 ? 1 : h <= 32 ? 2 : 3;
+  const int T = nang + (h * h + 32 * iv - 1) / (32 * iv) * 32;
+  const dim3 g(1, 1, P);
+  const size_t sm = j32_smem(m);
+  if (iv == 1) k_rr_jacobi32<1, 1><<<g, T, sm, s>>>(H, m, floor_abs, V, sweeps);
+  else if (iv == 2) k_rr_jacobi32<2, 1><<<g, T, sm, s>>>(H, m, floor_abs, V, sweeps);
+  else k_rr_jacobi32<3, 2><<<g, T, sm, s>>>(H, m, floor_abs, V, sweeps);
+  return cudaGetLastError();
+}
+
+cudaError_t small_attrs() {
+  static bool done = false;
+  if (done) return cudaSuccess;
+  cudaError_t e;
+  const int big = 200 * 1024;
+  const cudaFuncAttribute at = cudaFuncAttributeMaxDynamicSharedMemorySize;
+  if ((e = cudaFuncSetAttribute(k_rr_jacobi32<1, 1>, at, big)) ||
+      (e = cudaFuncSetAttribute(k_rr_jacobi32<2, 1>, at, big)) ||
+      (e = cudaFuncSetAttribute(k_rr_jacobi32<3, 2>, at, big)) ||
+      (e = cudaFuncSetAttribute(k_rr_sparse_jacobi, at, big)))
+    return e;
+  done = true;
+  return cudaSuccess;
+}
+
+}  // namespace
+
+cudaError_t small_eig(const SmallEig &a, cudaStream_t s, long long *launches) {
+  cudaError_t e = small_attrs();
+  if (e) return e;
+  const int P = a.P, m = a.m;
+  if (m < 4 || (m & 1) || m > kSiMaxBlock || P < 1 || P > 65535) return cudaErrorInvalidValue;
+  const long long mm = (long long)m * m;
+  auto slot = [&](int i) { return PSet{a.scratch.b0 + i * mm, a.scratch.b1 + i * mm, a.scratch.stride}; };
+  PSet X = slot(0), Xn = slot(1);
+  const PSet Y = slot(2), G = slot(3), S = slot(4), V = slot(5), W = slot(6);
+  // couplings below this share of the largest eigenvalue are rounding of the
+  // products (full: of H itself), and are left alone
+  const int floor_exp = a.full ? 51 : 44;
+  const float noise = ldexpf(1.0f, -(floor_exp + 1));
+  const int t = (m + 7) / 8;
+  auto op = [&](PSet A, int ta, PSet B, double bs, double bd, PSet Out) {
+    return MmOp{A, B, B, B, Out, ta, 0, bs, bd, m, m};
+  };
+  auto mm1 = [&](const MmOp &o) {
+    k_se_mm<<<dim3(t, t, P), 256, 0, s>>>(o, o, P, m, noise);
+    *launches += 1;
+  };
+  auto mm2 = [&](const MmOp &o, const MmOp &q) {
+    if (2 * P > 65535) {              // grid.z holds both products of every problem
+      mm1(o);
+      mm1(q);
+      return;
+    }
+    k_se_mm<<<dim3(t, t, 2 * P), 256, 0, s>>>(o, q, P, m, noise);
+    *launches += 1;
+  };
+  // H is symmetric: H^T Y is read along its rows
+  if (a.full) {
+    // a dense H: the first FP32 pass stops at its rounding (2^-24), the second
+    // one resolves what lies below; a graded H is resolved by the first
+    if ((e = launch_j32(a.H, m, ldexpf(1.0f, a.graded ? -56 : -24), X, a.sweeps, P, s))) return e;
+    mm1(op(X, 1, X, 1.0, 0.0, G));
+    mm1(op(X, 0, G, -0.5, 1.5, Xn));
+    mm1(op(a.H, 1, Xn, 1.0, 0.0, Y));
+    mm1(op(Xn, 1, Y, 1.0, 0.0, S));
+    if ((e = launch_j32(S, m, ldexpf(1.0f, -56), V, a.sweeps, P, s))) return e;
+    mm1(op(Xn, 0, V, 1.0, 0.0, X));
+    *launches += 2;
+  } else {
+    // pairs are resolved down to 2^-46 of the largest eigenvalue here (entries
+    // between small diagonal entries keep FP32 relative accuracy): stopping at
+    // 2^-30 costs no fewer sweeps and left hundreds of rotations to the last stage
+    if ((e = launch_j32(a.H, m, ldexpf(1.0f, -46), X, a.sweeps, P, s))) return e;
+    *launches += 1;
+  }
+  for (int pass = 0; pass < 3; ++pass) {
+    mm2(op(X, 1, X, 1.0, 0.0, G), op(a.H, 1, X, 1.0, 0.0, Y));
+    mm1(op(X, 1, Y, 1.0, 0.0, S));
+    mm1(MmOp{X, X, S, G, Xn, 0, 1, 1.0, 0.0, m, m});
+    const PSet q = X;
+    X = Xn;
+    Xn = q;
+  }
+  mm1(op(a.H, 1, X, 1.0, 0.0, Y));
+  mm1(op(X, 1, Y, 1.0, 0.0, S));
+  k_rr_sparse_jacobi<<<dim3(1, 1, P), kSparseThreads, sparse_smem(m), s>>>(S, m, floor_exp, W, a.theta, a.flag,
+                                                                          a.rounds);
+  *launches += 1;
+  mm1(MmOp{X, W, W, W, a.out, 0, 0, 1.0, 0.0, a.rows, a.cols});
+  return cudaGetLastError();
+}
+
+cudaError_t eig_one(PSet G, PSet X, PSet theta, int m, int P, cudaStream_t s, long long *launches) {
+  k_eig_one<<<(P + 127) / 128, 128, 0, s>>>(G, X, theta, m, P);
+  *launches += 1;
+  return cudaGetLastError();
+}
+
+}  // namespace hotrg

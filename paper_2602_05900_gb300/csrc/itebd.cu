@@ -259,6 +259,7 @@ hotrg_status itebd_update(hotrg_itebd *c) {
   sb.k = n;
   sb.m = jacobi_block(n);
   sb.G = pset_linear(warm ? c->theta : c->rho, c->sM);
+  sb.graded = warm;
   long long nl = 0;
   ICK(c, jacobi_full(sb, c->si_work, st, &nl));
   const SiOut o = si_outputs(c->si_work, G, n, sb.m);
