@@ -907,18 +907,12 @@ cudaError_t si_solve(const SiBatch &b, double *work, double tol, int max_iter, c
   const bool xs = b.xs;
   const bool xs_small = xs && (double)P * n * m * m >= kXsSmallWork;
   XsOperand gs{};
-  int xsplit = 1, gsplit = 1;
   // slices of a row-major (rows x K) view of problem z's buffer at src
   auto xs_slot = [&](long long off, long long scoff, int rows, int K) {
     return XsOperand{work + off, work + scoff, rows, K, xs_pitch(K), kSiSlices, P, L.per * 4, L.per};
   };
   if (xs) {
     gs = XsOperand{work + L.oGs, work + L.oGsc, n, n, L.xsp, kSiSlices, P, L.per * 4, L.per};
-    const int tiles = ((n + 127) / 128) * ((m + 95) / 96) * P;
-    xsplit = std::max(xs_min_split(n), std::min(kSplitMax, (2 * 152 + tiles - 1) / tiles));
-    while (xsplit > xs_min_split(n) && (n + xsplit - 1) / xsplit < 128) --xsplit;
-    const int gtiles = ((m + 79) / 80) * P;
-    gsplit = std::max(xs_min_split(n), std::min(std::min(kChunkMax, n / 64), (2 * 152 + gtiles - 1) / gtiles));
     if ((e = xs_split(b.G, map1(n), map1(1), gs, s))) return e;
     nl += 1;
   }
@@ -938,16 +932,9 @@ cudaError_t si_solve(const SiBatch &b, double *work, double tol, int max_iter, c
       const XsOperand xsl = xs_slot(L.oSb, L.oSbsc, m, n);     // rows of X^T
       cudaError_t r = xs_split(src, map1(n), map1(1), xsl, s);
       if (r) return r;
-      if (xsplit == 1) {
-        r = xs_gemm(gs, xsl, n, m, n, dst.b0, map1(1), map1(n), L.per, 1, 0, b.err, s);
-        nl += 2;
-      } else {
-        r = xs_gemm(gs, xsl, n, m, n, B.Yp.b0, map1(1), map1(n), L.per, xsplit, L.nm, b.err, s);
-        if (r) return r;
-        k_si_sum_split<<<dim3(grid_1d(L.nm, P), 1, P), 256, 0, s>>>(B.Yp, dst, xsplit, L.nm, src, B.sig, sh);
-        shifted = true;
-        nl += 3;
-      }
+      r = xs_gemm(gs, xsl, n, m, n, dst.b0, map1(1), map1(n), L.per, 1, 0, b.err, s, XsShift{sh != 0, src, B.sig});
+      shifted = true;
+      nl += 2;
       return r ? r : cudaGetLastError();
     }
     if (L.S == 1) {
@@ -1000,10 +987,9 @@ cudaError_t si_solve(const SiBatch &b, double *work, double tol, int max_iter, c
       if ((r = xs_split(A, map1(n), map1(1), a, s))) return r;
       const bool one = same(A, Bm);
       if (!one && (r = xs_split(Bm, map1(n), map1(1), bb, s))) return r;
-      if ((r = xs_gemm(a, one ? a : bb, m, m, n, B.Cp.b0, map1(m), map1(1), L.per, gsplit, L.mm,
-                       b.err, s)))
+      if ((r = xs_gemm(a, one ? a : bb, m, m, n, B.Cp.b0, map1(m), map1(1), L.per, 1, 0, b.err, s)))
         return r;
-      k_si_gram_reduce<<<dim3(grid_1d(L.mm, P), 1, P), 256, 0, s>>>(B.Cp, out, gsplit, m, 0, ns);
+      k_si_gram_reduce<<<dim3(grid_1d(L.mm, P), 1, P), 256, 0, s>>>(B.Cp, out, 1, m, 0, ns);
       nl += one ? 3 : 4;
       return cudaGetLastError();
     }

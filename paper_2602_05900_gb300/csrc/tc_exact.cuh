@@ -7,15 +7,15 @@
 // exact BF16 value (a "slice").  The product of two rows is then the sum over
 // slice pairs (s, t) of exact BF16 x BF16 products; pairs with s + t <= S + 1
 // are kept (the rest lie below 2^-6(S+1) of the leading term).  Pairs with the
-// same s + t = d share one FP32 accumulator in tensor memory; for d <= 6 every
-// partial sum is an integer multiple of 2^-6d below 2^24 of that unit as long as
-// K <= kXsMaxK (the d = 6 sum has five terms of at most 2^11, 2^10, 2^10,
-// 2^10, 2^11 per k), so those accumulators are exact whatever the order of
-// summation, and all d >= 7 pairs share one more, inexact but 2^-30 smaller,
-// accumulator (the tensor cores' FP32 accumulation truncates, so its error
-// grows with K; one level lower it set the error floor near 2^-44).  The
-// epilogue combines the exact accumulators in 64-bit integer arithmetic, adds
-// the small one and the row and column scales in FP64.  With
+// same s + t = d share one FP32 accumulator in tensor memory, an integer
+// multiple of 2^-6d.  For d <= 6 its partial sums stay below 2^24 of that unit
+// as long as K <= kXsMaxK (the d = 6 sum has five terms of at most 2^11, 2^10,
+// 2^10, 2^10, 2^11 per k), so those accumulators are exact whatever the order of
+// summation; the d >= 7 ones are 2^-30 smaller and exact but for saturated
+// digits at the longest K.  The epilogue combines the accumulators into one
+// 64-bit integer in units of 2^-50 (below the rounding of the digits), sums the
+// K parts of a tile exactly (a cluster of CTAs, through distributed shared
+// memory), and converts and scales once.  With
 // S slices the result is within about 2^-(6S-1) of max|A_i.| max|B_j.| per
 // term; the eigensolver's products G X use S = 8 (about 2^-47: FP64-grade).
 #pragma once
@@ -27,8 +27,8 @@
 namespace hotrg {
 
 constexpr int kXsBits = 6;        // bits per slice digit
-constexpr int kXsExactDiagonals = 5;  // digit sums d = 2..6 accumulate exactly
-constexpr int kXsMaxK = 2336;     // largest K (multiple of 32) with 7 2^10 K < 2^24
+constexpr int kXsMaxK = 2336;     // longest K part of one CTA (multiple of 32) with 7 2^10 K < 2^24
+constexpr int kXsMaxSumK = 8192;  // longest K of one launch: the integer sums stay below 2^63
 constexpr int kXsMaxSlices = 8;
 constexpr int kXsStagedK = 128;  // strided-K operands up to this K are sliced through shared memory
 
@@ -60,21 +60,28 @@ cudaError_t xs_split(PSet src, IdxMap rm, IdxMap km, const XsOperand &dst, cudaS
 cudaError_t xs_split_scaled(PSet src, IdxMap rm, IdxMap km, PSet kscale, int kmode,
                             const XsOperand &dst, cudaStream_t s);
 
+// Optional addition of a product's launch: C += sig[1] X (X laid out like C), and
+// sig[0] <- sig[1].
+struct XsShift {
+  bool on = false;
+  PSet X{nullptr, nullptr, 0}, sig{nullptr, nullptr, 0};
+};
+
 // C(m, n) = sum_k A(m, k) B(n, k) in FP64 for every instance z, written to
 // C + z * cstride + cm(m) + cn(n).  The K range is cut into `ksplit` equal
-// parts (each <= kXsMaxK); part p is written at C + p * pstride (the caller
+// parts (each <= kXsMaxSumK); part p is written at C + p * pstride (the caller
 // sums the parts).  A.S == B.S, A.batch == B.batch.  err_flag receives 2 if a
 // bounded wait runs out.
 cudaError_t xs_gemm(const XsOperand &A, const XsOperand &B, int M, int N, int K, double *C,
                     IdxMap cm, IdxMap cn, long long cstride, int ksplit, long long pstride,
-                    int *err_flag, cudaStream_t s);
+                    int *err_flag, cudaStream_t s, const XsShift &shift = XsShift{});
 
 // C[m * ldc + n] = sum_p parts[p * pstride + m * N + n] (row-major parts).
 cudaError_t xs_sum_parts(const double *parts, int nparts, long long pstride, int M, int N,
                          double *C, long long ldc, cudaStream_t s);
 
-// Smallest number of K parts with each part <= kXsMaxK.
-inline int xs_min_split(int K) { return (K + kXsMaxK - 1) / kXsMaxK; }
+// Smallest number of launch parts with each part <= kXsMaxSumK.
+inline int xs_min_split(int K) { return (K + kXsMaxSumK - 1) / kXsMaxSumK; }
 
 }  // namespace hotrg
 
