@@ -1,0 +1,542 @@
+// Orthogonalisation kernels of the subspace iteration (eig_si.cu).
+//
+// One CholeskyQR pass of an n x m block is two launches:
+//
+//   k_gram_chol32  one 8-CTA cluster per problem: FP32 Gram matrix of the CTAs'
+//                  rows (runs of 16 rows in FP32, added up in two floats), the
+//                  partials summed in FP64 through distributed shared memory,
+//                  then W by one CTA;
+//   k_si_rotate    Out = A W in FP64 (the span of the block is kept to FP64
+//                  whatever the accuracy of W).
+//
+// What bounds them: the factorisation is a chain of m dependent pivots
+// (broadcast of a row through shared memory, one barrier, a reciprocal, the
+// updates), kept free of FP64 (conversions included: FP32 -> FP64 by an
+// instruction on that chain cost 10 us of 31); the rotation is FP64 arithmetic
+// (two FMAs per clock and SM), so its tiles are sized to spread n m^2 / 2 FMAs
+// over all SMs.  Measured at n = 1024, m = 48, two problems: Gram partials, their
+// sum and the factor as three launches took 14.7 + 9.6 + 28 us and take 21.1 us
+// as one; the rotation 19.1 us and 9.2 us; an FP64 Gram matrix with its sum
+// 50 us and 16 us; the FP64 factor (one rank-1 update and three barriers per
+// column before) 115 us and 34 us.
+#include <cooperative_groups.h>
+#include <math.h>
+
+#include <algorithm>
+
+#include "eig_orth.cuh"
+#include "eig_si.cuh"
+
+namespace cg = cooperative_groups;
+
+namespace hotrg {
+namespace {
+
+constexpr int kOrthCluster = 8;
+constexpr int kSlab = 32;                    // rows staged at a time
+constexpr float kChol32Retry = 0x1.0p-12f;   // diagonal shift of a retried FP32 factorisation
+
+// FP64 <-> FP32 by integer arithmetic (the conversion instructions run at the
+// FP64 rate); subnormal FP32 values are taken as zero.
+__device__ __forceinline__ float to_f32(double x) {
+  const unsigned long long b = static_cast<unsigned long long>(__double_as_longlong(x));
+  const unsigned long long a = b & 0x7FFFFFFFFFFFFFFFull;
+  const long long r = (long long)((a + 0x0FFFFFFFull + ((a >> 29) & 1)) >> 29) - (896ll << 23);   // to nearest even
+  const unsigned f = r < (1 << 23) ? 0u : r >= (255ll << 23) ? (a > 0x7FF0000000000000ull ? 0x7FC00000u : 0x7F800000u)
+                                                              : (unsigned)r;
+  return __uint_as_float(f | ((unsigned)(b >> 32) & 0x80000000u));
+}
+__device__ __forceinline__ double to_f64(float x) {
+  const unsigned b = __float_as_uint(x), a = b & 0x7FFFFFFFu;
+  const unsigned long long r = a < (1u << 23) ? 0ull
+                               : a >= 0x7F800000u ? (0x7FF0000000000000ull | ((unsigned long long)(a & 0x7FFFFFu) << 29))
+                                                  : ((unsigned long long)a << 29) + (896ull << 52);
+  return __longlong_as_double((long long)(r | ((unsigned long long)(b & 0x80000000u) << 32)));
+}
+
+__device__ __forceinline__ float reciprocal(float p) { return __frcp_rn(p); }
+__device__ __forceinline__ double reciprocal(double p) {     // p within the FP32 range
+  double r = (double)__frcp_rn((float)p);
+  r = fma(r, fma(-p, r, 1.0), r);
+  return fma(r, fma(-p, r, 1.0), r);
+}
+__device__ __forceinline__ float inv_sqrt(float x) { return rsqrtf(x); }
+__device__ __forceinline__ double inv_sqrt(double x) { return rsqrt_fp64(x); }
+
+// Factor and inverse in one elimination, 256 threads as 16 x 16, thread (ty, tx)
+// holding the entries (ty + 16 u, tx + 16 v) in registers: element (i, k) is the
+// scaled matrix for k >= i and the growing L^-1 (L = R^T) for k < i, which
+// starts at zero.  Step j: row j goes through shared memory (two buffers, one
+// barrier per step); its pivot, its part right of the diagonal (which, the
+// matrix being symmetric, also holds the multipliers of the rows below) and its
+// L^-1 part (k < j, and 1 at k = j) update every row i > j.  At the end the
+// L^-1 rows over the square roots of the pivots are the columns of
+// W = diag(d) R^-1 = diag(d) L^-T.  Which row values an entry takes depends on
+// its tile alone off the diagonal tiles (right of them the matrix part, left of
+// them the L^-1 part), so the updates carry no tests.
+//
+// Nearly dependent columns break the unshifted factorisation; attempt a adds
+// shift(a) to the unit diagonal.  cmat(i, k), i <= k: the unscaled matrix.
+template <class T, int U, class Cmat, class Shift>
+__device__ void chol_inverse(Cmat cmat, Shift shift, int attempts, int m, double *W, int *flag, T *rowbuf, T *d,
+                             T *piv) {
+  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
+  constexpr int LD = 16 * U;
+  for (int j = tid; j < LD; j += 256) {
+    const T cjj = j < m ? cmat(j, j) : T(0);
+    d[j] = (cjj > T(0) && isfinite(cjj)) ? inv_sqrt(cjj) : T(1);
+    piv[j] = T(1);
+  }
+  __syncthreads();
+  T e[U][U];
+  bool bad = true;
+  for (int attempt = 0; attempt < attempts && bad; ++attempt) {
+    const T sh = shift(attempt);
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+#pragma unroll
+      for (int v = 0; v < U; ++v) {
+        const int i = ty + 16 * u, k = tx + 16 * v;
+        e[u][v] = (i <= k && k < m) ? cmat(i, k) * (d[i] * d[k]) + (i == k ? sh : T(0)) : T(0);
+      }
+    bad = false;
+    for (int j = 0; j < m; ++j) {
+      T *buf = rowbuf + (j & 1) * LD;
+      if (ty == (j & 15)) {
+        const int ju = j >> 4;
+#pragma unroll
+        for (int v = 0; v < U; ++v) {
+          T x = e[0][v];             // selected, not indexed: e stays in registers
+#pragma unroll
+          for (int u = 1; u < U; ++u) x = ju == u ? e[u][v] : x;
+          buf[tx + 16 * v] = x;
+        }
+      }
+      __syncthreads();
+      const T p = buf[j];
+      if (!(p > T(0)) || !isfinite(p)) {       // the same for every thread
+        bad = true;
+        break;
+      }
+      if (tid == 0) piv[j] = p;
+      const T rinv = reciprocal(p);
+      T right[U], left[U], diag[U];
+#pragma unroll
+      for (int v = 0; v < U; ++v) {
+        const int k = tx + 16 * v;
+        right[v] = buf[k];
+        left[v] = k < j ? right[v] : k == j ? T(1) : T(0);
+        diag[v] = tx >= ty ? right[v] : left[v];
+      }
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        if (j >= 16 * u + 15) continue;        // every row of the tile is done
+        const int i = ty + 16 * u;
+        const T mult = i > j ? -(buf[i] * rinv) : T(0);
+#pragma unroll
+        for (int v = 0; v < U; ++v) e[u][v] = fma(mult, v > u ? right[v] : v < u ? left[v] : diag[v], e[u][v]);
+      }
+    }
+    __syncthreads();
+  }
+  if (bad) {
+    if (tid == 0) atomicExch(flag, 1);
+    return;
+  }
+  for (int j = tid; j < m; j += 256) piv[j] = inv_sqrt(piv[j]);
+  __syncthreads();
+#pragma unroll
+  for (int u = 0; u < U; ++u)
+#pragma unroll
+    for (int v = 0; v < U; ++v) {
+      const int i = ty + 16 * u, k = tx + 16 * v;
+      if (i < m && k < m) {
+        const T z = (k < i ? e[u][v] : k == i ? T(1) : T(0)) * piv[i] * d[k];
+        if constexpr (sizeof(T) == 4) W[k + (size_t)i * m] = to_f64(z);
+        else W[k + (size_t)i * m] = z;
+      }
+    }
+}
+
+// FP32 attempts: as given, then with kChol32Retry, which always succeeds and
+// leaves a basis with condition number below about kChol32Retry^-1/2 for the
+// next pass to finish
+struct Shift32 {
+  float s;
+  __device__ float operator()(int a) const { return a == 0 ? s : fmaxf(s, kChol32Retry); }
+};
+// FP64 attempts: as given, then 2^-26 and 2^-12 of the unit diagonal
+struct Shift64 {
+  double s;
+  __device__ double operator()(int a) const { return a == 0 ? s : fmax(s, a == 1 ? 0x1.0p-26 : 0x1.0p-12); }
+};
+
+template <int U>
+constexpr size_t gram_chol_smem(int m) {
+  return ((size_t)m * m) * (sizeof(float2) + sizeof(float)) +
+         (size_t)(kSlab * (16 * U + 1) + 4 * 16 * U) * sizeof(float);
+}
+
+template <int U>
+__global__ void __launch_bounds__(256) __cluster_dims__(kOrthCluster, 1, 1)
+    k_gram_chol32(PSet Yin, int n, int m, float shift, PSet Wout, int *flag) {
+  extern __shared__ float2 gsh[];
+  constexpr int LD = 16 * U;
+  float2 *part = gsh;                                              // m x m, upper triangle
+  float *tot = reinterpret_cast<float *>(part + (size_t)m * m);    // m x m, upper triangle (rank 0)
+  float *slab = tot + (size_t)m * m;                               // kSlab x (LD + 1)
+  float *rowbuf = slab + kSlab * (LD + 1);                         // 2 x LD
+  float *d = rowbuf + 2 * LD, *piv = d + LD;
+  cg::cluster_group cluster = cg::this_cluster();
+  const int rank = (int)cluster.block_rank(), z = blockIdx.z;
+  const double *y = Yin.at(z);
+  const int rp = (n + kOrthCluster - 1) / kOrthCluster;
+  const int r0 = rank * rp, r1 = min(n, r0 + rp);
+  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
+  // a run of 16 rows is summed in FP32, the runs in two floats (TwoSum, Knuth)
+  float hi[U][U], lo[U][U];
+#pragma unroll
+  for (int u = 0; u < U; ++u)
+#pragma unroll
+    for (int v = 0; v < U; ++v) hi[u][v] = lo[u][v] = 0.0f;
+  auto two_sum = [](float &h, float &l, float x) {
+    const float s = h + x, bb = s - h;
+    l += (h - (s - bb)) + (x - bb);
+    h = s;
+  };
+  constexpr int PER = kSlab * LD / 256;                        // staged elements per thread
+  double nxt[PER];
+  auto fetch = [&](int rr) {
+#pragma unroll
+    for (int k = 0; k < PER; ++k) {
+      const int e = tid + 256 * k, ii = e & (kSlab - 1), col = e / kSlab, row = rr + ii;
+      nxt[k] = (row < r1 && col < m) ? y[(size_t)col * n + row] : 0.0;
+    }
+  };
+  fetch(r0);
+  for (int rr = r0; rr < r1; rr += kSlab) {
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < PER; ++k) {
+      const int e = tid + 256 * k, ii = e & (kSlab - 1), col = e / kSlab;
+      slab[ii * (LD + 1) + col] = to_f32(nxt[k]);
+    }
+    __syncthreads();
+    fetch(rr + kSlab);
+#pragma unroll 1
+    for (int half = 0; half < kSlab; half += 16) {
+      float acc[U][U];
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+#pragma unroll
+        for (int v = 0; v < U; ++v) acc[u][v] = 0.0f;
+#pragma unroll 4
+      for (int ii = half; ii < half + 16; ++ii) {
+        float av[U], bv[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          av[u] = slab[ii * (LD + 1) + ty + 16 * u];
+          bv[u] = slab[ii * (LD + 1) + tx + 16 * u];
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+#pragma unroll
+          for (int v = u; v < U; ++v) acc[u][v] = fmaf(av[u], bv[v], acc[u][v]);
+      }
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+#pragma unroll
+        for (int v = u; v < U; ++v) two_sum(hi[u][v], lo[u][v], acc[u][v]);
+    }
+  }
+#pragma unroll
+  for (int u = 0; u < U; ++u)
+#pragma unroll
+    for (int v = u; v < U; ++v) {
+      const int a = ty + 16 * u, b = tx + 16 * v;
+      if (a <= b && b < m) part[a * m + b] = make_float2(hi[u][v], lo[u][v]);
+    }
+  cluster.sync();
+  // every CTA sums its share of the entries over the cluster, into rank 0
+  float *dst = cluster.map_shared_rank(tot, 0);
+  for (int e = rank * 256 + tid; e < m * m; e += kOrthCluster * 256) {
+    if (e / m > e % m) continue;
+    float2 v[kOrthCluster];
+#pragma unroll
+    for (int q = 0; q < kOrthCluster; ++q) v[q] = *cluster.map_shared_rank(part + e, q);
+    float h = v[0].x, l = v[0].y;
+#pragma unroll
+    for (int q = 1; q < kOrthCluster; ++q) {
+      two_sum(h, l, v[q].x);
+      l += v[q].y;
+    }
+    dst[e] = h + l;
+  }
+  cluster.sync();                    // the partials have been read, the totals written
+  if (rank != 0) return;
+  chol_inverse<float, U>([&](int i, int k) { return tot[i * m + k]; }, Shift32{shift}, 2, m, Wout.at(z), flag,
+                         rowbuf, d, piv);
+}
+
+template <int U>
+__global__ void __launch_bounds__(256) k_chol32(PSet Cin, int m, float shift, PSet Wout, int *flag) {
+  __shared__ float rowbuf[2 * 16 * U], d[16 * U], piv[16 * U];
+  const double *C = Cin.at(blockIdx.z);
+  chol_inverse<float, U>([&](int i, int k) { return to_f32(C[(size_t)i * m + k]); }, Shift32{shift}, 2, m,
+                         Wout.at(blockIdx.z), flag, rowbuf, d, piv);
+}
+
+// the same in FP64; only_if (optional): run for problem z only if only_if.at(z)[2] != 0
+template <int U>
+__global__ void __launch_bounds__(256) k_chol64(PSet Cin, int m, double shift, PSet Wout, int *flag, PSet only_if) {
+  if (only_if.b0 && only_if.at(blockIdx.z)[2] == 0.0) return;
+  __shared__ double rowbuf[2 * 16 * U], d[16 * U], piv[16 * U];
+  const double *C = Cin.at(blockIdx.z);
+  chol_inverse<double, U>([&](int i, int k) { return C[(size_t)i * m + k]; }, Shift64{shift}, 3, m,
+                          Wout.at(blockIdx.z), flag, rowbuf, d, piv);
+}
+
+// Cp[c] = A[rows of chunk c]^T B[same rows] in FP64 (m x m, row-major), 256
+// threads as 16 x 16 with entries (ty + 16 u, tx + 16 v): every thread works
+// whatever m is.  sym: entries u <= v only (all of the upper triangle).
+template <int U>
+__global__ void __launch_bounds__(256) k_si_gram(PSet A, PSet B, PSet Cp, int n, int m, int sym, int rows) {
+  constexpr int LD = 16 * U;
+  __shared__ double As[16][LD + 1];
+  __shared__ double Bs[16][LD + 1];
+  const int z = blockIdx.z, c = blockIdx.x;
+  const double *a = A.at(z);
+  const double *b = B.at(z);
+  const int r0 = c * rows, r1 = min(n, r0 + rows);
+  const int ty = threadIdx.x >> 4, tx = threadIdx.x & 15;
+  double acc[U][U];
+#pragma unroll
+  for (int u = 0; u < U; ++u)
+#pragma unroll
+    for (int v = 0; v < U; ++v) acc[u][v] = 0.0;
+  for (int rr = r0; rr < r1; rr += 16) {
+    for (int e = threadIdx.x; e < 16 * LD; e += 256) {
+      const int j = e >> 4, ii = e & 15;
+      const int row = rr + ii;
+      const bool in = row < r1 && j < m;
+      As[ii][j] = in ? a[(size_t)j * n + row] : 0.0;
+      if (!sym) Bs[ii][j] = in ? b[(size_t)j * n + row] : 0.0;
+    }
+    __syncthreads();
+    const double(*Br)[LD + 1] = sym ? As : Bs;
+#pragma unroll 2
+    for (int ii = 0; ii < 16; ++ii) {
+      double av[U], bv[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        av[u] = As[ii][ty + 16 * u];
+        bv[u] = Br[ii][tx + 16 * u];
+      }
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+#pragma unroll
+        for (int v = 0; v < U; ++v)
+          if (!sym || u <= v) acc[u][v] = fma(av[u], bv[v], acc[u][v]);
+    }
+    __syncthreads();
+  }
+  double *out = Cp.at(z) + (size_t)c * m * m;
+#pragma unroll
+  for (int u = 0; u < U; ++u)
+#pragma unroll
+    for (int v = 0; v < U; ++v) {
+      const int ia = ty + 16 * u, ib = tx + 16 * v;
+      if (ia < m && ib < m && (!sym || ia <= ib)) out[ia * m + ib] = acc[u][v];
+    }
+}
+
+// C = sum over the chunks (fixed order), symmetrised.  A block takes 64 entries,
+// four threads to an entry, each with its own run of chunks: the sum is bound
+// by load latency, so many loads are kept in flight.
+__global__ void __launch_bounds__(256) k_si_gram_reduce(PSet Cp, PSet C, int nchunks, int m, int sym) {
+  __shared__ double sum[4][64];
+  const int z = blockIdx.z, l = threadIdx.x & 63, g = threadIdx.x >> 6;
+  const long long mm = (long long)m * m;
+  const int e = blockIdx.x * 64 + l, a = e / m, b = e % m;
+  const bool in = e < m * m && a <= b;
+  const int per = (nchunks + 3) / 4, c0 = g * per, c1 = min(nchunks, c0 + per);
+  double s = 0.0;
+  if (in) {
+    const double *src = Cp.at(z);
+    const long long o = (long long)a * m + b, ot = (long long)b * m + a;
+    double v[4] = {0.0, 0.0, 0.0, 0.0}, w[4] = {0.0, 0.0, 0.0, 0.0};
+    int c = c0;
+    for (; c + 4 <= c1; c += 4) {
+#pragma unroll
+      for (int q = 0; q < 4; ++q) v[q] += src[(c + q) * mm + o];
+      if (!sym)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) w[q] += src[(c + q) * mm + ot];
+    }
+    for (; c < c1; ++c) {
+      v[0] += src[c * mm + o];
+      if (!sym) w[0] += src[c * mm + ot];
+    }
+    s = (v[0] + v[1]) + (v[2] + v[3]);
+    if (!sym) s = 0.5 * (s + ((w[0] + w[1]) + (w[2] + w[3])));
+  }
+  sum[g][l] = s;
+  __syncthreads();
+  if (g == 0 && in) {
+    s = (sum[0][l] + sum[1][l]) + (sum[2][l] + sum[3][l]);
+    C.at(z)[a * m + b] = s;
+    C.at(z)[b * m + a] = s;
+  }
+}
+
+// Out = A W: a CTA takes RT rows and all columns; a warp takes 32 / RT
+// neighbouring columns at a time (lanes run along the rows), so that for a
+// triangular W its sum stops at their last nonzero, and the warps take the
+// column groups forwards and backwards in turn (equal shares).  FP64-bound:
+// RT is chosen so that the CTAs fill the SMs.
+template <int RT>
+__global__ void __launch_bounds__(256) k_si_rotate(PSet A, PSet W, PSet Out, int n, int m, int tri) {
+  extern __shared__ double rsh[];
+  double *As = rsh;                       // [column][RT]
+  double *Ws = rsh + (size_t)m * RT;      // [column][m + 1]
+  constexpr int CPW = 32 / RT;
+  const int z = blockIdx.z, i0 = blockIdx.x * RT;
+  const double *a = A.at(z), *w = W.at(z);
+  for (int e = threadIdx.x; e < m * RT; e += 256) {
+    const int j = e / RT, r = e % RT;
+    As[e] = i0 + r < n ? a[(size_t)j * n + i0 + r] : 0.0;
+  }
+  for (int e = threadIdx.x; e < m * m; e += 256) {
+    const int c = e / m, j = e % m;
+    if (!tri || j <= c) Ws[c * (m + 1) + j] = w[e];
+    else Ws[c * (m + 1) + j] = 0.0;
+  }
+  __syncthreads();
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, r = lane % RT, cl = lane / RT;
+  const int ng = (m + CPW - 1) / CPW;
+  for (int k = 0; k * 8 < ng; ++k) {
+    const int g = k * 8 + ((k & 1) ? 7 - warp : warp);
+    if (g >= ng) continue;
+    const int c = min(g * CPW + cl, m - 1);
+    const int jend = tri ? min(m, g * CPW + CPW) : m;
+    double acc = 0.0;
+#pragma unroll 8
+    for (int j = 0; j < jend; ++j) acc = fma(As[j * RT + r], Ws[c * (m + 1) + j], acc);
+    if (g * CPW + cl < m && i0 + r < n) Out.at(z)[(size_t)c * n + i0 + r] = acc;
+  }
+}
+
+int tile_of(int m) { return m <= 32 ? 2 : (m + 15) / 16; }   // 16-wide tiles per dimension, 2..6
+
+template <int U>
+cudaError_t launch_gram_chol(PSet Y, int n, int m, float shift, PSet W, int *flag, int P, cudaStream_t s) {
+  static bool done = false;
+  if (!done) {
+    cudaError_t e = cudaFuncSetAttribute(k_gram_chol32<U>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)gram_chol_smem<U>(16 * U));
+    if (e) return e;
+    done = true;
+  }
+  k_gram_chol32<U><<<dim3(kOrthCluster, 1, P), 256, gram_chol_smem<U>(m), s>>>(Y, n, m, shift, W, flag);
+  return cudaGetLastError();
+}
+
+template <int RT>
+cudaError_t launch_rotate(PSet A, PSet W, PSet Out, int n, int m, bool tri, int P, cudaStream_t s) {
+  static bool done = false;
+  if (!done) {
+    cudaError_t e = cudaFuncSetAttribute(k_si_rotate<RT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)(sizeof(double) * kSiMaxBlock * (RT + kSiMaxBlock + 1)));
+    if (e) return e;
+    done = true;
+  }
+  k_si_rotate<RT><<<dim3((n + RT - 1) / RT, 1, P), 256, sizeof(double) * m * (RT + m + 1), s>>>(A, W, Out, n, m,
+                                                                                               tri ? 1 : 0);
+  return cudaGetLastError();
+}
+
+}  // namespace
+
+cudaError_t gram_reduce(PSet part, PSet out, int chunks, int m, bool sym, int P, cudaStream_t s,
+                        long long *launches) {
+  k_si_gram_reduce<<<dim3((m * m + 63) / 64, 1, P), 256, 0, s>>>(part, out, chunks, m, sym ? 1 : 0);
+  *launches += 1;
+  return cudaGetLastError();
+}
+
+cudaError_t gram64(PSet A, PSet B, bool sym, int n, int m, PSet part, PSet out, int P, cudaStream_t s,
+                   long long *launches) {
+  // chunks of 16 rows until two CTAs per SM have one; longer ones beyond that
+  // keep the partials (m x m doubles per chunk) few
+  const int want = std::max(1, std::min(kGramChunks, (304 + P - 1) / P));
+  const int rows = std::max(16, ((n + want - 1) / want + 15) / 16 * 16);
+  const int chunks = (n + rows - 1) / rows;
+  if (chunks > kGramChunks || m > kSiMaxBlock) return cudaErrorInvalidValue;
+  const dim3 g(chunks, 1, P);
+  switch (tile_of(m)) {
+    case 2: k_si_gram<2><<<g, 256, 0, s>>>(A, B, part, n, m, sym, rows); break;
+    case 3: k_si_gram<3><<<g, 256, 0, s>>>(A, B, part, n, m, sym, rows); break;
+    case 4: k_si_gram<4><<<g, 256, 0, s>>>(A, B, part, n, m, sym, rows); break;
+    case 5: k_si_gram<5><<<g, 256, 0, s>>>(A, B, part, n, m, sym, rows); break;
+    default: k_si_gram<6><<<g, 256, 0, s>>>(A, B, part, n, m, sym, rows); break;
+  }
+  *launches += 1;
+  cudaError_t e = cudaGetLastError();
+  return e ? e : gram_reduce(part, out, chunks, m, sym, P, s, launches);
+}
+
+cudaError_t cholqr32_factor(PSet Y, int n, int m, float shift, PSet W, int *flag, int P, cudaStream_t s,
+                            long long *launches) {
+  *launches += 1;
+  switch (tile_of(m)) {
+    case 2: return launch_gram_chol<2>(Y, n, m, shift, W, flag, P, s);
+    case 3: return launch_gram_chol<3>(Y, n, m, shift, W, flag, P, s);
+    case 4: return launch_gram_chol<4>(Y, n, m, shift, W, flag, P, s);
+    case 5: return launch_gram_chol<5>(Y, n, m, shift, W, flag, P, s);
+    case 6: return launch_gram_chol<6>(Y, n, m, shift, W, flag, P, s);
+  }
+  return cudaErrorInvalidValue;
+}
+
+cudaError_t chol32(PSet C, int m, float shift, PSet W, int *flag, int P, cudaStream_t s, long long *launches) {
+  const dim3 g(1, 1, P);
+  switch (tile_of(m)) {
+    case 2: k_chol32<2><<<g, 256, 0, s>>>(C, m, shift, W, flag); break;
+    case 3: k_chol32<3><<<g, 256, 0, s>>>(C, m, shift, W, flag); break;
+    case 4: k_chol32<4><<<g, 256, 0, s>>>(C, m, shift, W, flag); break;
+    case 5: k_chol32<5><<<g, 256, 0, s>>>(C, m, shift, W, flag); break;
+    case 6: k_chol32<6><<<g, 256, 0, s>>>(C, m, shift, W, flag); break;
+    default: return cudaErrorInvalidValue;
+  }
+  *launches += 1;
+  return cudaGetLastError();
+}
+
+cudaError_t chol64(PSet C, int m, double shift, PSet W, int *flag, PSet only_if, int P, cudaStream_t s,
+                   long long *launches) {
+  const dim3 g(1, 1, P);
+  switch (tile_of(m)) {
+    case 2: k_chol64<2><<<g, 256, 0, s>>>(C, m, shift, W, flag, only_if); break;
+    case 3: k_chol64<3><<<g, 256, 0, s>>>(C, m, shift, W, flag, only_if); break;
+    case 4: k_chol64<4><<<g, 256, 0, s>>>(C, m, shift, W, flag, only_if); break;
+    case 5: k_chol64<5><<<g, 256, 0, s>>>(C, m, shift, W, flag, only_if); break;
+    case 6: k_chol64<6><<<g, 256, 0, s>>>(C, m, shift, W, flag, only_if); break;
+    default: return cudaErrorInvalidValue;
+  }
+  *launches += 1;
+  return cudaGetLastError();
+}
+
+cudaError_t rotate_basis(PSet A, PSet W, PSet Out, int n, int m, bool tri, int P, cudaStream_t s,
+                         long long *launches) {
+  if (m > kSiMaxBlock) return cudaErrorInvalidValue;
+  *launches += 1;
+  // the tallest tile that still gives most of the 152 SMs a CTA (each CTA reads
+  // all of W)
+  const long long rows = (long long)n * P;
+  if (rows >= 16 * 120) return launch_rotate<16>(A, W, Out, n, m, tri, P, s);
+  if (rows >= 8 * 120) return launch_rotate<8>(A, W, Out, n, m, tri, P, s);
+  return launch_rotate<4>(A, W, Out, n, m, tri, P, s);
+}
+
+}  // namespace hotrg

@@ -33,6 +33,7 @@
 #include <algorithm>
 #include <vector>
 
+#include "eig_orth.cuh"
 #include "eig_si.cuh"
 #include "eig_small.cuh"
 #include "tc_exact.cuh"
@@ -41,15 +42,10 @@ namespace hotrg {
 namespace {
 
 constexpr int kSplitMax = 8;     // split-K partials of G X
-constexpr int kChunkMax = 256;   // row chunks of the Gram reduction
-constexpr int kRowsPerChunk = 16;
-constexpr int kCholThreads = 256;
-constexpr int kCholPanel = 8;      // columns per panel of the blocked FP32 Cholesky
 constexpr double kXsSmallWork = 32.0 * 1024 * 1024;   // FP64 FMAs of one n x m x m product batch
 constexpr int kSiSmallBatch = 8;      // problems up to which the solve is latency bound
 constexpr double kSiFloorTol = 1e-10;  // residuals accepted once they stop decreasing
 constexpr int kSiSlowIters = 24;       // iterations after which a residual below the floor is accepted
-constexpr float kChol32Retry = 0x1.0p-12f;   // diagonal shift of a retried FP32 CholeskyQR pass
 
 
 // splitmix64 finaliser (Steele, Lea, Flood 2014) -> uniform double in [-1, 1)
@@ -59,34 +55,6 @@ __device__ inline double hash_uniform(unsigned long long x) {
   x = (x ^ (x >> 27)) * 0x94D049BB133111EBull;
   x ^= x >> 31;
   return static_cast<double>(x >> 11) * 0x1.0p-52 - 1.0;
-}
-
-// GB300 executes FP64 square roots and divisions as long dependent instruction
-// sequences; on the latency-bound paths below they are replaced by an FP32
-// estimate refined with FP64 fused multiply-adds (Newton's method), which is
-// accurate to FP64 rounding after two steps.
-
-// 2^-e scaling factor with e the binary exponent of x (exact, x > 0 finite)
-__device__ inline double pow2_inv_of(double x) {
-  const long long bits = __double_as_longlong(x);
-  const int e = (int)((bits >> 52) & 0x7FF) - 1023;
-  return __longlong_as_double((long long)(1023 - e) << 52);
-}
-
-// 1/sqrt(x) for x > 0 to FP64 accuracy: FP32 seed on a power-of-two scaled
-// argument, two Newton steps y <- y (3 - x y^2) / 2 in FP64.
-__device__ inline double rsqrt_fp64(double x) {
-  const double s = pow2_inv_of(x);                  // x s in [1, 2)
-  const double xs = x * s;
-  double y = (double)rsqrtf((float)xs);
-  y = y * fma(-0.5 * xs, y * y, 1.5);
-  y = y * fma(-0.5 * xs, y * y, 1.5);
-  // 1/sqrt(x) = (1/sqrt(x s)) sqrt(s); s is a power of two
-  const long long sb = __double_as_longlong(s);
-  const int es = (int)((sb >> 52) & 0x7FF) - 1023;
-  double root_s = (es & 1) ? 1.4142135623730951 : 1.0;
-  root_s *= __longlong_as_double((long long)(1023 + (es >> 1)) << 52);
-  return y * root_s;
 }
 
 __global__ void k_si_init(PSet X, PSet warm, int has_warm, int kw, int n, int m) {
@@ -207,397 +175,6 @@ __global__ void k_si_sum_split(PSet part, PSet out, int S, long long nm, PSet X,
   if (shift && blockIdx.x == 0 && threadIdx.x == 0) sig.at(z)[0] = sg;
 }
 
-// Cp[c] = A[rows of chunk c]^T B[same rows]   (m x m, row-major a*m + b)
-template <typename Acc>
-__global__ void __launch_bounds__(256) k_si_gram(PSet A, PSet B, PSet Cp, int n, int m, int sym) {
-  __shared__ Acc As[16][kSiMaxBlock + 1];
-  __shared__ Acc Bs[16][kSiMaxBlock + 1];
-  const int z = blockIdx.z, c = blockIdx.x;
-  const double *a = A.at(z);
-  const double *b = B.at(z);
-  const int r0 = c * kRowsPerChunk, r1 = min(n, r0 + kRowsPerChunk);
-  const int ta = threadIdx.x >> 4, tb = threadIdx.x & 15;
-  constexpr int U = kSiMaxBlock / 16;   // 6 x 6 outputs per thread
-  // A^T A is symmetric: only the tiles on or above the diagonal are computed
-  const bool skip = sym && (ta > tb);
-  Acc acc[U][U];
-#pragma unroll
-  for (int u = 0; u < U; ++u)
-#pragma unroll
-    for (int v = 0; v < U; ++v) acc[u][v] = Acc(0);
-  for (int rr = r0; rr < r1; rr += 16) {
-    for (int e = threadIdx.x; e < 16 * m; e += 256) {
-      const int j = e >> 4, ii = e & 15;
-      const int row = rr + ii;
-      As[ii][j] = (row < r1) ? (Acc)a[(size_t)j * n + row] : Acc(0);
-      Bs[ii][j] = (row < r1) ? (Acc)b[(size_t)j * n + row] : Acc(0);
-    }
-    __syncthreads();
-#pragma unroll 4
-    for (int ii = 0; ii < 16 && !skip; ++ii) {
-      Acc av[U], bv[U];
-#pragma unroll
-      for (int u = 0; u < U; ++u) av[u] = As[ii][ta * U + u];
-#pragma unroll
-      for (int v = 0; v < U; ++v) bv[v] = Bs[ii][tb * U + v];
-#pragma unroll
-      for (int u = 0; u < U; ++u)
-#pragma unroll
-        for (int v = 0; v < U; ++v) acc[u][v] = fma(av[u], bv[v], acc[u][v]);
-    }
-    __syncthreads();
-  }
-  double *out = Cp.at(z) + (size_t)c * m * m;
-#pragma unroll
-  for (int u = 0; u < U; ++u)
-#pragma unroll
-    for (int v = 0; v < U; ++v) {
-      const int ia = ta * U + u, ib = tb * U + v;
-      if (ia < m && ib < m && !skip) out[ia * m + ib] = (double)acc[u][v];
-    }
-}
-
-// C = sum over row chunks of the Gram partials (fixed order), symmetrised.
-// sym: the partials hold only the upper tiles (A^T A).  ns: write instead the
-// Newton-Schulz polish W = (3 I - C) / 2 (column-major, = row-major by symmetry).
-__global__ void k_si_gram_reduce(PSet Cp, PSet C, int nchunks, int m, int sym, int ns) {
-  const int z = blockIdx.z;
-  const long long mm = (long long)m * m;
-  constexpr int U = kSiMaxBlock / 16;
-  for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < m * m; e += gridDim.x * blockDim.x) {
-    const int a = e / m, b = e % m;
-    if (b < a) continue;
-    const double *src = Cp.at(z);
-    double v0 = 0.0, v1 = 0.0, v2 = 0.0, v3 = 0.0;
-    double sv;
-    if (sym) {
-      // (a, b) lives in tile (a / U, b / U); a tile below the diagonal was skipped.
-      // Eight independent partial sums keep eight loads in flight (the chunk
-      // sums are load-latency bound), combined in a fixed order.
-      const bool upper = (a / U) <= (b / U);
-      const long long off = upper ? (long long)a * m + b : (long long)b * m + a;
-      double v4 = 0.0, v5 = 0.0, v6 = 0.0, v7 = 0.0;
-      int c = 0;
-      for (; c + 8 <= nchunks; c += 8) {
-        v0 += src[c * mm + off];
-        v1 += src[(c + 1) * mm + off];
-        v2 += src[(c + 2) * mm + off];
-        v3 += src[(c + 3) * mm + off];
-        v4 += src[(c + 4) * mm + off];
-        v5 += src[(c + 5) * mm + off];
-        v6 += src[(c + 6) * mm + off];
-        v7 += src[(c + 7) * mm + off];
-      }
-      for (; c < nchunks; ++c) v0 += src[c * mm + off];
-      sv = ((v0 + v1) + (v2 + v3)) + ((v4 + v5) + (v6 + v7));
-    } else {
-      double w0 = 0.0, w1 = 0.0, w2 = 0.0, w3 = 0.0;
-      int c = 0;
-      for (; c + 4 <= nchunks; c += 4) {
-        v0 += src[c * mm + a * m + b];
-        w0 += src[c * mm + b * m + a];
-        v1 += src[(c + 1) * mm + a * m + b];
-        w1 += src[(c + 1) * mm + b * m + a];
-        v2 += src[(c + 2) * mm + a * m + b];
-        w2 += src[(c + 2) * mm + b * m + a];
-        v3 += src[(c + 3) * mm + a * m + b];
-        w3 += src[(c + 3) * mm + b * m + a];
-      }
-      for (; c < nchunks; ++c) {
-        v0 += src[c * mm + a * m + b];
-        w0 += src[c * mm + b * m + a];
-      }
-      sv = 0.5 * (((v0 + v1) + (v2 + v3)) + ((w0 + w1) + (w2 + w3)));
-    }
-    if (ns) sv = (a == b ? 1.5 : 0.0) - 0.5 * sv;
-    C.at(z)[a * m + b] = sv;
-    C.at(z)[b * m + a] = sv;
-  }
-}
-
-// Shifted, column-scaled Cholesky in FP32 of a block's Gram matrix C and the
-// rotation W = diag(d) R^-1 (column-major, stored in FP64) such that Y W is
-// orthonormal up to FP32 accuracy: C_hat = diag(d) C diag(d) + shift I = R^T R,
-// d_j = 1 / sqrt(C_jj).  Used for the iterations between Rayleigh-Ritz steps,
-// where an approximately orthonormal basis is all the power iteration needs.
-__global__ void __launch_bounds__(kCholThreads) k_si_chol32(PSet Cin, int m, float shift, PSet Wout,
-                                                            int *flag) {
-  extern __shared__ float shf[];
-  const int ld = m + 1;
-  float *C = shf;                 // m x ld: C_hat, updated in place (rows below the step)
-  float *R = shf + m * ld;        // m x ld: the factor R (upper triangle)
-  float *d = R + m * ld;          // m
-  const int z = blockIdx.z;
-  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-  for (int j = threadIdx.x; j < m; j += blockDim.x) {
-    const double cjj = Cin.at(z)[(size_t)j * m + j];
-    d[j] = (cjj > 0.0 && isfinite(cjj)) ? (float)rsqrt_fp64(cjj) : 1.0f;
-  }
-  __shared__ int bad;
-  // A nearly dependent set of columns breaks the unshifted factorisation; the
-  // second attempt adds kChol32Retry to the unit diagonal, which always
-  // succeeds and leaves a basis with condition number below about
-  // kChol32Retry^-1/2 for the next pass to finish.
-  for (int attempt = 0; attempt < 2; ++attempt) {
-    const float sh = attempt == 0 ? shift : fmaxf(shift, kChol32Retry);
-    __syncthreads();
-    // coalesced reads, four in flight per thread
-    for (int e0 = threadIdx.x; e0 < m * m; e0 += 4 * blockDim.x) {
-      double v[4];
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const int e = e0 + u * blockDim.x;
-        v[u] = e < m * m ? Cin.at(z)[e] : 0.0;
-      }
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const int e = e0 + u * blockDim.x;
-        if (e < m * m) {
-          const int a = e / m, b = e % m;
-          C[a * ld + b] = (float)v[u] * (d[a] * d[b]) + (a == b ? sh : 0.0f);
-        }
-      }
-    }
-    if (threadIdx.x == 0) bad = 0;
-    __syncthreads();
-    // Blocked right-looking factorisation, panels of kCholPanel columns and two
-    // barriers per panel: (a) the threads of the first three warps (the ones
-    // that need it: m <= 96) factor the panel's diagonal block U^T U = C_jj
-    // redundantly in registers (identical inputs, identical results); (b) the
-    // panel's rows of R right of the block, U^T R_j,rest = C_j,rest, by forward
-    // substitution, one column per thread; (c) after the barrier, a failed pivot
-    // (published by thread 0) stops every thread, else the trailing update
-    // C_rest -= R_j,rest^T R_j,rest.
-    const bool factor = threadIdx.x < 96;
-    for (int j0 = 0; j0 < m; j0 += kCholPanel) {
-      const int w = min(kCholPanel, m - j0);
-      float U[kCholPanel][kCholPanel];
-      float uinv[kCholPanel];
-      bool ok = factor;
-      if (factor) {
-        // the block's upper triangle into registers first (rows past w: identity),
-        // then the dependent chain; 1 / u_ii by rsqrtf (an FP32 factor is all
-        // the pass needs: the FP64 rotation preserves the span whatever W is)
-#pragma unroll
-        for (int i = 0; i < kCholPanel; ++i)
-#pragma unroll
-          for (int b = i; b < kCholPanel; ++b)
-            U[i][b] = (i < w && b < w) ? C[(j0 + i) * ld + j0 + b] : (i == b ? 1.0f : 0.0f);
-#pragma unroll
-        for (int i = 0; i < kCholPanel; ++i) {
-          float dd = U[i][i];
-#pragma unroll
-          for (int k = 0; k < i; ++k) dd = fmaf(-U[k][i], U[k][i], dd);
-          ok = ok && dd > 0.0f && isfinite(dd);
-          const float r = rsqrtf(dd);
-          uinv[i] = r;
-          U[i][i] = dd * r;
-#pragma unroll
-          for (int b = i + 1; b < kCholPanel; ++b) {
-            float v = U[i][b];
-#pragma unroll
-            for (int k = 0; k < i; ++k) v = fmaf(-U[k][i], U[k][b], v);
-            U[i][b] = v * r;
-          }
-        }
-      }
-      if (factor && !ok && threadIdx.x == 0) bad = 1;
-      if (ok && threadIdx.x == 0) {
-#pragma unroll
-        for (int i = 0; i < kCholPanel; ++i)
-#pragma unroll
-          for (int b = i; b < kCholPanel; ++b)
-            if (b < w) R[(j0 + i) * ld + j0 + b] = U[i][b];
-      }
-      for (int l = j0 + w + threadIdx.x; ok && l < m; l += blockDim.x) {
-        // a panel with columns past it is a full one (w = kCholPanel)
-        float cv[kCholPanel], y[kCholPanel];
-#pragma unroll
-        for (int i = 0; i < kCholPanel; ++i) cv[i] = C[(j0 + i) * ld + l];
-#pragma unroll
-        for (int i = 0; i < kCholPanel; ++i) {
-          float v = cv[i];
-#pragma unroll
-          for (int k = 0; k < i; ++k) v = fmaf(-U[k][i], y[k], v);
-          y[i] = v * uinv[i];
-        }
-#pragma unroll
-        for (int i = 0; i < kCholPanel; ++i) R[(j0 + i) * ld + l] = y[i];
-      }
-      __syncthreads();
-      if (bad) break;
-      // a panel with a trailing part is a full one (w = kCholPanel); the
-      // thread's column a of the panel rows stays in registers
-      for (int a = j0 + w + ty; a < m; a += 16) {
-        float ra[kCholPanel];
-#pragma unroll
-        for (int i = 0; i < kCholPanel; ++i) ra[i] = R[(j0 + i) * ld + a];
-        for (int b = a + tx; b < m; b += 16) {
-          float v = C[a * ld + b];
-#pragma unroll
-          for (int i = 0; i < kCholPanel; ++i) v = fmaf(-ra[i], R[(j0 + i) * ld + b], v);
-          C[a * ld + b] = v;
-        }
-      }
-      __syncthreads();
-    }
-    __syncthreads();
-    if (!bad) break;
-  }
-  if (bad) {
-    if (threadIdx.x == 0) atomicExch(flag, 1);
-    return;
-  }
-  // W = diag(d) R^-1.  Z = R^-1 (upper triangular, in the now free C storage)
-  // by 8 x 8 blocks: (1) every diagonal block Z_II = R_II^-1 by back
-  // substitution, one thread per column; (2) the off-diagonal blocks by
-  // distance d = J - I, all blocks of one distance at once:
-  // Z_IJ = -Z_II sum_{K = I+1..J} R_IK Z_KJ (the blocks Z_KJ, K > I, have
-  // smaller distances).  Two barriers per distance: the dependent chains are
-  // at most 8 d long instead of m.
-  constexpr int BS = kCholPanel;
-  const int nb = (m + BS - 1) / BS;
-  float *Z = C;
-  float *Tt = d + m;                      // nb BS x BS scratch blocks: the sums of one distance
-  for (int e = threadIdx.x; e < m * ld; e += blockDim.x) Z[e] = 0.0f;
-  __syncthreads();
-  for (int t = threadIdx.x; t < nb * BS; t += blockDim.x) {
-    const int I = t / BS, cl = t % BS, i0 = I * BS, w = min(BS, m - i0);
-    if (cl < w) {
-      const int c = i0 + cl;
-      float zc[BS];
-#pragma unroll
-      for (int ii = BS - 1; ii >= 0; --ii) {
-        float v = 0.0f;
-        if (ii <= cl) {
-          const int i = i0 + ii;
-          v = (ii == cl) ? 1.0f : 0.0f;
-#pragma unroll
-          for (int kk = ii + 1; kk < BS; ++kk)
-            if (kk <= cl) v = fmaf(-R[i * ld + i0 + kk], zc[kk], v);
-          v /= R[i * ld + i];
-        }
-        zc[ii] = v;
-      }
-#pragma unroll
-      for (int ii = 0; ii < BS; ++ii)
-        if (ii <= cl) Z[(i0 + ii) * ld + c] = zc[ii];
-    }
-  }
-  __syncthreads();
-  for (int dist = 1; dist < nb; ++dist) {
-    const int nblk = nb - dist;
-    // T_IJ[i][j] = sum_{k in blocks I+1..J} R[i][k] Z[k][j]
-    for (int t = threadIdx.x; t < nblk * BS * BS; t += blockDim.x) {
-      const int I = t / (BS * BS), ij = t % (BS * BS), ii = ij / BS, jj = ij % BS;
-      const int J = I + dist, i = I * BS + ii, j = J * BS + jj;
-      float v = 0.0f;
-      if (i < m && j < m) {
-        const int k1 = min(m, J * BS + BS);
-        for (int k = (I + 1) * BS; k < k1; ++k) v = fmaf(R[i * ld + k], Z[k * ld + j], v);
-      }
-      Tt[t] = v;
-    }
-    __syncthreads();
-    // Z_IJ = -Z_II T_IJ
-    for (int t = threadIdx.x; t < nblk * BS * BS; t += blockDim.x) {
-      const int I = t / (BS * BS), ij = t % (BS * BS), ii = ij / BS, jj = ij % BS;
-      const int J = I + dist, i0 = I * BS, i = i0 + ii, j = J * BS + jj;
-      if (i < m && j < m) {
-        float v = 0.0f;
-        for (int l = ii; l < BS && i0 + l < m; ++l) v = fmaf(Z[i * ld + i0 + l], Tt[I * BS * BS + l * BS + jj], v);
-        Z[i * ld + j] = -v;
-      }
-    }
-    __syncthreads();
-  }
-  double *W = Wout.at(z);
-  for (int e = threadIdx.x; e < m * m; e += blockDim.x) {
-    const int c = e / m, j = e % m;           // W[j + c m]
-    W[e] = (j <= c) ? (double)Z[j * ld + c] * (double)d[j] : 0.0;
-  }
-}
-
-// Shifted, column-scaled Cholesky of a block's Gram matrix C and the rotation
-// W = diag(d) R^-1 (column-major) such that Y W is orthonormal:
-//   C_hat = diag(d) C diag(d) + shift I = R^T R,  d_j = 1 / sqrt(C_jj).
-__global__ void __launch_bounds__(kCholThreads) k_si_chol(PSet Cin, int m, double shift, PSet Wout,
-                                                          int *flag, PSet only_if) {
-  // only_if (optional): run for problem z only if only_if.at(z)[2] != 0
-  if (only_if.b0 && only_if.at(blockIdx.z)[2] == 0.0) return;
-  extern __shared__ double sh[];
-  const int ld = m + 1;
-  double *C = sh;                 // m x ld, upper triangle -> R
-  double *Z = sh + m * ld;        // m x ld, R^-1 (upper)
-  double *d = Z + m * ld;         // m
-  double *rinv = d + m;           // m: 1 / R_jj
-  const int z = blockIdx.z;
-  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-  for (int e = threadIdx.x; e < m * m; e += blockDim.x) C[(e / m) * ld + e % m] = Cin.at(z)[e];
-  __syncthreads();
-  for (int j = threadIdx.x; j < m; j += blockDim.x) {
-    const double cjj = C[j * ld + j];
-    d[j] = (cjj > 0.0 && isfinite(cjj)) ? rsqrt_fp64(cjj) : 1.0;   // 1 / column norm
-  }
-  __syncthreads();
-  __shared__ int bad;
-  // Nearly dependent columns break the factorisation: later attempts add a
-  // larger diagonal shift (2^-26, then 2^-12 of the unit diagonal), which
-  // always succeeds and leaves a basis the next pass finishes.
-  for (int attempt = 0; attempt < 3; ++attempt) {
-  const double shv = attempt == 0 ? shift : fmax(shift, attempt == 1 ? 0x1.0p-26 : 0x1.0p-12);
-  __syncthreads();
-  for (int e = threadIdx.x; e < m * m; e += blockDim.x) C[(e / m) * ld + e % m] = Cin.at(z)[e];
-  __syncthreads();
-  for (int a = ty; a < m; a += 16)
-    for (int b = tx; b < m; b += 16) C[a * ld + b] = C[a * ld + b] * (d[a] * d[b]) + (a == b ? shv : 0.0);
-  if (threadIdx.x == 0) bad = 0;
-  __syncthreads();
-  // right-looking Cholesky on the upper triangle
-  for (int j = 0; j < m; ++j) {
-    const double piv = C[j * ld + j];
-    if (!(piv > 0.0) || !isfinite(piv)) {
-      if (threadIdx.x == 0) bad = 1;
-      break;
-    }
-    const double ri = rsqrt_fp64(piv);          // 1 / R_jj
-    __syncthreads();
-    for (int l = j + 1 + threadIdx.x; l < m; l += blockDim.x) C[j * ld + l] *= ri;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      C[j * ld + j] = piv * ri;
-      rinv[j] = ri;
-    }
-    for (int a = j + 1 + ty; a < m; a += 16)
-      for (int b = a + tx; b < m; b += 16) C[a * ld + b] -= C[j * ld + a] * C[j * ld + b];
-    __syncthreads();
-  }
-  __syncthreads();
-  if (!bad) break;
-  }
-  if (bad) {
-    if (threadIdx.x == 0) atomicExch(flag, 1);
-    return;
-  }
-  // R^-1 by right-looking back substitution: Z = I, then for i = m-1 .. 0 scale
-  // row i by 1/R_ii and eliminate it from the rows above (depth m, not m^2)
-  for (int a = ty; a < m; a += 16)
-    for (int b = tx; b < m; b += 16) Z[a * ld + b] = (a == b) ? 1.0 : 0.0;
-  __syncthreads();
-  for (int i = m - 1; i >= 0; --i) {
-    for (int b = i + threadIdx.x; b < m; b += blockDim.x) Z[i * ld + b] *= rinv[i];
-    __syncthreads();
-    for (int a = ty; a < i; a += 16)
-      for (int b = i + tx; b < m; b += 16) Z[a * ld + b] = fma(-C[a * ld + i], Z[i * ld + b], Z[a * ld + b]);
-    __syncthreads();
-  }
-  double *W = Wout.at(z);
-  for (int e = threadIdx.x; e < m * m; e += blockDim.x) {
-    const int c = e / m, j = e % m;           // W[j + c m]
-    W[e] = (j <= c) ? Z[j * ld + c] * d[j] : 0.0;
-  }
-}
-
 // flags.at(z)[2] = 1 if max |C_ij - delta_ij| > 1/4 (the Newton-Schulz
 // iteration for C^-1/2 from I is then not to be trusted), else 0.
 __global__ void k_rr_far_from_identity(PSet C, int m, PSet flags) {
@@ -656,52 +233,6 @@ __global__ void __launch_bounds__(256) k_rr_mm(PSet A, int ta, PSet B, double bs
   }
 }
 
-// Out = A . W  (A, Out n x m column-major; W m x m column-major: W[j + c m])
-// tri: W is upper triangular (W[j, c] = 0 for j > c), so j-blocks past the tile's last column are skipped
-__global__ void __launch_bounds__(256) k_si_rotate(PSet A, PSet W, PSet Out, int n, int m, int tri) {
-  __shared__ double As[32][33];
-  __shared__ double Ws[32][33];
-  const int z = blockIdx.z;
-  const double *a = A.at(z);
-  const double *w = W.at(z);
-  const int i0 = blockIdx.x * 32, c0 = blockIdx.y * 32;
-  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
-  double acc[4] = {0.0, 0.0, 0.0, 0.0};
-  const int jend = tri ? min(m, c0 + 32) : m;
-  // skip the zero-padded tail of the last j-chunk and the groups of 8 columns
-  // that start past m (uniform per block; their loads are zero-filled, so only
-  // work is skipped; at m = 72 the padding was 44 % of the FMAs)
-  const int ugroups = min(4, (m - c0 + 7) / 8);
-  for (int j0 = 0; j0 < jend; j0 += 32) {
-    for (int e = threadIdx.x; e < 32 * 32; e += 256) {
-      const int jj = e >> 5, ii = e & 31;
-      const int row = i0 + ii, j = j0 + jj;
-      As[jj][ii] = (row < n && j < m) ? a[(size_t)j * n + row] : 0.0;
-      const int cc = c0 + jj;          // Ws[j][c]: load W[j + cc m] along j
-      const int jw = j0 + ii;
-      Ws[ii][jj] = (jw < m && cc < m) ? w[(size_t)cc * m + jw] : 0.0;
-    }
-    __syncthreads();
-    const int jn = min(32, jend - j0);
-#pragma unroll 8
-    for (int jj = 0; jj < jn; ++jj) {
-      const double av = As[jj][tx];
-#pragma unroll
-      for (int u = 0; u < 4; ++u)
-        if (u < ugroups) acc[u] = fma(av, Ws[jj][ty + 8 * u], acc[u]);
-    }
-    __syncthreads();
-  }
-  const int i = i0 + tx;
-  if (i < n) {
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const int c = c0 + ty + 8 * u;
-      if (c < m) Out.at(z)[(size_t)c * n + i] = acc[u];
-    }
-  }
-}
-
 // res[i] = ||Y_i - theta_i X_i|| / |theta_0|, i < k
 // res_i = ||y_i - theta_i x_i|| / theta_0, or 0 for a pair whose unshifted
 // value lies below half the shift (2^-41 Tr G: inside the band where G's own
@@ -753,7 +284,7 @@ __global__ void k_si_copy(PSet src, PSet dst, long long nm) {
 // ---- host helpers ----
 
 struct Layout {
-  int S, NC, m;
+  int S, m;
   long long nm, mm;
   long long per;   // doubles per problem
   // slot offsets (doubles) inside a problem's workspace
@@ -772,14 +303,13 @@ Layout layout(int P, int n, int m) {
   const int tiles = (n + 63) / 64;
   L.S = std::max(1, std::min(kSplitMax, (2 * 152 + tiles * P - 1) / std::max(1, tiles * P)));
   while (L.S > 1 && (n + L.S - 1) / L.S < 64) --L.S;
-  L.NC = std::min(kChunkMax, (n + kRowsPerChunk - 1) / kRowsPerChunk);
   auto up = [](long long v) { return (v + 31) / 32 * 32; };   // 256-byte aligned slots
   long long o = 0;
   L.oY = o; o += up(L.nm);
   L.oZ = o; o += up(L.nm);
   L.oX = o; o += up(L.nm);
   L.oYp = o; o += up(kSplitMax * L.nm);
-  L.oCp = o; o += up(kChunkMax * L.mm);
+  L.oCp = o; o += up(kGramChunks * L.mm);
   L.oC = o; o += up(L.mm);
   L.oW = o; o += up(L.mm);
   L.oRes = o; o += up(m);
@@ -822,24 +352,6 @@ Bufs carve(double *work, int P, const Layout &L) {
 }
 
 bool same(const PSet &a, const PSet &b) { return a.b0 == b.b0 && a.b1 == b.b1 && a.stride == b.stride; }
-
-size_t chol_smem(int m) { return (size_t)(2 * m * (m + 1) + 2 * m) * sizeof(double); }
-size_t chol32_smem(int m) {
-  const int nb = (m + kCholPanel - 1) / kCholPanel;
-  return (size_t)(2 * m * (m + 1) + m + nb * kCholPanel * kCholPanel) * sizeof(float);
-}
-
-cudaError_t set_attrs() {
-  static bool done = false;
-  if (done) return cudaSuccess;
-  cudaError_t e;
-  const int big = 200 * 1024;
-  if ((e = cudaFuncSetAttribute(k_si_chol, cudaFuncAttributeMaxDynamicSharedMemorySize, big)) ||
-      (e = cudaFuncSetAttribute(k_si_chol32, cudaFuncAttributeMaxDynamicSharedMemorySize, big)))
-    return e;
-  done = true;
-  return cudaSuccess;
-}
 
 int grid_1d(long long count, int P) {
   long long b = (count + 255) / 256;
@@ -884,8 +396,7 @@ cudaError_t jacobi_full(const SiBatch &b, double *work, cudaStream_t s, long lon
 
 cudaError_t si_solve(const SiBatch &b, double *work, double tol, int max_iter, cudaStream_t s,
                      SiResult *res, long long *launches) {
-  cudaError_t e = set_attrs();
-  if (e) return e;
+  cudaError_t e;
   const int P = b.P, n = b.n, m = b.m, k = b.k;
   if (P < 1 || P > 65535 || m > kSiMaxBlock || m > n || k > m || (m & 1))
     return cudaErrorInvalidValue;
@@ -893,7 +404,6 @@ cudaError_t si_solve(const SiBatch &b, double *work, double tol, int max_iter, c
   Bufs B = carve(work, P, L);
   PSet X = B.X, Y = B.Y, Z = B.Z;
   const dim3 gz(1, 1, P);
-  const dim3 grot((n + 31) / 32, (m + 31) / 32, P);
   const int chunk = ((n + L.S - 1) / L.S + 15) / 16 * 16;
   const double shift = 11.0 * ((double)n * m + (double)m * (m + 1)) * 1.1102230246251565e-16;
   long long nl = 0;
@@ -974,12 +484,10 @@ cudaError_t si_solve(const SiBatch &b, double *work, double tol, int max_iter, c
       nl += 3;
       return cudaSuccess;
     }
-    k_si_rotate<<<grot, 256, 0, s>>>(src, W, dst, n, m, tri);
-    nl += 1;
-    return cudaGetLastError();
+    return rotate_basis(src, W, dst, n, m, tri != 0, P, s, &nl);
   };
-  // C = A^T B (m x m), symmetrised; ns: write the Newton-Schulz polish (3I - C)/2 instead
-  auto gram = [&](PSet A, PSet Bm, bool sym, bool f32, bool ns, PSet out) -> cudaError_t {
+  // C = A^T B (m x m), symmetrised
+  auto gram = [&](PSet A, PSet Bm, bool sym, PSet out) -> cudaError_t {
     if (xs_small) {
       const XsOperand a = xs_slot(L.oSa, L.oSasc, m, n);       // columns of A
       const XsOperand bb = xs_slot(L.oSb, L.oSbsc, m, n);      // columns of B
@@ -989,32 +497,26 @@ cudaError_t si_solve(const SiBatch &b, double *work, double tol, int max_iter, c
       if (!one && (r = xs_split(Bm, map1(n), map1(1), bb, s))) return r;
       if ((r = xs_gemm(a, one ? a : bb, m, m, n, B.Cp.b0, map1(m), map1(1), L.per, 1, 0, b.err, s)))
         return r;
-      k_si_gram_reduce<<<dim3(grid_1d(L.mm, P), 1, P), 256, 0, s>>>(B.Cp, out, 1, m, 0, ns);
-      nl += one ? 3 : 4;
-      return cudaGetLastError();
+      nl += one ? 2 : 3;
+      return gram_reduce(B.Cp, out, 1, m, false, P, s, &nl);
     }
-    if (f32)
-      k_si_gram<float><<<dim3(L.NC, 1, P), 256, 0, s>>>(A, Bm, B.Cp, n, m, sym);
-    else
-      k_si_gram<double><<<dim3(L.NC, 1, P), 256, 0, s>>>(A, Bm, B.Cp, n, m, sym);
-    k_si_gram_reduce<<<dim3(grid_1d(L.mm, P), 1, P), 256, 0, s>>>(B.Cp, out, L.NC, m, sym, ns);
-    nl += 2;
-    return cudaGetLastError();
+    return gram64(A, Bm, sym, n, m, B.Cp, out, P, s, &nl);
   };
   // one CholeskyQR pass with an FP32 factorisation: dst = src W
   auto cholqr32 = [&](PSet src, PSet dst, float sh) -> cudaError_t {
-    cudaError_t r = gram(src, src, true, true, false, B.C);
-    if (r) return r;
-    k_si_chol32<<<gz, kCholThreads, chol32_smem(m), s>>>(B.C, m, sh, B.W, B.flag);
-    nl += 1;
+    cudaError_t r;
+    if (xs_small) {
+      if ((r = gram(src, src, true, B.C)) || (r = chol32(B.C, m, sh, B.W, B.flag, P, s, &nl))) return r;
+    } else if ((r = cholqr32_factor(src, n, m, sh, B.W, B.flag, P, s, &nl))) {
+      return r;
+    }
     return rot(src, B.W, dst, 1);
   };
   // one CholeskyQR pass in FP64 (robust for any conditioning with the shift)
   auto cholqr64 = [&](PSet src, PSet dst, double sh) -> cudaError_t {
-    cudaError_t r = gram(src, src, true, false, false, B.C);
+    cudaError_t r = gram(src, src, true, B.C);
     if (r) return r;
-    k_si_chol<<<gz, kCholThreads, chol_smem(m), s>>>(B.C, m, sh, B.W, B.flag, PSet{nullptr, nullptr, 0});
-    nl += 1;
+    if ((r = chol64(B.C, m, sh, B.W, B.flag, PSet{nullptr, nullptr, 0}, P, s, &nl))) return r;
     return rot(src, B.W, dst, 1);
   };
   // dst = orth(src) through tmp (src is overwritten).  After the first
@@ -1106,8 +608,8 @@ cudaError_t si_solve(const SiBatch &b, double *work, double tol, int max_iter, c
       PSet Wn = slot(0), Tn = slot(1);
       const PSet Ck = slot(2), Rr = slot(3);
       const dim3 gmm((m + 7) / 8, (m + 7) / 8, P), g1(grid_1d(L.mm, P), 1, P);
-      if ((e = gram(X, X, true, false, false, B.W))) return e;   // C0 (B.W until small_eig)
-      if ((e = gram(X, Y, false, false, false, B.C))) return e;  // X^T Y
+      if ((e = gram(X, X, true, B.W))) return e;   // C0 (B.W until small_eig)
+      if ((e = gram(X, Y, false, B.C))) return e;  // X^T Y
       k_rr_axpi<<<g1, 256, 0, s>>>(B.W, -0.5, 1.5, Wn, m);       // W1 = (3I - C0) / 2
       nl += 1;
       for (int ns = 0; ns < 3; ++ns) {                              // W <- W (3I - W^T C0 W) / 2
@@ -1121,8 +623,8 @@ cudaError_t si_solve(const SiBatch &b, double *work, double tol, int max_iter, c
       // check), W comes instead from a shifted FP64 Cholesky of C0 (X W is
       // then orthonormal for any conditioning the shift allows)
       k_rr_far_from_identity<<<gz, 256, 0, s>>>(B.W, m, B.sig);
-      k_si_chol<<<gz, kCholThreads, chol_smem(m), s>>>(B.W, m, shift, Wn, B.flag, B.sig);
-      nl += 2;
+      nl += 1;
+      if ((e = chol64(B.W, m, shift, Wn, B.flag, B.sig, P, s, &nl))) return e;
       k_rr_mm<<<gmm, 256, 0, s>>>(B.C, 0, Wn, 1.0, 0.0, Tn, m);     // (X^T Y) W
       k_rr_mm<<<gmm, 256, 0, s>>>(Wn, 1, Tn, 1.0, 0.0, Ck, m);      // H = W^T X^T Y W
       nl += 2;

@@ -29,18 +29,12 @@
 // most a few rotations for stage 4.
 #include <math.h>
 
-#include "eig_small.cuh"
+#include "eig_orth.cuh"
 #include "eig_si.cuh"
+#include "eig_small.cuh"
 
 namespace hotrg {
 namespace {
-
-// 2^-e scaling factor with e the binary exponent of x (exact, x > 0 finite)
-__device__ inline double pow2_inv_of(double x) {
-  const long long bits = __double_as_longlong(x);
-  const int e = (int)((bits >> 52) & 0x7FF) - 1023;
-  return __longlong_as_double((long long)(1023 - e) << 52);
-}
 
 // |h| truncated to FP32 with integer arithmetic (FP64 conversions run at the
 // FP64 rate); values below the FP32 range give 0
