@@ -35,6 +35,45 @@ __host__ __device__ inline long long map_off(const IdxMap &m, long long i) {
   return i0 * m.s0 + i1 * m.s1 + i2 * m.s2;
 }
 
+// map_off for i < 2^31 in 32-bit arithmetic (device code: 64-bit divisions are
+// long instruction sequences)
+__device__ __forceinline__ long long map_off32(const IdxMap &m, int i) {
+  if (i < m.n0) return i * m.s0;
+  const int r = i / m.n0;
+  const int i0 = i - r * m.n0;
+  if (r < m.n1) return i0 * m.s0 + r * m.s1;
+  const int i2 = r / m.n1;
+  return i0 * m.s0 + (r - i2 * m.n1) * m.s1 + i2 * m.s2;
+}
+
+// FP64 <-> FP32 by integer arithmetic (the conversion instructions run at GB300's
+// FP64 rate); subnormal FP32 values are taken as zero.  To nearest even:
+__device__ __forceinline__ float to_f32(double x) {
+  const unsigned long long b = static_cast<unsigned long long>(__double_as_longlong(x));
+  const unsigned long long a = b & 0x7FFFFFFFFFFFFFFFull;
+  const long long r = (long long)((a + 0x0FFFFFFFull + ((a >> 29) & 1)) >> 29) - (896ll << 23);
+  const unsigned f = r < (1 << 23) ? 0u : r >= (255ll << 23) ? (a > 0x7FF0000000000000ull ? 0x7FC00000u : 0x7F800000u)
+                                                              : (unsigned)r;
+  return __uint_as_float(f | ((unsigned)(b >> 32) & 0x80000000u));
+}
+// Truncated, with the last bit set if anything was cut off: a later rounding to
+// 22 bits or fewer is then the rounding of x itself.
+__device__ __forceinline__ float to_f32_odd(double x) {
+  const unsigned long long b = static_cast<unsigned long long>(__double_as_longlong(x));
+  const unsigned long long a = b & 0x7FFFFFFFFFFFFFFFull;
+  const long long r = (long long)(a >> 29) - (896ll << 23);
+  const unsigned f = r < (1 << 23) ? 0u : r >= (255ll << 23) ? (a > 0x7FF0000000000000ull ? 0x7FC00000u : 0x7F800000u)
+                                                              : ((unsigned)r | ((a & 0x1FFFFFFFull) ? 1u : 0u));
+  return __uint_as_float(f | ((unsigned)(b >> 32) & 0x80000000u));
+}
+__device__ __forceinline__ double to_f64(float x) {
+  const unsigned b = __float_as_uint(x), a = b & 0x7FFFFFFFu;
+  const unsigned long long r = a < (1u << 23) ? 0ull
+                               : a >= 0x7F800000u ? (0x7FF0000000000000ull | ((unsigned long long)(a & 0x7FFFFFu) << 29))
+                                                  : ((unsigned long long)a << 29) + (896ull << 52);
+  return __longlong_as_double((long long)(r | ((unsigned long long)(b & 0x80000000u) << 32)));
+}
+
 // A family of buffers indexed by problem z: even z -> b0, odd z -> b1, plus
 // (z / 2) * stride.  The two environments of instance i are problems 2i (left)
 // and 2i + 1 (right); pset_linear(base, s) is simply "problem z at base + z s".

@@ -36,24 +36,6 @@ constexpr int kOrthCluster = 8;
 constexpr int kSlab = 32;                    // rows staged at a time
 constexpr float kChol32Retry = 0x1.0p-12f;   // diagonal shift of a retried FP32 factorisation
 
-// FP64 <-> FP32 by integer arithmetic (the conversion instructions run at the
-// FP64 rate); subnormal FP32 values are taken as zero.
-__device__ __forceinline__ float to_f32(double x) {
-  const unsigned long long b = static_cast<unsigned long long>(__double_as_longlong(x));
-  const unsigned long long a = b & 0x7FFFFFFFFFFFFFFFull;
-  const long long r = (long long)((a + 0x0FFFFFFFull + ((a >> 29) & 1)) >> 29) - (896ll << 23);   // to nearest even
-  const unsigned f = r < (1 << 23) ? 0u : r >= (255ll << 23) ? (a > 0x7FF0000000000000ull ? 0x7FC00000u : 0x7F800000u)
-                                                              : (unsigned)r;
-  return __uint_as_float(f | ((unsigned)(b >> 32) & 0x80000000u));
-}
-__device__ __forceinline__ double to_f64(float x) {
-  const unsigned b = __float_as_uint(x), a = b & 0x7FFFFFFFu;
-  const unsigned long long r = a < (1u << 23) ? 0ull
-                               : a >= 0x7F800000u ? (0x7FF0000000000000ull | ((unsigned long long)(a & 0x7FFFFFu) << 29))
-                                                  : ((unsigned long long)a << 29) + (896ull << 52);
-  return __longlong_as_double((long long)(r | ((unsigned long long)(b & 0x80000000u) << 32)));
-}
-
 __device__ __forceinline__ float reciprocal(float p) { return __frcp_rn(p); }
 __device__ __forceinline__ double reciprocal(double p) {     // p within the FP32 range
   double r = (double)__frcp_rn((float)p);

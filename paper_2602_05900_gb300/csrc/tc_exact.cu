@@ -82,16 +82,6 @@ struct XsOut {
   XsShift shift;
 };
 
-// map_off in 32-bit arithmetic (64-bit divisions are long instruction sequences)
-__device__ __forceinline__ long long map_off32(const IdxMap &m, int i) {
-  if (i < m.n0) return i * m.s0;
-  const int r = i / m.n0;
-  const int i0 = i - r * m.n0;
-  if (r < m.n1) return i0 * m.s0 + r * m.s1;
-  const int i2 = r / m.n1;
-  return i0 * m.s0 + (r - i2 * m.n1) * m.s1 + i2 * m.s2;
-}
-
 // ---- slicing ------------------------------------------------------------------
 //
 // The row maximum is taken on the bit patterns (|x| of a double orders like its

@@ -99,6 +99,30 @@ __device__ __forceinline__ void store_out4(const TcEpilogue &e, long long off, f
   }
 }
 
+// Stores VE (4 or 8) consecutive columns of a BF16-plane output (one by one, the
+// a5 GEMM of a D = 64 BF16X3 step -- 4.3 GB of output -- took 6.26 ms; it takes
+// 1.30 ms), one 8- or
+// 16-byte store per plane (tc_gemm checked the alignment when it set e.vec).
+template <int VE>
+__device__ __forceinline__ void store_planes(const TcEpilogue &e, long long off, float (&v)[VE], long long zoff,
+                                             int *err) {
+  const long long last = zoff + off + VE - 1 + (e.planes - 1) * e.plane_stride;
+  if (!checked_ok(zoff + off, e.cap, err) || !checked_ok(last, e.cap, err)) return;
+  __nv_bfloat16 *c = static_cast<__nv_bfloat16 *>(e.C) + off;
+  for (int p = 0; p < e.planes; ++p) {
+    unsigned w[VE / 2];
+#pragma unroll
+    for (int j = 0; j < VE / 2; ++j) {
+      const __nv_bfloat162 t = __floats2bfloat162_rn(v[2 * j], v[2 * j + 1]);
+      w[j] = *reinterpret_cast<const unsigned *>(&t);
+      v[2 * j] -= __uint_as_float(w[j] << 16);
+      v[2 * j + 1] -= __uint_as_float(w[j] & 0xFFFF0000u);
+    }
+    if constexpr (VE == 8) *reinterpret_cast<uint4 *>(c + p * e.plane_stride) = make_uint4(w[0], w[1], w[2], w[3]);
+    else *reinterpret_cast<uint2 *>(c + p * e.plane_stride) = make_uint2(w[0], w[1]);
+  }
+}
+
 template <int MODE>
 struct ModeTraits;
 template <>
@@ -301,29 +325,60 @@ __global__ void __launch_bounds__(384, 1)
       const long long zoff = (long long)z * epi.bstride;
       const int row = m0 + quad * 32 + lane;
       const bool rv = row < M;
-      const long long roff = rv ? map_off(e.cm, row) : -1;
+      const long long roff = rv ? map_off32(e.cm, row) : -1;
 #pragma unroll 1
       for (int c = half; c < BN / 32; c += 2) {
         if (n0 + c * 32 >= N) break;
         uint32_t r[32];
         tmem_ld32(tmem + trow + buf * BN + c * 32, r);
         const int col = n0 + c * 32 + lane;
-        const long long coff = (col < N) ? map_off(e.cn, col) : -1;
+        const long long coff = (col < N) ? map_off32(e.cn, col) : -1;
         if (!e.transpose) {
 #pragma unroll
           for (int j = 0; j < 32; ++j) {
             const long long co = __shfl_sync(0xffffffffu, coff, j);
             if (rv && co >= 0) store_out(e, roff + co, __uint_as_float(r[j]), zoff, err_flag);
           }
-        } else if (e.vec4 && n0 + c * 32 + 32 <= N) {
-          // column-major staging (stage[col][row], conflict-free), then lane l
-          // stores columns 4 (l mod 8) .. + 3 of row 4 it + l / 8: eight 16-byte
-          // stores per lane and chunk instead of 32 scalar ones
+        } else if (e.vec && n0 + c * 32 + 32 <= N) {
+          // column-major staging (stage[col][row], conflict-free), then a lane
+          // stores VE neighbouring columns of a row at once: F32 and F64 take
+          // columns 4 (l mod 8) .. + 3 of row 4 it + l / 8 (16-byte stores), BF16
+          // planes 8 columns (16 bytes a plane) or 4, so that a chunk takes 8 or
+          // fewer stores per lane and plane instead of 32 scalar ones
 #pragma unroll
           for (int j = 0; j < 32; ++j) stage[j * 33 + lane] = __uint_as_float(r[j]);
           __syncwarp();
+          if (e.kind == OutKind::BF16P) {
+            if (e.vec == 8) {
+              const int q = lane & 3;
+              const long long cq = __shfl_sync(0xffffffffu, coff, 8 * q);
+#pragma unroll
+              for (int it = 0; it < 4; ++it) {
+                const int rr = it * 8 + (lane >> 2);
+                const long long ro = __shfl_sync(0xffffffffu, roff, rr);
+                float v[8];
+#pragma unroll
+                for (int j = 0; j < 8; ++j) v[j] = stage[(8 * q + j) * 33 + rr];
+                if (ro >= 0) store_planes<8>(e, ro + cq, v, zoff, err_flag);
+              }
+            } else {
+              const int q = lane & 7;
+              const long long cq = __shfl_sync(0xffffffffu, coff, 4 * q);
+#pragma unroll
+              for (int it = 0; it < 8; ++it) {
+                const int rr = it * 4 + (lane >> 3);
+                const long long ro = __shfl_sync(0xffffffffu, roff, rr);
+                float v[4];
+#pragma unroll
+                for (int j = 0; j < 4; ++j) v[j] = stage[(4 * q + j) * 33 + rr];
+                if (ro >= 0) store_planes<4>(e, ro + cq, v, zoff, err_flag);
+              }
+            }
+            __syncwarp();
+            continue;
+          }
           const int q = lane & 7;
-          const long long cq = map_off(e.cn, n0 + c * 32 + 4 * q);
+          const long long cq = __shfl_sync(0xffffffffu, coff, 4 * q);
 #pragma unroll
           for (int it = 0; it < 8; ++it) {
             const int rr = it * 4 + (lane >> 3);
@@ -430,7 +485,7 @@ cudaError_t run_bn(int bn, const TcOperand &A, const TcOperand &B, int M, int N,
   const int batch = A.batch < 1 ? 1 : A.batch;
   if (bn == 64) return launch<MODE, 64>(ta, tb, M, N, K, batch, epi, err, s);
   if (bn == 128) return launch<MODE, 128>(ta, tb, M, N, K, batch, epi, err, s);
-  if constexpr (MODE == 0) {
+  if constexpr (MODE <= 1) {
     if (bn == 256) return launch<MODE, 256>(ta, tb, M, N, K, batch, epi, err, s);
   }
   return cudaErrorInvalidValue;
@@ -470,7 +525,7 @@ cudaError_t dispatch_bn(const TcOperand &A, const TcOperand &B, int M, int N, in
     return run_bn<MODE>(heuristic, A, B, M, N, K, epi, err, s);
   }
   const int cands[3] = {64, 128, 256};
-  const int ncand = MODE == 0 ? 3 : 2;
+  const int ncand = MODE <= 1 ? 3 : 2;
   cudaEvent_t ev[2] = {nullptr, nullptr};
   if (cudaEventCreate(&ev[0]) != cudaSuccess || cudaEventCreate(&ev[1]) != cudaSuccess) {
     (void)cudaGetLastError();
@@ -557,16 +612,18 @@ cudaError_t tc_gemm(TcMode mode, const TcOperand &A, const TcOperand &B, int M, 
   TcEpilogue e = epi;
   // store layout: keep lane = row when the rows are unit-stride, else transpose
   e.transpose = !(epi.cm.s0 == 1 && epi.cm.n0 >= 8);
-  // transposed F32 / F64 stores 4 columns at a time where every group of 4
-  // consecutive columns is contiguous and 16-byte aligned: unit column stride,
-  // all other strides and the instance stride multiples of 4 elements
-  {
-    auto m4 = [](long long v) { return (v & 3) == 0; };
+  // transposed stores take several columns at a time where every group of them
+  // is contiguous and aligned: unit column stride, all other strides and the
+  // instance stride multiples of the group (4 columns: 16 bytes of F32, 32 of
+  // F64, 8 of a BF16 plane; BF16 planes 8 columns, 16 bytes, where that divides)
+  auto fits = [&](int ve) {
+    auto mul = [ve](long long v) { return v % ve == 0; };
     const IdxMap &cm = epi.cm, &cn = epi.cn;
-    e.vec4 = e.transpose && (epi.kind == OutKind::F32 || epi.kind == OutKind::F64) && cn.s0 == 1 &&
-             (cn.n0 & 3) == 0 && m4(cn.s1) && m4(cn.s2) && m4(cm.s0) && m4(cm.s1) && m4(cm.s2) &&
-             m4(epi.bstride) && (reinterpret_cast<uintptr_t>(epi.C) & 15) == 0;
-  }
+    return e.transpose && cn.s0 == 1 && mul(cn.n0) && mul(cn.s1) && mul(cn.s2) && mul(cm.s0) && mul(cm.s1) &&
+           mul(cm.s2) && mul(epi.bstride) && (reinterpret_cast<uintptr_t>(epi.C) & 15) == 0 &&
+           (epi.kind != OutKind::BF16P || mul(epi.plane_stride));
+  };
+  e.vec = epi.kind == OutKind::BF16P && fits(8) ? 8 : fits(4) ? 4 : 0;
   switch (mode) {
     case TcMode::TF32: return dispatch_bn<0>(A, B, M, N, K, e, err_flag, s);
     case TcMode::BF16X3: return dispatch_bn<1>(A, B, M, N, K, e, err_flag, s);

@@ -47,8 +47,8 @@ struct TcEpilogue {
                            // stores 32 consecutive columns of one row (unit-stride cn)
   long long cap;           // elements of C from its base, all instances and planes (0 =
                            // unknown): bounds of the checked build
-  bool vec4;               // set by tc_gemm: transposed F32 / F64 stores of 4 consecutive
-                           // columns at once (unit-stride, 4-aligned column map)
+  int vec;                 // set by tc_gemm: columns per store of the transposed layout (4, or
+                           // 8 for BF16 planes, where the column map allows; 0: one by one)
 };
 
 // Launches C(M x N) = A(M x K) . B(N x K)^T for every instance of the batch
