@@ -21,13 +21,15 @@
 //
 // Measured against the FP64 two-sided Jacobi on an 8-CTA cluster that this
 // replaced (its rounds cost 4 us, half of it FP64 arithmetic): an iTEBD update
-// of one chain at n = 60 took 3.63 ms and takes 0.74 ms, of 64 chains at n = 32
-// 3.39 ms and 0.51 ms, a D = 8 FP64 step (n = 64) 2.88 ms and 0.76 ms.
+// of one chain at n = 60 took 3.63 ms and takes 0.62 ms, of 64 chains at n = 32
+// 3.39 ms and 0.45 ms, a D = 8 FP64 step (n = 64) 2.88 ms and 0.65 ms.
 //
 // A CPU model of the four stages (dense, graded, rank-deficient and degenerate
 // matrices, m = 16 to 96) leaves residuals and orthonormality at 1e-15 and at
 // most a few rotations for stage 4.
 #include <math.h>
+
+#include <type_traits>
 
 #include "eig_orth.cuh"
 #include "eig_si.cuh"
@@ -84,46 +86,71 @@ __device__ inline void jacobi_angle(double hpp, double hqq, double hpq, double &
 constexpr int kJ32MaxSweeps = 30;
 constexpr float kJ32Rel2 = 1e-12f;   // a pair is rotated while h_pq^2 > this h_pp h_qq
 
-// Row pitch: congruent to h = m / 2 modulo 32, so that a warp whose lanes run
-// over the slots of one row and on into the next one touches consecutive banks.
-__host__ __device__ inline int j32_ld(int m) {
-  const int h = m / 2;
-  return m + (((h - m) % 32) + 32) % 32;
-}
-size_t j32_smem(int m) {
-  return (size_t)4 * m * j32_ld(m) * sizeof(float) + (size_t)2 * (m / 2) * sizeof(float2);
+// Layout of the kernel for up to HM pairs (h = m / 2 <= HM): tops of the slots at
+// rows and columns 0..h-1, bottoms HM further on, so that the four entries of a
+// block and the two buffers are compile-time offsets apart.  A warp takes 4 x 8
+// blocks, and the row pitch is 8 or 24 modulo the 32 banks: its four rows of
+// eight neighbours fall on different banks.  The angles of a whole sweep are
+// kept, of two sweeps in turn.
+template <int HM, int SPL>
+struct J32Cfg {
+  static constexpr int kLd = 2 * HM + 8;                     // row pitch
+  static constexpr int kA = 2 * HM * kLd;                    // floats of one matrix buffer
+  static constexpr int kRound = 16 * SPL;                    // slots of a round's angles (float2: c, s), >= HM
+  static constexpr int kSweep = (2 * HM - 1) * kRound;       // float2 of one sweep's angles
+  static constexpr size_t kSmem = 2 * kA * sizeof(float) + (2 * kSweep + kRound) * sizeof(float2);
+  static_assert(kSmem <= 200 * 1024, "shared memory");
+  static_assert(kLd % 32 == 8 || kLd % 32 == 24, "bank layout");
+};
+
+__device__ __forceinline__ float rsqrt_approx(float x) {
+  float r;
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
 }
 
 // FP32 cyclic Jacobi on the symmetric m x m matrix of problem z, all disjoint
 // pairs of a round at once (Eq. 6 per 2 x 2 block), Brent and Luk's systolic
-// order (Fig. 3): slot I holds the positions I (top) and h + I (bottom), a
-// round rotates every slot's pair and then moves the tops one slot up and the
-// bottoms one slot down (slot 0's top stays), so every pair meets once in the
-// m - 1 rounds of a sweep and a sweep ends with every index back in its place.
-// The permutation is the same in every round: a thread reads and writes the
-// same addresses all the time (two buffers in turn), with no index arithmetic.
+// order (Fig. 3): slot I holds a top and a bottom index, a round rotates every
+// slot's pair and then moves the tops one slot up and the bottoms one slot down
+// (slot 0's top stays), so every pair meets once in the m - 1 rounds of a sweep
+// and a sweep ends with every index back in its place.  The permutation is the
+// same in every round: a thread reads and writes the same addresses all the
+// time (two buffers in turn), with no index arithmetic.
 //
-// What bounds it: the chain angle -> barrier -> rotate -> barrier of a round,
-// and shared-memory wavefronts.  The matrix is kept as the blocks I <= J only,
-// and the rotation of V by a round's angles runs in the threads that wait for
-// the next round's angles.  IV, IA: blocks of V and of the matrix per thread.
+// What bounds it: the chain from one round's angles to the next, then
+// shared-memory wavefronts and issue slots.  So a round has one barrier: warps of
+// their own compute the next round's angles from this round's matrix and angles
+// (the two diagonal entries and the coupling that meet in a slot, rotated on the
+// spot) while the others rotate the matrix.  The angles use the approximate
+// reciprocal and square roots (an angle needs no more; c and s = t c keep
+// c^2 + s^2 = 1 to FP32 rounding).  The matrix is kept as the blocks I <= J only,
+// and V is off the chain: its rows sit in the registers of more warps (16 lanes a
+// row, SPL slots a lane; a round is a rotation and one shuffle each way), which
+// replay the angles of one sweep while the others run the next, and meet them
+// once per sweep.  A round at m = 60 took 0.55 us with two barriers and V in
+// shared memory, 0.42 us with V in registers, and takes 0.35 us (0.08 us of it the
+// barrier and the loop; the angles alone end at 0.22, the matrix alone at 0.28).  RPG: rows per
+// group of 16 lanes, IA: blocks of the matrix per thread.
 //
 // A pair is rotated while |h_pq| exceeds both floor_abs (of the largest
 // diagonal entry, scaled to [1, 2)) and 1e-6 of sqrt|h_pp h_qq|: entries
 // between two small diagonal entries are resolved to FP32 relative accuracy.
 // Vout (FP64, column-major) receives the accumulated rotation, its columns in
 // the order of the final diagonal (unsorted); *sweeps the largest sweep count.
-template <int IV, int IA>
+template <int HM, int SPL, int RPG, int IA>
 __global__ void __launch_bounds__(1024, 1)
-    k_rr_jacobi32(PSet Hin, int m, float floor_abs, PSet Vout, int *sweeps) {
-  extern __shared__ float jsh[];
-  const int h = m / 2, ld = j32_ld(m), sz = m * ld;
-  float *Abuf = jsh, *Vbuf = jsh + 2 * sz;
-  float2 *cs = reinterpret_cast<float2 *>(jsh + 4 * sz);     // [round parity][slot]
+    k_rr_jacobi32(PSet Hin, int m, float floor_abs, int nang, int nA, PSet Vout, int *sweeps) {
+  using C = J32Cfg<HM, SPL>;
+  extern __shared__ __align__(16) float jsh[];
+  float *Abuf = jsh;
+  float2 *ring = reinterpret_cast<float2 *>(jsh + 2 * C::kA);   // [sweep parity][round][slot]
+  float2 *spare = ring + 2 * C::kSweep;                         // angles nobody uses
   __shared__ double s_scale;
-  __shared__ int s_rot;
+  __shared__ int s_rot[2];                                   // by sweep parity
+  const int h = m / 2;
+  constexpr int ld = C::kLd;
   const int z = blockIdx.z, tid = threadIdx.x, T = blockDim.x;
-  const int nang = (h + 31) / 32 * 32;                       // threads that compute angles
   const double *H = Hin.at(z);
   if (tid < 32) {
     double v = 0.0;
@@ -131,154 +158,226 @@ __global__ void __launch_bounds__(1024, 1)
     for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(0xffffffffu, v, o));
     if (tid == 0) s_scale = (v > 0.0 && isfinite(v)) ? pow2_inv_of(v) : 1.0;
   }
+  for (int e = tid; e < 2 * C::kSweep; e += T) ring[e] = make_float2(1.0f, 0.0f);   // slots past h stay so
   __syncthreads();
   const double sc = s_scale;
+  auto at = [&](int i) { return i < h ? i : HM + i - h; };   // row or column of index i
   // H is symmetric by definition; its stored copy may not be (a projected
   // matrix whose basis amplifies rounding), and the two-sided rotations of an
   // unsymmetric matrix do not settle: read the symmetric part
   for (int e = tid; e < m * m; e += T) {
     const int a = e / m, b = e % m;
-    Abuf[a * ld + b] = (float)(0.5 * (H[e] + H[(size_t)b * m + a]) * sc);
-    Vbuf[a * ld + b] = (a == b) ? 1.0f : 0.0f;
+    Abuf[at(a) * ld + at(b)] = to_f32(0.5 * (H[e] + H[(size_t)b * m + a]) * sc);
   }
-  // where a position moves after a round, and the stored place of an entry
-  auto next = [&](int x) {
-    if (x < h) return x == 0 ? 0 : (x < h - 1 ? x + 1 : m - 1);
-    return x == h ? 1 : x - 1;
-  };
-  auto place = [&](int r, int c) {
-    const int br = r < h ? r : r - h, bc = c < h ? c : c - h;
-    const bool swap = br > bc || (br == bc && r >= h && c < h);
-    return swap ? c * ld + r : r * ld + c;
-  };
-  // this thread's blocks of the matrix (upper triangle of blocks, folded into
-  // rows of h + 1 blocks) and of V
-  int aI[IA], aJ[IA], aw[IA][4];
-  bool aok[IA];
-#pragma unroll
-  for (int k = 0; k < IA; ++k) {
-    const int idx = tid + k * T, r = idx / (h + 1), c = idx % (h + 1);
-    const bool lower = c >= h - r;
-    aok[k] = r < (h + 1) / 2 && !(lower && r == h - 1 - r);
-    const int I = lower ? h - 1 - r : r, J = lower ? I + (c - (h - r)) : r + c;
-    aI[k] = aok[k] ? I : 0;
-    aJ[k] = aok[k] ? J : 0;
-    const int tI = next(aI[k]), bI = next(h + aI[k]), tJ = next(aJ[k]), bJ = next(h + aJ[k]);
-    aw[k][0] = place(tI, tJ);
-    aw[k][1] = place(tI, bJ);
-    aw[k][2] = place(bI, tJ);
-    aw[k][3] = place(bI, bJ);
-  }
-  int vr[IV], vJ[IV], vt[IV], vb[IV];
-  bool vok[IV];
-#pragma unroll
-  for (int k = 0; k < IV; ++k) {
-    const int idx = tid - nang + k * (T - nang);
-    vok[k] = tid >= nang && idx < h * h;
-    const int R = vok[k] ? idx / h : 0, J = vok[k] ? idx % h : 0;
-    vJ[k] = J;
-    vr[k] = R * ld + J;
-    vt[k] = R * ld + next(J);
-    vb[k] = R * ld + next(h + J);
-  }
-  int cur = 0, vcur = 0;
-  // V <- V J with the angles of round parity par, columns moved to their new slots
-  auto rotate_v = [&](int par) {
-    const float *src = Vbuf + vcur * sz;
-    float *dst = Vbuf + (vcur ^ 1) * sz;
-#pragma unroll
-    for (int k = 0; k < IV; ++k)
-      if (vok[k]) {
-        const float2 g = cs[par * h + vJ[k]];
-        const float x0 = src[vr[k]], y0 = src[vr[k] + h];
-        const float x1 = src[vr[k] + h * ld], y1 = src[vr[k] + h * ld + h];
-        dst[vt[k]] = g.x * x0 - g.y * y0;
-        dst[vb[k]] = g.y * x0 + g.x * y0;
-        dst[vt[k] + h * ld] = g.x * x1 - g.y * y1;
-        dst[vb[k] + h * ld] = g.y * x1 + g.x * y1;
-      }
-    vcur ^= 1;
-  };
   __syncthreads();
-  int sweep = 0;
-  for (; sweep < kJ32MaxSweeps; ++sweep) {
-    // a sweep that would find nothing to rotate is not run
-    if (tid == 0) s_rot = 0;
-    __syncthreads();
-    {
-      const float *A = Abuf + cur * sz;
-      bool any = false;
+  if (tid < nA) {
+    // ---- angles: first nang threads (thread k: slot k); the matrix: up to nA
+    auto bar = [&]() { asm volatile("bar.sync 1, %0;" ::"r"(nA) : "memory"); };
+    // where an index moves after a round (slot order), and the stored place of an entry
+    auto next = [&](int x) {
+      if (x < h) return x == 0 ? 0 : (x < h - 1 ? x + 1 : m - 1);
+      return x == h ? 1 : x - 1;
+    };
+    auto place = [&](int r, int c) {
+      const int br = r < h ? r : r - h, bc = c < h ? c : c - h;
+      const bool swap = br > bc || (br == bc && r >= h && c < h);
+      return swap ? at(c) * ld + at(r) : at(r) * ld + at(c);
+    };
+    auto angle = [&](float app, float aqq, float apq) {
+      float c = 1.0f, sv = 0.0f;
+      if (fabsf(apq) > floor_abs && apq * apq > kJ32Rel2 * fabsf(app * aqq)) {
+        // half-angle form of the smaller rotation: with r = hypot(d, 2 g),
+        // c^2 = (1 + |d| / r) / 2 and s = sign(d) g / (r c)
+        const float d = aqq - app, ir = rsqrt_approx(fmaf(d, d, 4.0f * apq * apq));
+        const float w = fmaf(0.5f * fabsf(d), ir, 0.5f), ic = rsqrt_approx(w);
+        c = w * ic;
+        sv = copysignf(apq * ir, d) * (apq < 0.0f ? -ic : ic);
+      }
+      return make_float2(c, sv);
+    };
+    // the indices that meet in slot k after a round: their slots and kinds now
+    const bool is_angle = tid < nang;
+    const int k0 = tid < h ? tid : 0;
+    const int tS = k0 == 0 ? 0 : k0 == 1 ? 0 : k0 - 1, qS = k0 == h - 1 ? h - 1 : k0 + 1;
+    const bool t_top = k0 != 1, q_top = k0 == h - 1;
+    const int lo = tS < qS ? tS : qS, hi = tS < qS ? qS : tS;
+    const bool lo_top = tS < qS ? t_top : q_top, hi_top = tS < qS ? q_top : t_top;
+    // this thread's blocks: tiles of 4 x 8 blocks that reach above the diagonal,
+    // one per warp and k, their 32 blocks over the lanes
+    int aI[IA], aJ[IA], at0[IA], ab0[IA], aw[IA][4];
+    bool aok[IA];
+#pragma unroll
+    for (int k = 0; k < IA; ++k) {
+      int left = (tid - nang) / 32 + k * ((nA - nang) / 32), ti = 0;
+      while (left >= (h + 7) / 8 - ti / 2 && 4 * ti < h) left -= (h + 7) / 8 - ti / 2, ++ti;
+      const int I = 4 * ti + ((tid & 31) >> 3), J = 8 * (ti / 2 + left) + (tid & 7);
+      aok[k] = !is_angle && I <= J && J < h;
+      aI[k] = aok[k] ? I : 0;
+      aJ[k] = aok[k] ? J : 0;
+      const int tI = next(aI[k]), bI = next(h + aI[k]), tJ = next(aJ[k]), bJ = next(h + aJ[k]);
+      at0[k] = aI[k] * ld + aJ[k];
+      ab0[k] = (HM + aI[k]) * ld + aJ[k];
+      aw[k][0] = place(tI, tJ);
+      aw[k][1] = place(tI, bJ);
+      aw[k][2] = place(bI, tJ);
+      aw[k][3] = place(bI, bJ);
+    }
+    // rotates the matrix by the angles cs into the other buffer, and computes the
+    // next round's angles into cs_next
+    auto do_round = [&](auto cur, const float2 *cs, float2 *cs_next) {
+      constexpr int CUR = decltype(cur)::value;
+      const float *A = Abuf + CUR * C::kA;
+      float *B = Abuf + (CUR ^ 1) * C::kA;
+      if (is_angle) {
+        if (tid < h) {
+          // row of the rotation that makes a slot's new top (c, -s) or bottom (s, c)
+          const float2 gl = cs[lo], gh = cs[hi];
+          const float ul = lo_top ? gl.x : gl.y, vl = lo_top ? -gl.y : gl.x;
+          const float uh = hi_top ? gh.x : gh.y, vh = hi_top ? -gh.y : gh.x;
+          const float *dl = A + lo * ld + lo, *dh = A + hi * ld + hi, *x = A + lo * ld + hi;
+          const float l00 = dl[0], l01 = dl[HM], l11 = dl[HM * ld + HM];
+          const float h00 = dh[0], h01 = dh[HM], h11 = dh[HM * ld + HM];
+          const float x00 = x[0], x01 = x[HM], x10 = x[HM * ld], x11 = x[HM * ld + HM];
+          const float nl = ul * (ul * l00 + vl * l01) + vl * (ul * l01 + vl * l11);
+          const float nh = uh * (uh * h00 + vh * h01) + vh * (uh * h01 + vh * h11);
+          const float nx = ul * (uh * x00 + vh * x01) + vl * (uh * x10 + vh * x11);
+          cs_next[tid] = tS < qS ? angle(nl, nh, nx) : angle(nh, nl, nx);
+        }
+        bar();
+        return;
+      }
 #pragma unroll
       for (int k = 0; k < IA; ++k)
         if (aok[k]) {
-          const int I = aI[k], J = aJ[k];
-          const float dI[2] = {A[I * ld + I], A[(h + I) * ld + h + I]};
-          const float dJ[2] = {A[J * ld + J], A[(h + J) * ld + h + J]};
-#pragma unroll
-          for (int a = 0; a < 2; ++a)
-#pragma unroll
-            for (int b = 0; b < 2; ++b) {
-              if (I == J && !(a == 0 && b == 1)) continue;
-              const float v = A[(I + a * h) * ld + J + b * h];
-              any = any || (fabsf(v) > floor_abs && v * v > kJ32Rel2 * fabsf(dI[a] * dJ[b]));
-            }
+          const bool own = aI[k] == aJ[k];
+          const float2 gI = cs[aI[k]], gJ = cs[aJ[k]];
+          const float a00 = A[at0[k]], a01 = A[at0[k] + HM], a11 = A[ab0[k] + HM];
+          const float a10 = own ? a01 : A[ab0[k]];
+          const float b00 = gJ.x * a00 - gJ.y * a01, b01 = gJ.y * a00 + gJ.x * a01;
+          const float b10 = gJ.x * a10 - gJ.y * a11, b11 = gJ.y * a10 + gJ.x * a11;
+          const float n00 = gI.x * b00 - gI.y * b10, n11 = gI.y * b01 + gI.x * b11;
+          float n01 = gI.x * b01 - gI.y * b11, n10 = gI.y * b00 + gI.x * b10;
+          // a rotated slot's own coupling is zero; one left alone keeps it
+          if (own) n01 = n10 = gI.y != 0.0f ? 0.0f : a01;
+          B[aw[k][0]] = n00;
+          B[aw[k][1]] = n01;
+          B[aw[k][2]] = n10;
+          B[aw[k][3]] = n11;
         }
-      if (any) s_rot = 1;
-    }
-    __syncthreads();
-    const int more = s_rot;
-    __syncthreads();
-    if (!more) break;
-    for (int r = 0; r < m - 1; ++r) {
-      if (tid < h) {
-        const float *A = Abuf + cur * sz;
-        const float app = A[tid * ld + tid], aqq = A[(h + tid) * ld + h + tid], apq = A[tid * ld + h + tid];
-        float c = 1.0f, sv = 0.0f;
-        if (fabsf(apq) > floor_abs && apq * apq > kJ32Rel2 * fabsf(app * aqq)) {
-          const float tau = (aqq - app) / (2.0f * apq);
-          const float t = copysignf(1.0f, tau) / (fabsf(tau) + sqrtf(fmaf(tau, tau, 1.0f)));
-          c = rsqrtf(fmaf(t, t, 1.0f));
-          sv = t * c;
-        }
-        cs[(r & 1) * h + tid] = make_float2(c, sv);
-      }
-      if (r > 0) rotate_v((r - 1) & 1);
-      __syncthreads();
-      {
-        const float *A = Abuf + cur * sz;
-        float *B = Abuf + (cur ^ 1) * sz;
+      bar();
+    };
+    int cur = 0, sweep = 0;
+    for (; sweep <= kJ32MaxSweeps; ++sweep) {
+      // a sweep that would find nothing to rotate is not run
+      float2 *cs = ring + (sweep & 1) * C::kSweep;
+      if (tid == 0) s_rot[sweep & 1] = 0;
+      bar();
+      if (sweep < kJ32MaxSweeps) {
+        const float *A = Abuf + cur * C::kA;
+        bool any = false;
 #pragma unroll
         for (int k = 0; k < IA; ++k)
           if (aok[k]) {
-            const int I = aI[k], J = aJ[k], o = I * ld + J;
-            const float2 gI = cs[(r & 1) * h + I], gJ = cs[(r & 1) * h + J];
-            const float a00 = A[o], a01 = A[o + h], a11 = A[o + h * ld + h];
-            const float a10 = I == J ? a01 : A[o + h * ld];
-            const float b00 = gJ.x * a00 - gJ.y * a01, b01 = gJ.y * a00 + gJ.x * a01;
-            const float b10 = gJ.x * a10 - gJ.y * a11, b11 = gJ.y * a10 + gJ.x * a11;
-            const float n00 = gI.x * b00 - gI.y * b10, n11 = gI.y * b01 + gI.x * b11;
-            float n01 = gI.x * b01 - gI.y * b11, n10 = gI.y * b00 + gI.x * b10;
-            // a rotated slot's own coupling is zero; one left alone keeps it
-            if (I == J) n01 = n10 = gI.y != 0.0f ? 0.0f : a01;
-            B[aw[k][0]] = n00;
-            B[aw[k][1]] = n01;
-            B[aw[k][2]] = n10;
-            B[aw[k][3]] = n11;
+            const int I = aI[k], J = aJ[k];
+            const float dI[2] = {A[I * ld + I], A[(HM + I) * ld + HM + I]};
+            const float dJ[2] = {A[J * ld + J], A[(HM + J) * ld + HM + J]};
+#pragma unroll
+            for (int a = 0; a < 2; ++a)
+#pragma unroll
+              for (int b = 0; b < 2; ++b) {
+                if (I == J && !(a == 0 && b == 1)) continue;
+                const float v = A[(a ? ab0[k] : at0[k]) + b * HM];
+                any = any || (fabsf(v) > floor_abs && v * v > kJ32Rel2 * fabsf(dI[a] * dJ[b]));
+              }
           }
+        if (any) s_rot[sweep & 1] = 1;
+      }
+      __syncthreads();     // the last sweep's angles are ready; V has used up those of the one before
+      if (!s_rot[sweep & 1]) break;
+      if (tid < h) {
+        const float *A = Abuf + cur * C::kA;
+        cs[tid] = angle(A[tid * ld + tid], A[(HM + tid) * ld + HM + tid], A[tid * ld + HM + tid]);
+      }
+      bar();
+      for (int r = 0; r < m - 1; ++r, cs += C::kRound) {
+        // the last round's successor is the next sweep's first: computed there
+        float2 *nx = r < m - 2 ? cs + C::kRound : spare;
+        if (cur == 0) do_round(std::integral_constant<int, 0>{}, cs, nx);
+        else do_round(std::integral_constant<int, 1>{}, cs, nx);
         cur ^= 1;
       }
-      __syncthreads();
     }
-    rotate_v((m - 2) & 1);
-    // the next sweep's test synchronises before the angles are written again
-  }
-  __syncthreads();
-  if (tid == 0) atomicMax(sweeps, sweep);
-  const float *V = Vbuf + vcur * sz;
-  double *out = Vout.at(z);
-  for (int e = tid; e < m * m; e += T) {
-    const int c = e / m, j = e % m;            // out[j + c m] = V[j][c]
-    out[e] = (double)V[j * ld + c];
+    if (tid == 0) atomicMax(sweeps, sweep);
+  } else {
+    // ---- V: RPG rows per group of 16 lanes, slots SPL l .. SPL l + SPL - 1 of a row in lane l
+    const int l = tid & 15, row0 = (tid - nA) / 16 * RPG;
+    float t[RPG][SPL], b[RPG][SPL];
+    bool last[SPL];
+#pragma unroll
+    for (int q = 0; q < SPL; ++q) {
+      const int sl = l * SPL + q;
+      last[q] = sl == h - 1;
+#pragma unroll
+      for (int r = 0; r < RPG; ++r) {
+        t[r][q] = row0 + r == sl ? 1.0f : 0.0f;
+        b[r][q] = row0 + r == h + sl ? 1.0f : 0.0f;
+      }
+    }
+    const bool l0 = l == 0;
+    for (int sweep = 0;; ++sweep) {
+      __syncthreads();
+      const bool more = s_rot[sweep & 1] != 0;
+      if (sweep > 0) {
+        const float2 *cs = ring + ((sweep - 1) & 1) * C::kSweep + l * SPL;
+        float2 g[SPL];
+#pragma unroll
+        for (int q = 0; q < SPL; ++q) g[q] = cs[q];
+        for (int r = 0; r < m - 1; ++r) {
+          float2 gn[SPL];
+          cs += r < m - 2 ? C::kRound : 0;          // the next round's angles, ahead of their use
+#pragma unroll
+          for (int q = 0; q < SPL; ++q) gn[q] = cs[q];
+#pragma unroll
+          for (int i = 0; i < RPG; ++i) {
+#pragma unroll
+            for (int q = 0; q < SPL; ++q) {
+              const float x = t[i][q], y = b[i][q];
+              t[i][q] = g[q].x * x - g[q].y * y;
+              b[i][q] = g[q].y * x + g[q].x * y;
+            }
+            // tops one slot up (slot 0's stays, slot 0's bottom follows into slot 1),
+            // bottoms one slot down (the last top turns round)
+            const float up = __shfl_up_sync(0xffffffffu, SPL == 1 && l0 ? b[i][0] : t[i][SPL - 1], 1, 16);
+            const float dn = __shfl_down_sync(0xffffffffu, b[i][0], 1, 16);
+            float nt[SPL], nb[SPL];
+#pragma unroll
+            for (int q = 0; q < SPL; ++q) {
+              nt[q] = q == 0 ? (l0 ? t[i][0] : up) : (q == 1 && l0 ? b[i][0] : t[i][q > 0 ? q - 1 : 0]);
+              nb[q] = last[q] ? t[i][q] : q == SPL - 1 ? dn : b[i][q < SPL - 1 ? q + 1 : q];
+            }
+#pragma unroll
+            for (int q = 0; q < SPL; ++q) {
+              t[i][q] = nt[q];
+              b[i][q] = nb[q];
+            }
+          }
+#pragma unroll
+          for (int q = 0; q < SPL; ++q) g[q] = gn[q];
+        }
+      }
+      if (!more) break;
+    }
+    double *out = Vout.at(z);
+#pragma unroll
+    for (int i = 0; i < RPG; ++i)
+#pragma unroll
+      for (int q = 0; q < SPL; ++q) {
+        const int sl = l * SPL + q, row = row0 + i;
+        if (row < m && sl < h) {
+          out[row + (size_t)sl * m] = to_f64(t[i][q]);             // out[j + c m] = V[j][c]
+          out[row + (size_t)(h + sl) * m] = to_f64(b[i][q]);
+        }
+      }
   }
 }
 
@@ -532,31 +631,37 @@ __global__ void k_eig_one(PSet G, PSet X, PSet theta, int m, int P) {
   for (int i = 1; i < m; ++i) theta.at(z)[i] = 0.0;
 }
 
-cudaError_t launch_j32(PSet H, int m, float floor_abs, PSet V, int *sweeps, int P, cudaStream_t s) {
+template <int HM, int SPL, int RPG, int IA>
+cudaError_t run_j32(PSet H, int m, float floor_abs, PSet V, int *sweeps, int P, cudaStream_t s) {
+  const auto kern = k_rr_jacobi32<HM, SPL, RPG, IA>;
+  static bool done = false;
+  if (!done) {
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)J32Cfg<HM, SPL>::kSmem);
+    if (e) return e;
+    done = true;
+  }
+  // threads of the angles, of the matrix (4 x 8 blocks per warp, IA of them in turn) and of V
   const int h = m / 2, nang = (h + 31) / 32 * 32;
-  // blocks of V per thread, so that the threads (and half of the matrix's
-  // blocks, at most IA per thread) fit 1024
-  const int iv = h <= 25 ? 1 : h <= 32 ? 2 : 3;
-  const int T = nang + (h * h + 32 * iv - 1) / (32 * iv) * 32;
-  const dim3 g(1, 1, P);
-  const size_t sm = j32_smem(m);
-  if (iv == 1) k_rr_jacobi32<1, 1><<<g, T, sm, s>>>(H, m, floor_abs, V, sweeps);
-  else if (iv == 2) k_rr_jacobi32<2, 1><<<g, T, sm, s>>>(H, m, floor_abs, V, sweeps);
-  else k_rr_jacobi32<3, 2><<<g, T, sm, s>>>(H, m, floor_abs, V, sweeps);
+  int tiles = 0;
+  for (int ti = 0; 4 * ti < h; ++ti) tiles += (h + 7) / 8 - ti / 2;
+  const int nA = nang + (tiles + IA - 1) / IA * 32;
+  const int nV = ((m + RPG - 1) / RPG + 1) / 2 * 32;
+  kern<<<dim3(1, 1, P), nA + nV, J32Cfg<HM, SPL>::kSmem, s>>>(H, m, floor_abs, nang, nA, V, sweeps);
   return cudaGetLastError();
+}
+
+cudaError_t launch_j32(PSet H, int m, float floor_abs, PSet V, int *sweeps, int P, cudaStream_t s) {
+  if (m <= 32) return run_j32<16, 1, 2, 1>(H, m, floor_abs, V, sweeps, P, s);
+  if (m <= 48) return run_j32<24, 2, 3, 1>(H, m, floor_abs, V, sweeps, P, s);
+  if (m <= 64) return run_j32<32, 2, 3, 1>(H, m, floor_abs, V, sweeps, P, s);
+  return run_j32<48, 3, 5, 3>(H, m, floor_abs, V, sweeps, P, s);
 }
 
 cudaError_t small_attrs() {
   static bool done = false;
   if (done) return cudaSuccess;
-  cudaError_t e;
-  const int big = 200 * 1024;
-  const cudaFuncAttribute at = cudaFuncAttributeMaxDynamicSharedMemorySize;
-  if ((e = cudaFuncSetAttribute(k_rr_jacobi32<1, 1>, at, big)) ||
-      (e = cudaFuncSetAttribute(k_rr_jacobi32<2, 1>, at, big)) ||
-      (e = cudaFuncSetAttribute(k_rr_jacobi32<3, 2>, at, big)) ||
-      (e = cudaFuncSetAttribute(k_rr_sparse_jacobi, at, big)))
-    return e;
+  const cudaError_t e = cudaFuncSetAttribute(k_rr_sparse_jacobi, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+  if (e) return e;
   done = true;
   return cudaSuccess;
 }
