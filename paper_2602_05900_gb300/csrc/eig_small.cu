@@ -11,11 +11,12 @@
 //      small eigenvalues of a dense H only through the FP32 rounding of the
 //      large entries; S is graded, and its small block is resolved at its own
 //      scale.
-//   3. Three refinement passes X <- X (I + E) (Ogita and Aishima's iteration):
+//   3. Two refinement passes X <- X (I + E) (Ogita and Aishima's iteration):
 //      with G = X^T X, S = X^T H X and lambda_i = s_ii / g_ii,
 //      E_ij = (s_ij - lambda_j g_ij) / (lambda_j - lambda_i) for separated pairs
 //      and -g_ij / 2 inside clusters and for couplings at rounding level:
-//      quadratic convergence of the vectors and of their orthonormality at once.
+//      quadratic convergence of the vectors and of their orthonormality at once;
+//      then two Newton-Schulz steps for the orthonormality the last pass left.
 //   4. S = X^T H X once more, and exact 2 x 2 rotations (k_rr_sparse_jacobi) of
 //      the pairs that still need one: those in clusters of near-equal values.
 //
@@ -30,6 +31,7 @@
 #include <math.h>
 
 #include <type_traits>
+#include <utility>
 
 #include "eig_orth.cuh"
 #include "eig_si.cuh"
@@ -391,6 +393,7 @@ constexpr double kSfsCluster = 1e3;   // a pair is separated if |gap| > kSfsClus
 struct MmOp {
   PSet A, B, S, G, Out;
   int ta, refine;
+  int sym;               // the product is symmetric: only its upper tiles are computed, and mirrored
   double bs, bd;
   int rows, cols;
 };
@@ -410,7 +413,7 @@ __global__ void __launch_bounds__(256) k_se_mm(MmOp op0, MmOp op1, int P, int m,
   const MmOp &o = second ? op1 : op0;
   const int z = second ? (int)blockIdx.z - P : (int)blockIdx.z;
   const int i0 = blockIdx.x * 8, j0 = blockIdx.y * 8;
-  if (i0 >= o.rows || j0 >= o.cols) return;
+  if (i0 >= o.rows || j0 >= o.cols || (o.sym && i0 > j0)) return;
   const double *a = o.A.at(z);
   if (o.ta) {
     for (int e = threadIdx.x; e < 8 * m; e += blockDim.x) {
@@ -451,7 +454,7 @@ __global__ void __launch_bounds__(256) k_se_mm(MmOp op0, MmOp op1, int P, int m,
         if (k == j) {
           v = 1.5 - 0.5 * g;                                  // 1 + (1 - g) / 2
         } else {
-          const double s = 0.5 * (S[(size_t)j * m + k] + S[(size_t)k * m + j]);
+          const double s = S[(size_t)j * m + k];
           const double gap = lam[j] - lam[k];
           const double num = fma(-lam[j], g, s);
           const float off = mag32(fma(0.5 * gap, g, num));    // s - (lam_j + lam_k) g / 2
@@ -472,9 +475,11 @@ __global__ void __launch_bounds__(256) k_se_mm(MmOp op0, MmOp op1, int P, int m,
   __syncthreads();
   if (threadIdx.x < 64) {
     const int i = i0 + ti, j = j0 + tj;
-    if (i < o.rows && j < o.cols)
-      o.Out.at(z)[(size_t)j * o.rows + i] =
-          (part[0][ti][tj] + part[1][ti][tj]) + (part[2][ti][tj] + part[3][ti][tj]);
+    if (i < o.rows && j < o.cols) {
+      const double v = (part[0][ti][tj] + part[1][ti][tj]) + (part[2][ti][tj] + part[3][ti][tj]);
+      o.Out.at(z)[(size_t)j * o.rows + i] = v;
+      if (o.sym && i0 != j0) o.Out.at(z)[(size_t)i * o.rows + j] = v;
+    }
   }
 }
 
@@ -492,7 +497,7 @@ __global__ void __launch_bounds__(256) k_se_mm(MmOp op0, MmOp op1, int P, int m,
 // in theta, Wout columns in the same order.  The search compares FP32
 // magnitudes taken from the bits (an FP64 comparison of every entry would cost
 // more than the rotations: m^2 of them at two per clock).
-constexpr int kSparseRounds = 16;
+constexpr int kSparseRounds = 32;
 constexpr int kSparseThreads = 1024;
 
 size_t sparse_smem(int m) {
@@ -683,8 +688,9 @@ cudaError_t small_eig(const SmallEig &a, cudaStream_t s, long long *launches) {
   const float noise = ldexpf(1.0f, -(floor_exp + 1));
   const int t = (m + 7) / 8;
   auto op = [&](PSet A, int ta, PSet B, double bs, double bd, PSet Out) {
-    return MmOp{A, B, B, B, Out, ta, 0, bs, bd, m, m};
+    return MmOp{A, B, B, B, Out, ta, 0, 0, bs, bd, m, m};
   };
+  auto sym = [&](PSet A, PSet B, PSet Out) { return MmOp{A, B, B, B, Out, 1, 0, 1, 1.0, 0.0, m, m}; };   // A^T B
   auto mm1 = [&](const MmOp &o) {
     k_se_mm<<<dim3(t, t, P), 256, 0, s>>>(o, o, P, m, noise);
     *launches += 1;
@@ -703,10 +709,10 @@ cudaError_t small_eig(const SmallEig &a, cudaStream_t s, long long *launches) {
     // a dense H: the first FP32 pass stops at its rounding (2^-24), the second
     // one resolves what lies below; a graded H is resolved by the first
     if ((e = launch_j32(a.H, m, ldexpf(1.0f, a.graded ? -56 : -24), X, a.sweeps, P, s))) return e;
-    mm1(op(X, 1, X, 1.0, 0.0, G));
+    mm1(sym(X, X, G));
     mm1(op(X, 0, G, -0.5, 1.5, Xn));
     mm1(op(a.H, 1, Xn, 1.0, 0.0, Y));
-    mm1(op(Xn, 1, Y, 1.0, 0.0, S));
+    mm1(sym(Xn, Y, S));
     if ((e = launch_j32(S, m, ldexpf(1.0f, -56), V, a.sweeps, P, s))) return e;
     mm1(op(Xn, 0, V, 1.0, 0.0, X));
     *launches += 2;
@@ -717,20 +723,25 @@ cudaError_t small_eig(const SmallEig &a, cudaStream_t s, long long *launches) {
     if ((e = launch_j32(a.H, m, ldexpf(1.0f, -46), X, a.sweeps, P, s))) return e;
     *launches += 1;
   }
-  for (int pass = 0; pass < 3; ++pass) {
-    mm2(op(X, 1, X, 1.0, 0.0, G), op(a.H, 1, X, 1.0, 0.0, Y));
-    mm1(op(X, 1, Y, 1.0, 0.0, S));
-    mm1(MmOp{X, X, S, G, Xn, 0, 1, 1.0, 0.0, m, m});
-    const PSet q = X;
-    X = Xn;
-    Xn = q;
+  for (int pass = 0; pass < 2; ++pass) {
+    mm2(sym(X, X, G), op(a.H, 1, X, 1.0, 0.0, Y));
+    mm1(sym(X, Y, S));
+    mm1(MmOp{X, X, S, G, Xn, 0, 1, 0, 1.0, 0.0, m, m});
+    std::swap(X, Xn);
+  }
+  // orthonormal to rounding: barely separated pairs take E up to 1 / kSfsCluster,
+  // whose square is what a pass leaves
+  for (int ns = 0; ns < 2; ++ns) {
+    mm1(sym(X, X, G));
+    mm1(op(X, 0, G, -0.5, 1.5, Xn));
+    std::swap(X, Xn);
   }
   mm1(op(a.H, 1, X, 1.0, 0.0, Y));
-  mm1(op(X, 1, Y, 1.0, 0.0, S));
+  mm1(sym(X, Y, S));
   k_rr_sparse_jacobi<<<dim3(1, 1, P), kSparseThreads, sparse_smem(m), s>>>(S, m, floor_exp, W, a.theta, a.flag,
                                                                           a.rounds);
   *launches += 1;
-  mm1(MmOp{X, W, W, W, a.out, 0, 0, 1.0, 0.0, a.rows, a.cols});
+  mm1(MmOp{X, W, W, W, a.out, 0, 0, 0, 1.0, 0.0, a.rows, a.cols});
   return cudaGetLastError();
 }
 

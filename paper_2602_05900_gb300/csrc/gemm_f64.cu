@@ -6,7 +6,7 @@
 // outputs per thread, K staged through shared memory in chunks of 16 with a
 // register prefetch of the next chunk; grid.z runs over the instances of a batch.
 // GEMMs with at most 64 outputs and K >= 256 take a block-per-output dot kernel,
-// GEMMs with M, N <= 128 a 16 x 16-tile kernel.
+// GEMMs with few 64 x 64 tiles a kernel of 16 x 16 or 8 x 8 tiles.
 #include "common.cuh"
 
 namespace hotrg {
@@ -160,41 +160,91 @@ __global__ void __launch_bounds__(NT) k_dot_f64(MappedGemm g) {
 
 constexpr long long kDotMaxOutputs = 64, kDotMinK = 256;
 
-// Small GEMMs (M, N <= 128): 16 x 16 output tiles, one output per thread, K in
-// chunks of 16 through shared memory.  A 64 x 64 tiling would put such a product
-// on at most four SMs, and GB300's FP64 rate per SM (about 2 FMA per clock) makes
-// the number of SMs, not the tile efficiency, the limit.
-constexpr int ST = 16;
-constexpr int kSmallMax = 128;
-
+// GEMMs whose 64 x 64 tiles would not give every SM two blocks: TM x TM output
+// tiles (16: one output per thread; 8: the sum over k also split four ways and
+// combined in a fixed order).  GB300's FP64 rate (about 2 FMA per clock and SM)
+// makes the number of SMs the limit, not the operand traffic of a small tile:
+// a 16 x 16 x 32 chunk is 4096 clocks of FMAs for 1024 loads.  Measured at D = 8
+// (a6: 512 x 64 x 64) 60 us with 64 x 64 tiles on eight SMs, 4.4 us with this; a 13 x 13 x
+// 169 product of a chain step 21 us and 3.5 us.
+template <int TM, bool K_FAST_A, bool K_FAST_B>
 __global__ void __launch_bounds__(256) k_gemm_f64_small(MappedGemm g) {
-  __shared__ double As[ST][ST + 1], Bs[ST][ST + 1];   // [k][row]
-  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-  const long long m0 = (long long)blockIdx.x * ST, n0 = (long long)blockIdx.y * ST;
+  constexpr int KS = 256 / (TM * TM);             // k split over the threads
+  constexpr int KC = TM == 8 ? 64 : 32;           // k per chunk
+  constexpr int NL = TM * KC / 256;               // loads per thread, operand and chunk
+  __shared__ double As[KC][TM + 1], Bs[KC][TM + 1];   // [k][row]
+  __shared__ double part[KS][TM][TM + 1];
+  __shared__ long long rowA[TM], rowB[TM];
+  const int tid = threadIdx.x, ks = tid / (TM * TM), tx = tid % TM, ty = tid / TM % TM;
+  const int m0 = blockIdx.x * TM, n0 = blockIdx.y * TM;
   const long long zA = blockIdx.z * g.bA, zB = blockIdx.z * g.bB, zC = blockIdx.z * g.bC;
   g.A += zA;
   g.B += zB;
   g.C += zC;
-  // loads: thread (ty, tx) brings A(m0 + ty, k0 + tx) and B(n0 + ty, k0 + tx)
-  const long long ar = (m0 + ty < g.M) ? map_off(g.am, m0 + ty) : -1;
-  const long long br = (n0 + ty < g.N) ? map_off(g.bn, n0 + ty) : -1;
-  double acc = 0.0;
-  for (int k0 = 0; k0 < g.K; k0 += ST) {
-    const int k = k0 + tx;
-    const bool kv = k < g.K;
-    const long long oa = ar + (kv ? map_off(g.ak, k) : 0), ob = br + (kv ? map_off(g.bk, k) : 0);
-    As[tx][ty] = (ar >= 0 && kv && checked_ok(zA + oa, g.capA, g.err)) ? g.A[oa] : 0.0;
-    Bs[tx][ty] = (br >= 0 && kv && checked_ok(zB + ob, g.capB, g.err)) ? g.B[ob] : 0.0;
-    __syncthreads();
+  if (tid < TM) rowA[tid] = m0 + tid < g.M ? map_off32(g.am, m0 + tid) : -1;
+  else if (tid < 2 * TM) rowB[tid - TM] = n0 + tid - TM < g.N ? map_off32(g.bn, n0 + tid - TM) : -1;
+  __syncthreads();
+  // consecutive threads on consecutive k where the k map is unit-stride, else on rows
+  auto coords = [&](bool fast, int i, int &r, int &k) {
+    const int e = tid + i * 256;
+    r = fast ? e / KC : e % TM;
+    k = fast ? e % KC : e / TM;
+  };
+  double ra[NL], rb[NL];
+  auto fetch = [&](int k0) {
 #pragma unroll
-    for (int kk = 0; kk < ST; ++kk) acc = fma(As[kk][ty], Bs[kk][tx], acc);
+    for (int i = 0; i < NL; ++i) {
+      int r, k;
+      coords(K_FAST_A, i, r, k);
+      const long long oa = rowA[r] + (k0 + k < g.K ? map_off32(g.ak, k0 + k) : 0);
+      ra[i] = rowA[r] >= 0 && k0 + k < g.K && checked_ok(zA + oa, g.capA, g.err) ? g.A[oa] : 0.0;
+      coords(K_FAST_B, i, r, k);
+      const long long ob = rowB[r] + (k0 + k < g.K ? map_off32(g.bk, k0 + k) : 0);
+      rb[i] = rowB[r] >= 0 && k0 + k < g.K && checked_ok(zB + ob, g.capB, g.err) ? g.B[ob] : 0.0;
+    }
+  };
+  double acc = 0.0;
+  fetch(0);
+  for (int k0 = 0; k0 < g.K; k0 += KC) {
+#pragma unroll
+    for (int i = 0; i < NL; ++i) {
+      int r, k;
+      coords(K_FAST_A, i, r, k);
+      As[k][r] = ra[i];
+      coords(K_FAST_B, i, r, k);
+      Bs[k][r] = rb[i];
+    }
+    __syncthreads();
+    if (k0 + KC < g.K) fetch(k0 + KC);
+    const int kn = min(KC, g.K - k0);
+#pragma unroll 8
+    for (int k = ks; k < kn; k += KS) acc = fma(As[k][ty], Bs[k][tx], acc);
     __syncthreads();
   }
-  const long long m = m0 + ty, n = n0 + tx;
+  if constexpr (KS > 1) {
+    part[ks][ty][tx] = acc;
+    __syncthreads();
+    if (ks > 0) return;
+    acc = (part[0][ty][tx] + part[1 % KS][ty][tx]) + (part[2 % KS][ty][tx] + part[3 % KS][ty][tx]);
+  }
+  const int m = m0 + ty, n = n0 + tx;
   if (m < g.M && n < g.N) {
-    const long long oc = map_off(g.cm, m) + map_off(g.cn, n);
+    const long long oc = map_off32(g.cm, m) + map_off32(g.cn, n);
     if (checked_ok(zC + oc, g.capC, g.err)) g.C[oc] = acc;
   }
+}
+
+template <int TM>
+cudaError_t launch_small(const MappedGemm &g, cudaStream_t s) {
+  const dim3 grid((unsigned)((g.M + TM - 1) / TM), (unsigned)((g.N + TM - 1) / TM),
+                  (unsigned)(g.batch < 1 ? 1 : g.batch));
+  if (grid.y > 65535u || grid.z > 65535u) return cudaErrorInvalidConfiguration;
+  const bool ka = (g.ak.s0 == 1), kb = (g.bk.s0 == 1);
+  if (ka && kb) k_gemm_f64_small<TM, true, true><<<grid, 256, 0, s>>>(g);
+  else if (ka) k_gemm_f64_small<TM, true, false><<<grid, 256, 0, s>>>(g);
+  else if (kb) k_gemm_f64_small<TM, false, true><<<grid, 256, 0, s>>>(g);
+  else k_gemm_f64_small<TM, false, false><<<grid, 256, 0, s>>>(g);
+  return cudaGetLastError();
 }
 
 }  // namespace
@@ -206,13 +256,11 @@ cudaError_t gemm_f64(const MappedGemm &g, cudaStream_t s) {
     k_dot_f64<<<dim3((unsigned)(g.M * g.N), 1, (unsigned)(g.batch < 1 ? 1 : g.batch)), NT, 0, s>>>(g);
     return cudaGetLastError();
   }
-  if (g.M <= kSmallMax && g.N <= kSmallMax) {
-    if (g.batch > 65535) return cudaErrorInvalidConfiguration;
-    const dim3 gs((unsigned)((g.M + ST - 1) / ST), (unsigned)((g.N + ST - 1) / ST),
-                  (unsigned)(g.batch < 1 ? 1 : g.batch));
-    k_gemm_f64_small<<<gs, 256, 0, s>>>(g);
-    return cudaGetLastError();
-  }
+  // 64 x 64 tiles once they give the 152 SMs two blocks each, 16 x 16 ones while
+  // those do, else 8 x 8
+  const long long batch = g.batch < 1 ? 1 : g.batch;
+  auto tiles = [&](long long t) { return ((g.M + t - 1) / t) * ((g.N + t - 1) / t) * batch; };
+  if (tiles(BM) < 2 * 152) return tiles(16) < 2 * 152 ? launch_small<8>(g, s) : launch_small<16>(g, s);
   dim3 grid((unsigned)((g.M + BM - 1) / BM), (unsigned)((g.N + BN - 1) / BN),
             (unsigned)(g.batch < 1 ? 1 : g.batch));
   if (grid.y > 65535u || grid.z > 65535u) return cudaErrorInvalidConfiguration;
