@@ -1,31 +1,12 @@
 // hotrg_dgemm_emu: the exact-slice tensor-core GEMM (tc_exact.cuh) as a
 // stand-alone FP64 GEMM entry point (declared in include/hotrg.h).
-#include <string.h>
-
-#include <vector>
-
 #include "../../include/hotrg.h"
+#include "dev_pool.cuh"
 #include "tc_exact.cuh"
 
 using namespace hotrg;
 
 namespace {
-
-struct Scratch {
-  std::vector<void *> ptrs;
-  ~Scratch() {
-    for (void *p : ptrs) cudaFree(p);
-  }
-  void *get(size_t bytes) {
-    void *p = nullptr;
-    if (cudaMalloc(&p, bytes + 256) != cudaSuccess) {
-      (void)cudaGetLastError();
-      return nullptr;
-    }
-    ptrs.push_back(p);
-    return p;
-  }
-};
 
 hotrg_status from_cuda(cudaError_t e) {
   if (e == cudaSuccess) return HOTRG_OK;
@@ -43,18 +24,22 @@ extern "C" hotrg_status hotrg_dgemm_emu(int M, int N, int K, const double *A, lo
     return HOTRG_EINVAL;
   if (M == 0 || N == 0) return HOTRG_OK;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  Scratch sc;
-  const int pitch = xs_pitch(K);
-  XsOperand a{sc.get(sizeof(short) * xs_elems(M, K, slices)), nullptr, M, K, pitch, slices, 1, 0, 0};
-  XsOperand b{sc.get(sizeof(short) * xs_elems(N, K, slices)), nullptr, N, K, pitch, slices, 1, 0, 0};
-  a.scale = static_cast<double *>(sc.get(sizeof(double) * M));
-  b.scale = static_cast<double *>(sc.get(sizeof(double) * N));
-  int *err = static_cast<int *>(sc.get(sizeof(int)));
-  const int ksplit = xs_min_split(K);
-  double *parts = ksplit > 1 ? static_cast<double *>(sc.get(sizeof(double) * ksplit * (size_t)M * N))
-                             : nullptr;
-  if (!a.slices || !b.slices || !a.scale || !b.scale || !err || (ksplit > 1 && !parts))
+  const int pitch = xs_pitch(K), ksplit = xs_min_split(K);
+  // one buffer: both operands' slices and row scales, the K parts, the error flag
+  auto up = [](size_t v) { return (v + 255) / 256 * 256; };
+  const size_t sa = up(sizeof(short) * xs_elems(M, K, slices)), sb = up(sizeof(short) * xs_elems(N, K, slices));
+  const size_t ca = up(sizeof(double) * M), cb = up(sizeof(double) * N);
+  const size_t cp = ksplit > 1 ? up(sizeof(double) * ksplit * (size_t)M * N) : 0;
+  StreamBuffer buf(s);
+  if (buf.alloc(sa + sb + ca + cb + cp + 256) != cudaSuccess) {
+    (void)cudaGetLastError();
     return HOTRG_ENOMEM;
+  }
+  char *p = buf.data();
+  XsOperand a{p, reinterpret_cast<double *>(p + sa + sb), M, K, pitch, slices, 1, 0, 0};
+  XsOperand b{p + sa, reinterpret_cast<double *>(p + sa + sb + ca), N, K, pitch, slices, 1, 0, 0};
+  double *parts = cp ? reinterpret_cast<double *>(p + sa + sb + ca + cb) : nullptr;
+  int *err = reinterpret_cast<int *>(p + sa + sb + ca + cb + cp);
   cudaError_t e;
   PSet pa{const_cast<double *>(A), const_cast<double *>(A), 0};
   PSet pb{const_cast<double *>(B), const_cast<double *>(B), 0};

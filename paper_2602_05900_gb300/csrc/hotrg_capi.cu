@@ -36,6 +36,7 @@
 
 #include "../../include/hotrg.h"
 #include "common.cuh"
+#include "dev_pool.cuh"
 #include "eig_si.cuh"
 #include "tc_exact.cuh"
 #include "tc_gemm.cuh"
@@ -284,7 +285,7 @@ struct hotrg_ctx {
   int *err = nullptr;
   hotrg_status status = HOTRG_OK;
   std::string msg;
-  std::vector<void *> allocs;
+  DeviceBuffers mem;
 };
 
 namespace {
@@ -310,12 +311,11 @@ hotrg_status fail(hotrg_ctx *c, hotrg_status s, const std::string &m) {
 template <typename T>
 hotrg_status dalloc(hotrg_ctx *c, T **p, size_t count) {
   void *q = nullptr;
-  cudaError_t e = cudaMalloc(&q, count * sizeof(T) + 256);
+  cudaError_t e = c->mem.alloc(&q, count * sizeof(T) + 256);
   if (e != cudaSuccess) {
     (void)cudaGetLastError();
-    return fail(c, HOTRG_ENOMEM, "cudaMalloc of " + std::to_string(count * sizeof(T)) + " bytes failed");
+    return fail(c, HOTRG_ENOMEM, "allocation of " + std::to_string(count * sizeof(T)) + " bytes failed");
   }
-  c->allocs.push_back(q);
   *p = static_cast<T *>(q);
   return HOTRG_OK;
 }
@@ -405,7 +405,7 @@ hotrg_status alloc_group(hotrg_ctx *c, Group &g) {
   } else {
     g.sC1 = round_up(nmax, 32);
     if ((s = dalloc(c, &g.c1, 6 * g.sC1 * G))) return s;
-    const int r = g.tc.init(c->prec, g.D0, g.D_cut, G, g.stream, c->err);
+    const int r = g.tc.init(c->prec, g.D0, g.D_cut, G, g.stream, c->err, c->mem);
     if (r == 2) return fail(c, HOTRG_ENOMEM, "tensor-core operand buffers do not fit");
     if (r) return fail(c, HOTRG_ECUDA, "tensor-core path initialisation failed");
   }
@@ -473,6 +473,7 @@ hotrg_status create_ctx(int n, const double *const *T0s, const int *D0s, const i
     if ((s = dalloc(c, &g.si_work, (size_t)si_workspace_doubles(2 * g.G, nsi, kSiMaxBlock))))
       return bail(s);
   }
+  if (c->mem.ready() != cudaSuccess) return bail(HOTRG_ECUDA);
   if (cudaMemsetAsync(c->err, 0, sizeof(int), c->stream) != cudaSuccess) return bail(HOTRG_ECUDA);
   for (auto &gp : c->groups) {
     Group &g = *gp;
@@ -989,7 +990,7 @@ void hotrg_destroy(hotrg_ctx *c) {
   cudaStreamSynchronize(c->stream);
   for (auto &g : c->groups)
     if (g->own_stream && g->stream) cudaStreamSynchronize(g->stream);
-  for (void *p : c->allocs) cudaFree(p);
+  c->mem.free_all();
   delete c;
 }
 

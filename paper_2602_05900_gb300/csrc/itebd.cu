@@ -29,6 +29,7 @@
 #include <vector>
 
 #include "common.cuh"
+#include "dev_pool.cuh"
 #include "eig_si.cuh"
 #include "hotrg.h"
 #include "xxz.cuh"
@@ -169,7 +170,7 @@ struct hotrg_itebd {
   int nb[2] = {-1, -1};
   double *si_work = nullptr;
   int *err = nullptr;
-  std::vector<void *> allocs;
+  DeviceBuffers mem;
   hotrg_status status = HOTRG_OK;
   std::string msg;
 };
@@ -194,11 +195,10 @@ hotrg_status ifail(hotrg_itebd *c, hotrg_status s, const std::string &m) {
 template <typename T>
 hotrg_status ialloc(hotrg_itebd *c, T **p, long long count) {
   void *q = nullptr;
-  if (cudaMalloc(&q, sizeof(T) * (size_t)std::max(1LL, count)) != cudaSuccess) {
+  if (c->mem.alloc(&q, sizeof(T) * (size_t)std::max(1LL, count)) != cudaSuccess) {
     (void)cudaGetLastError();
     return ifail(c, HOTRG_ENOMEM, "device allocation failed");
   }
-  c->allocs.push_back(q);
   *p = static_cast<T *>(q);
   return HOTRG_OK;
 }
@@ -334,7 +334,7 @@ hotrg_status hotrg_itebd_create(int n, const double *couplings, int D_b, int D0,
   c->sL = (Db + 31) / 32 * 32;
   c->sM = (twoD * twoD + 31) / 32 * 32;
   auto bail = [&](hotrg_status s) {
-    for (void *p : c->allocs) cudaFree(p);
+    cudaStreamSynchronize(c->stream);
     delete c;
     return s;
   };
@@ -351,6 +351,7 @@ hotrg_status hotrg_itebd_create(int n, const double *couplings, int D_b, int D0,
       (s = ialloc(c, &c->si_work, si_workspace_doubles(n, (int)twoD, jacobi_block((int)twoD)))) ||
       (s = ialloc(c, &c->err, 4LL)))
     return bail(s);
+  if (c->mem.ready() != cudaSuccess) return bail(HOTRG_ECUDA);
   // host-side initial state and per-chain operators
   std::vector<double> hT((size_t)(c->sT * n), 0.0), hQ((size_t)(c->sT * n), 0.0);
   std::vector<double> hL((size_t)(c->sL * n), 0.0), hO((size_t)(c->sL * n), 0.0);
@@ -453,7 +454,6 @@ const char *hotrg_itebd_last_error(const hotrg_itebd *c) { return c ? c->msg.c_s
 void hotrg_itebd_destroy(hotrg_itebd *c) {
   if (!c) return;
   cudaStreamSynchronize(c->stream);
-  for (void *p : c->allocs) cudaFree(p);
   delete c;
 }
 

@@ -9,6 +9,7 @@
 // separate pass.
 #include <cuda_bf16.h>
 
+#include "dev_pool.cuh"
 #include "tc_chain.cuh"
 #include "tc_gemm.cuh"
 #include "tc_path.cuh"
@@ -30,16 +31,6 @@ struct TcPath::Impl {
   void *P = nullptr, *Q = nullptr;
   int *err = nullptr;
   std::size_t capT = 0, capP = 0;  // elements per plane
-  ~Impl() {
-    cudaFree(opT);
-    cudaFree(part);
-    cudaFree(opU5);
-    cudaFree(opT5);
-    cudaFree(opT6);
-    cudaFree(opU7);
-    cudaFree(P);
-    cudaFree(Q);
-  }
 };
 
 namespace {
@@ -122,20 +113,11 @@ __global__ void __launch_bounds__(256) k_gather(const double *src, long long sSr
   }
 }
 
-void *alloc(std::size_t bytes) {
-  void *p = nullptr;
-  if (cudaMalloc(&p, bytes + 256) != cudaSuccess) {
-    (void)cudaGetLastError();
-    return nullptr;
-  }
-  return p;
-}
-
 }  // namespace
 
 TcPath::~TcPath() { delete impl_; }
 
-int TcPath::init(hotrg_prec prec, int D0, int D_cut, int G, cudaStream_t s, int *err_flag) {
+int TcPath::init(hotrg_prec prec, int D0, int D_cut, int G, cudaStream_t s, int *err_flag, DeviceBuffers &mem) {
   impl_ = new Impl();
   Impl &I = *impl_;
   I.mode = prec == HOTRG_TF32 ? TcMode::TF32 : (prec == HOTRG_BF16X3 ? TcMode::BF16X3 : TcMode::BF16X6);
@@ -153,6 +135,12 @@ int TcPath::init(hotrg_prec prec, int D0, int D_cut, int G, cudaStream_t s, int 
   I.sTop = ((long long)I.capT * I.planes + 63) / 64 * 64;
   I.sPop = ((long long)I.capP * I.planes + 63) / 64 * 64;
   const std::size_t bt = (std::size_t)I.sTop * G * I.eb, bp = (std::size_t)I.sPop * G * I.eb;
+  auto alloc = [&](std::size_t bytes) -> void * {
+    void *p = nullptr;
+    if (mem.alloc(&p, bytes + 256) == cudaSuccess) return p;
+    (void)cudaGetLastError();
+    return nullptr;
+  };
   if (!(I.opT = alloc(4 * bt)) || !(I.part = alloc(4 * bt))) return 2;
   if (!(I.opU5 = alloc(bt)) || !(I.opT5 = alloc(bt)) || !(I.opT6 = alloc(bt)) ||
       !(I.opU7 = alloc(bt)) || !(I.P = alloc(bp)) || !(I.Q = alloc(bp)))

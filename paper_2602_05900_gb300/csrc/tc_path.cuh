@@ -8,6 +8,7 @@
 
 #include "../../include/hotrg.h"
 #include "common.cuh"
+#include "dev_pool.cuh"
 
 namespace hotrg {
 
@@ -16,7 +17,8 @@ class TcPath {
   ~TcPath();
   // 0 on success, 1 CUDA error, 2 allocation failure.  err_flag (device int)
   // receives 2 if a kernel's bounded wait runs out.
-  int init(hotrg_prec prec, int D0, int D_cut, int G, cudaStream_t s, int *err_flag);
+  // Buffers come from `mem`, which outlives this object.
+  int init(hotrg_prec prec, int D0, int D_cut, int G, cudaStream_t s, int *err_flag, DeviceBuffers &mem);
   // Both chains return 0 or the CUDA error of the failing call.
   // a2 + a3: environments G_L, G_R (FP64, [x1,x2,u1,u2], instance stride sG) of a
   // Y step on the strided view (sx, sxp, sy, syp) of T (instance stride sT) with
