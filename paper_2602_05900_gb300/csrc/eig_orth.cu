@@ -25,6 +25,7 @@
 #include <algorithm>
 
 #include "eig_orth.cuh"
+#include "launch.cuh"
 #include "eig_si.cuh"
 
 namespace cg = cooperative_groups;
@@ -162,6 +163,7 @@ constexpr size_t gram_chol_smem(int m) {
 template <int U>
 __global__ void __launch_bounds__(256) __cluster_dims__(kOrthCluster, 1, 1)
     k_gram_chol32(PSet Yin, int n, int m, float shift, PSet Wout, int *flag) {
+  pdl_enter();
   extern __shared__ float2 gsh[];
   constexpr int LD = 16 * U;
   float2 *part = gsh;                                              // m x m, upper triangle
@@ -262,6 +264,7 @@ __global__ void __launch_bounds__(256) __cluster_dims__(kOrthCluster, 1, 1)
 
 template <int U>
 __global__ void __launch_bounds__(256) k_chol32(PSet Cin, int m, float shift, PSet Wout, int *flag) {
+  pdl_enter();
   __shared__ float rowbuf[2 * 16 * U], d[16 * U], piv[16 * U];
   const double *C = Cin.at(blockIdx.z);
   chol_inverse<float, U>([&](int i, int k) { return to_f32(C[(size_t)i * m + k]); }, Shift32{shift}, 2, m,
@@ -271,6 +274,7 @@ __global__ void __launch_bounds__(256) k_chol32(PSet Cin, int m, float shift, PS
 // the same in FP64; only_if (optional): run for problem z only if only_if.at(z)[2] != 0
 template <int U>
 __global__ void __launch_bounds__(256) k_chol64(PSet Cin, int m, double shift, PSet Wout, int *flag, PSet only_if) {
+  pdl_enter();
   if (only_if.b0 && only_if.at(blockIdx.z)[2] == 0.0) return;
   __shared__ double rowbuf[2 * 16 * U], d[16 * U], piv[16 * U];
   const double *C = Cin.at(blockIdx.z);
@@ -283,6 +287,7 @@ __global__ void __launch_bounds__(256) k_chol64(PSet Cin, int m, double shift, P
 // whatever m is.  sym: entries u <= v only (all of the upper triangle).
 template <int U>
 __global__ void __launch_bounds__(256) k_si_gram(PSet A, PSet B, PSet Cp, int n, int m, int sym, int rows) {
+  pdl_enter();
   constexpr int LD = 16 * U;
   __shared__ double As[16][LD + 1];
   __shared__ double Bs[16][LD + 1];
@@ -336,6 +341,7 @@ __global__ void __launch_bounds__(256) k_si_gram(PSet A, PSet B, PSet Cp, int n,
 // four threads to an entry, each with its own run of chunks: the sum is bound
 // by load latency, so many loads are kept in flight.
 __global__ void __launch_bounds__(256) k_si_gram_reduce(PSet Cp, PSet C, int nchunks, int m, int sym) {
+  pdl_enter();
   __shared__ double sum[4][64];
   const int z = blockIdx.z, l = threadIdx.x & 63, g = threadIdx.x >> 6;
   const long long mm = (long long)m * m;
@@ -378,6 +384,7 @@ __global__ void __launch_bounds__(256) k_si_gram_reduce(PSet Cp, PSet C, int nch
 // RT is chosen so that the CTAs fill the SMs.
 template <int RT>
 __global__ void __launch_bounds__(256) k_si_rotate(PSet A, PSet W, PSet Out, int n, int m, int tri) {
+  pdl_enter();
   extern __shared__ double rsh[];
   double *As = rsh;                       // [column][RT]
   double *Ws = rsh + (size_t)m * RT;      // [column][m + 1]
@@ -419,7 +426,7 @@ cudaError_t launch_gram_chol(PSet Y, int n, int m, float shift, PSet W, int *fla
     if (e) return e;
     done = true;
   }
-  k_gram_chol32<U><<<dim3(kOrthCluster, 1, P), 256, gram_chol_smem<U>(m), s>>>(Y, n, m, shift, W, flag);
+  launch_pdl(k_gram_chol32<U>, dim3(kOrthCluster, 1, P), 256, gram_chol_smem<U>(m), s, Y, n, m, shift, W, flag);
   return cudaGetLastError();
 }
 
@@ -432,6 +439,9 @@ cudaError_t launch_rotate(PSet A, PSet W, PSet Out, int n, int m, bool tri, int 
     if (e) return e;
     done = true;
   }
+  // a plain launch: started early, its blocks would be dealt out while the factor's
+  // cluster still holds SMs, and the others would get two (D = 48 job: 57.6 ms
+  // started early, 55.5 ms like this)
   k_si_rotate<RT><<<dim3((n + RT - 1) / RT, 1, P), 256, sizeof(double) * m * (RT + m + 1), s>>>(A, W, Out, n, m,
                                                                                                tri ? 1 : 0);
   return cudaGetLastError();
@@ -441,7 +451,7 @@ cudaError_t launch_rotate(PSet A, PSet W, PSet Out, int n, int m, bool tri, int 
 
 cudaError_t gram_reduce(PSet part, PSet out, int chunks, int m, bool sym, int P, cudaStream_t s,
                         long long *launches) {
-  k_si_gram_reduce<<<dim3((m * m + 63) / 64, 1, P), 256, 0, s>>>(part, out, chunks, m, sym ? 1 : 0);
+  launch_pdl(k_si_gram_reduce, dim3((m * m + 63) / 64, 1, P), 256, 0, s, part, out, chunks, m, sym ? 1 : 0);
   *launches += 1;
   return cudaGetLastError();
 }
@@ -456,11 +466,11 @@ cudaError_t gram64(PSet A, PSet B, bool sym, int n, int m, PSet part, PSet out, 
   if (chunks > kGramChunks || m > kSiMaxBlock) return cudaErrorInvalidValue;
   const dim3 g(chunks, 1, P);
   switch (tile_of(m)) {
-    case 2: k_si_gram<2><<<g, 256, 0, s>>>(A, B, part, n, m, sym, rows); break;
-    case 3: k_si_gram<3><<<g, 256, 0, s>>>(A, B, part, n, m, sym, rows); break;
-    case 4: k_si_gram<4><<<g, 256, 0, s>>>(A, B, part, n, m, sym, rows); break;
-    case 5: k_si_gram<5><<<g, 256, 0, s>>>(A, B, part, n, m, sym, rows); break;
-    default: k_si_gram<6><<<g, 256, 0, s>>>(A, B, part, n, m, sym, rows); break;
+    case 2: launch_pdl(k_si_gram<2>, g, 256, 0, s, A, B, part, n, m, sym, rows); break;
+    case 3: launch_pdl(k_si_gram<3>, g, 256, 0, s, A, B, part, n, m, sym, rows); break;
+    case 4: launch_pdl(k_si_gram<4>, g, 256, 0, s, A, B, part, n, m, sym, rows); break;
+    case 5: launch_pdl(k_si_gram<5>, g, 256, 0, s, A, B, part, n, m, sym, rows); break;
+    default: launch_pdl(k_si_gram<6>, g, 256, 0, s, A, B, part, n, m, sym, rows); break;
   }
   *launches += 1;
   cudaError_t e = cudaGetLastError();
@@ -483,11 +493,11 @@ cudaError_t cholqr32_factor(PSet Y, int n, int m, float shift, PSet W, int *flag
 cudaError_t chol32(PSet C, int m, float shift, PSet W, int *flag, int P, cudaStream_t s, long long *launches) {
   const dim3 g(1, 1, P);
   switch (tile_of(m)) {
-    case 2: k_chol32<2><<<g, 256, 0, s>>>(C, m, shift, W, flag); break;
-    case 3: k_chol32<3><<<g, 256, 0, s>>>(C, m, shift, W, flag); break;
-    case 4: k_chol32<4><<<g, 256, 0, s>>>(C, m, shift, W, flag); break;
-    case 5: k_chol32<5><<<g, 256, 0, s>>>(C, m, shift, W, flag); break;
-    case 6: k_chol32<6><<<g, 256, 0, s>>>(C, m, shift, W, flag); break;
+    case 2: launch_pdl(k_chol32<2>, g, 256, 0, s, C, m, shift, W, flag); break;
+    case 3: launch_pdl(k_chol32<3>, g, 256, 0, s, C, m, shift, W, flag); break;
+    case 4: launch_pdl(k_chol32<4>, g, 256, 0, s, C, m, shift, W, flag); break;
+    case 5: launch_pdl(k_chol32<5>, g, 256, 0, s, C, m, shift, W, flag); break;
+    case 6: launch_pdl(k_chol32<6>, g, 256, 0, s, C, m, shift, W, flag); break;
     default: return cudaErrorInvalidValue;
   }
   *launches += 1;
@@ -498,11 +508,11 @@ cudaError_t chol64(PSet C, int m, double shift, PSet W, int *flag, PSet only_if,
                    long long *launches) {
   const dim3 g(1, 1, P);
   switch (tile_of(m)) {
-    case 2: k_chol64<2><<<g, 256, 0, s>>>(C, m, shift, W, flag, only_if); break;
-    case 3: k_chol64<3><<<g, 256, 0, s>>>(C, m, shift, W, flag, only_if); break;
-    case 4: k_chol64<4><<<g, 256, 0, s>>>(C, m, shift, W, flag, only_if); break;
-    case 5: k_chol64<5><<<g, 256, 0, s>>>(C, m, shift, W, flag, only_if); break;
-    case 6: k_chol64<6><<<g, 256, 0, s>>>(C, m, shift, W, flag, only_if); break;
+    case 2: launch_pdl(k_chol64<2>, g, 256, 0, s, C, m, shift, W, flag, only_if); break;
+    case 3: launch_pdl(k_chol64<3>, g, 256, 0, s, C, m, shift, W, flag, only_if); break;
+    case 4: launch_pdl(k_chol64<4>, g, 256, 0, s, C, m, shift, W, flag, only_if); break;
+    case 5: launch_pdl(k_chol64<5>, g, 256, 0, s, C, m, shift, W, flag, only_if); break;
+    case 6: launch_pdl(k_chol64<6>, g, 256, 0, s, C, m, shift, W, flag, only_if); break;
     default: return cudaErrorInvalidValue;
   }
   *launches += 1;

@@ -34,6 +34,7 @@
 #include <vector>
 
 #include "eig_orth.cuh"
+#include "launch.cuh"
 #include "eig_si.cuh"
 #include "eig_small.cuh"
 #include "tc_exact.cuh"
@@ -58,6 +59,7 @@ __device__ inline double hash_uniform(unsigned long long x) {
 }
 
 __global__ void k_si_init(PSet X, PSet warm, int has_warm, int kw, int n, int m) {
+  pdl_enter();
   const int z = blockIdx.z;
   const long long total = (long long)n * m;
   for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < total;
@@ -72,6 +74,7 @@ __global__ void k_si_init(PSet X, PSet warm, int has_warm, int kw, int n, int m)
 
 // Out_s = G[rows i0.., cols in split s] . X[those rows, :]  (X, Out column-major n x m)
 __global__ void __launch_bounds__(256) k_si_gemm(PSet G, PSet X, PSet Out, int n, int m, int chunk) {
+  pdl_enter();
   __shared__ double Gs[16][65];
   __shared__ double Xs[16][kSiMaxBlock];
   const int z = blockIdx.z;
@@ -122,6 +125,7 @@ __global__ void __launch_bounds__(256) k_si_gemm(PSet G, PSet X, PSet Out, int n
 // Y = (G + sig[0] I) X, sig[1] the shift of the next product (equal to it in
 // this solver; kept apart so that a shift change can never mix the two).
 __global__ void k_si_sigma_init(PSet sig, PSet trace, double factor) {
+  pdl_enter();
   const int z = blockIdx.z;
   if (threadIdx.x == 0) {
     const double t = trace.at(z)[0];
@@ -133,6 +137,7 @@ __global__ void k_si_sigma_init(PSet sig, PSet trace, double factor) {
 
 // Y += sig[1] X; block (0, 0, z) records sig[0] = sig[1] (the shift now in Y)
 __global__ void k_si_shift_add(PSet Y, PSet X, PSet sig, long long nm) {
+  pdl_enter();
   const int z = blockIdx.z;
   const double sg = sig.at(z)[1];
   for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < nm;
@@ -143,6 +148,7 @@ __global__ void k_si_shift_add(PSet Y, PSet X, PSet sig, long long nm) {
 
 // theta_z[i] -= sig[0] for i < m (the shift of the last Rayleigh-Ritz step)
 __global__ void k_si_unshift(PSet theta, PSet sig, int m) {
+  pdl_enter();
   const int z = blockIdx.z;
   const double sg = sig.at(z)[0];
   for (int i = threadIdx.x; i < m; i += blockDim.x) theta.at(z)[i] -= sg;
@@ -151,6 +157,7 @@ __global__ void k_si_unshift(PSet theta, PSet sig, int m) {
 // ks[j] = power of two within a factor 2 of 1 / sqrt(C_jj) (1 if C_jj is not
 // positive and finite): the column scales of a CholeskyQR basis change
 __global__ void k_si_colscale(PSet C, PSet ks, int m) {
+  pdl_enter();
   const int z = blockIdx.z;
   for (int j = threadIdx.x; j < m; j += blockDim.x) {
     const double c = C.at(z)[(size_t)j * m + j];
@@ -163,6 +170,7 @@ __global__ void k_si_colscale(PSet C, PSet ks, int m) {
 // out = sum of the S K-parts; with shift, + sig[1] X as well (the iteration's
 // shift, the same fma as k_si_shift_add) and sig[0] = sig[1]
 __global__ void k_si_sum_split(PSet part, PSet out, int S, long long nm, PSet X, PSet sig, int shift) {
+  pdl_enter();
   const int z = blockIdx.z;
   const double sg = shift ? sig.at(z)[1] : 0.0;
   for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < nm;
@@ -178,6 +186,7 @@ __global__ void k_si_sum_split(PSet part, PSet out, int S, long long nm, PSet X,
 // flags.at(z)[2] = 1 if max |C_ij - delta_ij| > 1/4 (the Newton-Schulz
 // iteration for C^-1/2 from I is then not to be trusted), else 0.
 __global__ void k_rr_far_from_identity(PSet C, int m, PSet flags) {
+  pdl_enter();
   const int z = blockIdx.z;
   double v = 0.0;
   for (int e = threadIdx.x; e < m * m; e += blockDim.x) {
@@ -197,6 +206,7 @@ __global__ void k_rr_far_from_identity(PSet C, int m, PSet flags) {
 
 // Out = a A + b I for m x m matrices of every problem z.
 __global__ void k_rr_axpi(PSet A, double a, double b, PSet Out, int m) {
+  pdl_enter();
   const int z = blockIdx.z;
   for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < m * m; e += gridDim.x * blockDim.x)
     Out.at(z)[e] = a * A.at(z)[e] + ((e % m == e / m) ? b : 0.0);
@@ -207,6 +217,7 @@ __global__ void k_rr_axpi(PSet A, double a, double b, PSet Out, int m) {
 // k is split four ways across the CTA's threads and combined in a fixed order.
 __global__ void __launch_bounds__(256) k_rr_mm(PSet A, int ta, PSet B, double bs, double bd,
                                                PSet Out, int m) {
+  pdl_enter();
   __shared__ double As[8][kSiMaxBlock + 1];   // op(A) rows i0..i0+7, all k
   __shared__ double Bs[8][kSiMaxBlock + 1];   // B columns j0..j0+7, all k
   __shared__ double part[4][8][9];
@@ -240,6 +251,7 @@ __global__ void __launch_bounds__(256) k_rr_mm(PSet A, int ta, PSet B, double bs
 // is as good as another)
 __global__ void k_si_residual(PSet X, PSet Y, PSet theta, PSet res, PSet sig, int use_sig, int n,
                               int k) {
+  pdl_enter();
   const int z = blockIdx.z, i = blockIdx.x;
   const double th = theta.at(z)[i];
   if (use_sig && th - sig.at(z)[0] <= 0.5 * sig.at(z)[1] && i > 0) {
@@ -266,6 +278,7 @@ __global__ void k_si_residual(PSet X, PSet Y, PSet theta, PSet res, PSet sig, in
 
 // G (n x n) into an m x m zero-padded square (m = n or n + 1) for the direct Jacobi path.
 __global__ void k_si_copy_square(PSet G, PSet out, int n, int m) {
+  pdl_enter();
   const int z = blockIdx.z;
   for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < m * m; e += gridDim.x * blockDim.x) {
     const int a = e / m, b = e % m;
@@ -275,6 +288,7 @@ __global__ void k_si_copy_square(PSet G, PSet out, int n, int m) {
 
 // Copy of problem z's n x m block from src to dst (final placement of Ritz vectors).
 __global__ void k_si_copy(PSet src, PSet dst, long long nm) {
+  pdl_enter();
   const int z = blockIdx.z;
   for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < nm;
        e += (long long)gridDim.x * blockDim.x)
@@ -385,7 +399,7 @@ cudaError_t jacobi_full(const SiBatch &b, double *work, cudaStream_t s, long lon
   if ((e = cudaMemsetAsync(B.flag, 0, 4 * sizeof(int), s))) return e;
   PSet H = b.G;
   if (m != n) {
-    k_si_copy_square<<<dim3(grid_1d((long long)m * m, P), 1, P), 256, 0, s>>>(b.G, B.C, n, m);
+    launch_pdl(k_si_copy_square, dim3(grid_1d((long long)m * m, P), 1, P), 256, 0, s, b.G, B.C, n, m);
     if ((e = cudaGetLastError())) return e;
     *launches += 1;
     H = B.C;
@@ -428,7 +442,7 @@ cudaError_t si_solve(const SiBatch &b, double *work, double tol, int max_iter, c
   }
   auto add_shift = [&](PSet src, PSet dst) -> cudaError_t {
     if (!b.has_trace) return cudaSuccess;
-    k_si_shift_add<<<dim3(grid_1d(L.nm, P), 1, P), 256, 0, s>>>(dst, src, B.sig, L.nm);
+    launch_pdl(k_si_shift_add, dim3(grid_1d(L.nm, P), 1, P), 256, 0, s, dst, src, B.sig, L.nm);
     nl += 1;
     return cudaGetLastError();
   };
@@ -448,11 +462,11 @@ cudaError_t si_solve(const SiBatch &b, double *work, double tol, int max_iter, c
       return r ? r : cudaGetLastError();
     }
     if (L.S == 1) {
-      k_si_gemm<<<dim3((n + 63) / 64, 1, P), 256, 0, s>>>(b.G, src, dst, n, m, chunk);
+      launch_pdl(k_si_gemm, dim3((n + 63) / 64, 1, P), 256, 0, s, b.G, src, dst, n, m, chunk);
       nl += 1;
     } else {
-      k_si_gemm<<<dim3((n + 63) / 64, L.S, P), 256, 0, s>>>(b.G, src, B.Yp, n, m, chunk);
-      k_si_sum_split<<<dim3(grid_1d(L.nm, P), 1, P), 256, 0, s>>>(B.Yp, dst, L.S, L.nm, src, B.sig, sh);
+      launch_pdl(k_si_gemm, dim3((n + 63) / 64, L.S, P), 256, 0, s, b.G, src, B.Yp, n, m, chunk);
+      launch_pdl(k_si_sum_split, dim3(grid_1d(L.nm, P), 1, P), 256, 0, s, B.Yp, dst, L.S, L.nm, src, B.sig, sh);
       shifted = true;
       nl += 2;
     }
@@ -474,7 +488,7 @@ cudaError_t si_solve(const SiBatch &b, double *work, double tol, int max_iter, c
       const PSet ks = pset_linear(work + L.oKs, L.per);
       cudaError_t r;
       if (tri) {
-        k_si_colscale<<<dim3(1, 1, P), 128, 0, s>>>(B.C, ks, m);
+        launch_pdl(k_si_colscale, dim3(1, 1, P), 128, 0, s, B.C, ks, m);
         nl += 1;
       }
       if ((r = xs_split_scaled(src, map1(1), map1(n), ks, tri ? 1 : 0, a, s)) ||
@@ -565,10 +579,10 @@ cudaError_t si_solve(const SiBatch &b, double *work, double tol, int max_iter, c
 
   if ((e = cudaMemsetAsync(B.flag, 0, 4 * sizeof(int), s))) return e;
   if (b.has_trace) {
-    k_si_sigma_init<<<dim3(1, 1, P), 32, 0, s>>>(B.sig, b.trace, b.shift_rel);
+    launch_pdl(k_si_sigma_init, dim3(1, 1, P), 32, 0, s, B.sig, b.trace, b.shift_rel);
     nl += 1;
   }
-  k_si_init<<<dim3(grid_1d(L.nm, P), 1, P), 256, 0, s>>>(X, b.warm, b.has_warm ? 1 : 0, b.kw, n, m);
+  launch_pdl(k_si_init, dim3(grid_1d(L.nm, P), 1, P), 256, 0, s, X, b.warm, b.has_warm ? 1 : 0, b.kw, n, m);
   nl += 1;
   // a random or partly warm start is orthogonalised (well conditioned); a start
   // from all m Ritz vectors of the previous solve is orthonormal to FP64 accuracy
@@ -610,34 +624,34 @@ cudaError_t si_solve(const SiBatch &b, double *work, double tol, int max_iter, c
       const dim3 gmm((m + 7) / 8, (m + 7) / 8, P), g1(grid_1d(L.mm, P), 1, P);
       if ((e = gram(X, X, true, B.W))) return e;   // C0 (B.W until small_eig)
       if ((e = gram(X, Y, false, B.C))) return e;  // X^T Y
-      k_rr_axpi<<<g1, 256, 0, s>>>(B.W, -0.5, 1.5, Wn, m);       // W1 = (3I - C0) / 2
+      launch_pdl(k_rr_axpi, g1, 256, 0, s, B.W, -0.5, 1.5, Wn, m);       // W1 = (3I - C0) / 2
       nl += 1;
       for (int ns = 0; ns < 3; ++ns) {                              // W <- W (3I - W^T C0 W) / 2
-        k_rr_mm<<<gmm, 256, 0, s>>>(B.W, 0, Wn, 1.0, 0.0, Tn, m);   // C0 W
-        k_rr_mm<<<gmm, 256, 0, s>>>(Wn, 1, Tn, 1.0, 0.0, Ck, m);    // W^T C0 W
-        k_rr_mm<<<gmm, 256, 0, s>>>(Wn, 0, Ck, -0.5, 1.5, Tn, m);   // next W
+        launch_pdl(k_rr_mm, gmm, 256, 0, s, B.W, 0, Wn, 1.0, 0.0, Tn, m);   // C0 W
+        launch_pdl(k_rr_mm, gmm, 256, 0, s, Wn, 1, Tn, 1.0, 0.0, Ck, m);    // W^T C0 W
+        launch_pdl(k_rr_mm, gmm, 256, 0, s, Wn, 0, Ck, -0.5, 1.5, Tn, m);   // next W
         std::swap(Wn, Tn);
         nl += 3;
       }
       // where X is far from orthonormal (nearly dependent columns at a first
       // check), W comes instead from a shifted FP64 Cholesky of C0 (X W is
       // then orthonormal for any conditioning the shift allows)
-      k_rr_far_from_identity<<<gz, 256, 0, s>>>(B.W, m, B.sig);
+      launch_pdl(k_rr_far_from_identity, gz, 256, 0, s, B.W, m, B.sig);
       nl += 1;
       if ((e = chol64(B.W, m, shift, Wn, B.flag, B.sig, P, s, &nl))) return e;
-      k_rr_mm<<<gmm, 256, 0, s>>>(B.C, 0, Wn, 1.0, 0.0, Tn, m);     // (X^T Y) W
-      k_rr_mm<<<gmm, 256, 0, s>>>(Wn, 1, Tn, 1.0, 0.0, Ck, m);      // H = W^T X^T Y W
+      launch_pdl(k_rr_mm, gmm, 256, 0, s, B.C, 0, Wn, 1.0, 0.0, Tn, m);     // (X^T Y) W
+      launch_pdl(k_rr_mm, gmm, 256, 0, s, Wn, 1, Tn, 1.0, 0.0, Ck, m);      // H = W^T X^T Y W
       nl += 2;
       if ((e = cudaGetLastError())) return e;
       const SmallEig se{P, m, Ck, slot(4), false, false, B.W, m, m, B.th, B.flag, B.sweeps, B.flag + 3};
       if ((e = small_eig(se, s, &nl))) return e;                    // H = Z Theta Z^T (Z in B.W)
-      k_rr_mm<<<gmm, 256, 0, s>>>(Wn, 0, B.W, 1.0, 0.0, Rr, m);     // R = W Z
+      launch_pdl(k_rr_mm, gmm, 256, 0, s, Wn, 0, B.W, 1.0, 0.0, Rr, m);     // R = W Z
       nl += 1;
       if ((e = rot(X, Rr, Z, 0))) return e;
       std::swap(X, Z);
       if ((e = rot(Y, Rr, Z, 0))) return e;
       std::swap(Y, Z);
-      k_si_residual<<<dim3(k, 1, P), 256, 0, s>>>(X, Y, B.th, B.res, B.sig, b.has_trace ? 1 : 0, n, k);
+      launch_pdl(k_si_residual, dim3(k, 1, P), 256, 0, s, X, Y, B.th, B.res, B.sig, b.has_trace ? 1 : 0, n, k);
       nl += 2;
       ++res->rr;
       if ((e = cudaMemcpy2DAsync(hres.data(), sizeof(double) * k, B.res.at(0), sizeof(double) * L.per,
@@ -720,12 +734,12 @@ cudaError_t si_solve(const SiBatch &b, double *work, double tol, int max_iter, c
   }
   res->iterations = it;
   if (b.has_trace) {
-    k_si_unshift<<<dim3(1, 1, P), 128, 0, s>>>(B.th, B.sig, m);
+    launch_pdl(k_si_unshift, dim3(1, 1, P), 128, 0, s, B.th, B.sig, m);
     nl += 1;
   }
   // the Ritz vectors end in the workspace's X slot
   if (!same(X, B.X)) {
-    k_si_copy<<<dim3(grid_1d(L.nm, P), 1, P), 256, 0, s>>>(X, B.X, L.nm);
+    launch_pdl(k_si_copy, dim3(grid_1d(L.nm, P), 1, P), 256, 0, s, X, B.X, L.nm);
     nl += 1;
   }
   *launches += nl;

@@ -34,6 +34,7 @@
 #include <utility>
 
 #include "eig_orth.cuh"
+#include "launch.cuh"
 #include "eig_si.cuh"
 #include "eig_small.cuh"
 
@@ -143,6 +144,7 @@ __device__ __forceinline__ float rsqrt_approx(float x) {
 template <int HM, int SPL, int RPG, int IA>
 __global__ void __launch_bounds__(1024, 1)
     k_rr_jacobi32(PSet Hin, int m, float floor_abs, int nang, int nA, PSet Vout, int *sweeps) {
+  pdl_enter();
   using C = J32Cfg<HM, SPL>;
   extern __shared__ __align__(16) float jsh[];
   float *Abuf = jsh;
@@ -404,6 +406,7 @@ struct MmOp {
 // cycles of one SM, about the launch's own latency: smaller tiles would only
 // re-read more, larger ones leave SMs idle.
 __global__ void __launch_bounds__(256) k_se_mm(MmOp op0, MmOp op1, int P, int m, float noise) {
+  pdl_enter();
   __shared__ double As[8][kSiMaxBlock + 1];   // op(A) rows i0..i0+7, all k
   __shared__ double Bs[8][kSiMaxBlock + 1];   // B' columns j0..j0+7, all k
   __shared__ double part[4][8][9];
@@ -507,6 +510,7 @@ size_t sparse_smem(int m) {
 
 __global__ void __launch_bounds__(kSparseThreads, 1)
     k_rr_sparse_jacobi(PSet Hin, int m, int floor_exp, PSet Wout, PSet theta, int *flag, int *rounds_out) {
+  pdl_enter();
   extern __shared__ double ssh[];
   const int ld = m + 1, maxsel = m / 2 + 1;
   double *H = ssh;                                  // row-major, symmetric part of Hin
@@ -629,6 +633,7 @@ __global__ void __launch_bounds__(kSparseThreads, 1)
 }
 
 __global__ void k_eig_one(PSet G, PSet X, PSet theta, int m, int P) {
+  pdl_enter();
   const int z = blockIdx.x * blockDim.x + threadIdx.x;
   if (z >= P) return;
   X.at(z)[0] = 1.0;
@@ -651,7 +656,8 @@ cudaError_t run_j32(PSet H, int m, float floor_abs, PSet V, int *sweeps, int P, 
   for (int ti = 0; 4 * ti < h; ++ti) tiles += (h + 7) / 8 - ti / 2;
   const int nA = nang + (tiles + IA - 1) / IA * 32;
   const int nV = ((m + RPG - 1) / RPG + 1) / 2 * 32;
-  kern<<<dim3(1, 1, P), nA + nV, J32Cfg<HM, SPL>::kSmem, s>>>(H, m, floor_abs, nang, nA, V, sweeps);
+  const size_t smem = J32Cfg<HM, SPL>::kSmem;
+  launch_pdl(kern, dim3(1, 1, P), nA + nV, smem, s, H, m, floor_abs, nang, nA, V, sweeps);
   return cudaGetLastError();
 }
 
@@ -692,7 +698,7 @@ cudaError_t small_eig(const SmallEig &a, cudaStream_t s, long long *launches) {
   };
   auto sym = [&](PSet A, PSet B, PSet Out) { return MmOp{A, B, B, B, Out, 1, 0, 1, 1.0, 0.0, m, m}; };   // A^T B
   auto mm1 = [&](const MmOp &o) {
-    k_se_mm<<<dim3(t, t, P), 256, 0, s>>>(o, o, P, m, noise);
+    launch_pdl(k_se_mm, dim3(t, t, P), 256, 0, s, o, o, P, m, noise);
     *launches += 1;
   };
   auto mm2 = [&](const MmOp &o, const MmOp &q) {
@@ -701,7 +707,7 @@ cudaError_t small_eig(const SmallEig &a, cudaStream_t s, long long *launches) {
       mm1(q);
       return;
     }
-    k_se_mm<<<dim3(t, t, 2 * P), 256, 0, s>>>(o, q, P, m, noise);
+    launch_pdl(k_se_mm, dim3(t, t, 2 * P), 256, 0, s, o, q, P, m, noise);
     *launches += 1;
   };
   // H is symmetric: H^T Y is read along its rows
@@ -738,7 +744,7 @@ cudaError_t small_eig(const SmallEig &a, cudaStream_t s, long long *launches) {
   }
   mm1(op(a.H, 1, X, 1.0, 0.0, Y));
   mm1(sym(X, Y, S));
-  k_rr_sparse_jacobi<<<dim3(1, 1, P), kSparseThreads, sparse_smem(m), s>>>(S, m, floor_exp, W, a.theta, a.flag,
+  launch_pdl(k_rr_sparse_jacobi, dim3(1, 1, P), kSparseThreads, sparse_smem(m), s, S, m, floor_exp, W, a.theta, a.flag,
                                                                           a.rounds);
   *launches += 1;
   mm1(MmOp{X, W, W, W, a.out, 0, 0, 0, 1.0, 0.0, a.rows, a.cols});
@@ -746,7 +752,7 @@ cudaError_t small_eig(const SmallEig &a, cudaStream_t s, long long *launches) {
 }
 
 cudaError_t eig_one(PSet G, PSet X, PSet theta, int m, int P, cudaStream_t s, long long *launches) {
-  k_eig_one<<<(P + 127) / 128, 128, 0, s>>>(G, X, theta, m, P);
+  launch_pdl(k_eig_one, (P + 127) / 128, 128, 0, s, G, X, theta, m, P);
   *launches += 1;
   return cudaGetLastError();
 }

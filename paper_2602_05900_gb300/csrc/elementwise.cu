@@ -5,6 +5,7 @@
 #include <math.h>
 
 #include "common.cuh"
+#include "launch.cuh"
 
 namespace hotrg {
 namespace {
@@ -42,6 +43,7 @@ __device__ double block_sum(double v) {
 // shared memory, so every global access is coalesced.  Each off-diagonal pair
 // (i, j) gets 0.5 (G_ij + G_ji) in both places; diagonal entries are unchanged.
 __global__ void __launch_bounds__(256) k_symmetrize_tiled(double *G, int n, long long sG) {
+  pdl_enter();
   __shared__ double A[32][33], B[32][33];
   G += blockIdx.y * sG;
   const int T = (n + 31) / 32;
@@ -77,6 +79,7 @@ __global__ void __launch_bounds__(256) k_symmetrize_tiled(double *G, int n, long
 // (problems side * per_side + i) to out[i sOut + side]
 __global__ void k_trace_diag(const double *G, int n, long long sG, double *out, long long sOut,
                              int per_side) {
+  pdl_enter();
   G += blockIdx.x * sG;
   double v = 0.0;
   for (int i = threadIdx.x; i < n; i += blockDim.x) v += G[(long long)i * n + i];
@@ -89,6 +92,7 @@ __global__ void k_trace_diag(const double *G, int n, long long sG, double *out, 
 }
 
 __global__ void k_identity(double *U, int n, long long sU) {
+  pdl_enter();
   U += blockIdx.y * sU;
   const long long total = (long long)n * n;
   for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < total;
@@ -100,6 +104,7 @@ __global__ void k_identity(double *U, int n, long long sU) {
 // like their bit patterns, so the combine is an integer atomicMax.
 __global__ void k_maxabs(const double *T, long long count, long long sT, unsigned long long *out,
                          long long sOut) {
+  pdl_enter();
   T += blockIdx.y * sT;
   double v = 0.0;
   for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < count;
@@ -115,6 +120,7 @@ __global__ void k_maxabs(const double *T, long long count, long long sT, unsigne
 __global__ void k_scale(double *T, long long count, long long sT, const unsigned long long *maxbits,
                         long long sMax, double *logsum, long long sLog, double inv_two_pow_n,
                         double *ln_c_out, long long sLnc, int *err) {
+  pdl_enter();
   const long long inst = blockIdx.y;
   T += inst * sT;
   const double c = __longlong_as_double((long long)maxbits[inst * sMax]);
@@ -138,6 +144,7 @@ __global__ void k_scale(double *T, long long count, long long sT, const unsigned
 // one block per instance
 __global__ void k_periodic_trace(const double *T, int Dx, int Dy, long long sT, double *out,
                                  long long sOut) {
+  pdl_enter();
   T += blockIdx.x * sT;
   double v = 0.0;
   const long long sx = (long long)Dx * Dy * Dy + (long long)Dy * Dy;  // step along x == x'
@@ -153,6 +160,7 @@ __global__ void k_periodic_trace(const double *T, int Dx, int Dy, long long sT, 
 // Tx[x][x'] = sum_y T[x][x'][y][y]: one thread per output element of every
 // instance (grid.y); the Dy summands of an element lie Dy + 1 apart.
 __global__ void k_trace_y(const double *T, double *Tx, int Dx, int Dy, long long sT) {
+  pdl_enter();
   const int e = blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= Dx * Dx) return;
   const double *t = T + blockIdx.y * sT + (long long)e * Dy * Dy;
@@ -165,6 +173,7 @@ __global__ void k_trace_y(const double *T, double *Tx, int Dx, int Dy, long long
 // the eigenvalues (a few dozen adds), so no separate launch or host round trip
 // is needed; block (0, i) also writes instance i's record and spectrum.
 __global__ void k_select(SelectArgs a) {
+  pdl_enter();
   __shared__ int s_side;
   __shared__ int s_arg;
   __shared__ double wbest[32];
@@ -233,6 +242,7 @@ __global__ void k_select(SelectArgs a) {
 __global__ void k_spectrum_no_cut(PSet w, int n, int desc, const double *tr, long long sTr,
                                   double *record, long long sRec, double *spectrum,
                                   long long sSpec) {
+  pdl_enter();
   const int inst = blockIdx.x;
   if (threadIdx.x == 0) {
     const double *wv = w.at(inst);
@@ -260,13 +270,13 @@ int grid_for(long long count, int threads, int batch) {
 cudaError_t symmetrize_trace(double *G, int n, long long sG, double *trace_out, long long sTr,
                              int batch, cudaStream_t s, int per_side) {
   const int T = (n + 31) / 32;
-  k_symmetrize_tiled<<<dim3(T * (T + 1) / 2, batch), 256, 0, s>>>(G, n, sG);
-  k_trace_diag<<<batch, 1024, 0, s>>>(G, n, sG, trace_out, sTr, per_side);
+  launch_pdl(k_symmetrize_tiled, dim3(T * (T + 1) / 2, batch), 256, 0, s, G, n, sG);
+  launch_pdl(k_trace_diag, batch, 1024, 0, s, G, n, sG, trace_out, sTr, per_side);
   return cudaGetLastError();
 }
 
 cudaError_t identity_isometry(double *U, int n, long long sU, int batch, cudaStream_t s) {
-  k_identity<<<dim3(grid_for((long long)n * n, 256, batch), batch), 256, 0, s>>>(U, n, sU);
+  launch_pdl(k_identity, dim3(grid_for((long long)n * n, 256, batch), batch), 256, 0, s, U, n, sU);
   return cudaGetLastError();
 }
 
@@ -279,34 +289,34 @@ cudaError_t maxabs_scale_log(double *T, long long count, long long sT, double *s
                                     batch, s);
   if (e != cudaSuccess) return e;
   const dim3 g(grid_for(count, 256, batch), batch);
-  k_maxabs<<<g, 256, 0, s>>>(T, count, sT, bits, sScratch);
-  k_scale<<<g, 256, 0, s>>>(T, count, sT, bits, sScratch, logsum, sLog, inv_two_pow_n, ln_c_out,
+  launch_pdl(k_maxabs, g, 256, 0, s, T, count, sT, bits, sScratch);
+  launch_pdl(k_scale, g, 256, 0, s, T, count, sT, bits, sScratch, logsum, sLog, inv_two_pow_n, ln_c_out,
                             sLnc, err_flag);
   return cudaGetLastError();
 }
 
 cudaError_t periodic_trace(const double *T, int Dx, int Dy, long long sT, double *out,
                            long long sOut, int batch, cudaStream_t s) {
-  k_periodic_trace<<<batch, 1024, 0, s>>>(T, Dx, Dy, sT, out, sOut);
+  launch_pdl(k_periodic_trace, batch, 1024, 0, s, T, Dx, Dy, sT, out, sOut);
   return cudaGetLastError();
 }
 
 cudaError_t trace_y(const double *T, double *Tx, int Dx, int Dy, long long sT, int batch,
                     cudaStream_t s) {
   const int n = Dx * Dx;
-  k_trace_y<<<dim3((n + 255) / 256, batch), 256, 0, s>>>(T, Tx, Dx, Dy, sT);
+  launch_pdl(k_trace_y, dim3((n + 255) / 256, batch), 256, 0, s, T, Tx, Dx, Dy, sT);
   return cudaGetLastError();
 }
 
 cudaError_t select_isometry(const SelectArgs &a, cudaStream_t s) {
-  k_select<<<dim3(a.Dn, a.batch), 256, 0, s>>>(a);
+  launch_pdl(k_select, dim3(a.Dn, a.batch), 256, 0, s, a);
   return cudaGetLastError();
 }
 
 cudaError_t spectrum_no_cut(PSet w, int n, int desc, const double *tr, long long sTr,
                             double *record, long long sRec, double *spectrum, long long sSpec,
                             int batch, cudaStream_t s) {
-  k_spectrum_no_cut<<<batch, 32, 0, s>>>(w, n, desc, tr, sTr, record, sRec, spectrum, sSpec);
+  launch_pdl(k_spectrum_no_cut, batch, 32, 0, s, w, n, desc, tr, sTr, record, sRec, spectrum, sSpec);
   return cudaGetLastError();
 }
 

@@ -8,6 +8,7 @@
 // GEMMs with at most 64 outputs and K >= 256 take a block-per-output dot kernel,
 // GEMMs with few 64 x 64 tiles a kernel of 16 x 16 or 8 x 8 tiles.
 #include "common.cuh"
+#include "launch.cuh"
 
 namespace hotrg {
 namespace {
@@ -16,6 +17,7 @@ constexpr int BM = 64, BN = 64, BK = 16, NT = 256;
 
 template <bool K_FAST_A, bool K_FAST_B>
 __global__ void __launch_bounds__(NT) k_gemm_f64(MappedGemm g) {
+  pdl_enter();
   __shared__ double As[2][BK][BM + 1];
   __shared__ double Bs[2][BK][BN + 1];
   __shared__ long long rowA[BM], rowB[BN];
@@ -135,6 +137,7 @@ __global__ void __launch_bounds__(NT) k_gemm_f64(MappedGemm g) {
 // legs are trivial, K = E^2): one block per output element, K strided over the
 // threads and combined by a fixed-order tree, so the result is deterministic.
 __global__ void __launch_bounds__(NT) k_dot_f64(MappedGemm g) {
+  pdl_enter();
   __shared__ double red[NT];
   const long long e = blockIdx.x;
   const long long m = e / g.N, n = e % g.N;
@@ -169,6 +172,7 @@ constexpr long long kDotMaxOutputs = 64, kDotMinK = 256;
 // 169 product of a chain step 21 us and 3.5 us.
 template <int TM, bool K_FAST_A, bool K_FAST_B>
 __global__ void __launch_bounds__(256) k_gemm_f64_small(MappedGemm g) {
+  pdl_enter();
   constexpr int KS = 256 / (TM * TM);             // k split over the threads
   constexpr int KC = TM == 8 ? 64 : 32;           // k per chunk
   constexpr int NL = TM * KC / 256;               // loads per thread, operand and chunk
@@ -240,10 +244,10 @@ cudaError_t launch_small(const MappedGemm &g, cudaStream_t s) {
                   (unsigned)(g.batch < 1 ? 1 : g.batch));
   if (grid.y > 65535u || grid.z > 65535u) return cudaErrorInvalidConfiguration;
   const bool ka = (g.ak.s0 == 1), kb = (g.bk.s0 == 1);
-  if (ka && kb) k_gemm_f64_small<TM, true, true><<<grid, 256, 0, s>>>(g);
-  else if (ka) k_gemm_f64_small<TM, true, false><<<grid, 256, 0, s>>>(g);
-  else if (kb) k_gemm_f64_small<TM, false, true><<<grid, 256, 0, s>>>(g);
-  else k_gemm_f64_small<TM, false, false><<<grid, 256, 0, s>>>(g);
+  if (ka && kb) launch_pdl(k_gemm_f64_small<TM, true, true>, grid, 256, 0, s, g);
+  else if (ka) launch_pdl(k_gemm_f64_small<TM, true, false>, grid, 256, 0, s, g);
+  else if (kb) launch_pdl(k_gemm_f64_small<TM, false, true>, grid, 256, 0, s, g);
+  else launch_pdl(k_gemm_f64_small<TM, false, false>, grid, 256, 0, s, g);
   return cudaGetLastError();
 }
 
@@ -253,7 +257,7 @@ cudaError_t gemm_f64(const MappedGemm &g, cudaStream_t s) {
   if (g.M <= 0 || g.N <= 0) return cudaSuccess;
   if ((long long)g.M * g.N <= kDotMaxOutputs && g.K >= kDotMinK) {
     if (g.batch > 65535) return cudaErrorInvalidConfiguration;
-    k_dot_f64<<<dim3((unsigned)(g.M * g.N), 1, (unsigned)(g.batch < 1 ? 1 : g.batch)), NT, 0, s>>>(g);
+    launch_pdl(k_dot_f64, dim3((unsigned)(g.M * g.N), 1, (unsigned)(g.batch < 1 ? 1 : g.batch)), NT, 0, s, g);
     return cudaGetLastError();
   }
   // 64 x 64 tiles once they give the 152 SMs two blocks each, 16 x 16 ones while
@@ -265,10 +269,10 @@ cudaError_t gemm_f64(const MappedGemm &g, cudaStream_t s) {
             (unsigned)(g.batch < 1 ? 1 : g.batch));
   if (grid.y > 65535u || grid.z > 65535u) return cudaErrorInvalidConfiguration;
   const bool ka = (g.ak.s0 == 1), kb = (g.bk.s0 == 1);
-  if (ka && kb) k_gemm_f64<true, true><<<grid, NT, 0, s>>>(g);
-  else if (ka) k_gemm_f64<true, false><<<grid, NT, 0, s>>>(g);
-  else if (kb) k_gemm_f64<false, true><<<grid, NT, 0, s>>>(g);
-  else k_gemm_f64<false, false><<<grid, NT, 0, s>>>(g);
+  if (ka && kb) launch_pdl(k_gemm_f64<true, true>, grid, NT, 0, s, g);
+  else if (ka) launch_pdl(k_gemm_f64<true, false>, grid, NT, 0, s, g);
+  else if (kb) launch_pdl(k_gemm_f64<false, true>, grid, NT, 0, s, g);
+  else launch_pdl(k_gemm_f64<false, false>, grid, NT, 0, s, g);
   return cudaGetLastError();
 }
 

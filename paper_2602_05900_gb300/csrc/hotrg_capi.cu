@@ -38,6 +38,7 @@
 #include "common.cuh"
 #include "dev_pool.cuh"
 #include "eig_si.cuh"
+#include "launch.cuh"
 #include "tc_exact.cuh"
 #include "tc_gemm.cuh"
 #include "tc_path.cuh"
@@ -1026,7 +1027,10 @@ hotrg_status hotrg_step(hotrg_ctx *c, hotrg_dir dir) {
     th.reserve(c->groups.size());
     const int step = c->nsteps;
     for (size_t i = 0; i < c->groups.size(); ++i)
-      th.emplace_back([c, &st, i, dir, step] { st[i] = step_group(c, *c->groups[i], dir, step); });
+      th.emplace_back([c, &st, i, dir, step] {
+        pdl_allowed() = false;
+        st[i] = step_group(c, *c->groups[i], dir, step);
+      });
     for (auto &t : th) t.join();
     cudaEventDestroy(start);
     for (auto &g : c->groups) CK_CUDA(c, cudaStreamSynchronize(g->stream));

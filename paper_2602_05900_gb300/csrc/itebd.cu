@@ -29,6 +29,7 @@
 #include <vector>
 
 #include "common.cuh"
+#include "launch.cuh"
 #include "dev_pool.cuh"
 #include "eig_si.cuh"
 #include "hotrg.h"
@@ -43,6 +44,7 @@ constexpr int kItebdMaxD = kSiMaxBlock / 2;    // 2 D_b <= 96: the direct Jacobi
 // phit[i][A][B][m] = sum_ab g[AB][ab] phi[i][a][b][m], theta = lam[i] phit
 __global__ void k_itebd_gate(const double *phi, double *phit, double *theta, const double *gates,
                              const double *lam, int Dl, int Dr, long long sM, long long sL) {
+  pdl_enter();
   const long long z = blockIdx.y;
   phi += z * sM;
   phit += z * sM;
@@ -71,6 +73,7 @@ __global__ void k_itebd_gate(const double *phi, double *phit, double *theta, con
 // rnorm = 1 / sqrt(sum_{k < Dn} w_k), the factor that keeps the state normalised
 __global__ void k_itebd_schmidt(PSet w, int m, int Dn, double *lam, long long sL, double *disc,
                                 double *rnorm, int *err) {
+  pdl_enter();
   const int z = blockIdx.x;
   const double *wz = w.at(z);
   __shared__ double keep;
@@ -93,6 +96,7 @@ __global__ void k_itebd_schmidt(PSet w, int m, int Dn, double *lam, long long sL
 
 // P' *= rnorm of its chain
 __global__ void k_itebd_scale(double *P, long long count, long long sT, const double *rnorm) {
+  pdl_enter();
   const long long z = blockIdx.y;
   const double r = rnorm[z];
   for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < count;
@@ -102,6 +106,7 @@ __global__ void k_itebd_scale(double *P, long long count, long long sT, const do
 
 // Q'[j][B][m] = Y[(B m), j] for j < Dn: the first Dn columns of the column-major Y
 __global__ void k_itebd_take(PSet Y, long long count, double *Q, long long sT) {
+  pdl_enter();
   const long long z = blockIdx.y;
   const double *y = Y.at((int)z);
   for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < count;
@@ -112,6 +117,7 @@ __global__ void k_itebd_take(PSet Y, long long count, double *Q, long long sT) {
 // one block per chain: <theta|h|theta> / <theta|theta>, theta = lam[i] phi[i][a][b][m]
 __global__ void k_itebd_energy(const double *phi, const double *lam, const double *hs, int Dl, int Dr,
                                long long sM, long long sL, double *out, int slot) {
+  pdl_enter();
   const long long z = blockIdx.x;
   phi += z * sM;
   lam += z * sL;
@@ -227,7 +233,7 @@ hotrg_status itebd_update(hotrg_itebd *c) {
   MappedGemm g1{kPhys * Dl, kPhys * Dr, Dm, P, map1(Dm), map1(1), Q, map1(1), map1(kPhys * Dr),
                 c->phi, map1(kPhys * Dr), map1(1), G, c->sT, c->sT, c->sM};
   ICK(c, gemm_f64(g1, st));
-  k_itebd_gate<<<dim3(grid1((long long)Dl * Dr), G), 256, 0, st>>>(c->phi, c->phit, c->theta, c->gates,
+  launch_pdl(k_itebd_gate, dim3(grid1((long long)Dl * Dr), G), 256, 0, st, c->phi, c->phit, c->theta, c->gates,
                                                                    c->l[c->iL], Dl, Dr, c->sM, c->sL);
   ICK(c, cudaGetLastError());
   // rho = theta^T theta, symmetrised
@@ -263,7 +269,7 @@ hotrg_status itebd_update(hotrg_itebd *c) {
   long long nl = 0;
   ICK(c, jacobi_full(sb, c->si_work, st, &nl));
   const SiOut o = si_outputs(c->si_work, G, n, sb.m);
-  k_itebd_schmidt<<<G, 64, 0, st>>>(o.theta, sb.m, Dn, c->l[iN], c->sL, c->disc, c->rnorm, c->err);
+  launch_pdl(k_itebd_schmidt, G, 64, 0, st, o.theta, sb.m, Dn, c->l[iN], c->sL, c->disc, c->rnorm, c->err);
   ICK(c, cudaGetLastError());
   // the new basis V' = V W (or W cold), column-major n x n, into Vn
   const long long ys = o.X.b1 - o.X.b0;
@@ -272,7 +278,7 @@ hotrg_status itebd_update(hotrg_itebd *c) {
                   G, c->sM, ys, c->sM};
     ICK(c, gemm_f64(w3, st));
   } else {
-    k_itebd_take<<<dim3(grid1((long long)n * n), G), 256, 0, st>>>(o.X, (long long)n * n, c->Vn, c->sM);
+    launch_pdl(k_itebd_take, dim3(grid1((long long)n * n), G), 256, 0, st, o.X, (long long)n * n, c->Vn, c->sM);
     ICK(c, cudaGetLastError());
   }
   std::swap(c->Vb[par], c->Vn);
@@ -282,10 +288,10 @@ hotrg_status itebd_update(hotrg_itebd *c) {
   MappedGemm g3{kPhys * Dl, Dn, n, c->phit, map1(n), map1(1), Y.b0, map1(n), map1(1), Pn, map1(Dn),
                 map1(1), G, c->sM, c->sM, c->sT};
   ICK(c, gemm_f64(g3, st));
-  k_itebd_scale<<<dim3(grid1((long long)kPhys * Dl * Dn), G), 256, 0, st>>>(Pn, (long long)kPhys * Dl * Dn,
+  launch_pdl(k_itebd_scale, dim3(grid1((long long)kPhys * Dl * Dn), G), 256, 0, st, Pn, (long long)kPhys * Dl * Dn,
                                                                            c->sT, c->rnorm);
   ICK(c, cudaGetLastError());
-  k_itebd_take<<<dim3(grid1((long long)Dn * n), G), 256, 0, st>>>(Y, (long long)Dn * n, Qn, c->sT);
+  launch_pdl(k_itebd_take, dim3(grid1((long long)Dn * n), G), 256, 0, st, Y, (long long)Dn * n, Qn, c->sT);
   ICK(c, cudaGetLastError());
   // the next bond: (P, Q, lam) <- (Q', P', lam'); lam_other <- lam
   c->iP = iQn;
@@ -405,12 +411,12 @@ hotrg_status hotrg_itebd_energy(hotrg_itebd *c, double *out_n) {
   MappedGemm g1{kPhys * o, kPhys * o, m, P, map1(m), map1(1), Q, map1(1), map1(kPhys * o), c->phi,
                 map1(kPhys * o), map1(1), G, c->sT, c->sT, c->sM};
   ICK(c, gemm_f64(g1, st));
-  k_itebd_energy<<<G, 256, 0, st>>>(c->phi, c->l[c->iL], c->hs, o, o, c->sM, c->sL, c->energy, 0);
+  launch_pdl(k_itebd_energy, G, 256, 0, st, c->phi, c->l[c->iL], c->hs, o, o, c->sM, c->sL, c->energy, 0);
   ICK(c, cudaGetLastError());
   MappedGemm g2{kPhys * m, kPhys * m, o, Q, map1(o), map1(1), P, map1(1), map1(kPhys * m), c->phi,
                 map1(kPhys * m), map1(1), G, c->sT, c->sT, c->sM};
   ICK(c, gemm_f64(g2, st));
-  k_itebd_energy<<<G, 256, 0, st>>>(c->phi, c->l[c->iO], c->hs, m, m, c->sM, c->sL, c->energy, 1);
+  launch_pdl(k_itebd_energy, G, 256, 0, st, c->phi, c->l[c->iO], c->hs, m, m, c->sM, c->sL, c->energy, 1);
   ICK(c, cudaGetLastError());
   std::vector<double> h(2 * (size_t)G);
   ICK(c, cudaMemcpyAsync(h.data(), c->energy, sizeof(double) * h.size(), cudaMemcpyDeviceToHost, st));

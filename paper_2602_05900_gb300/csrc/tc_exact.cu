@@ -35,6 +35,7 @@
 #include <algorithm>
 
 #include "tc_exact.cuh"
+#include "launch.cuh"
 #include "tcgen05.cuh"
 
 namespace cg = cooperative_groups;
@@ -202,6 +203,7 @@ __global__ void __launch_bounds__(256) k_xs_split(PSet src, int R, int K, IdxMap
                                                   __nv_bfloat16 *dst, int pitch, long long bstride,
                                                   double *scale, long long sstride, PSet kscale,
                                                   int kmode) {
+  pdl_enter();
   const int z = blockIdx.z;
   const int r = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
   if (r >= R) return;
@@ -220,6 +222,7 @@ __global__ void __launch_bounds__(kXsRowThreads) k_xs_split_row(PSet src, int R,
                                                                 __nv_bfloat16 *dst, int pitch,
                                                                 long long bstride, double *scale,
                                                                 long long sstride, PSet kscale, int kmode) {
+  pdl_enter();
   const int z = blockIdx.z, r = blockIdx.x;
   const double *a = src.at(z), *ks = kmode ? kscale.at(z) : nullptr;
   const long long ro = map_off32(rm, r);
@@ -246,6 +249,7 @@ __global__ void __launch_bounds__(256) k_xs_split_staged(PSet src, int R, int K,
                                                          IdxMap km, __nv_bfloat16 *dst, int pitch,
                                                          long long bstride, double *scale,
                                                          long long sstride, PSet kscale, int kmode) {
+  pdl_enter();
   __shared__ double tile[32][kXsStagedK + 1];
   const int z = blockIdx.z;
   const int r0 = blockIdx.x * 32;
@@ -333,6 +337,8 @@ __global__ void __launch_bounds__(kXsThreads, 1)
   __syncthreads();
   fence_after();
   const uint32_t tmem = tmem_base_sh;
+  // the operands are the kernel before's: everything above needs none of them
+  pdl_enter();
 
   if (warp == 0 && lane == 0) {
     int i = 0;
@@ -551,13 +557,14 @@ cudaError_t launch_xs(const XsOperand &A, const XsOperand &B, int M, int N, int 
   cfg.blockDim = dim3(kXsThreads, 1, 1);
   cfg.dynamicSmemBytes = C::SMEM;
   cfg.stream = s;
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeClusterDimension;
   attr[0].val.clusterDim.x = csplit;
   attr[0].val.clusterDim.y = 1;
   attr[0].val.clusterDim.z = 1;
+  attr[1] = pdl_attribute();
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = 2;
   return cudaLaunchKernelEx(&cfg, k_xs_gemm<S, BN>, ta, tb, M, N, K, kbp, ntn, csplit, o, err, wait_limit(),
                             stall);
 }
@@ -609,7 +616,7 @@ cudaError_t xs_split_scaled(PSet src, IdxMap rm, IdxMap km, PSet kscale, int kmo
     switch (d.S) {
 #define XS_STAGED_CASE(SS)                                                                    \
   case SS:                                                                                    \
-    k_xs_split_staged<SS><<<gs, 256, 0, s>>>(src, d.rows, d.K, rm, km, dst, d.pitch, d.bstride, \
+    launch_pdl(k_xs_split_staged<SS>, gs, 256, 0, s, src, d.rows, d.K, rm, km, dst, d.pitch, d.bstride, \
                                              d.scale, d.sstride, kscale, kmode);              \
     break;
       XS_STAGED_CASE(1) XS_STAGED_CASE(2) XS_STAGED_CASE(3) XS_STAGED_CASE(4)
@@ -623,7 +630,7 @@ cudaError_t xs_split_scaled(PSet src, IdxMap rm, IdxMap km, PSet kscale, int kmo
     switch (d.S) {
 #define XS_ROW_CASE(SS)                                                                       \
   case SS:                                                                                    \
-    k_xs_split_row<SS><<<gr, kXsRowThreads, 0, s>>>(src, d.rows, d.K, rm, km, dst, d.pitch, d.bstride,  \
+    launch_pdl(k_xs_split_row<SS>, gr, kXsRowThreads, 0, s, src, d.rows, d.K, rm, km, dst, d.pitch, d.bstride,  \
                                           d.scale, d.sstride, kscale, kmode);                 \
     break;
       XS_ROW_CASE(1) XS_ROW_CASE(2) XS_ROW_CASE(3) XS_ROW_CASE(4)
@@ -635,7 +642,7 @@ cudaError_t xs_split_scaled(PSet src, IdxMap rm, IdxMap km, PSet kscale, int kmo
   switch (d.S) {
 #define XS_SPLIT_CASE(SS)                                                                     \
   case SS:                                                                                    \
-    k_xs_split<SS><<<g, 256, 0, s>>>(src, d.rows, d.K, rm, km, dst, d.pitch, d.bstride,       \
+    launch_pdl(k_xs_split<SS>, g, 256, 0, s, src, d.rows, d.K, rm, km, dst, d.pitch, d.bstride,       \
                                      d.scale, d.sstride, kscale, kmode);                      \
     break;
     XS_SPLIT_CASE(1) XS_SPLIT_CASE(2) XS_SPLIT_CASE(3) XS_SPLIT_CASE(4)
@@ -678,6 +685,7 @@ namespace {
 
 __global__ void k_xs_sum_parts(const double *parts, int nparts, long long pstride, int M, int N,
                                double *C, long long ldc) {
+  pdl_enter();
   const long long total = (long long)M * N;
   for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < total;
        e += (long long)gridDim.x * blockDim.x) {
@@ -694,7 +702,7 @@ cudaError_t xs_sum_parts(const double *parts, int nparts, long long pstride, int
   const long long total = (long long)M * N;
   long long b = (total + 255) / 256;
   if (b > 152 * 8) b = 152 * 8;
-  k_xs_sum_parts<<<(int)(b < 1 ? 1 : b), 256, 0, s>>>(parts, nparts, pstride, M, N, C, ldc);
+  launch_pdl(k_xs_sum_parts, (int)(b < 1 ? 1 : b), 256, 0, s, parts, nparts, pstride, M, N, C, ldc);
   return cudaGetLastError();
 }
 
@@ -706,6 +714,7 @@ namespace {
 // C(cm(m) + cn(n)) of instance z = sum_p parts[((p * batch + z) * M + m) * N + n]
 __global__ void k_xs_scatter_parts(const double *parts, int nparts, int batch, int M, int N,
                                    double *C, IdxMap cm, IdxMap cn, long long bC) {
+  pdl_enter();
   const int z = blockIdx.y;
   const long long mn = (long long)M * N;
   for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < mn;
@@ -753,7 +762,7 @@ cudaError_t gemm_xs(const MappedGemm &g, int S, const XsWork &w, int *err_flag, 
   long long blocks = (mn + 255) / 256;
   const long long cap = (152LL * 8 + batch - 1) / batch;
   if (blocks > cap) blocks = cap;
-  k_xs_scatter_parts<<<dim3((unsigned)(blocks < 1 ? 1 : blocks), batch), 256, 0, s>>>(
+  launch_pdl(k_xs_scatter_parts, dim3((unsigned)(blocks < 1 ? 1 : blocks), batch), 256, 0, s, 
       w.parts, ks, batch, g.M, g.N, g.C, g.cm, g.cn, g.bC);
   return cudaGetLastError();
 }
