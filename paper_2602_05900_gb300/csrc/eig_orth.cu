@@ -49,14 +49,16 @@ __device__ __forceinline__ double inv_sqrt(double x) { return rsqrt_fp64(x); }
 // Factor and inverse in one elimination, 256 threads as 16 x 16, thread (ty, tx)
 // holding the entries (ty + 16 u, tx + 16 v) in registers: element (i, k) is the
 // scaled matrix for k >= i and the growing L^-1 (L = R^T) for k < i, which
-// starts at zero.  Step j: row j goes through shared memory (two buffers, one
-// barrier per step); its pivot, its part right of the diagonal (which, the
-// matrix being symmetric, also holds the multipliers of the rows below) and its
-// L^-1 part (k < j, and 1 at k = j) update every row i > j.  At the end the
-// L^-1 rows over the square roots of the pivots are the columns of
+// starts at zero.  A step takes two pivots j, j + 1 (m is even): rows j and j + 1
+// go through shared memory (two buffers, one barrier per step); every thread
+// eliminates row j from its part of row j + 1, and both update every row below.
+// A row's part right of the diagonal also holds (the matrix being symmetric) the
+// multipliers of the rows below, its L^-1 part is k < j, and 1 at k = j.  At the
+// end the L^-1 rows over the square roots of the pivots are the columns of
 // W = diag(d) R^-1 = diag(d) L^-T.  Which row values an entry takes depends on
 // its tile alone off the diagonal tiles (right of them the matrix part, left of
-// them the L^-1 part), so the updates carry no tests.
+// them the L^-1 part), so the updates carry no tests.  One pivot per barrier took
+// 14 us at m = 48 and 41 at m = 88, two take 10 and 28 us.
 //
 // Nearly dependent columns break the unshifted factorisation; attempt a adds
 // shift(a) to the unit diagonal.  cmat(i, k), i <= k: the unscaled matrix.
@@ -83,10 +85,11 @@ __device__ void chol_inverse(Cmat cmat, Shift shift, int attempts, int m, double
         e[u][v] = (i <= k && k < m) ? cmat(i, k) * (d[i] * d[k]) + (i == k ? sh : T(0)) : T(0);
       }
     bad = false;
-    for (int j = 0; j < m; ++j) {
-      T *buf = rowbuf + (j & 1) * LD;
-      if (ty == (j & 15)) {
+    for (int j = 0; j < m; j += 2) {
+      T *b0 = rowbuf + (j & 2) * LD, *b1 = b0 + LD;
+      if (ty == (j & 15) || ty == (j & 15) + 1) {          // j is even: both rows lie in one tile
         const int ju = j >> 4;
+        T *buf = ty == (j & 15) ? b0 : b1;
 #pragma unroll
         for (int v = 0; v < U; ++v) {
           T x = e[0][v];             // selected, not indexed: e stays in registers
@@ -96,28 +99,42 @@ __device__ void chol_inverse(Cmat cmat, Shift shift, int attempts, int m, double
         }
       }
       __syncthreads();
-      const T p = buf[j];
-      if (!(p > T(0)) || !isfinite(p)) {       // the same for every thread
+      const T p0 = b0[j], c01 = b0[j + 1];
+      const T r0 = reciprocal(p0), l = c01 * r0;           // row j + 1 loses l times row j
+      const T p1 = fma(-l, c01, b1[j + 1]);
+      if (!(p0 > T(0)) || !isfinite(p0) || !(p1 > T(0)) || !isfinite(p1)) {   // the same for every thread
         bad = true;
         break;
       }
-      if (tid == 0) piv[j] = p;
-      const T rinv = reciprocal(p);
-      T right[U], left[U], diag[U];
+      if (tid == 0) {
+        piv[j] = p0;
+        piv[j + 1] = p1;
+      }
+      const T r1 = reciprocal(p1);
+      T right0[U], left0[U], diag0[U], right1[U], left1[U], diag1[U];
 #pragma unroll
       for (int v = 0; v < U; ++v) {
         const int k = tx + 16 * v;
-        right[v] = buf[k];
-        left[v] = k < j ? right[v] : k == j ? T(1) : T(0);
-        diag[v] = tx >= ty ? right[v] : left[v];
+        const T x0 = b0[k], x1 = b1[k];
+        right0[v] = x0;
+        left0[v] = k < j ? x0 : k == j ? T(1) : T(0);
+        diag0[v] = tx >= ty ? right0[v] : left0[v];
+        right1[v] = fma(-l, x0, x1);
+        left1[v] = fma(-l, left0[v], k < j ? x1 : k == j + 1 ? T(1) : T(0));
+        diag1[v] = tx >= ty ? right1[v] : left1[v];
       }
 #pragma unroll
       for (int u = 0; u < U; ++u) {
         if (j >= 16 * u + 15) continue;        // every row of the tile is done
         const int i = ty + 16 * u;
-        const T mult = i > j ? -(buf[i] * rinv) : T(0);
+        const T x0 = b0[i];
+        const T m0 = i > j ? -(x0 * r0) : T(0), m1 = i > j + 1 ? -(fma(-l, x0, b1[i]) * r1) : T(0);
 #pragma unroll
-        for (int v = 0; v < U; ++v) e[u][v] = fma(mult, v > u ? right[v] : v < u ? left[v] : diag[v], e[u][v]);
+        for (int v = 0; v < U; ++v) {
+          const T a0 = v > u ? right0[v] : v < u ? left0[v] : diag0[v];
+          const T a1 = v > u ? right1[v] : v < u ? left1[v] : diag1[v];
+          e[u][v] = fma(m1, a1, fma(m0, a0, e[u][v]));
+        }
       }
     }
     __syncthreads();
@@ -157,7 +174,7 @@ struct Shift64 {
 template <int U>
 constexpr size_t gram_chol_smem(int m) {
   return ((size_t)m * m) * (sizeof(float2) + sizeof(float)) +
-         (size_t)(kSlab * (16 * U + 1) + 4 * 16 * U) * sizeof(float);
+         (size_t)(kSlab * (16 * U + 1) + 6 * 16 * U) * sizeof(float);
 }
 
 template <int U>
@@ -169,8 +186,8 @@ __global__ void __launch_bounds__(256) __cluster_dims__(kOrthCluster, 1, 1)
   float2 *part = gsh;                                              // m x m, upper triangle
   float *tot = reinterpret_cast<float *>(part + (size_t)m * m);    // m x m, upper triangle (rank 0)
   float *slab = tot + (size_t)m * m;                               // kSlab x (LD + 1)
-  float *rowbuf = slab + kSlab * (LD + 1);                         // 2 x LD
-  float *d = rowbuf + 2 * LD, *piv = d + LD;
+  float *rowbuf = slab + kSlab * (LD + 1);                         // 2 x 2 x LD
+  float *d = rowbuf + 4 * LD, *piv = d + LD;
   cg::cluster_group cluster = cg::this_cluster();
   const int rank = (int)cluster.block_rank(), z = blockIdx.z;
   const double *y = Yin.at(z);
@@ -265,35 +282,42 @@ __global__ void __launch_bounds__(256) __cluster_dims__(kOrthCluster, 1, 1)
 template <int U>
 __global__ void __launch_bounds__(256) k_chol32(PSet Cin, int m, float shift, PSet Wout, int *flag) {
   pdl_enter();
-  __shared__ float rowbuf[2 * 16 * U], d[16 * U], piv[16 * U];
+  __shared__ float rowbuf[4 * 16 * U], d[16 * U], piv[16 * U];
   const double *C = Cin.at(blockIdx.z);
   chol_inverse<float, U>([&](int i, int k) { return to_f32(C[(size_t)i * m + k]); }, Shift32{shift}, 2, m,
                          Wout.at(blockIdx.z), flag, rowbuf, d, piv);
 }
 
-// the same in FP64; only_if (optional): run for problem z only if only_if.at(z)[2] != 0
+// the same in FP64; only_if (optional): run for problem z only if only_if.at(z)[2]
+// != 0, and without a first shift if it is 1
 template <int U>
 __global__ void __launch_bounds__(256) k_chol64(PSet Cin, int m, double shift, PSet Wout, int *flag, PSet only_if) {
   pdl_enter();
-  if (only_if.b0 && only_if.at(blockIdx.z)[2] == 0.0) return;
-  __shared__ double rowbuf[2 * 16 * U], d[16 * U], piv[16 * U];
+  const double cond = only_if.b0 ? only_if.at(blockIdx.z)[2] : 2.0;
+  if (cond == 0.0) return;
+  __shared__ double rowbuf[4 * 16 * U], d[16 * U], piv[16 * U];
   const double *C = Cin.at(blockIdx.z);
-  chol_inverse<double, U>([&](int i, int k) { return C[(size_t)i * m + k]; }, Shift64{shift}, 3, m,
+  chol_inverse<double, U>([&](int i, int k) { return C[(size_t)i * m + k]; }, Shift64{cond == 1.0 ? 0.0 : shift}, 3, m,
                           Wout.at(blockIdx.z), flag, rowbuf, d, piv);
 }
 
-// Cp[c] = A[rows of chunk c]^T B[same rows] in FP64 (m x m, row-major), 256
-// threads as 16 x 16 with entries (ty + 16 u, tx + 16 v): every thread works
-// whatever m is.  sym: entries u <= v only (all of the upper triangle).
+// Cp[c] = A[rows of chunk c]^T B[same rows] in FP64 (m x m, row-major; the second
+// product's chunks follow the first's), 256 threads as 16 x 16 with entries
+// (ty + 16 u, tx + 16 v): every thread works whatever m is.  Of a symmetric
+// product, entries u <= v only (all of the upper triangle).
 template <int U>
-__global__ void __launch_bounds__(256) k_si_gram(PSet A, PSet B, PSet Cp, int n, int m, int sym, int rows) {
+__global__ void __launch_bounds__(256) k_si_gram(PSet A, PSet B0, PSet B1, PSet Cp, int n, int m, int P, int rows) {
   pdl_enter();
   constexpr int LD = 16 * U;
   __shared__ double As[16][LD + 1];
   __shared__ double Bs[16][LD + 1];
-  const int z = blockIdx.z, c = blockIdx.x;
+  // problem z's products A^T B0 and, from blockIdx.z = P on, A^T B1; one with
+  // B == A is symmetric
+  const bool second = (int)blockIdx.z >= P;
+  const int z = second ? (int)blockIdx.z - P : (int)blockIdx.z, c = blockIdx.x;
   const double *a = A.at(z);
-  const double *b = B.at(z);
+  const double *b = (second ? B1 : B0).at(z);
+  const bool sym = a == b;
   const int r0 = c * rows, r1 = min(n, r0 + rows);
   const int ty = threadIdx.x >> 4, tx = threadIdx.x & 15;
   double acc[U][U];
@@ -310,24 +334,39 @@ __global__ void __launch_bounds__(256) k_si_gram(PSet A, PSet B, PSet Cp, int n,
       if (!sym) Bs[ii][j] = in ? b[(size_t)j * n + row] : 0.0;
     }
     __syncthreads();
-    const double(*Br)[LD + 1] = sym ? As : Bs;
+    // a test of sym at every FMA would cost as much as the FMAs it saves
+    if (sym) {
 #pragma unroll 2
-    for (int ii = 0; ii < 16; ++ii) {
-      double av[U], bv[U];
+      for (int ii = 0; ii < 16; ++ii) {
+        double av[U], bv[U];
 #pragma unroll
-      for (int u = 0; u < U; ++u) {
-        av[u] = As[ii][ty + 16 * u];
-        bv[u] = Br[ii][tx + 16 * u];
+        for (int u = 0; u < U; ++u) {
+          av[u] = As[ii][ty + 16 * u];
+          bv[u] = As[ii][tx + 16 * u];
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+#pragma unroll
+          for (int v = u; v < U; ++v) acc[u][v] = fma(av[u], bv[v], acc[u][v]);
       }
+    } else {
+#pragma unroll 2
+      for (int ii = 0; ii < 16; ++ii) {
+        double av[U], bv[U];
 #pragma unroll
-      for (int u = 0; u < U; ++u)
+        for (int u = 0; u < U; ++u) {
+          av[u] = As[ii][ty + 16 * u];
+          bv[u] = Bs[ii][tx + 16 * u];
+        }
 #pragma unroll
-        for (int v = 0; v < U; ++v)
-          if (!sym || u <= v) acc[u][v] = fma(av[u], bv[v], acc[u][v]);
+        for (int u = 0; u < U; ++u)
+#pragma unroll
+          for (int v = 0; v < U; ++v) acc[u][v] = fma(av[u], bv[v], acc[u][v]);
+      }
     }
     __syncthreads();
   }
-  double *out = Cp.at(z) + (size_t)c * m * m;
+  double *out = Cp.at(z) + (size_t)(second ? gridDim.x + c : c) * m * m;
 #pragma unroll
   for (int u = 0; u < U; ++u)
 #pragma unroll
@@ -340,17 +379,22 @@ __global__ void __launch_bounds__(256) k_si_gram(PSet A, PSet B, PSet Cp, int n,
 // C = sum over the chunks (fixed order), symmetrised.  A block takes 64 entries,
 // four threads to an entry, each with its own run of chunks: the sum is bound
 // by load latency, so many loads are kept in flight.
-__global__ void __launch_bounds__(256) k_si_gram_reduce(PSet Cp, PSet C, int nchunks, int m, int sym) {
+// blockIdx.z as in k_si_gram; sym0, sym1: whether the products are symmetric.
+__global__ void __launch_bounds__(256) k_si_gram_reduce(PSet Cp, PSet C0, PSet C1, int nchunks, int m, int P, int sym0,
+                                                        int sym1) {
   pdl_enter();
   __shared__ double sum[4][64];
-  const int z = blockIdx.z, l = threadIdx.x & 63, g = threadIdx.x >> 6;
+  const bool second = (int)blockIdx.z >= P;
+  const int z = second ? (int)blockIdx.z - P : (int)blockIdx.z, l = threadIdx.x & 63, g = threadIdx.x >> 6;
+  const bool sym = second ? sym1 : sym0;
+  const PSet &C = second ? C1 : C0;
   const long long mm = (long long)m * m;
   const int e = blockIdx.x * 64 + l, a = e / m, b = e % m;
   const bool in = e < m * m && a <= b;
   const int per = (nchunks + 3) / 4, c0 = g * per, c1 = min(nchunks, c0 + per);
   double s = 0.0;
   if (in) {
-    const double *src = Cp.at(z);
+    const double *src = Cp.at(z) + (second ? nchunks * mm : 0);
     const long long o = (long long)a * m + b, ot = (long long)b * m + a;
     double v[4] = {0.0, 0.0, 0.0, 0.0}, w[4] = {0.0, 0.0, 0.0, 0.0};
     int c = c0;
@@ -383,14 +427,17 @@ __global__ void __launch_bounds__(256) k_si_gram_reduce(PSet Cp, PSet C, int nch
 // column groups forwards and backwards in turn (equal shares).  FP64-bound:
 // RT is chosen so that the CTAs fill the SMs.
 template <int RT>
-__global__ void __launch_bounds__(256) k_si_rotate(PSet A, PSet W, PSet Out, int n, int m, int tri) {
+__global__ void __launch_bounds__(256) k_si_rotate(PSet A0, PSet A1, PSet W, PSet Out0, PSet Out1, int n, int m, int P,
+                                                   int tri) {
   pdl_enter();
   extern __shared__ double rsh[];
   double *As = rsh;                       // [column][RT]
   double *Ws = rsh + (size_t)m * RT;      // [column][m + 1]
   constexpr int CPW = 32 / RT;
-  const int z = blockIdx.z, i0 = blockIdx.x * RT;
-  const double *a = A.at(z), *w = W.at(z);
+  const bool second = (int)blockIdx.z >= P;      // A0 W, and from blockIdx.z = P on A1 W
+  const int z = second ? (int)blockIdx.z - P : (int)blockIdx.z, i0 = blockIdx.x * RT;
+  const double *a = (second ? A1 : A0).at(z), *w = W.at(z);
+  double *out = (second ? Out1 : Out0).at(z);
   for (int e = threadIdx.x; e < m * RT; e += 256) {
     const int j = e / RT, r = e % RT;
     As[e] = i0 + r < n ? a[(size_t)j * n + i0 + r] : 0.0;
@@ -411,7 +458,7 @@ __global__ void __launch_bounds__(256) k_si_rotate(PSet A, PSet W, PSet Out, int
     double acc = 0.0;
 #pragma unroll 8
     for (int j = 0; j < jend; ++j) acc = fma(As[j * RT + r], Ws[c * (m + 1) + j], acc);
-    if (g * CPW + cl < m && i0 + r < n) Out.at(z)[(size_t)c * n + i0 + r] = acc;
+    if (g * CPW + cl < m && i0 + r < n) out[(size_t)c * n + i0 + r] = acc;
   }
 }
 
@@ -431,7 +478,8 @@ cudaError_t launch_gram_chol(PSet Y, int n, int m, float shift, PSet W, int *fla
 }
 
 template <int RT>
-cudaError_t launch_rotate(PSet A, PSet W, PSet Out, int n, int m, bool tri, int P, cudaStream_t s) {
+cudaError_t launch_rotate(PSet A0, PSet A1, PSet W, PSet Out0, PSet Out1, int count, int n, int m, bool tri, int P,
+                          cudaStream_t s) {
   static bool done = false;
   if (!done) {
     cudaError_t e = cudaFuncSetAttribute(k_si_rotate<RT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -442,8 +490,8 @@ cudaError_t launch_rotate(PSet A, PSet W, PSet Out, int n, int m, bool tri, int 
   // a plain launch: started early, its blocks would be dealt out while the factor's
   // cluster still holds SMs, and the others would get two (D = 48 job: 57.6 ms
   // started early, 55.5 ms like this)
-  k_si_rotate<RT><<<dim3((n + RT - 1) / RT, 1, P), 256, sizeof(double) * m * (RT + m + 1), s>>>(A, W, Out, n, m,
-                                                                                               tri ? 1 : 0);
+  k_si_rotate<RT><<<dim3((n + RT - 1) / RT, 1, count * P), 256, sizeof(double) * m * (RT + m + 1), s>>>(
+      A0, A1, W, Out0, Out1, n, m, P, tri ? 1 : 0);
   return cudaGetLastError();
 }
 
@@ -451,30 +499,36 @@ cudaError_t launch_rotate(PSet A, PSet W, PSet Out, int n, int m, bool tri, int 
 
 cudaError_t gram_reduce(PSet part, PSet out, int chunks, int m, bool sym, int P, cudaStream_t s,
                         long long *launches) {
-  launch_pdl(k_si_gram_reduce, dim3((m * m + 63) / 64, 1, P), 256, 0, s, part, out, chunks, m, sym ? 1 : 0);
+  launch_pdl(k_si_gram_reduce, dim3((m * m + 63) / 64, 1, P), 256, 0, s, part, out, out, chunks, m, P, sym ? 1 : 0, 0);
   *launches += 1;
   return cudaGetLastError();
 }
 
-cudaError_t gram64(PSet A, PSet B, bool sym, int n, int m, PSet part, PSet out, int P, cudaStream_t s,
-                   long long *launches) {
+cudaError_t gram64(PSet A, PSet B0, PSet out0, const PSet *B1, const PSet *out1, int n, int m, PSet part, int P,
+                   cudaStream_t s, long long *launches) {
   // chunks of 16 rows until two CTAs per SM have one; longer ones beyond that
   // keep the partials (m x m doubles per chunk) few
-  const int want = std::max(1, std::min(kGramChunks, (304 + P - 1) / P));
+  const int count = B1 && 2 * P <= 65535 ? 2 : 1;
+  const int want = std::max(1, std::min(kGramChunks / count, (304 + P * count - 1) / (P * count)));
   const int rows = std::max(16, ((n + want - 1) / want + 15) / 16 * 16);
   const int chunks = (n + rows - 1) / rows;
-  if (chunks > kGramChunks || m > kSiMaxBlock) return cudaErrorInvalidValue;
-  const dim3 g(chunks, 1, P);
+  if (chunks * count > kGramChunks || m > kSiMaxBlock) return cudaErrorInvalidValue;
+  const PSet b1 = count == 2 ? *B1 : B0, o1 = count == 2 ? *out1 : out0;
+  const dim3 g(chunks, 1, count * P);
   switch (tile_of(m)) {
-    case 2: launch_pdl(k_si_gram<2>, g, 256, 0, s, A, B, part, n, m, sym, rows); break;
-    case 3: launch_pdl(k_si_gram<3>, g, 256, 0, s, A, B, part, n, m, sym, rows); break;
-    case 4: launch_pdl(k_si_gram<4>, g, 256, 0, s, A, B, part, n, m, sym, rows); break;
-    case 5: launch_pdl(k_si_gram<5>, g, 256, 0, s, A, B, part, n, m, sym, rows); break;
-    default: launch_pdl(k_si_gram<6>, g, 256, 0, s, A, B, part, n, m, sym, rows); break;
+    case 2: launch_pdl(k_si_gram<2>, g, 256, 0, s, A, B0, b1, part, n, m, P, rows); break;
+    case 3: launch_pdl(k_si_gram<3>, g, 256, 0, s, A, B0, b1, part, n, m, P, rows); break;
+    case 4: launch_pdl(k_si_gram<4>, g, 256, 0, s, A, B0, b1, part, n, m, P, rows); break;
+    case 5: launch_pdl(k_si_gram<5>, g, 256, 0, s, A, B0, b1, part, n, m, P, rows); break;
+    default: launch_pdl(k_si_gram<6>, g, 256, 0, s, A, B0, b1, part, n, m, P, rows); break;
   }
-  *launches += 1;
+  auto same = [](const PSet &x, const PSet &y) { return x.b0 == y.b0 && x.b1 == y.b1 && x.stride == y.stride; };
+  launch_pdl(k_si_gram_reduce, dim3((m * m + 63) / 64, 1, count * P), 256, 0, s, part, out0, o1, chunks, m, P,
+             same(A, B0) ? 1 : 0, same(A, b1) ? 1 : 0);
+  *launches += 2;
   cudaError_t e = cudaGetLastError();
-  return e ? e : gram_reduce(part, out, chunks, m, sym, P, s, launches);
+  if (e || !B1 || count == 2) return e;
+  return gram64(A, *B1, *out1, nullptr, nullptr, n, m, part, P, s, launches);
 }
 
 cudaError_t cholqr32_factor(PSet Y, int n, int m, float shift, PSet W, int *flag, int P, cudaStream_t s,
@@ -519,16 +573,20 @@ cudaError_t chol64(PSet C, int m, double shift, PSet W, int *flag, PSet only_if,
   return cudaGetLastError();
 }
 
-cudaError_t rotate_basis(PSet A, PSet W, PSet Out, int n, int m, bool tri, int P, cudaStream_t s,
-                         long long *launches) {
+cudaError_t rotate_basis(PSet A0, PSet Out0, const PSet *A1, const PSet *Out1, PSet W, int n, int m, bool tri, int P,
+                         cudaStream_t s, long long *launches) {
   if (m > kSiMaxBlock) return cudaErrorInvalidValue;
+  const int count = A1 && 2 * P <= 65535 ? 2 : 1;
+  const PSet a1 = count == 2 ? *A1 : A0, o1 = count == 2 ? *Out1 : Out0;
   *launches += 1;
   // the tallest tile that still gives most of the 152 SMs a CTA (each CTA reads
   // all of W)
-  const long long rows = (long long)n * P;
-  if (rows >= 16 * 120) return launch_rotate<16>(A, W, Out, n, m, tri, P, s);
-  if (rows >= 8 * 120) return launch_rotate<8>(A, W, Out, n, m, tri, P, s);
-  return launch_rotate<4>(A, W, Out, n, m, tri, P, s);
+  const long long rows = (long long)n * P * count;
+  const cudaError_t e = rows >= 16 * 120  ? launch_rotate<16>(A0, a1, W, Out0, o1, count, n, m, tri, P, s)
+                        : rows >= 8 * 120 ? launch_rotate<8>(A0, a1, W, Out0, o1, count, n, m, tri, P, s)
+                                          : launch_rotate<4>(A0, a1, W, Out0, o1, count, n, m, tri, P, s);
+  if (e || !A1 || count == 2) return e;
+  return rotate_basis(*A1, *Out1, nullptr, nullptr, W, n, m, tri, P, s, launches);
 }
 
 }  // namespace hotrg

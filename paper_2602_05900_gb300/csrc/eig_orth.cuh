@@ -39,10 +39,10 @@ __device__ inline double rsqrt_fp64(double x) {
 // Number of row chunks whose partial Gram matrices gram64 writes (m x m doubles
 // each, at most kGramChunks per problem).
 constexpr int kGramChunks = 256;
-// out = A^T B (m x m, symmetrised; A, B n x m column-major); sym: A == B.
-// part: kGramChunks m x m slots of problem z.
-cudaError_t gram64(PSet A, PSet B, bool sym, int n, int m, PSet part, PSet out, int P, cudaStream_t s,
-                   long long *launches);
+// out0 = A^T B0 and (optional) out1 = A^T B1 (m x m, symmetrised; A, B n x m
+// column-major).  part: kGramChunks m x m slots of problem z.
+cudaError_t gram64(PSet A, PSet B0, PSet out0, const PSet *B1, const PSet *out1, int n, int m, PSet part, int P,
+                   cudaStream_t s, long long *launches);
 // out = sum of `chunks` m x m partials of A^T B, symmetrised (sym: only their
 // upper triangles are valid).
 cudaError_t gram_reduce(PSet part, PSet out, int chunks, int m, bool sym, int P, cudaStream_t s,
@@ -57,13 +57,14 @@ cudaError_t cholqr32_factor(PSet Y, int n, int m, float shift, PSet W, int *flag
 // ... or from a given C:
 cudaError_t chol32(PSet C, int m, float shift, PSet W, int *flag, int P, cudaStream_t s, long long *launches);
 
-// The same in FP64 (W to FP64 accuracy); for problem z only if only_if.at(z)[2] != 0
-// (only_if.b0 null: always).
+// The same in FP64 (W to FP64 accuracy); for problem z only if only_if.at(z)[2] != 0,
+// and without a shift at first if it is 1 (only_if.b0 null: always, shifted).
 cudaError_t chol64(PSet C, int m, double shift, PSet W, int *flag, PSet only_if, int P, cudaStream_t s,
                    long long *launches);
 
-// Out = A W (A, Out n x m column-major, W m x m column-major; tri: W upper triangular)
-cudaError_t rotate_basis(PSet A, PSet W, PSet Out, int n, int m, bool tri, int P, cudaStream_t s,
-                         long long *launches);
+// Out0 = A0 W and (optional) Out1 = A1 W (A, Out n x m column-major, W m x m
+// column-major; tri: W upper triangular)
+cudaError_t rotate_basis(PSet A0, PSet Out0, const PSet *A1, const PSet *Out1, PSet W, int n, int m, bool tri, int P,
+                         cudaStream_t s, long long *launches);
 
 }  // namespace hotrg

@@ -183,41 +183,44 @@ __global__ void k_si_sum_split(PSet part, PSet out, int S, long long nm, PSet X,
   if (shift && blockIdx.x == 0 && threadIdx.x == 0) sig.at(z)[0] = sg;
 }
 
-// flags.at(z)[2] = 1 if max |C_ij - delta_ij| > 1/4 (the Newton-Schulz
-// iteration for C^-1/2 from I is then not to be trusted), else 0.
-__global__ void k_rr_far_from_identity(PSet C, int m, PSet flags) {
+// Start of W = C^-1/2: W1 = (3 I - C) / 2, and how far C is from I (largest entry
+// of C - I): flags[2] = 0 up to kNearChol (Newton-Schulz converges to rounding in
+// two steps: the norm of C - I is at most 96 times that, 3/8 of its square the error
+// of W1, and a step squares it again), 1 up to 1/4, else 2; flags[3] = 1 where
+// one step is enough.
+constexpr float kNearChol = 1e-4f, kNearOne = 3e-6f;
+
+__global__ void __launch_bounds__(1024) k_rr_start(PSet Cin, int m, PSet W, PSet flags) {
   pdl_enter();
   const int z = blockIdx.z;
-  double v = 0.0;
+  const double *C = Cin.at(z);
+  float far = 0.0f;
   for (int e = threadIdx.x; e < m * m; e += blockDim.x) {
-    const double d = C.at(z)[e] - ((e % m == e / m) ? 1.0 : 0.0);
-    v = fmax(v, (d == d) ? fabs(d) : INFINITY);
+    const double one = (e % m == e / m) ? 1.0 : 0.0, c = C[e];
+    W.at(z)[e] = fma(-0.5, c, 1.5 * one);
+    const float d = fabsf(to_f32(c - one));
+    far = fmaxf(far, d == d ? d : INFINITY);
   }
-  for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(0xffffffffu, v, o));
-  __shared__ double part[32];
-  if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = v;
+  for (int o = 16; o > 0; o >>= 1) far = fmaxf(far, __shfl_xor_sync(0xffffffffu, far, o));
+  __shared__ float part[32];
+  if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = far;
   __syncthreads();
   if (threadIdx.x == 0) {
-    double w = 0.0;
-    for (int i = 0; i < (int)(blockDim.x >> 5); ++i) w = fmax(w, part[i]);
-    flags.at(z)[2] = (w > 0.25) ? 1.0 : 0.0;
+    for (int i = 0; i < (int)(blockDim.x >> 5); ++i) far = fmaxf(far, part[i]);
+    flags.at(z)[2] = far > 0.25f ? 2.0 : far > kNearChol ? 1.0 : 0.0;
+    flags.at(z)[3] = far <= kNearOne ? 1.0 : 0.0;
   }
-}
-
-// Out = a A + b I for m x m matrices of every problem z.
-__global__ void k_rr_axpi(PSet A, double a, double b, PSet Out, int m) {
-  pdl_enter();
-  const int z = blockIdx.z;
-  for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < m * m; e += gridDim.x * blockDim.x)
-    Out.at(z)[e] = a * A.at(z)[e] + ((e % m == e / m) ? b : 0.0);
 }
 
 // Out = op(A) (bs B + bd I) for m x m column-major FP64 matrices of every
 // problem z (op(A) = A^T if ta).  One CTA per 8 x 8 output tile; the sum over
 // k is split four ways across the CTA's threads and combined in a fixed order.
+// unless (optional): nothing is done for problem z where unless.at(z)[3] != 0;
+// copy (optional): receives the result too.
 __global__ void __launch_bounds__(256) k_rr_mm(PSet A, int ta, PSet B, double bs, double bd,
-                                               PSet Out, int m) {
+                                               PSet Out, int m, PSet unless, PSet copy) {
   pdl_enter();
+  if (unless.b0 && unless.at(blockIdx.z)[3] != 0.0) return;
   __shared__ double As[8][kSiMaxBlock + 1];   // op(A) rows i0..i0+7, all k
   __shared__ double Bs[8][kSiMaxBlock + 1];   // B columns j0..j0+7, all k
   __shared__ double part[4][8][9];
@@ -239,8 +242,11 @@ __global__ void __launch_bounds__(256) k_rr_mm(PSet A, int ta, PSet B, double bs
   __syncthreads();
   if (threadIdx.x < 64) {
     const int i = i0 + ti, j = j0 + tj;
-    if (i < m && j < m)
-      Out.at(z)[(size_t)j * m + i] = (part[0][ti][tj] + part[1][ti][tj]) + (part[2][ti][tj] + part[3][ti][tj]);
+    if (i < m && j < m) {
+      const double v = (part[0][ti][tj] + part[1][ti][tj]) + (part[2][ti][tj] + part[3][ti][tj]);
+      Out.at(z)[(size_t)j * m + i] = v;
+      if (copy.b0) copy.at(z)[(size_t)j * m + i] = v;
+    }
   }
 }
 
@@ -416,7 +422,7 @@ cudaError_t si_solve(const SiBatch &b, double *work, double tol, int max_iter, c
     return cudaErrorInvalidValue;
   const Layout L = layout(P, n, m);
   Bufs B = carve(work, P, L);
-  PSet X = B.X, Y = B.Y, Z = B.Z;
+  PSet X = B.X, Y = B.Y, Z = B.Z, Y2 = B.Yp;   // Y2: free but during an FP64 SIMT product
   const dim3 gz(1, 1, P);
   const int chunk = ((n + L.S - 1) / L.S + 15) / 16 * 16;
   const double shift = 11.0 * ((double)n * m + (double)m * (m + 1)) * 1.1102230246251565e-16;
@@ -498,29 +504,32 @@ cudaError_t si_solve(const SiBatch &b, double *work, double tol, int max_iter, c
       nl += 3;
       return cudaSuccess;
     }
-    return rotate_basis(src, W, dst, n, m, tri != 0, P, s, &nl);
+    return rotate_basis(src, dst, nullptr, nullptr, W, n, m, tri != 0, P, s, &nl);
   };
-  // C = A^T B (m x m), symmetrised
-  auto gram = [&](PSet A, PSet Bm, bool sym, PSet out) -> cudaError_t {
+  // C = A^T A (m x m), and with Bm out2 = A^T Bm, symmetrised
+  auto gram = [&](PSet A, PSet out, const PSet *Bm, const PSet *out2) -> cudaError_t {
     if (xs_small) {
       const XsOperand a = xs_slot(L.oSa, L.oSasc, m, n);       // columns of A
       const XsOperand bb = xs_slot(L.oSb, L.oSbsc, m, n);      // columns of B
       cudaError_t r;
-      if ((r = xs_split(A, map1(n), map1(1), a, s))) return r;
-      const bool one = same(A, Bm);
-      if (!one && (r = xs_split(Bm, map1(n), map1(1), bb, s))) return r;
-      if ((r = xs_gemm(a, one ? a : bb, m, m, n, B.Cp.b0, map1(m), map1(1), L.per, 1, 0, b.err, s)))
+      if ((r = xs_split(A, map1(n), map1(1), a, s)) ||
+          (r = xs_gemm(a, a, m, m, n, B.Cp.b0, map1(m), map1(1), L.per, 1, 0, b.err, s)))
         return r;
-      nl += one ? 2 : 3;
-      return gram_reduce(B.Cp, out, 1, m, false, P, s, &nl);
+      nl += 2;
+      if ((r = gram_reduce(B.Cp, out, 1, m, false, P, s, &nl)) || !Bm) return r;
+      if ((r = xs_split(*Bm, map1(n), map1(1), bb, s)) ||
+          (r = xs_gemm(a, bb, m, m, n, B.Cp.b0, map1(m), map1(1), L.per, 1, 0, b.err, s)))
+        return r;
+      nl += 2;
+      return gram_reduce(B.Cp, *out2, 1, m, false, P, s, &nl);
     }
-    return gram64(A, Bm, sym, n, m, B.Cp, out, P, s, &nl);
+    return gram64(A, A, out, Bm, out2, n, m, B.Cp, P, s, &nl);
   };
   // one CholeskyQR pass with an FP32 factorisation: dst = src W
   auto cholqr32 = [&](PSet src, PSet dst, float sh) -> cudaError_t {
     cudaError_t r;
     if (xs_small) {
-      if ((r = gram(src, src, true, B.C)) || (r = chol32(B.C, m, sh, B.W, B.flag, P, s, &nl))) return r;
+      if ((r = gram(src, B.C, nullptr, nullptr)) || (r = chol32(B.C, m, sh, B.W, B.flag, P, s, &nl))) return r;
     } else if ((r = cholqr32_factor(src, n, m, sh, B.W, B.flag, P, s, &nl))) {
       return r;
     }
@@ -528,7 +537,7 @@ cudaError_t si_solve(const SiBatch &b, double *work, double tol, int max_iter, c
   };
   // one CholeskyQR pass in FP64 (robust for any conditioning with the shift)
   auto cholqr64 = [&](PSet src, PSet dst, double sh) -> cudaError_t {
-    cudaError_t r = gram(src, src, true, B.C);
+    cudaError_t r = gram(src, B.C, nullptr, nullptr);
     if (r) return r;
     if ((r = chol64(B.C, m, sh, B.W, B.flag, PSet{nullptr, nullptr, 0}, P, s, &nl))) return r;
     return rot(src, B.W, dst, 1);
@@ -621,38 +630,47 @@ cudaError_t si_solve(const SiBatch &b, double *work, double tol, int max_iter, c
       auto slot = [&](int i) { return PSet{B.Cp.b0 + i * L.mm, B.Cp.b1 + i * L.mm, B.Cp.stride}; };
       PSet Wn = slot(0), Tn = slot(1);
       const PSet Ck = slot(2), Rr = slot(3);
-      const dim3 gmm((m + 7) / 8, (m + 7) / 8, P), g1(grid_1d(L.mm, P), 1, P);
-      if ((e = gram(X, X, true, B.W))) return e;   // C0 (B.W until small_eig)
-      if ((e = gram(X, Y, false, B.C))) return e;  // X^T Y
-      launch_pdl(k_rr_axpi, g1, 256, 0, s, B.W, -0.5, 1.5, Wn, m);       // W1 = (3I - C0) / 2
+      const dim3 gmm((m + 7) / 8, (m + 7) / 8, P);
+      const PSet always{nullptr, nullptr, 0};
+      if ((e = gram(X, B.W, &Y, &B.C))) return e;   // C0 (B.W until small_eig) and X^T Y
+      launch_pdl(k_rr_start, gz, 1024, 0, s, B.W, m, Wn, B.sig);
       nl += 1;
-      for (int ns = 0; ns < 3; ++ns) {                              // W <- W (3I - W^T C0 W) / 2
-        launch_pdl(k_rr_mm, gmm, 256, 0, s, B.W, 0, Wn, 1.0, 0.0, Tn, m);   // C0 W
-        launch_pdl(k_rr_mm, gmm, 256, 0, s, Wn, 1, Tn, 1.0, 0.0, Ck, m);    // W^T C0 W
-        launch_pdl(k_rr_mm, gmm, 256, 0, s, Wn, 0, Ck, -0.5, 1.5, Tn, m);   // next W
-        std::swap(Wn, Tn);
-        nl += 3;
-      }
-      // where X is far from orthonormal (nearly dependent columns at a first
-      // check), W comes instead from a shifted FP64 Cholesky of C0 (X W is
-      // then orthonormal for any conditioning the shift allows)
-      launch_pdl(k_rr_far_from_identity, gz, 256, 0, s, B.W, m, B.sig);
-      nl += 1;
+      // W <- W (3I - W^T C0 W) / 2 twice, the second time only where it is needed
+      // (Tn holds the result either way)
+      const PSet T2 = slot(4 + kSmallEigSlots);
+      launch_pdl(k_rr_mm, gmm, 256, 0, s, B.W, 0, Wn, 1.0, 0.0, Ck, m, always, always);   // C0 W
+      launch_pdl(k_rr_mm, gmm, 256, 0, s, Wn, 1, Ck, 1.0, 0.0, Rr, m, always, always);    // W^T C0 W
+      launch_pdl(k_rr_mm, gmm, 256, 0, s, Wn, 0, Rr, -0.5, 1.5, Tn, m, always, T2);
+      launch_pdl(k_rr_mm, gmm, 256, 0, s, B.W, 0, T2, 1.0, 0.0, Ck, m, B.sig, always);
+      launch_pdl(k_rr_mm, gmm, 256, 0, s, T2, 1, Ck, 1.0, 0.0, Rr, m, B.sig, always);
+      launch_pdl(k_rr_mm, gmm, 256, 0, s, T2, 0, Rr, -0.5, 1.5, Tn, m, B.sig, always);
+      nl += 6;
+      std::swap(Wn, Tn);
+      // where X is further from orthonormal (nearly dependent columns at a first
+      // check), W comes instead from an FP64 Cholesky of C0, shifted where C0 is far
+      // from I (X W is then orthonormal for any conditioning the shift allows)
       if ((e = chol64(B.W, m, shift, Wn, B.flag, B.sig, P, s, &nl))) return e;
-      launch_pdl(k_rr_mm, gmm, 256, 0, s, B.C, 0, Wn, 1.0, 0.0, Tn, m);     // (X^T Y) W
-      launch_pdl(k_rr_mm, gmm, 256, 0, s, Wn, 1, Tn, 1.0, 0.0, Ck, m);      // H = W^T X^T Y W
+      launch_pdl(k_rr_mm, gmm, 256, 0, s, B.C, 0, Wn, 1.0, 0.0, Tn, m, always, always);     // (X^T Y) W
+      launch_pdl(k_rr_mm, gmm, 256, 0, s, Wn, 1, Tn, 1.0, 0.0, Ck, m, always, always);      // H = W^T X^T Y W
       nl += 2;
       if ((e = cudaGetLastError())) return e;
       const SmallEig se{P, m, Ck, slot(4), false, false, B.W, m, m, B.th, B.flag, B.sweeps, B.flag + 3};
       if ((e = small_eig(se, s, &nl))) return e;                    // H = Z Theta Z^T (Z in B.W)
-      launch_pdl(k_rr_mm, gmm, 256, 0, s, Wn, 0, B.W, 1.0, 0.0, Rr, m);     // R = W Z
+      launch_pdl(k_rr_mm, gmm, 256, 0, s, Wn, 0, B.W, 1.0, 0.0, Rr, m, always, always);     // R = W Z
       nl += 1;
-      if ((e = rot(X, Rr, Z, 0))) return e;
-      std::swap(X, Z);
-      if ((e = rot(Y, Rr, Z, 0))) return e;
-      std::swap(Y, Z);
+      if (xs_small) {
+        if ((e = rot(X, Rr, Z, 0))) return e;
+        std::swap(X, Z);
+        if ((e = rot(Y, Rr, Z, 0))) return e;
+        std::swap(Y, Z);
+      } else {
+        // X -> Z and Y -> the first K-part slot in one launch, then renamed
+        if ((e = rotate_basis(X, Z, &Y, &Y2, Rr, n, m, false, P, s, &nl))) return e;
+        std::swap(X, Z);
+        std::swap(Y, Y2);
+      }
       launch_pdl(k_si_residual, dim3(k, 1, P), 256, 0, s, X, Y, B.th, B.res, B.sig, b.has_trace ? 1 : 0, n, k);
-      nl += 2;
+      nl += 1;
       ++res->rr;
       if ((e = cudaMemcpy2DAsync(hres.data(), sizeof(double) * k, B.res.at(0), sizeof(double) * L.per,
                                  sizeof(double) * k, P, cudaMemcpyDeviceToHost, s)))
