@@ -43,7 +43,12 @@ namespace hotrg {
 namespace {
 
 constexpr int kSplitMax = 8;     // split-K partials of G X
-constexpr double kXsSmallWork = 32.0 * 1024 * 1024;   // FP64 FMAs of one n x m x m product batch
+// FP64 FMAs of one n x m x m product batch from which its rotations and Gram
+// matrices run as exact-slice products: few problems are latency bound and stay
+// with the single FP64 launches longer (24-instance sweep: 150.4 ms with 2^25 for
+// all, 142.4 ms like this; with 2^22 for all the one pair of a D = 32 run, 2^22.2,
+// took 65 ms against 50)
+constexpr double kXsSmallWork = 0x1p25, kXsBatchWork = 0x1p23;
 constexpr int kSiSmallBatch = 8;      // problems up to which the solve is latency bound
 constexpr double kSiFloorTol = 1e-10;  // residuals accepted once they stop decreasing
 constexpr int kSiSlowIters = 24;       // iterations after which a residual below the floor is accepted
@@ -432,10 +437,10 @@ cudaError_t si_solve(const SiBatch &b, double *work, double tol, int max_iter, c
   // Gram matrices X^T Y) run as exact-slice tensor-core GEMMs (FP64-grade, see
   // tc_exact.cuh) unless the caller asked for the FP64 SIMT kernels.  The
   // n x m x m rotations and Gram matrices go to the tensor cores only when the
-  // batch makes them FP64-throughput bound (P n m^2 >= kXsSmallWork); below
+  // batch makes them FP64-throughput bound; below
   // that the single SIMT launch beats the slice-and-multiply sequence.
   const bool xs = b.xs;
-  const bool xs_small = xs && (double)P * n * m * m >= kXsSmallWork;
+  const bool xs_small = xs && (double)P * n * m * m >= (P > kSiSmallBatch ? kXsBatchWork : kXsSmallWork);
   XsOperand gs{};
   // slices of a row-major (rows x K) view of problem z's buffer at src
   auto xs_slot = [&](long long off, long long scoff, int rows, int K) {
