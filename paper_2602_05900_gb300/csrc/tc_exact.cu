@@ -737,14 +737,39 @@ void xs_gemm_needs(int M, int N, int K, int S, int batch, long long need[5]) {
   need[4] = ks > 1 ? (long long)ks * batch * M * N : 0;
 }
 
+bool xs_fits(int M, int N, int K, int S, int batch, const XsWork &w) {
+  long long need[5];
+  xs_gemm_needs(M, N, K, S, batch, need);
+  return need[0] <= w.cap_a && need[1] <= w.cap_b && need[2] <= w.cap_sa && need[3] <= w.cap_sb &&
+         need[4] <= w.cap_parts;
+}
+
+bool syrk_xs_fits(int M, int K, int batch, int S, const XsWork &w) {
+  return M > 0 && K > 0 && batch <= kXsMaxBatch && xs_min_split(K) == 1 && xs_fits(M, 0, K, S, batch, w);
+}
+
+cudaError_t syrk_xs(const MappedGemm *g, int count, int S, const XsWork &w, int *err_flag, cudaStream_t s) {
+  const int M = g[0].M, K = g[0].K, G = g[0].batch < 1 ? 1 : g[0].batch;
+  if (count < 1 || !syrk_xs_fits(M, K, count * G, S, w))
+    return cudaErrorInvalidValue;
+  const long long ea = xs_elems(M, K, S);
+  cudaError_t e;
+  for (int v = 0; v < count; ++v) {
+    const MappedGemm &q = g[v];
+    if (q.M != M || q.N != M || q.K != K || q.C != g[0].C + v * G * g[0].bC) return cudaErrorInvalidValue;
+    const PSet pa{const_cast<double *>(q.A), const_cast<double *>(q.A) + q.bA, 2 * q.bA};
+    const XsOperand a{static_cast<__nv_bfloat16 *>(w.sa) + v * G * ea, w.sca + (long long)v * G * M, M, K, xs_pitch(K), S,
+                      G, ea, M};
+    if ((e = xs_split(pa, q.am, q.ak, a, s))) return e;
+  }
+  const XsOperand all{w.sa, w.sca, M, K, xs_pitch(K), S, count * G, ea, M};
+  return xs_gemm(all, all, M, M, K, g[0].C, g[0].cm, g[0].cn, g[0].bC, 1, 0, err_flag, s);
+}
+
 cudaError_t gemm_xs(const MappedGemm &g, int S, const XsWork &w, int *err_flag, cudaStream_t s) {
   if (g.M <= 0 || g.N <= 0) return cudaSuccess;
   const int batch = g.batch < 1 ? 1 : g.batch;
-  long long need[5];
-  xs_gemm_needs(g.M, g.N, g.K, S, batch, need);
-  if (need[0] > w.cap_a || need[1] > w.cap_b || need[2] > w.cap_sa || need[3] > w.cap_sb ||
-      need[4] > w.cap_parts)
-    return cudaErrorInvalidValue;
+  if (!xs_fits(g.M, g.N, g.K, S, batch, w)) return cudaErrorInvalidValue;
   const long long ea = xs_elems(g.M, g.K, S), eb = xs_elems(g.N, g.K, S);
   XsOperand a{w.sa, w.sca, g.M, g.K, xs_pitch(g.K), S, batch, ea, g.M};
   XsOperand b{w.sb, w.scb, g.N, g.K, xs_pitch(g.K), S, batch, eb, g.N};

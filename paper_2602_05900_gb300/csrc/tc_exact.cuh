@@ -28,6 +28,7 @@ namespace hotrg {
 
 constexpr int kXsBits = 6;        // bits per slice digit
 constexpr int kXsMaxK = 2336;     // longest K part of one CTA (multiple of 32) with 7 2^10 K < 2^24
+constexpr int kXsMaxBatch = 65535;  // instances of one launch (grid limit)
 constexpr int kXsMaxSumK = 8192;  // longest K of one launch: the integer sums stay below 2^63
 constexpr int kXsMaxSlices = 8;
 constexpr int kXsStagedK = 128;  // strided-K operands up to this K are sliced through shared memory
@@ -107,5 +108,15 @@ void xs_gemm_needs(int M, int N, int K, int S, int batch, long long need[5]);
 // gathered and sliced, K is split into exact parts, the result is written in
 // FP64 through g's output maps.
 cudaError_t gemm_xs(const MappedGemm &g, int S, const XsWork &w, int *err_flag, cudaStream_t s);
+
+// Whether gemm_xs of that size fits the scratch.
+bool xs_fits(int M, int N, int K, int S, int batch, const XsWork &w);
+
+// `count` products C_v(m, n) = sum_k A_v(m, k) A_v(n, k) of the same sizes and output
+// maps (g[v].B is not read), C_v = g[0].C + v * batch * bC: every operand is sliced
+// once and all products are one launch.  The scratch has to fit count * batch
+// instances of A (syrk_xs_fits with that batch; K <= kXsMaxSumK).
+bool syrk_xs_fits(int M, int K, int batch, int S, const XsWork &w);
+cudaError_t syrk_xs(const MappedGemm *g, int count, int S, const XsWork &w, int *err_flag, cudaStream_t s);
 
 }  // namespace hotrg
