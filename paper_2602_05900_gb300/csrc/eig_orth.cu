@@ -301,6 +301,152 @@ __global__ void __launch_bounds__(256) k_chol64(PSet Cin, int m, double shift, P
                           Wout.at(blockIdx.z), flag, rowbuf, d, piv);
 }
 
+// Sums of two FP32 numbers, ~2^-44 of the value: twelve FP32 instructions for a
+// multiply-add (Dekker's product by fused multiply-add, Knuth's sum), where the
+// FP64 unit takes the time of 64 for one.
+struct F2 { float h, l; };
+__device__ __forceinline__ F2 f2_norm(float h, float l) {
+  const float s = __fadd_rn(h, l);
+  return F2{s, __fsub_rn(l, __fsub_rn(s, h))};
+}
+__device__ __forceinline__ F2 f2_mul(F2 a, F2 b) {
+  const float p = __fmul_rn(a.h, b.h);
+  return F2{p, fmaf(a.h, b.l, fmaf(a.l, b.h, fmaf(a.h, b.h, -p)))};
+}
+// c + a b, the low part not yet normalised
+__device__ __forceinline__ F2 f2_fma(F2 a, F2 b, F2 c) {
+  const F2 p = f2_mul(a, b);
+  const float s = __fadd_rn(c.h, p.h), t = __fsub_rn(s, c.h);
+  const float r = __fadd_rn(__fsub_rn(c.h, __fsub_rn(s, t)), __fsub_rn(p.h, t));
+  return F2{s, __fadd_rn(c.l, __fadd_rn(p.l, r))};
+}
+__device__ __forceinline__ F2 f2_neg(F2 a) { return F2{-a.h, -a.l}; }
+__device__ __forceinline__ F2 f2_reciprocal(F2 p) {
+  const float r = __frcp_rn(p.h);
+  return F2{r, __fmul_rn(r, fmaf(-p.l, r, fmaf(-p.h, r, 1.0f)))};
+}
+__device__ __forceinline__ F2 f2_rsqrt(F2 p) {          // one Newton step y + y (1 - p y^2) / 2
+  const float y = rsqrtf(p.h);
+  const float q = __fmul_rn(p.h, y), ql = fmaf(p.h, y, -q);
+  return F2{y, 0.5f * y * (fmaf(-q, y, 1.0f) - y * fmaf(p.l, y, ql))};
+}
+
+// Cholesky factor (see lr_factor), laid out and stepped like chol_inverse without
+// the inverse: the rows of R = L^T go to shared memory once each, as they become
+// pivots, so a step (two pivots) has one barrier and no buffer is reused.  The
+// square roots of the pivots are taken at the end, off the chain of steps.  L only
+// has to be one matrix whose columns the caller rotates: what it misses of H is
+// seen, and removed, by the FP64 passes after it.  In FP64 the kernel was bound by
+// that unit (87 us at m = 60; 29 us in pairs of FP32 numbers); FP32 alone takes
+// the caller four more sweeps, which cost as much as FP64.
+template <int U>
+__global__ void __launch_bounds__(256) k_lr_factor(PSet Hin, int m, PSet Lout, PSet Bout) {
+  pdl_enter();
+  constexpr int LD = 16 * U;
+  extern __shared__ __align__(16) F2 lr_rows[];       // m rows of LD: row j as it was published
+  __shared__ F2 rs[LD], ls[LD / 2];                   // pivot, then 1 / sqrt of it; row j + 1's multiple of row j
+  __shared__ int s_exp;
+  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
+  const double *H = Hin.at(blockIdx.z);
+  double *L = Lout.at(blockIdx.z), *B = Bout.at(blockIdx.z);
+  if (tid == 0) s_exp = 0;
+  __syncthreads();
+  double x[U][U];
+  int ex = 0;
+#pragma unroll
+  for (int u = 0; u < U; ++u)
+#pragma unroll
+    for (int v = u; v < U; ++v) {
+      const int i = ty + 16 * u, k = tx + 16 * v;
+      x[u][v] = i <= k && k < m ? H[(size_t)i * m + k] : 0.0;
+      ex = max(ex, (__double2hiint(x[u][v]) >> 20) & 0x7FF);
+    }
+  for (int o = 16; o > 0; o >>= 1) ex = max(ex, __shfl_xor_sync(0xffffffffu, ex, o));
+  if ((tid & 31) == 0) atomicMax(&s_exp, ex);
+  __syncthreads();
+  ex = s_exp;
+  // 2^-(exponent); a matrix of zeros, or with entries no scale helps, keeps its own
+  const double sc = ex > 0 && ex < 2046 ? __longlong_as_double((long long)(2046 - ex) << 52) : 1.0;
+  F2 e[U][U];
+#pragma unroll
+  for (int u = 0; u < U; ++u)
+#pragma unroll
+    for (int v = u; v < U; ++v) {
+      const double y = fma(x[u][v], sc, ty + 16 * u == tx + 16 * v ? kLrShift : 0.0);
+      const float h = to_f32(y);
+      e[u][v] = F2{h, to_f32(y - to_f64(h))};
+    }
+  bool bad = false;
+  for (int j = 0; j < m; j += 2) {
+    F2 *b0 = lr_rows + (size_t)j * LD, *b1 = b0 + LD;
+    if (ty == (j & 15) || ty == (j & 15) + 1) {          // j is even: both rows lie in one tile
+      const int ju = j >> 4;
+      F2 *buf = ty == (j & 15) ? b0 : b1;
+#pragma unroll
+      for (int v = 0; v < U; ++v) {
+        F2 w = e[0][v];              // selected, not indexed: e stays in registers
+#pragma unroll
+        for (int u = 1; u <= v; ++u) w = ju == u ? e[u][v] : w;
+        buf[tx + 16 * v] = f2_norm(w.h, w.l);
+      }
+    }
+    __syncthreads();
+    const F2 p0 = b0[j], c01 = b0[j + 1];
+    const F2 r0 = f2_reciprocal(p0), l = f2_neg(f2_mul(c01, r0));
+    const F2 q1 = f2_fma(l, c01, b1[j + 1]), p1 = f2_norm(q1.h, q1.l);
+    if (!(p0.h > kLrPivot) || !isfinite(p0.h) || !(p1.h > kLrPivot) || !isfinite(p1.h)) {   // the same for every thread
+      bad = true;
+      break;
+    }
+    if (tid == 0) {
+      rs[j] = p0;
+      rs[j + 1] = p1;
+      ls[j >> 1] = l;
+    }
+    const F2 r1 = f2_reciprocal(p1);
+    F2 x0[U], x1[U];
+#pragma unroll
+    for (int v = 0; v < U; ++v) {
+      x0[v] = b0[tx + 16 * v];
+      const F2 w = f2_fma(l, x0[v], b1[tx + 16 * v]);
+      x1[v] = f2_norm(w.h, w.l);
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      if (j >= 16 * u + 14) continue;        // every row of the tile is done
+      const int i = ty + 16 * u;
+      if (i <= j + 1) continue;
+      const F2 y0 = b0[i], w = f2_fma(l, y0, b1[i]), y1 = f2_norm(w.h, w.l);
+      const F2 m0 = f2_neg(f2_mul(y0, r0)), m1 = f2_neg(f2_mul(y1, r1));
+#pragma unroll
+      for (int v = u; v < U; ++v) e[u][v] = f2_fma(m1, x1[v], f2_fma(m0, x0[v], e[u][v]));
+    }
+  }
+  __syncthreads();
+  if (bad) {
+    for (int q = tid; q < m * m; q += 256) {
+      const int i = q % m, k = q / m;
+      L[q] = i == k ? 1.0 : 0.0;
+      B[q] = 0.5 * (H[q] + H[(size_t)i * m + k]);
+    }
+    return;
+  }
+  if (tid < m) rs[tid] = f2_rsqrt(rs[tid]);
+  __syncthreads();
+  for (int q = tid; q < m * m; q += 256) {
+    const int i = q % m, k = q / m;          // L(i, k) = R(k, i)
+    double v = 0.0;
+    if (i >= k) {
+      F2 w = lr_rows[(size_t)k * LD + i];
+      if (k & 1) w = f2_fma(ls[k >> 1], lr_rows[(size_t)(k - 1) * LD + i], w);
+      w = f2_mul(f2_norm(w.h, w.l), rs[k]);
+      v = to_f64(w.h) + to_f64(w.l);
+    }
+    L[q] = v;
+    B[q] = v;
+  }
+}
+
 // Cp[c] = A[rows of chunk c]^T B[same rows] in FP64 (m x m, row-major; the second
 // product's chunks follow the first's), 256 threads as 16 x 16 with entries
 // (ty + 16 u, tx + 16 v): every thread works whatever m is.  Of a symmetric
@@ -571,6 +717,31 @@ cudaError_t chol64(PSet C, int m, double shift, PSet W, int *flag, PSet only_if,
   }
   *launches += 1;
   return cudaGetLastError();
+}
+
+template <int U>
+static cudaError_t launch_lr(PSet H, int m, PSet L, PSet B, int P, cudaStream_t s) {
+  constexpr size_t smem = (size_t)(16 * U) * (16 * U) * sizeof(F2);
+  static bool done = false;
+  if (!done) {
+    const cudaError_t e = cudaFuncSetAttribute(k_lr_factor<U>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e) return e;
+    done = true;
+  }
+  launch_pdl(k_lr_factor<U>, dim3(1, 1, P), 256, smem, s, H, m, L, B);
+  return cudaGetLastError();
+}
+
+cudaError_t lr_factor(PSet H, int m, PSet L, PSet B, int P, cudaStream_t s, long long *launches) {
+  *launches += 1;
+  switch (tile_of(m)) {
+    case 2: return launch_lr<2>(H, m, L, B, P, s);
+    case 3: return launch_lr<3>(H, m, L, B, P, s);
+    case 4: return launch_lr<4>(H, m, L, B, P, s);
+    case 5: return launch_lr<5>(H, m, L, B, P, s);
+    case 6: return launch_lr<6>(H, m, L, B, P, s);
+  }
+  return cudaErrorInvalidValue;
 }
 
 cudaError_t rotate_basis(PSet A0, PSet Out0, const PSet *A1, const PSet *Out1, PSet W, int n, int m, bool tri, int P,

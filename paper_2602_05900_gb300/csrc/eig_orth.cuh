@@ -62,6 +62,15 @@ cudaError_t chol32(PSet C, int m, float shift, PSet W, int *flag, int P, cudaStr
 cudaError_t chol64(PSet C, int m, double shift, PSet W, int *flag, PSet only_if, int P, cudaStream_t s,
                    long long *launches);
 
+// H (m x m, symmetric) scaled by the power of two that brings its largest
+// entry into [1, 2), plus kLrShift I, = L L^T to ~2^-44 sqrt(h_ii h_jj): L (column-major, zeros above the
+// diagonal) and B = L.  A pivot below kLrPivot (H is not positive semidefinite to
+// rounding) makes L = I and B = H of that problem: L^T B is similar to H either way,
+// up to the scale and the shift.
+constexpr double kLrShift = 0x1p-28;
+constexpr float kLrPivot = 0x1p-30f;
+cudaError_t lr_factor(PSet H, int m, PSet L, PSet B, int P, cudaStream_t s, long long *launches);
+
 // Out0 = A0 W and (optional) Out1 = A1 W (A, Out n x m column-major, W m x m
 // column-major; tri: W upper triangular)
 cudaError_t rotate_basis(PSet A0, PSet Out0, const PSet *A1, const PSet *Out1, PSet W, int n, int m, bool tri, int P,

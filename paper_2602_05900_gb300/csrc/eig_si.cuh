@@ -35,7 +35,7 @@ struct SiBatch {
   double shift_rel;      // initial shift / Tr G
   int first_check;       // expected convergence iteration (first Rayleigh-Ritz step of small batches)
   double floor_tol;      // residual accepted once it stops decreasing (0: the FP64 default, 1e-10)
-  bool graded;           // jacobi_full: G is nearly diagonal already (a warm start)
+  bool graded;           // jacobi_full: G = V^T (M^T M) V with a V that nearly diagonalises it (a warm start)
 };
 
 // Where a solve leaves its results inside the workspace: Ritz vectors of

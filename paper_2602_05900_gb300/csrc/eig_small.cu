@@ -11,7 +11,17 @@
 //      small eigenvalues of a dense H only through the FP32 rounding of the
 //      large entries; S is graded, and its small block is resolved at its own
 //      scale.
-//   3. Two refinement passes X <- X (I + E) (Ogita and Aishima's iteration):
+//      Warm starts (from kLrMinSize rows) take another way to
+//      X: H + shift = L L^T, FP32 passes on L^T L, which is similar to it and far
+//      nearer to diagonal where the spectrum is graded (Rutishauser's LR step; the
+//      preconditioning of Veselic and Hari's one-sided Jacobi method), and
+//      X = L V, made orthonormal by a refinement pass that normalises the columns
+//      and a Newton-Schulz step.  An FP32 rotation contaminates a column
+//      with ~1e-13 of the leading eigenvalue, so the shift is 2^-28 of it: with 2^-48
+//      columns belonging to eigenvalues of 1e-18 lost their orthogonality.  Over
+//      graded, rank-deficient, degenerate and random environments of 34 to 96 rows
+//      both passes together took 1445 sweeps without the factor and take 617 in a CPU model.
+//   3. Two refinement passes (one after the factored route) X <- X (I + E) (Ogita and Aishima's iteration):
 //      with G = X^T X, S = X^T H X and lambda_i = s_ii / g_ii,
 //      E_ij = (s_ij - lambda_j g_ij) / (lambda_j - lambda_i) for separated pairs
 //      and -g_ij / 2 inside clusters and for couplings at rounding level:
@@ -22,8 +32,8 @@
 //
 // Measured against the FP64 two-sided Jacobi on an 8-CTA cluster that this
 // replaced (its rounds cost 4 us, half of it FP64 arithmetic): an iTEBD update
-// of one chain at n = 60 took 3.63 ms and takes 0.62 ms, of 64 chains at n = 32
-// 3.39 ms and 0.45 ms, a D = 8 FP64 step (n = 64) 2.88 ms and 0.65 ms.
+// of one chain at n = 60 took 3.63 ms and takes 0.37 ms, of 64 chains at n = 32
+// 3.39 ms and 0.36 ms, a D = 8 FP64 step (n = 64) 2.88 ms and 0.43 ms.
 //
 // A CPU model of the four stages (dense, graded, rank-deficient and degenerate
 // matrices, m = 16 to 96) leaves residuals and orthonormality at 1e-15 and at
@@ -87,6 +97,21 @@ __device__ inline void jacobi_angle(double hpp, double hqq, double hpq, double &
 // ---- stage 1: FP32 cyclic Jacobi ---------------------------------------------
 
 constexpr int kJ32MaxSweeps = 30;
+// Warm starts of at least this size are factored: 30 iTEBD updates, ms without and
+// with the factor, one chain n = 8 3.09 / 3.16, 14 3.69 / 3.78, 16 4.31 / 4.05,
+// 32 6.72 / 5.83, 60 15.2 / 11.0, 96 37.9 / 26.6; 64 chains n = 8 3.90 / 4.03,
+// 16 5.58 / 5.45, 32 11.3 / 10.8, 60 38.8 / 36.5.  Cold environments save three
+// sweeps, which the six additional launches cost again (D = 8 run 8.46 / 8.44 ms, in
+// TF32 9.15 / 9.64).
+constexpr int kLrMinSize = 16;
+
+// Where the first pass of a factored matrix stops: between the columns of length
+// sqrt(kLrShift), 2^-12 of it leaves couplings of 2e-4 in X^T X, which the
+// refinement squares.  Without a floor FP32 noise between equal small entries was
+// rotated up to the sweep limit.
+constexpr float kLrFloor = 0x1p-40f;
+
+
 constexpr float kJ32Rel2 = 1e-12f;   // a pair is rotated while h_pq^2 > this h_pp h_qq
 
 // Layout of the kernel for up to HM pairs (h = m / 2 <= HM): tops of the slots at
@@ -394,7 +419,7 @@ constexpr double kSfsCluster = 1e3;   // a pair is separated if |gap| > kSfsClus
 // truncated to rows x cols, column-major with ld = rows.
 struct MmOp {
   PSet A, B, S, G, Out;
-  int ta, refine;
+  int ta, refine;        // refine: 1, or 2 where A's columns still have to be normalised
   int sym;               // the product is symmetric: only its upper tiles are computed, and mirrored
   double bs, bd;
   int rows, cols;
@@ -410,7 +435,7 @@ __global__ void __launch_bounds__(256) k_se_mm(MmOp op0, MmOp op1, int P, int m,
   __shared__ double As[8][kSiMaxBlock + 1];   // op(A) rows i0..i0+7, all k
   __shared__ double Bs[8][kSiMaxBlock + 1];   // B' columns j0..j0+7, all k
   __shared__ double part[4][8][9];
-  __shared__ double lam[kSiMaxBlock];
+  __shared__ double lam[kSiMaxBlock], rn[kSiMaxBlock];
   __shared__ float s_mx;
   const bool second = (int)blockIdx.z >= P;
   const MmOp &o = second ? op1 : op0;
@@ -438,8 +463,18 @@ __global__ void __launch_bounds__(256) k_se_mm(MmOp op0, MmOp op1, int P, int m,
   } else {
     const double *S = o.S.at(z), *G = o.G.at(z);
     // lambda = s / g to first order in g - 1 (V is orthonormal to 1e-5 or better)
-    for (int k = threadIdx.x; k < m; k += blockDim.x)
-      lam[k] = S[(size_t)k * m + k] * (2.0 - G[(size_t)k * m + k]);
+    // or exactly, for columns of any length: then A diag(rn) is what is refined
+    const bool norm = o.refine == 2;
+    for (int k = threadIdx.x; k < m; k += blockDim.x) {
+      const double s = S[(size_t)k * m + k], g = G[(size_t)k * m + k];
+      if (norm) {
+        const double r = g > 0.0 ? rsqrt_fp64(g) : 1.0;
+        rn[k] = r;
+        lam[k] = s * r * r;
+      } else {
+        lam[k] = s * (2.0 - g);
+      }
+    }
     __syncthreads();
     if (threadIdx.x < 32) {
       float v = 0.0f;
@@ -453,11 +488,16 @@ __global__ void __launch_bounds__(256) k_se_mm(MmOp op0, MmOp op1, int P, int m,
       const int r = e / m, k = e % m, j = j0 + r;
       double v = 0.0;
       if (j < m) {
-        const double g = G[(size_t)j * m + k];
+        double g = G[(size_t)j * m + k];
         if (k == j) {
-          v = 1.5 - 0.5 * g;                                  // 1 + (1 - g) / 2
+          v = norm ? rn[k] : 1.5 - 0.5 * g;                   // 1 + (1 - g) / 2
         } else {
-          const double s = S[(size_t)j * m + k];
+          double s = S[(size_t)j * m + k];
+          if (norm) {
+            const double w = rn[k] * rn[j];
+            g *= w;
+            s *= w;
+          }
           const double gap = lam[j] - lam[k];
           const double num = fma(-lam[j], g, s);
           const float off = mag32(fma(0.5 * gap, g, num));    // s - (lam_j + lam_k) g / 2
@@ -465,6 +505,7 @@ __global__ void __launch_bounds__(256) k_se_mm(MmOp op0, MmOp op1, int P, int m,
           // order of 1e-7 of a coupling that the next pass sees
           if (mag32(gap) > (float)kSfsCluster * off && off > fl) v = (double)((float)num / (float)gap);
           else v = -0.5 * g;
+          if (norm) v *= rn[k];
         }
       }
       Bs[r][k] = v;
@@ -711,7 +752,33 @@ cudaError_t small_eig(const SmallEig &a, cudaStream_t s, long long *launches) {
     *launches += 1;
   };
   // H is symmetric: H^T Y is read along its rows
-  if (a.full) {
+  auto refine = [&](int kind) {
+    mm2(sym(X, X, G), op(a.H, 1, X, 1.0, 0.0, Y));
+    mm1(sym(X, Y, S));
+    mm1(MmOp{X, X, S, G, Xn, 0, kind, 0, 1.0, 0.0, m, m});
+    std::swap(X, Xn);
+  };
+  auto newton_schulz = [&]() {
+    mm1(sym(X, X, G));
+    mm1(op(X, 0, G, -0.5, 1.5, Xn));
+    std::swap(X, Xn);
+  };
+  const bool lr = a.full && a.graded && m >= kLrMinSize;
+  if (lr) {
+    // L^T L in place of H = L L^T (see the file comment)
+    if ((e = lr_factor(a.H, m, Y, G, P, s, launches))) return e;
+    mm1(sym(Y, G, S));
+    if ((e = launch_j32(S, m, kLrFloor, V, a.sweeps, P, s))) return e;
+    mm1(op(Y, 0, V, 1.0, 0.0, X));
+    refine(2);
+    newton_schulz();
+    mm1(op(a.H, 1, X, 1.0, 0.0, Y));
+    mm1(sym(X, Y, S));
+    if ((e = launch_j32(S, m, ldexpf(1.0f, -56), V, a.sweeps, P, s))) return e;
+    mm1(op(X, 0, V, 1.0, 0.0, Xn));
+    std::swap(X, Xn);
+    *launches += 2;
+  } else if (a.full) {
     // a dense H: the first FP32 pass stops at its rounding (2^-24), the second
     // one resolves what lies below; a graded H is resolved by the first
     if ((e = launch_j32(a.H, m, ldexpf(1.0f, a.graded ? -56 : -24), X, a.sweeps, P, s))) return e;
@@ -729,19 +796,12 @@ cudaError_t small_eig(const SmallEig &a, cudaStream_t s, long long *launches) {
     if ((e = launch_j32(a.H, m, ldexpf(1.0f, -46), X, a.sweeps, P, s))) return e;
     *launches += 1;
   }
-  for (int pass = 0; pass < 2; ++pass) {
-    mm2(sym(X, X, G), op(a.H, 1, X, 1.0, 0.0, Y));
-    mm1(sym(X, Y, S));
-    mm1(MmOp{X, X, S, G, Xn, 0, 1, 0, 1.0, 0.0, m, m});
-    std::swap(X, Xn);
-  }
+  refine(1);
+  if (!lr) refine(1);
   // orthonormal to rounding: barely separated pairs take E up to 1 / kSfsCluster,
   // whose square is what a pass leaves
-  for (int ns = 0; ns < 2; ++ns) {
-    mm1(sym(X, X, G));
-    mm1(op(X, 0, G, -0.5, 1.5, Xn));
-    std::swap(X, Xn);
-  }
+  newton_schulz();
+  newton_schulz();
   mm1(op(a.H, 1, X, 1.0, 0.0, Y));
   mm1(sym(X, Y, S));
   launch_pdl(k_rr_sparse_jacobi, dim3(1, 1, P), kSparseThreads, sparse_smem(m), s, S, m, floor_exp, W, a.theta, a.flag,

@@ -19,7 +19,8 @@ struct SmallEig {
   bool full;             // resolve every pair to FP64 rounding of H (direct solves); else to
                          // 2^-44 of the largest eigenvalue (Rayleigh-Ritz steps, whose H
                          // carries that much rounding)
-  bool graded;           // full only: H is already nearly diagonal or graded (a warm start)
+  bool graded;           // full only: H is positive semidefinite to rounding and already nearly
+                         // diagonal (a warm start); a hint, the result does not depend on it
   PSet out;              // leading eigenvectors: rows x cols, column-major, ld = rows
   int rows, cols;        // rows, cols <= m
   PSet theta;            // m eigenvalues, descending

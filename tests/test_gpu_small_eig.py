@@ -51,3 +51,23 @@ def test_rank_one_start(pkg, D_b):
     with pkg.Itebd([(1.0, 1.0, 0.05)], D_b) as c:
         lam = c.step(4).lam()
     assert np.abs(lam - np.pad(st.lam, (0, lam.size - st.lam.size))).max() <= 1e-7
+
+
+@pytest.mark.parametrize("D_b", [7, 8, 17, 24, 25, 33, 40, 41, 48])
+def test_factored_warm_starts(pkg, D_b):
+    """Warm solves at the edges of the Cholesky factor's 16-wide tiles (and of the
+    rule that chooses it: 16 rows and more), two different chains in one batch."""
+    J = [(1.0, 0.7, 0.05), (0.6, 1.3, 0.05)]
+    init = [random_mps(D_b, seed=300 + D_b + 50 * i) for i in range(2)]
+    runs = [it.ItebdRun(P, Q, lam, np.ones(D_b) / np.sqrt(D_b)) for P, Q, lam in init]
+    with pkg.Itebd(J, D_b, init=init) as c:
+        for _ in range(6):
+            c.step(1)
+            for i, st in enumerate(runs):
+                old = st.lam
+                st.P, st.Q, st.lam, _ = it.update(st.P, st.Q, st.lam, hz.bond_gate(*J[i]), D_b)
+                st.lam_other = old
+        for i, st in enumerate(runs):
+            assert np.abs(c.lam(i) - st.lam).max() <= 1e-10
+            want = it.site_energy(st, hz.bond_hamiltonian(J[i][0], J[i][1]))
+            assert abs(float(c.energy()[i]) - want) <= 1e-11
