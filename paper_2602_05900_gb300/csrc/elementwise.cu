@@ -16,12 +16,6 @@ __device__ inline double warp_sum(double v) {
   return v;
 }
 
-__device__ inline double warp_max(double v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(0xffffffffu, v, o));
-  return v;
-}
-
 // Block-wide sum over up to 1024 threads; result valid in thread 0.
 __device__ double block_sum(double v) {
   __shared__ double part[32];
@@ -100,32 +94,52 @@ __global__ void k_identity(double *U, int n, long long sU) {
     U[e] = (e % n == e / n) ? 1.0 : 0.0;
 }
 
-// Max |T| per instance by a grid-stride reduction; non-negative doubles order
-// like their bit patterns, so the combine is an integer atomicMax.
-__global__ void k_maxabs(const double *T, long long count, long long sT, unsigned long long *out,
-                         long long sOut) {
+// Max |T| per instance; non-negative doubles order like their bit patterns, so the
+// search is integer arithmetic (an FP64 comparison of every element cost as much as
+// its load) and the blocks combine by one integer atomicMax each (one per warp was
+// bound by the atomics: mean of a D = 32 run 14.4 us, 4.5 us now).
+__global__ void __launch_bounds__(256) k_maxabs(const double *T, long long count, long long sT,
+                                                unsigned long long *out, long long sOut) {
   pdl_enter();
-  T += blockIdx.y * sT;
-  double v = 0.0;
-  for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < count;
-       e += (long long)gridDim.x * blockDim.x) {
-    const double a = fabs(T[e]);
-    v = (a != a) ? INFINITY : fmax(v, a);   // NaN poisons the norm
+  constexpr unsigned long long kAbs = 0x7FFFFFFFFFFFFFFFull, kInf = 0x7FF0000000000000ull;
+  const unsigned long long *t = reinterpret_cast<const unsigned long long *>(T + blockIdx.y * sT);
+  const long long step = (long long)gridDim.x * 256;
+  long long e = blockIdx.x * 256ll + threadIdx.x;
+  unsigned long long v = 0;
+  for (; e + 3 * step < count; e += 4 * step) {
+    const unsigned long long a = t[e] & kAbs, b = t[e + step] & kAbs, c = t[e + 2 * step] & kAbs,
+                             d = t[e + 3 * step] & kAbs;
+    v = max(v, max(max(a, b), max(c, d)));
   }
-  v = warp_max(v);
-  if ((threadIdx.x & 31) == 0)
-    atomicMax(out + blockIdx.y * sOut, (unsigned long long)__double_as_longlong(v));
+  for (; e < count; e += step) v = max(v, t[e] & kAbs);
+  for (int o = 16; o > 0; o >>= 1) v = max(v, __shfl_xor_sync(0xffffffffu, v, o));
+  __shared__ unsigned long long part[8];
+  if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = v;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int w = 1; w < 8; ++w) v = max(v, part[w]);
+    atomicMax(out + blockIdx.y * sOut, v > kInf ? kInf : v);   // NaN poisons the norm
+  }
 }
 
-__global__ void k_scale(double *T, long long count, long long sT, const unsigned long long *maxbits,
-                        long long sMax, double *logsum, long long sLog, double inv_two_pow_n,
-                        double *ln_c_out, long long sLnc, int *err) {
+// T /= c: the correctly rounded quotient from the reciprocal of c by Markstein's
+// theorem (q = T r, then q + r (T - q c)): three FP64 instructions per element, a
+// division costs three times that (mean of a D = 32 run 15.1 us, 11.4 us now; D = 48
+// 43.8 us, 26.6 us).
+// Quotients or divisors near the ends of the exponent range, where the remainder
+// would not be exact, are divided.
+__global__ void __launch_bounds__(256) k_scale(double *T, long long count, long long sT,
+                                               const unsigned long long *maxbits, long long sMax, double *logsum,
+                                               long long sLog, double inv_two_pow_n, double *ln_c_out,
+                                               long long sLnc, int *err) {
   pdl_enter();
   const long long inst = blockIdx.y;
   T += inst * sT;
   const double c = __longlong_as_double((long long)maxbits[inst * sMax]);
   const bool ok = (c > 0.0) && isfinite(c);
-  if (blockIdx.x == 0 && threadIdx.x == 0) {
+  __shared__ double s_r;
+  if (threadIdx.x == 0) s_r = ok ? 1.0 / c : 0.0;
+  if (blockIdx.x == 0 && threadIdx.x == 32) {
     if (ok) {
       const double lc = log(c);
       logsum[inst * sLog] += lc * inv_two_pow_n;
@@ -135,10 +149,28 @@ __global__ void k_scale(double *T, long long count, long long sT, const unsigned
       if (ln_c_out) ln_c_out[inst * sLnc] = NAN;
     }
   }
-  if (!ok) return;
-  for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < count;
-       e += (long long)gridDim.x * blockDim.x)
-    T[e] = T[e] / c;
+  if (!ok) return;                        // the same for every thread
+  __syncthreads();
+  const double r = s_r;
+  auto expo = [](double x) { return (__double2hiint(x) >> 20) & 0x7FF; };
+  // T and c at 2^-500 or above and c at 2^500 or below: q c, the remainder and q are normal
+  const bool c_mid = expo(c) > 1023 - 500 && expo(c) < 1023 + 500;
+  auto quotient = [&](double a) {
+    if (__double_as_longlong(a) << 1 == 0) return a;      // keeps the sign of a zero
+    if (!c_mid || expo(a) <= 1023 - 500) return a / c;
+    const double q = a * r;
+    return fma(fma(-q, c, a), r, q);
+  };
+  const long long step = (long long)gridDim.x * 256;
+  long long e = blockIdx.x * 256ll + threadIdx.x;
+  for (; e + 3 * step < count; e += 4 * step) {
+    const double x0 = T[e], x1 = T[e + step], x2 = T[e + 2 * step], x3 = T[e + 3 * step];
+    T[e] = quotient(x0);
+    T[e + step] = quotient(x1);
+    T[e + 2 * step] = quotient(x2);
+    T[e + 3 * step] = quotient(x3);
+  }
+  for (; e < count; e += step) T[e] = quotient(T[e]);
 }
 
 // one block per instance
@@ -170,42 +202,49 @@ __global__ void k_trace_y(const double *T, double *Tx, int Dx, int Dy, long long
 }
 
 // grid (kept column a, instance).  Every block recomputes the side choice from
-// the eigenvalues (a few dozen adds), so no separate launch or host round trip
-// is needed; block (0, i) also writes instance i's record and spectrum.
+// the eigenvalues (a few dozen adds, each side's in its own warp from shared memory,
+// in the order of the values), so no separate launch or host round trip is needed;
+// block (0, i) also writes instance i's record and spectrum.  Bound by those adds:
+// D = 32 19.3 us with one thread for both sums and the spectrum, 9.0 us now.
 __global__ void k_select(SelectArgs a) {
   pdl_enter();
-  __shared__ int s_side;
   __shared__ int s_arg;
   __shared__ double wbest[32];
   __shared__ int warg[32];
   const int col = blockIdx.x, inst = blockIdx.y;
   const double *wL = a.w.at(2 * inst), *wR = a.w.at(2 * inst + 1);
   const double *tr = a.tr + inst * a.sTr;
+  extern __shared__ double vals[];            // [side][a.m]
+  __shared__ double s_eps[2];
   // i-th largest eigenvalue / its vector, whatever order the solver returned
   auto val = [&](const double *w, int i) { return a.desc ? w[i] : w[a.m - 1 - i]; };
   auto vecidx = [&](int i) { return a.desc ? i : a.m - 1 - i; };
-  if (threadIdx.x == 0) {
-    double sumL = 0.0, sumR = 0.0;
-    for (int i = 0; i < a.Dn; ++i) {
-      sumL += val(wL, i);
-      sumR += val(wR, i);
-    }
-    const double epsL = tr[0] - sumL, epsR = tr[1] - sumR;
-    s_side = (epsL <= epsR) ? 0 : 1;
-    if (col == 0) {
-      const double *w = s_side == 0 ? wL : wR;
-      const double l1 = val(w, 0);
-      double *rec = a.record + inst * a.sRec;
-      double *spec = a.spectrum + inst * a.sSpec;
+  for (int i = threadIdx.x; i < 2 * a.m; i += blockDim.x) vals[i] = i < a.m ? val(wL, i) : val(wR, i - a.m);
+  __syncthreads();
+  if (threadIdx.x == 0 || threadIdx.x == 32) {
+    const int side = threadIdx.x >> 5;
+    const double *w = vals + side * a.m;
+    double sum = 0.0;
+    for (int i = 0; i < a.Dn; ++i) sum += w[i];
+    s_eps[side] = tr[side] - sum;
+  }
+  __syncthreads();
+  const double epsL = s_eps[0], epsR = s_eps[1];
+  const int s_side = epsL <= epsR ? 0 : 1;
+  if (col == 0) {
+    const double *w = vals + s_side * a.m;
+    const double l1 = w[0];
+    double *rec = a.record + inst * a.sRec;
+    double *spec = a.spectrum + inst * a.sSpec;
+    if (threadIdx.x == 64) {
       rec[0] = (double)s_side;
       rec[1] = epsL;
       rec[2] = epsR;
-      rec[3] = (a.m > a.Dn) ? (val(w, a.Dn - 1) - val(w, a.Dn)) / l1 : INFINITY;
+      rec[3] = (a.m > a.Dn) ? (w[a.Dn - 1] - w[a.Dn]) / l1 : INFINITY;
       rec[4] = tr[0];
-      for (int i = 0; i < a.m; ++i) spec[i] = val(w, i) / l1;
     }
+    for (int i = threadIdx.x; i < a.m; i += blockDim.x) spec[i] = w[i] / l1;
   }
-  __syncthreads();
   const double *v = a.v.at(2 * inst + s_side) + (long long)vecidx(col) * a.n;
   // sign convention: the component of largest magnitude (first on ties) is positive
   double best = -1.0;
@@ -288,7 +327,7 @@ cudaError_t maxabs_scale_log(double *T, long long count, long long sT, double *s
   cudaError_t e = cudaMemset2DAsync(bits, sScratch * sizeof(double), 0, sizeof(unsigned long long),
                                     batch, s);
   if (e != cudaSuccess) return e;
-  const dim3 g(grid_for(count, 256, batch), batch);
+  const dim3 g(grid_for((count + 3) / 4, 256, batch), batch);
   launch_pdl(k_maxabs, g, 256, 0, s, T, count, sT, bits, sScratch);
   launch_pdl(k_scale, g, 256, 0, s, T, count, sT, bits, sScratch, logsum, sLog, inv_two_pow_n, ln_c_out,
                             sLnc, err_flag);
@@ -309,7 +348,7 @@ cudaError_t trace_y(const double *T, double *Tx, int Dx, int Dy, long long sT, i
 }
 
 cudaError_t select_isometry(const SelectArgs &a, cudaStream_t s) {
-  launch_pdl(k_select, dim3(a.Dn, a.batch), 256, 0, s, a);
+  launch_pdl(k_select, dim3(a.Dn, a.batch), 256, 2 * (size_t)a.m * sizeof(double), s, a);
   return cudaGetLastError();
 }
 
