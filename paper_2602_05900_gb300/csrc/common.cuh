@@ -148,6 +148,8 @@ cudaError_t gemm_f64(const MappedGemm &g, cudaStream_t s);
 // trace_out[i sTr + side].
 cudaError_t symmetrize_trace(double *G, int n, long long sG, double *trace_out, long long sTr,
                              int batch, cudaStream_t s, int per_side = 0);
+// The same without the trace.
+cudaError_t symmetrize(double *G, int n, long long sG, int batch, cudaStream_t s);
 cudaError_t identity_isometry(double *U, int n, long long sU, int batch, cudaStream_t s);
 // T /= max|T| per instance, logsum += ln(max) * inv_two_pow_n, ln_c_out (may be null)
 // receives ln(max); scratch holds one word per instance (stride sScratch doubles).

@@ -306,10 +306,16 @@ int grid_for(long long count, int threads, int batch) {
 
 }  // namespace
 
-cudaError_t symmetrize_trace(double *G, int n, long long sG, double *trace_out, long long sTr,
-                             int batch, cudaStream_t s, int per_side) {
+cudaError_t symmetrize(double *G, int n, long long sG, int batch, cudaStream_t s) {
   const int T = (n + 31) / 32;
   launch_pdl(k_symmetrize_tiled, dim3(T * (T + 1) / 2, batch), 256, 0, s, G, n, sG);
+  return cudaGetLastError();
+}
+
+cudaError_t symmetrize_trace(double *G, int n, long long sG, double *trace_out, long long sTr,
+                             int batch, cudaStream_t s, int per_side) {
+  const cudaError_t e = symmetrize(G, n, sG, batch, s);
+  if (e != cudaSuccess) return e;
   launch_pdl(k_trace_diag, batch, 1024, 0, s, G, n, sG, trace_out, sTr, per_side);
   return cudaGetLastError();
 }

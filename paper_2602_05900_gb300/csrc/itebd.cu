@@ -5,15 +5,15 @@
 //
 //   phi   = P Q                        FP64 GEMM, rows (i, a), columns (b, m)
 //   phit  = g phi, theta = lam phit    k_itebd_gate
-//   rho   = theta^T theta              FP64 GEMM + symmetrise: the bond's right
-//                                      reduced density matrix (2D x 2D)
-//   Y, w  = eig(rho)                   cluster two-sided Jacobi (Sec. II.B, Eqs. 5-6),
+//   rho   = theta^T theta              FP64 GEMM: the bond's right reduced
+//                                      density matrix (2D x 2D)
+//   Y, w  = eig(rho)                   Jacobi (Sec. II.B, Eqs. 5-6; eig_small.cu),
 //                                      warm-started from the same kind of bond's
 //                                      last eigenbasis V: eig(V^T rho V), Y = V W
 //   lam'  = sqrt(w[:D']) / norm        k_itebd_schmidt (+ the discarded weight)
-//   P'    = phit Y[:, :D'] / |s|       FP64 GEMM + k_itebd_scale (keeps the state
+//   P'    = phit Y[:, :D'] / |s|       FP64 GEMM + k_itebd_finish (keeps the state
 //                                      normalised under the non-unitary gate)
-//   Q'    = Y[:, :D']^T                k_itebd_take (Y is column-major: a copy)
+//   Q'    = Y[:, :D']^T                k_itebd_finish (Y is column-major: a copy)
 //
 // then (P, Q, lam) <- (Q', P', lam') for the other kind of bond.  The singular
 // values of theta are the square roots of rho's eigenvalues (the paper's SVD of a
@@ -70,41 +70,53 @@ __global__ void k_itebd_gate(const double *phi, double *phit, double *theta, con
 
 // one block per chain: lam'[k] = sqrt(w_k) / sqrt(sum_{k < Dn} w_k) with w = max(eig, 0);
 // disc = sum_{k >= Dn} w_k / sum_k w_k over the m eigenvalues (descending);
-// rnorm = 1 / sqrt(sum_{k < Dn} w_k), the factor that keeps the state normalised
-__global__ void k_itebd_schmidt(PSet w, int m, int Dn, double *lam, long long sL, double *disc,
-                                double *rnorm, int *err) {
+// rnorm = 1 / sqrt(sum_{k < Dn} w_k), the factor that keeps the state normalised.
+// One value per thread (m <= kItebdMaxN): a chain of FP64 adds and square roots, 14.2 us
+// at m = 60 with one thread for the sums, 4.0 us with a tree.
+constexpr int kItebdMaxN = 96;
+__global__ void __launch_bounds__(kItebdMaxN) k_itebd_schmidt(PSet w, int m, int Dn, double *lam, long long sL,
+                                                              double *disc, double *rnorm, int *err) {
   pdl_enter();
-  const int z = blockIdx.x;
-  const double *wz = w.at(z);
-  __shared__ double keep;
-  if (threadIdx.x == 0) {
-    double a = 0.0, b = 0.0;
-    for (int k = 0; k < m; ++k) {
-      const double v = fmax(wz[k], 0.0);
-      b += v;
-      if (k < Dn) a += v;
-    }
-    keep = a;
-    disc[z] = b > 0.0 ? (b - a) / b : NAN;
-    rnorm[z] = 1.0 / sqrt(a);
-    if (!(a > 0.0) || !isfinite(b)) atomicExch(err, 1);
+  const int z = blockIdx.x, k = threadIdx.x;
+  const double v = k < m ? fmax(w.at(z)[k], 0.0) : 0.0;
+  double a = k < Dn ? v : 0.0, b = v;
+  for (int o = 16; o > 0; o >>= 1) {
+    a += __shfl_xor_sync(0xffffffffu, a, o);
+    b += __shfl_xor_sync(0xffffffffu, b, o);
+  }
+  __shared__ double pa[3], pb[3];
+  if ((k & 31) == 0) {
+    pa[k >> 5] = a;
+    pb[k >> 5] = b;
   }
   __syncthreads();
-  const double inv = 1.0 / sqrt(keep);
-  for (int k = threadIdx.x; k < Dn; k += blockDim.x) lam[z * sL + k] = sqrt(fmax(wz[k], 0.0)) * inv;
+  a = (pa[0] + pa[1]) + pa[2];
+  b = (pb[0] + pb[1]) + pb[2];
+  const double inv = 1.0 / sqrt(a);
+  if (k < Dn) lam[z * sL + k] = sqrt(v) * inv;
+  if (k == 0) {
+    rnorm[z] = inv;
+    if (!(a > 0.0) || !isfinite(b)) atomicExch(err, 1);
+  }
+  if (k == 64) disc[z] = b > 0.0 ? (b - a) / b : NAN;
 }
 
-// P' *= rnorm of its chain
-__global__ void k_itebd_scale(double *P, long long count, long long sT, const double *rnorm) {
+// P' *= rnorm of its chain (first cP elements of the launch), and
+// Q'[j][B][m] = Y[(B m), j] for j < Dn: the first Dn columns of the column-major Y
+__global__ void k_itebd_finish(double *P, long long cP, const double *rnorm, PSet Y, long long cQ, double *Q,
+                               long long sT) {
   pdl_enter();
   const long long z = blockIdx.y;
   const double r = rnorm[z];
-  for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < count;
-       e += (long long)gridDim.x * blockDim.x)
-    P[z * sT + e] *= r;
+  const double *y = Y.at((int)z);
+  for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < cP + cQ;
+       e += (long long)gridDim.x * blockDim.x) {
+    if (e < cP) P[z * sT + e] *= r;
+    else Q[z * sT + e - cP] = y[e - cP];
+  }
 }
 
-// Q'[j][B][m] = Y[(B m), j] for j < Dn: the first Dn columns of the column-major Y
+// the first `count` elements of Y
 __global__ void k_itebd_take(PSet Y, long long count, double *Q, long long sT) {
   pdl_enter();
   const long long z = blockIdx.y;
@@ -168,7 +180,7 @@ struct hotrg_itebd {
   double *l[3] = {};              // Schmidt values: lam, lam_other, lam'
   int iL = 0, iO = 1;
   double *phi = nullptr, *phit = nullptr, *theta = nullptr, *rho = nullptr;
-  double *gates = nullptr, *hs = nullptr, *disc = nullptr, *energy = nullptr, *trace = nullptr;
+  double *gates = nullptr, *hs = nullptr, *disc = nullptr, *energy = nullptr;
   double *rnorm = nullptr;
   // warm start: the last full eigenbasis of each kind of bond (n x n column-major,
   // n = nb[parity], -1 = none) and a buffer for the next one
@@ -236,11 +248,11 @@ hotrg_status itebd_update(hotrg_itebd *c) {
   launch_pdl(k_itebd_gate, dim3(grid1((long long)Dl * Dr), G), 256, 0, st, c->phi, c->phit, c->theta, c->gates,
                                                                    c->l[c->iL], Dl, Dr, c->sM, c->sL);
   ICK(c, cudaGetLastError());
-  // rho = theta^T theta, symmetrised
+  // rho = theta^T theta: rho_ij and rho_ji are the same sums of the same products,
+  // so it is symmetric to the last bit
   MappedGemm g2{n, n, kPhys * Dl, c->theta, map1(1), map1(n), c->theta, map1(1), map1(n),
                 c->rho, map1(n), map1(1), G, c->sM, c->sM, c->sM};
   ICK(c, gemm_f64(g2, st));
-  ICK(c, symmetrize_trace(c->rho, n, c->sM, c->trace, 1, G, st));
   // Warm start: two updates ago the same kind of bond had eigenbasis V; near the
   // fixed point rho is nearly diagonal in it, so the Jacobi runs on
   // rho~ = V^T rho V (a few sweeps instead of ~11 from scratch) and the basis
@@ -256,7 +268,7 @@ hotrg_status itebd_update(hotrg_itebd *c) {
     MappedGemm w2{n, n, n, Vold, map1(n), map1(1), c->phi, map1(1), map1(n), c->theta, map1(n), map1(1),
                   G, c->sM, c->sM, c->sM};
     ICK(c, gemm_f64(w2, st));
-    ICK(c, symmetrize_trace(c->theta, n, c->sM, c->trace, 1, G, st));
+    ICK(c, symmetrize(c->theta, n, c->sM, G, st));
   }
   // all n eigenpairs (the full basis is kept for the next warm start)
   SiBatch sb{};
@@ -269,7 +281,7 @@ hotrg_status itebd_update(hotrg_itebd *c) {
   long long nl = 0;
   ICK(c, jacobi_full(sb, c->si_work, st, &nl));
   const SiOut o = si_outputs(c->si_work, G, n, sb.m);
-  launch_pdl(k_itebd_schmidt, G, 64, 0, st, o.theta, sb.m, Dn, c->l[iN], c->sL, c->disc, c->rnorm, c->err);
+  launch_pdl(k_itebd_schmidt, G, kItebdMaxN, 0, st, o.theta, sb.m, Dn, c->l[iN], c->sL, c->disc, c->rnorm, c->err);
   ICK(c, cudaGetLastError());
   // the new basis V' = V W (or W cold), column-major n x n, into Vn
   const long long ys = o.X.b1 - o.X.b0;
@@ -288,10 +300,8 @@ hotrg_status itebd_update(hotrg_itebd *c) {
   MappedGemm g3{kPhys * Dl, Dn, n, c->phit, map1(n), map1(1), Y.b0, map1(n), map1(1), Pn, map1(Dn),
                 map1(1), G, c->sM, c->sM, c->sT};
   ICK(c, gemm_f64(g3, st));
-  launch_pdl(k_itebd_scale, dim3(grid1((long long)kPhys * Dl * Dn), G), 256, 0, st, Pn, (long long)kPhys * Dl * Dn,
-                                                                           c->sT, c->rnorm);
-  ICK(c, cudaGetLastError());
-  launch_pdl(k_itebd_take, dim3(grid1((long long)Dn * n), G), 256, 0, st, Y, (long long)Dn * n, Qn, c->sT);
+  const long long cP = (long long)kPhys * Dl * Dn, cQ = (long long)Dn * n;
+  launch_pdl(k_itebd_finish, dim3(grid1(cP + cQ), G), 256, 0, st, Pn, cP, c->rnorm, Y, cQ, Qn, c->sT);
   ICK(c, cudaGetLastError());
   // the next bond: (P, Q, lam) <- (Q', P', lam'); lam_other <- lam
   c->iP = iQn;
@@ -351,7 +361,7 @@ hotrg_status hotrg_itebd_create(int n, const double *couplings, int D_b, int D0,
       (s = ialloc(c, &c->theta, c->sM * n)) || (s = ialloc(c, &c->rho, c->sM * n)) ||
       (s = ialloc(c, &c->gates, 16LL * n)) || (s = ialloc(c, &c->hs, 16LL * n)) ||
       (s = ialloc(c, &c->disc, (long long)n)) || (s = ialloc(c, &c->energy, 2LL * n)) ||
-      (s = ialloc(c, &c->trace, (long long)n)) || (s = ialloc(c, &c->rnorm, (long long)n)) ||
+      (s = ialloc(c, &c->rnorm, (long long)n)) ||
       (s = ialloc(c, &c->Vb[0], c->sM * n)) || (s = ialloc(c, &c->Vb[1], c->sM * n)) ||
       (s = ialloc(c, &c->Vn, c->sM * n)) ||
       (s = ialloc(c, &c->si_work, si_workspace_doubles(n, (int)twoD, jacobi_block((int)twoD)))) ||
