@@ -999,7 +999,7 @@ def itebd_report(pkg, torch, d_values=(4, 8, 12, 16, 20, 24, 30, 48), batch=64, 
     energy per site against the Bethe-ansatz value."""
     e0 = 0.25 - math.log(2.0)      # Bethe-ansatz ground-state energy per site (J = 1)
     res = {"workload": f"AF Heisenberg chain, tau = 0.05, Neel start, {warm} + {n} updates; "
-                       f"FP64 (GEMMs, cluster Jacobi eig of the 2D_b x 2D_b bond density matrix)",
+                       f"FP64 (GEMMs, Jacobi eig of the 2D_b x 2D_b bond density matrix)",
            "per_D": {}}
     for D in d_values:
         row = {}
@@ -1044,10 +1044,10 @@ def itebd_cpu_baseline(d_values=(8, 16, 30), budget_s=4.0, warm=60):
 
 ITEBD_METRIC = "iTEBD update steps/s, AF Heisenberg chain (tau = 0.05), FP64"
 ITEBD_WORKLOADS = {"itebd_heisenberg_d30": 30, "itebd_heisenberg_d16": 16}
-# kernels per warm-started update: phi GEMM, gate, rho GEMM, symmetrise (2), V^T rho V
-# (2 GEMMs + symmetrise (2)), Jacobi (copy, solve, take), Schmidt, V W GEMM, P' GEMM,
-# scale, take
-ITEBD_LAUNCHES_PER_UPDATE = 17
+# kernels per warm-started update of 16 rows and more: phi GEMM, gate, rho GEMM, V^T rho V
+# (2 GEMMs + symmetrise), the eigensolver (factor, two FP32 Jacobi passes, 20 m x m products,
+# sparse Jacobi), Schmidt, V W GEMM, P' GEMM, scale and copy
+ITEBD_LAUNCHES_PER_UPDATE = 34
 
 
 def run_itebd_line(args, world, rank, local):
@@ -1086,11 +1086,11 @@ def run_itebd_line(args, world, rank, local):
            "config": {"workload": args.workload, "D_b": D, "tau": 0.05, "chains_per_gpu": 1,
                       "l2": "per-update working set is tiny (< 1 MB); one flush before the timed region",
                       "parallelism": f"replicas x{world}"},
-           "roofline": {"kernel": "k_si_jacobi (cluster Jacobi of the 2D_b x 2D_b bond density matrix)",
+           "roofline": {"kernel": "k_rr_jacobi32 (FP32 Jacobi passes of the 2D_b x 2D_b bond density matrix)",
                         "bound": "latency", "achieved": None, "peak": None, "unit": None, "frac": None,
                         "traffic": None,
-                        "note": "one problem of size 2D_b on 8 SMs: bound by the per-round latency of the "
-                                "rotation-angle chain and the cluster barrier, not by a throughput peak"},
+                        "note": "one problem of size 2D_b on one SM: bound by the per-round latency of the "
+                                "rotation-angle chain and its barrier, not by a throughput peak"},
            "energy_per_site": e, "energy_minus_bethe": e - (0.25 - math.log(2.0)),
            "gpu_launches": ITEBD_LAUNCHES_PER_UPDATE * args.steps, "clocks": clk.summary()}
     if rank == 0 and not args.quick:
@@ -1177,7 +1177,7 @@ def run_quantum_line(args, world, rank, local):
                       "D_cut": q.D_cut, "Dy": 4, "precision": prec,
                       "l2": f"flushed before every update step ({L2_FLUSH_BYTES >> 20} MiB write)",
                       "parallelism": f"replicas x{world}"},
-           "roofline": {"kernel": "eigensolver stage (k_si_jacobi, k_si_chol32, k_si_rotate, k_xs_gemm)",
+           "roofline": {"kernel": "eigensolver stage (k_xs_gemm, k_gram_chol32, k_si_rotate, k_rr_jacobi32)",
                         "bound": "latency", "achieved": None, "peak": None, "unit": None, "frac": None,
                         "traffic": None,
                         "share_of_step": round(ms.get("eig", 0.0) / max(1e-9, sum(ms.values())), 4),

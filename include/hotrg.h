@@ -80,7 +80,7 @@ typedef enum { HOTRG_DIR_X = 0, HOTRG_DIR_Y = 1 } hotrg_dir;
  *                 every operand row is scaled by a power of two and rounded to
  *                 6S bits, the digit products are exact and their leading sums
  *                 accumulate exactly on the tensor cores (K split into parts of
- *                 at most 2336), intermediates are FP64.  About 2^-(6S+1) per
+ *                 at most 2336, summed as integers), intermediates are FP64.  About 2^-(6S+1) per
  *                 term relative to the row maxima; aimed at free energies
  *                 within 1e-9 of the FP64 result.
  */
@@ -107,8 +107,8 @@ typedef struct {
   double eig_residual; /* max_i<=D' ||G u_i - lambda_i u_i|| / lambda_1 (path 2)    */
   int eig_rr;       /* Rayleigh-Ritz steps of the subspace iteration (path 2)      */
   int eig_sweeps;   /* most rounds of the FP64 finishing Jacobi of one Rayleigh-Ritz
-                       step (path 2): rotations still needed after the first-order
-                       corrections (0: none)                                        */
+                       step (path 2): rotations still needed after the refinement
+                       (0: none)                                                    */
   int eig_sweeps32; /* most FP32 Jacobi sweeps of one Rayleigh-Ritz step (path 2)  */
 } hotrg_step_info_t;
 
@@ -242,7 +242,8 @@ hotrg_status hotrg_create(const double *T0, int D0, int D_cut, hotrg_prec prec,
  * rescale and log-sum update.  See the header comment for the synchronisation.
  * The leading D'+1 eigenpairs of each environment come from a batched FP64
  * eigensolver (both environments at once): for Dx^2 <= 96 a parallel two-sided
- * Jacobi diagonalisation of the whole matrix (Sec. II.B, Eqs. 5-6), otherwise
+ * Jacobi diagonalisation of the whole matrix (Sec. II.B, Eqs. 5-6; FP32 rotations,
+ * refined in FP64), otherwise
  * block subspace iteration with Rayleigh-Ritz steps solved by the same Jacobi
  * method, stopped at a residual of 1e-12 relative to the largest eigenvalue.
  * If that bound is not reached within HOTRG_OPT_EIG_MAX_ITERS iterations the
@@ -458,9 +459,10 @@ hotrg_status hotrg_batch_get_tensor(hotrg_ctx *ctx, int inst, double *host_out, 
  * leading digit sums (K is split into parts of at most 2336 for that), and
  * combined in 64-bit integer and FP64 arithmetic.  Error per term about
  * 2^-(6 slices) relative to the row maxima max|A_i.| max|B_j.| (slices = 8:
- * about 1e-15 of max|A_i.| max|B_j.| K).  4 <= slices <= 8, K >= 1, lda, ldb >= K, ldc >= N.  Allocates its scratch
- * (about 2 slices (M + N) K bytes) with cudaMalloc, runs on `stream` and
- * synchronises it before returning.  Returns HOTRG_OK, HOTRG_EINVAL,
+ * about 1e-15 of max|A_i.| max|B_j.| K).  4 <= slices <= 8, K >= 1, lda, ldb >= K,
+ * ldc >= N.  Takes its scratch (about 2 slices (M + N) K bytes) from the library's
+ * bounded memory pool (blocks of 1 GiB and more from cudaMalloc), runs on `stream`
+ * and synchronises it before returning.  Returns HOTRG_OK, HOTRG_EINVAL,
  * HOTRG_ENOMEM, HOTRG_ECUDA, or HOTRG_ETIMEOUT if a bounded device wait ran
  * out.  A row with a non-finite entry gives NaN in its outputs.
  */
