@@ -551,7 +551,7 @@ cudaError_t launch_xs(const XsOperand &A, const XsOperand &B, int M, int N, int 
                         ((long long)ntn * ntm * batch * osplit * csplit * 2 <= 152 && kpart >= 128 * csplit)))
     csplit *= 2;
   const int kbp = (nkb + osplit * csplit - 1) / (osplit * csplit);
-  if (kbp * C::BK > kXsMaxK || ntm > 65535 || batch > 65535) return cudaErrorInvalidValue;
+  if (kbp * C::BK > kXsMaxK || csplit * kbp * C::BK > kXsMaxSumK || ntm > 65535 || batch > 65535) return cudaErrorInvalidValue;
   const int stall = take_stall(kStallGemm) ? 1 : 0;
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3((unsigned)csplit * ntn * osplit, ntm, batch);

@@ -29,7 +29,11 @@ namespace hotrg {
 constexpr int kXsBits = 6;        // bits per slice digit
 constexpr int kXsMaxK = 2336;     // longest K part of one CTA (multiple of 32) with 7 2^10 K < 2^24
 constexpr int kXsMaxBatch = 65535;  // instances of one launch (grid limit)
-constexpr int kXsMaxSumK = 8192;  // longest K of one launch: the integer sums stay below 2^63
+// Longest K of one launch.  A scaled element can round up to exactly 1, so a term
+// reaches 2^50 units (its dropped digit pairs add at most 2^-24 of that) and the
+// sum of 8192 of them 2^63: K stays below.  31 256, so that the parts of a
+// launch divide into 1, 2, 4 or 8 of whole K blocks and never cover more.
+constexpr int kXsMaxSumK = 7936;
 constexpr int kXsMaxSlices = 8;
 constexpr int kXsStagedK = 128;  // strided-K operands up to this K are sliced through shared memory
 
