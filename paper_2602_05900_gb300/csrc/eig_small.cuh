@@ -14,7 +14,8 @@ constexpr int kSmallEigSlots = 7;   // m x m scratch matrices per problem
 
 struct SmallEig {
   int P, m;              // problems, matrix size
-  PSet H;                // symmetric m x m matrix of problem z (its symmetric part is used)
+  PSet H;                // m x m matrix of problem z, symmetric to the last bit (of the products
+                         // with it only one triangle is computed)
   PSet scratch;          // kSmallEigSlots consecutive m x m slots of problem z
   bool full;             // resolve every pair to FP64 rounding of H (direct solves); else to
                          // 2^-44 of the largest eigenvalue (Rayleigh-Ritz steps, whose H
