@@ -221,13 +221,11 @@ __global__ void __launch_bounds__(1024) k_rr_start(PSet Cin, int m, PSet W, PSet
 // problem z (op(A) = A^T if ta).  One CTA per 8 x 8 output tile; the sum over
 // k is split four ways across the CTA's threads and combined in a fixed order.
 // unless (optional): nothing is done for problem z where unless.at(z)[3] != 0;
-// copy (optional): receives the result too.  sym: the product is symmetric but for
-// rounding; only i <= j is computed, and mirrored, so that it is so to the last bit.
+// copy (optional): receives the result too.
 __global__ void __launch_bounds__(256) k_rr_mm(PSet A, int ta, PSet B, double bs, double bd,
-                                               PSet Out, int m, PSet unless, PSet copy, int sym) {
+                                               PSet Out, int m, PSet unless, PSet copy) {
   pdl_enter();
   if (unless.b0 && unless.at(blockIdx.z)[3] != 0.0) return;
-  if (sym && blockIdx.x > blockIdx.y) return;
   __shared__ double As[8][kSiMaxBlock + 1];   // op(A) rows i0..i0+7, all k
   __shared__ double Bs[8][kSiMaxBlock + 1];   // B columns j0..j0+7, all k
   __shared__ double part[4][8][9];
@@ -251,10 +249,51 @@ __global__ void __launch_bounds__(256) k_rr_mm(PSet A, int ta, PSet B, double bs
     const int i = i0 + ti, j = j0 + tj;
     if (i < m && j < m) {
       const double v = (part[0][ti][tj] + part[1][ti][tj]) + (part[2][ti][tj] + part[3][ti][tj]);
-      if (sym && i > j) return;
       Out.at(z)[(size_t)j * m + i] = v;
-      if (sym) Out.at(z)[(size_t)i * m + j] = v;
       if (copy.b0) copy.at(z)[(size_t)j * m + i] = v;
+    }
+  }
+}
+
+// Out = (A^T B + B^T A) / 2, symmetric to the last bit, with the tiles and sums of
+// k_rr_mm: the mean of the two triangles of H = W^T (X^T Y W).  Where W is large (a
+// block that holds numerically null directions) the triangles differ by far more
+// than small_eig resolves; given as they are they took its last stage 200 to 280
+// rounds (5 at most now), and one of them for both costs the iteration more steps
+// than their mean (Ising beta = 8, D = 13 to 24, BF16X3: 186 and 117 in twelve steps).
+__global__ void __launch_bounds__(256) k_rr_sym(PSet A, PSet B, PSet Out, int m) {
+  pdl_enter();
+  if (blockIdx.x > blockIdx.y) return;
+  __shared__ double As[2][8][kSiMaxBlock + 1], Bs[2][8][kSiMaxBlock + 1];   // columns of tile I, of tile J
+  __shared__ double part[2][4][8][9];
+  const int z = blockIdx.z, i0 = blockIdx.x * 8, j0 = blockIdx.y * 8;
+  const double *a = A.at(z), *b = B.at(z);
+  for (int e = threadIdx.x; e < 8 * m; e += blockDim.x) {
+    const int r = e / m, k = e % m;
+    const int i = i0 + r, j = j0 + r;
+    As[0][r][k] = i < m ? a[(size_t)i * m + k] : 0.0;
+    As[1][r][k] = j < m ? a[(size_t)j * m + k] : 0.0;
+    Bs[0][r][k] = i < m ? b[(size_t)i * m + k] : 0.0;
+    Bs[1][r][k] = j < m ? b[(size_t)j * m + k] : 0.0;
+  }
+  __syncthreads();
+  const int ti = threadIdx.x & 7, tj = (threadIdx.x >> 3) & 7, ks = threadIdx.x >> 6;
+  double ab = 0.0, ba = 0.0;
+  for (int k = ks; k < m; k += 4) {
+    ab = fma(As[0][ti][k], Bs[1][tj][k], ab);
+    ba = fma(Bs[0][ti][k], As[1][tj][k], ba);
+  }
+  part[0][ks][ti][tj] = ab;
+  part[1][ks][ti][tj] = ba;
+  __syncthreads();
+  if (threadIdx.x < 64) {
+    const int i = i0 + ti, j = j0 + tj;
+    if (i < m && j < m) {
+      double v[2];
+      for (int q = 0; q < 2; ++q) v[q] = (part[q][0][ti][tj] + part[q][1][ti][tj]) + (part[q][2][ti][tj] + part[q][3][ti][tj]);
+      const double h = 0.5 * (v[0] + v[1]);
+      Out.at(z)[(size_t)j * m + i] = h;
+      if (i0 != j0) Out.at(z)[(size_t)i * m + j] = h;
     }
   }
 }
@@ -647,27 +686,25 @@ cudaError_t si_solve(const SiBatch &b, double *work, double tol, int max_iter, c
       // W <- W (3I - W^T C0 W) / 2 twice, the second time only where it is needed
       // (Tn holds the result either way)
       const PSet T2 = slot(4 + kSmallEigSlots);
-      launch_pdl(k_rr_mm, gmm, 256, 0, s, B.W, 0, Wn, 1.0, 0.0, Ck, m, always, always, 0);   // C0 W
-      launch_pdl(k_rr_mm, gmm, 256, 0, s, Wn, 1, Ck, 1.0, 0.0, Rr, m, always, always, 0);    // W^T C0 W
-      launch_pdl(k_rr_mm, gmm, 256, 0, s, Wn, 0, Rr, -0.5, 1.5, Tn, m, always, T2, 0);
-      launch_pdl(k_rr_mm, gmm, 256, 0, s, B.W, 0, T2, 1.0, 0.0, Ck, m, B.sig, always, 0);
-      launch_pdl(k_rr_mm, gmm, 256, 0, s, T2, 1, Ck, 1.0, 0.0, Rr, m, B.sig, always, 0);
-      launch_pdl(k_rr_mm, gmm, 256, 0, s, T2, 0, Rr, -0.5, 1.5, Tn, m, B.sig, always, 0);
+      launch_pdl(k_rr_mm, gmm, 256, 0, s, B.W, 0, Wn, 1.0, 0.0, Ck, m, always, always);   // C0 W
+      launch_pdl(k_rr_mm, gmm, 256, 0, s, Wn, 1, Ck, 1.0, 0.0, Rr, m, always, always);    // W^T C0 W
+      launch_pdl(k_rr_mm, gmm, 256, 0, s, Wn, 0, Rr, -0.5, 1.5, Tn, m, always, T2);
+      launch_pdl(k_rr_mm, gmm, 256, 0, s, B.W, 0, T2, 1.0, 0.0, Ck, m, B.sig, always);
+      launch_pdl(k_rr_mm, gmm, 256, 0, s, T2, 1, Ck, 1.0, 0.0, Rr, m, B.sig, always);
+      launch_pdl(k_rr_mm, gmm, 256, 0, s, T2, 0, Rr, -0.5, 1.5, Tn, m, B.sig, always);
       nl += 6;
       std::swap(Wn, Tn);
       // where X is further from orthonormal (nearly dependent columns at a first
       // check), W comes instead from an FP64 Cholesky of C0, shifted where C0 is far
       // from I (X W is then orthonormal for any conditioning the shift allows)
       if ((e = chol64(B.W, m, shift, Wn, B.flag, B.sig, P, s, &nl))) return e;
-      launch_pdl(k_rr_mm, gmm, 256, 0, s, B.C, 0, Wn, 1.0, 0.0, Tn, m, always, always, 0);     // (X^T Y) W
-      // H = W^T X^T Y W: where W is large (a first check on nearly dependent columns)
-      // its two triangles differ by far more than small_eig resolves, so one is taken
-      launch_pdl(k_rr_mm, gmm, 256, 0, s, Wn, 1, Tn, 1.0, 0.0, Ck, m, always, always, 1);
+      launch_pdl(k_rr_mm, gmm, 256, 0, s, B.C, 0, Wn, 1.0, 0.0, Tn, m, always, always);     // (X^T Y) W
+      launch_pdl(k_rr_sym, gmm, 256, 0, s, Wn, Tn, Ck, m);                                  // H = W^T X^T Y W
       nl += 2;
       if ((e = cudaGetLastError())) return e;
       const SmallEig se{P, m, Ck, slot(4), false, false, B.W, m, m, B.th, B.flag, B.sweeps, B.flag + 3};
       if ((e = small_eig(se, s, &nl))) return e;                    // H = Z Theta Z^T (Z in B.W)
-      launch_pdl(k_rr_mm, gmm, 256, 0, s, Wn, 0, B.W, 1.0, 0.0, Rr, m, always, always, 0);     // R = W Z
+      launch_pdl(k_rr_mm, gmm, 256, 0, s, Wn, 0, B.W, 1.0, 0.0, Rr, m, always, always);     // R = W Z
       nl += 1;
       if (xs_small) {
         if ((e = rot(X, Rr, Z, 0))) return e;
