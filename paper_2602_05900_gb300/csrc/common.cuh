@@ -47,11 +47,12 @@ __device__ __forceinline__ long long map_off32(const IdxMap &m, int i) {
 }
 
 // FP64 <-> FP32 by integer arithmetic (the conversion instructions run at GB300's
-// FP64 rate); subnormal FP32 values are taken as zero.  To nearest even:
-__device__ __forceinline__ float to_f32(double x) {
+// FP64 rate); subnormal FP32 values are taken as zero.  x 2^(1023 - bias), to nearest
+// even (200 <= bias <= 1900: the exponent field that becomes 1):
+__device__ __forceinline__ float to_f32(double x, int bias = 1023) {
   const unsigned long long b = static_cast<unsigned long long>(__double_as_longlong(x));
   const unsigned long long a = b & 0x7FFFFFFFFFFFFFFFull;
-  const long long r = (long long)((a + 0x0FFFFFFFull + ((a >> 29) & 1)) >> 29) - (896ll << 23);
+  const long long r = (long long)((a + 0x0FFFFFFFull + ((a >> 29) & 1)) >> 29) - ((long long)(bias - 127) << 23);
   const unsigned f = r < (1 << 23) ? 0u : r >= (255ll << 23) ? (a > 0x7FF0000000000000ull ? 0x7FC00000u : 0x7F800000u)
                                                               : (unsigned)r;
   return __uint_as_float(f | ((unsigned)(b >> 32) & 0x80000000u));

@@ -51,15 +51,23 @@
 namespace hotrg {
 namespace {
 
-// |h| truncated to FP32 with integer arithmetic (FP64 conversions run at the
-// FP64 rate); values below the FP32 range give 0
-__device__ inline float mag32(double h) {
-  const unsigned hi = (unsigned)__double2hiint(h) & 0x7FFFFFFFu, lo = (unsigned)__double2loint(h);
-  const int e = (int)(hi >> 20) - 896;
+// Couplings, gaps and quotients of the FP64 stages are judged in FP32, relative
+// to the largest diagonal entry: its exponent field (kept within the range in which
+// every product below stays normal; that of 1 for a zero diagonal) is the bias of
+// their conversions, so that a matrix of any scale is treated alike.
+__device__ inline unsigned abs_hi(double h) { return (unsigned)__double2hiint(h) & 0x7FFFFFFFu; }
+__device__ inline int scale_bias(unsigned hi) { return hi >> 20 ? min(max((int)(hi >> 20), 200), 1900) : 1023; }
+__device__ inline unsigned warp_max(unsigned v) { return __reduce_max_sync(0xffffffffu, v); }
+
+// |h| 2^(1023 - bias) truncated to FP32 with integer arithmetic (FP64 conversions
+// run at the FP64 rate); values below the FP32 range give 0
+__device__ inline float mag32(unsigned hi, unsigned lo, int bias) {
+  const int e = (int)(hi >> 20) - (bias - 127);
   if (e <= 0) return 0.0f;
   if (e >= 255) return INFINITY;
   return __uint_as_float(((unsigned)e << 23) | ((hi & 0xFFFFFu) << 3) | (lo >> 29));
 }
+__device__ inline float mag32(double h, int bias) { return mag32(abs_hi(h), (unsigned)__double2loint(h), bias); }
 
 __device__ inline void jacobi_angle(double hpp, double hqq, double hpq, double &c, double &s) {
   // solve h_pq t^2 + (h_qq - h_pp) t - h_pq = 0 for the smaller root (Golub &
@@ -436,7 +444,7 @@ __global__ void __launch_bounds__(256) k_se_mm(MmOp op0, MmOp op1, int P, int m,
   __shared__ double Bs[8][kSiMaxBlock + 1];   // B' columns j0..j0+7, all k
   __shared__ double part[4][8][9];
   __shared__ double lam[kSiMaxBlock], rn[kSiMaxBlock];
-  __shared__ float s_mx;
+  __shared__ unsigned s_mx;
   const bool second = (int)blockIdx.z >= P;
   const MmOp &o = second ? op1 : op0;
   const int z = second ? (int)blockIdx.z - P : (int)blockIdx.z;
@@ -477,13 +485,14 @@ __global__ void __launch_bounds__(256) k_se_mm(MmOp op0, MmOp op1, int P, int m,
     }
     __syncthreads();
     if (threadIdx.x < 32) {
-      float v = 0.0f;
-      for (int k = threadIdx.x; k < m; k += 32) v = fmaxf(v, mag32(lam[k]));
-      for (int s = 16; s > 0; s >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, s));
+      unsigned v = 0;
+      for (int k = threadIdx.x; k < m; k += 32) v = max(v, abs_hi(lam[k]));
+      v = warp_max(v);
       if (threadIdx.x == 0) s_mx = v;
     }
     __syncthreads();
-    const float fl = noise * s_mx;
+    const int bias = scale_bias(s_mx);
+    const float fl = noise * mag32(s_mx, 0, bias);
     for (int e = threadIdx.x; e < 8 * m; e += blockDim.x) {
       const int r = e / m, k = e % m, j = j0 + r;
       double v = 0.0;
@@ -500,10 +509,11 @@ __global__ void __launch_bounds__(256) k_se_mm(MmOp op0, MmOp op1, int P, int m,
           }
           const double gap = lam[j] - lam[k];
           const double num = fma(-lam[j], g, s);
-          const float off = mag32(fma(0.5 * gap, g, num));    // s - (lam_j + lam_k) g / 2
+          const float off = mag32(fma(0.5 * gap, g, num), bias);    // s - (lam_j + lam_k) g / 2
           // the quotient needs FP32 accuracy only: what it misses is of the
           // order of 1e-7 of a coupling that the next pass sees
-          if (mag32(gap) > (float)kSfsCluster * off && off > fl) v = (double)((float)num / (float)gap);
+          if (mag32(gap, bias) > (float)kSfsCluster * off && off > fl)
+            v = to_f64(to_f32(num, bias) / to_f32(gap, bias));
           else v = -0.5 * g;
           if (norm) v *= rn[k];
         }
@@ -562,7 +572,6 @@ __global__ void __launch_bounds__(kSparseThreads, 1)
   int *selp = best + m, *selq = selp + maxsel;
   float *rt = reinterpret_cast<float *>(selq + maxsel);   // sqrt|h_pp|
   __shared__ int nsel;
-  __shared__ float s_floor;
   const int z = blockIdx.z;
   const double *hin = Hin.at(z);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nwarps = blockDim.x >> 5;
@@ -572,27 +581,25 @@ __global__ void __launch_bounds__(kSparseThreads, 1)
     W[r * ld + c] = r == c ? 1.0 : 0.0;
   }
   __syncthreads();
-  if (threadIdx.x < 32) {
-    float v = 0.0f;
-    for (int i = threadIdx.x; i < m; i += 32) v = fmaxf(v, mag32(H[i * ld + i]));
-    for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
-    if (threadIdx.x == 0) s_floor = ldexpf(v, -floor_exp);
-  }
+  unsigned mx = 0;                                  // every warp on its own: no barrier
+  for (int i = lane; i < m; i += 32) mx = max(mx, abs_hi(H[i * ld + i]));
+  mx = warp_max(mx);
+  const int bias = scale_bias(mx);
+  const float fl = ldexpf(mag32(mx, 0, bias), -floor_exp);
   int round = 0;
   bool done = false;
   for (; round < kSparseRounds * m; ++round) {
-    for (int p = threadIdx.x; p < m; p += blockDim.x) rt[p] = sqrtf(mag32(H[p * ld + p]));
+    for (int p = threadIdx.x; p < m; p += blockDim.x) rt[p] = sqrtf(mag32(H[p * ld + p], bias));
     if (threadIdx.x == 0) nsel = 0;
     __syncthreads();
     // (1) each row's best partner (one warp per row); rows p and q both read the
     // entry above the diagonal, so they agree on it
-    const float fl = s_floor;
     for (int p = warp; p < m; p += nwarps) {
       float bv = 0.0f;
       int bq = -1;
       const float rp = 1e-15f * rt[p];
       for (int q = lane; q < m; q += 32) {
-        const float hv = mag32(q > p ? H[p * ld + q] : H[q * ld + p]);
+        const float hv = mag32(q > p ? H[p * ld + q] : H[q * ld + p], bias);
         if (q != p && hv > fl && hv > rp * rt[q] && hv > bv) {
           bv = hv;
           bq = q;
