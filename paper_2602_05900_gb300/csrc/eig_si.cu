@@ -45,9 +45,12 @@ namespace {
 constexpr int kSplitMax = 8;     // split-K partials of G X
 // FP64 FMAs of one n x m x m product batch from which its rotations and Gram
 // matrices run as exact-slice products: few problems are latency bound and stay
-// with the single FP64 launches longer (24-instance sweep: 150.4 ms with 2^25 for
-// all, 142.4 ms like this; with 2^22 for all the one pair of a D = 32 run, 2^22.2,
-// took 65 ms against 50)
+// with the single FP64 launches longer (24-instance TF32 sweep: 150.4 ms with 2^25
+// for all, 142.4 ms like this; with 2^22 for all the one pair of a D = 32 run, 2^22.2,
+// took 65 ms against 50).  The lower line is for environments of reduced precision
+// only, whose isometries are rounded to 2^-24 or coarser before they are used: the
+// slices leave U^T U within 1e-13 of I, the FP64 launches within 2e-15 (five D = 32
+// instances: 1.7e-13 and 1.4e-15).
 constexpr double kXsSmallWork = 0x1p25, kXsBatchWork = 0x1p23;
 constexpr int kSiSmallBatch = 8;      // problems up to which the solve is latency bound
 constexpr double kSiFloorTol = 1e-10;  // residuals accepted once they stop decreasing
@@ -483,7 +486,8 @@ cudaError_t si_solve(const SiBatch &b, double *work, double tol, int max_iter, c
   // batch makes them FP64-throughput bound; below
   // that the single SIMT launch beats the slice-and-multiply sequence.
   const bool xs = b.xs;
-  const bool xs_small = xs && (double)P * n * m * m >= (P > kSiSmallBatch ? kXsBatchWork : kXsSmallWork);
+  const bool batch = P > kSiSmallBatch && b.floor_tol > 0.0;
+  const bool xs_small = xs && (double)P * n * m * m >= (batch ? kXsBatchWork : kXsSmallWork);
   XsOperand gs{};
   // slices of a row-major (rows x K) view of problem z's buffer at src
   auto xs_slot = [&](long long off, long long scoff, int rows, int K) {

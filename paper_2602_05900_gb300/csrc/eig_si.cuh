@@ -34,7 +34,8 @@ struct SiBatch {
   bool has_trace;
   double shift_rel;      // initial shift / Tr G
   int first_check;       // expected convergence iteration (first Rayleigh-Ritz step of small batches)
-  double floor_tol;      // residual accepted once it stops decreasing (0: the FP64 default, 1e-10)
+  double floor_tol;      // residual accepted once it stops decreasing (0: G of FP64 grade, 1e-10; else G
+                         // carries that much rounding)
   bool graded;           // jacobi_full: G = V^T (M^T M) V with a V that nearly diagonalises it (a warm start)
 };
 
