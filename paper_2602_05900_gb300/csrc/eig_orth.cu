@@ -25,6 +25,7 @@
 #include <algorithm>
 
 #include "eig_orth.cuh"
+#include "kernel_attr.cuh"
 #include "launch.cuh"
 #include "eig_si.cuh"
 
@@ -612,13 +613,9 @@ int tile_of(int m) { return m <= 32 ? 2 : (m + 15) / 16; }   // 16-wide tiles pe
 
 template <int U>
 cudaError_t launch_gram_chol(PSet Y, int n, int m, float shift, PSet W, int *flag, int P, cudaStream_t s) {
-  static bool done = false;
-  if (!done) {
-    cudaError_t e = cudaFuncSetAttribute(k_gram_chol32<U>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)gram_chol_smem<U>(16 * U));
-    if (e) return e;
-    done = true;
-  }
+  static SmemLimit limit;
+  if (cudaError_t e = limit.raise(reinterpret_cast<const void *>(k_gram_chol32<U>), (int)gram_chol_smem<U>(16 * U)))
+    return e;
   launch_pdl(k_gram_chol32<U>, dim3(kOrthCluster, 1, P), 256, gram_chol_smem<U>(m), s, Y, n, m, shift, W, flag);
   return cudaGetLastError();
 }
@@ -626,13 +623,10 @@ cudaError_t launch_gram_chol(PSet Y, int n, int m, float shift, PSet W, int *fla
 template <int RT>
 cudaError_t launch_rotate(PSet A0, PSet A1, PSet W, PSet Out0, PSet Out1, int count, int n, int m, bool tri, int P,
                           cudaStream_t s) {
-  static bool done = false;
-  if (!done) {
-    cudaError_t e = cudaFuncSetAttribute(k_si_rotate<RT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)(sizeof(double) * kSiMaxBlock * (RT + kSiMaxBlock + 1)));
-    if (e) return e;
-    done = true;
-  }
+  static SmemLimit limit;
+  if (cudaError_t e = limit.raise(reinterpret_cast<const void *>(k_si_rotate<RT>),
+                                  (int)(sizeof(double) * kSiMaxBlock * (RT + kSiMaxBlock + 1))))
+    return e;
   // a plain launch: started early, its blocks would be dealt out while the factor's
   // cluster still holds SMs, and the others would get two (D = 48 job: 57.6 ms
   // started early, 55.5 ms like this)
@@ -722,12 +716,8 @@ cudaError_t chol64(PSet C, int m, double shift, PSet W, int *flag, PSet only_if,
 template <int U>
 static cudaError_t launch_lr(PSet H, int m, PSet L, PSet B, int P, cudaStream_t s) {
   constexpr size_t smem = (size_t)(16 * U) * (16 * U) * sizeof(F2);
-  static bool done = false;
-  if (!done) {
-    const cudaError_t e = cudaFuncSetAttribute(k_lr_factor<U>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e) return e;
-    done = true;
-  }
+  static SmemLimit limit;
+  if (cudaError_t e = limit.raise(reinterpret_cast<const void *>(k_lr_factor<U>), (int)smem)) return e;
   launch_pdl(k_lr_factor<U>, dim3(1, 1, P), 256, smem, s, H, m, L, B);
   return cudaGetLastError();
 }

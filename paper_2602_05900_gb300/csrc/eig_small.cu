@@ -44,6 +44,7 @@
 #include <utility>
 
 #include "eig_orth.cuh"
+#include "kernel_attr.cuh"
 #include "launch.cuh"
 #include "eig_si.cuh"
 #include "eig_small.cuh"
@@ -692,12 +693,8 @@ __global__ void k_eig_one(PSet G, PSet X, PSet theta, int m, int P) {
 template <int HM, int SPL, int RPG, int IA>
 cudaError_t run_j32(PSet H, int m, float floor_abs, PSet V, int *sweeps, int P, cudaStream_t s) {
   const auto kern = k_rr_jacobi32<HM, SPL, RPG, IA>;
-  static bool done = false;
-  if (!done) {
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)J32Cfg<HM, SPL>::kSmem);
-    if (e) return e;
-    done = true;
-  }
+  static SmemLimit limit;
+  if (cudaError_t e = limit.raise(reinterpret_cast<const void *>(kern), (int)J32Cfg<HM, SPL>::kSmem)) return e;
   // threads of the angles, of the matrix (4 x 8 blocks per warp, IA of them in turn) and of V
   const int h = m / 2, nang = (h + 31) / 32 * 32;
   int tiles = 0;
@@ -717,12 +714,8 @@ cudaError_t launch_j32(PSet H, int m, float floor_abs, PSet V, int *sweeps, int 
 }
 
 cudaError_t small_attrs() {
-  static bool done = false;
-  if (done) return cudaSuccess;
-  const cudaError_t e = cudaFuncSetAttribute(k_rr_sparse_jacobi, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-  if (e) return e;
-  done = true;
-  return cudaSuccess;
+  static SmemLimit limit;
+  return limit.raise(reinterpret_cast<const void *>(k_rr_sparse_jacobi), 200 * 1024);
 }
 
 }  // namespace

@@ -24,6 +24,7 @@
 #include <cuda.h>
 #include <cudaTypedefs.h>
 
+#include "kernel_attr.cuh"
 #include "tc_chain.cuh"
 #include "tcgen05.cuh"
 
@@ -369,19 +370,9 @@ cudaError_t launch_chain(const ChainArgs &a, cudaStream_t s) {
       !make_map_f32(&tt, a.T6, DE, DE, a.pitchT, a.batch, a.sT6, 128) ||
       !make_map_f32(&tu, a.U7, n, a.Dn, a.pitchU, a.batch, a.sU7, 32))
     return cudaErrorInvalidValue;
-  static bool attr_set = false;
-  if (!attr_set) {
-    cudaError_t e = cudaFuncSetAttribute(k_tc_chain<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM);
-    if (e != cudaSuccess) return e;
-    attr_set = true;
-  }
-  static int nsm = 0;
-  if (nsm == 0) {
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || nsm < 1)
-      nsm = 148;
-  }
+  static SmemLimit limit;
+  if (cudaError_t e = limit.raise(reinterpret_cast<const void *>(k_tc_chain<D>), C::SMEM)) return e;
+  const int nsm = sm_count();
   const long long units = (long long)(DE / C::BN) * (a.Dn * DE / C::BM) * a.batch;
   const int grid = (int)(units < nsm ? units : nsm);
   const int stall = take_stall(kStallChain) ? 1 : 0;

@@ -36,6 +36,7 @@
 #include <algorithm>
 
 #include "tc_exact.cuh"
+#include "kernel_attr.cuh"
 #include "launch.cuh"
 #include "tcgen05.cuh"
 
@@ -529,13 +530,8 @@ template <int S, int BN>
 cudaError_t launch_xs(const XsOperand &A, const XsOperand &B, int M, int N, int K,
                       const XsOut &o, int osplit, int *err, cudaStream_t s) {
   using C = XsCfg<S, BN>;
-  static bool attr_set = false;
-  if (!attr_set) {
-    cudaError_t e = cudaFuncSetAttribute(k_xs_gemm<S, BN>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM);
-    if (e != cudaSuccess) return e;
-    attr_set = true;
-  }
+  static SmemLimit limit;
+  if (cudaError_t e = limit.raise(reinterpret_cast<const void *>(k_xs_gemm<S, BN>), C::SMEM)) return e;
   CUtensorMap ta, tb;
   if (!make_xs_map(&ta, A, C::BM, C::ROW) || !make_xs_map(&tb, B, BN, C::ROW))
     return cudaErrorInvalidValue;

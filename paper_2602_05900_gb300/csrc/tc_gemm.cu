@@ -20,6 +20,7 @@
 #include <mutex>
 #include <tuple>
 
+#include "kernel_attr.cuh"
 #include "tc_gemm.cuh"
 #include "tcgen05.cuh"
 
@@ -455,20 +456,9 @@ cudaError_t launch(const CUtensorMap &ta, const CUtensorMap &tb, int M, int N, i
                    const TcEpilogue &epi, int *err, cudaStream_t s) {
   const int stall = take_stall(kStallGemm) ? 1 : 0;
   using C = Cfg<MODE, BN>;
-  static bool attr_set = false;
-  if (!attr_set) {
-    cudaError_t e = cudaFuncSetAttribute(k_tc_gemm<MODE, BN>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM);
-    if (e != cudaSuccess) return e;
-    attr_set = true;
-  }
-  static int nsm = 0;
-  if (nsm == 0) {
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || nsm < 1)
-      nsm = 148;
-  }
+  static SmemLimit limit;
+  if (cudaError_t e = limit.raise(reinterpret_cast<const void *>(k_tc_gemm<MODE, BN>), C::SMEM)) return e;
+  const int nsm = sm_count();
   const long long tiles = (long long)((N + BN - 1) / BN) * ((M + C::BM - 1) / C::BM) * batch;
   const int grid = (int)(tiles < nsm ? tiles : nsm);
   k_tc_gemm<MODE, BN><<<grid, 384, C::SMEM, s>>>(ta, tb, M, N, K, batch, epi, err, wait_limit(),
