@@ -362,8 +362,7 @@ hotrg_status hotrg_set_option(hotrg_ctx *ctx, int option, int value);
  * context's stream.  hotrg_profile_read synchronises the stream and returns
  * the device time per stage accumulated since the profiler was (re)enabled,
  * the algorithmic flops per stage (each flop counted once: split products
- * and zero padding are not counted), and the number of kernels the library
- * itself launched (library-internal eigensolver kernels are not counted).
+ * and zero padding are not counted), and the number of kernels launched.
  */
 enum {
   HOTRG_ST_PREP = 0, HOTRG_ST_ENV, HOTRG_ST_GRAM, HOTRG_ST_EIG, HOTRG_ST_PROJ_P,

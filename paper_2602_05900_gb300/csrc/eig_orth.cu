@@ -637,9 +637,8 @@ cudaError_t launch_rotate(PSet A0, PSet A1, PSet W, PSet Out0, PSet Out1, int co
 
 }  // namespace
 
-cudaError_t gram_reduce(PSet part, PSet out, int chunks, int m, bool sym, int P, cudaStream_t s,
-                        long long *launches) {
-  launch_pdl(k_si_gram_reduce, dim3((m * m + 63) / 64, 1, P), 256, 0, s, part, out, out, chunks, m, P, sym ? 1 : 0, 0);
+cudaError_t gram_reduce(PSet part, PSet out, int chunks, int m, int P, cudaStream_t s, long long *launches) {
+  launch_pdl(k_si_gram_reduce, dim3((m * m + 63) / 64, 1, P), 256, 0, s, part, out, out, chunks, m, P, 0, 0);
   *launches += 1;
   return cudaGetLastError();
 }

@@ -43,10 +43,8 @@ constexpr int kGramChunks = 256;
 // column-major).  part: kGramChunks m x m slots of problem z.
 cudaError_t gram64(PSet A, PSet B0, PSet out0, const PSet *B1, const PSet *out1, int n, int m, PSet part, int P,
                    cudaStream_t s, long long *launches);
-// out = sum of `chunks` m x m partials of A^T B, symmetrised (sym: only their
-// upper triangles are valid).
-cudaError_t gram_reduce(PSet part, PSet out, int chunks, int m, bool sym, int P, cudaStream_t s,
-                        long long *launches);
+// out = sum of `chunks` m x m partials of A^T B, symmetrised.
+cudaError_t gram_reduce(PSet part, PSet out, int chunks, int m, int P, cudaStream_t s, long long *launches);
 
 // W = diag(d) R^-1 (column-major, upper triangular) with R^T R = diag(d) C diag(d)
 // + shift I, d_j = 1 / sqrt(C_jj), in FP32: Y W is orthonormal to FP32 accuracy.

@@ -568,12 +568,12 @@ cudaError_t si_solve(const SiBatch &b, double *work, double tol, int max_iter, c
           (r = xs_gemm(a, a, m, m, n, B.Cp.b0, map1(m), map1(1), L.per, 1, 0, b.err, s)))
         return r;
       nl += 2;
-      if ((r = gram_reduce(B.Cp, out, 1, m, false, P, s, &nl)) || !Bm) return r;
+      if ((r = gram_reduce(B.Cp, out, 1, m, P, s, &nl)) || !Bm) return r;
       if ((r = xs_split(*Bm, map1(n), map1(1), bb, s)) ||
           (r = xs_gemm(a, bb, m, m, n, B.Cp.b0, map1(m), map1(1), L.per, 1, 0, b.err, s)))
         return r;
       nl += 2;
-      return gram_reduce(B.Cp, *out2, 1, m, false, P, s, &nl);
+      return gram_reduce(B.Cp, *out2, 1, m, P, s, &nl);
     }
     return gram64(A, A, out, Bm, out2, n, m, B.Cp, P, s, &nl);
   };

@@ -543,10 +543,17 @@ hotrg_status step_group(hotrg_ctx *c, Group &g, hotrg_dir dir, int step) {
     Q = g.c1 + 5 * b;
     sPart = sPQ = g.sC1;
   }
-  // FP64 SIMT or exact-slice tensor-core GEMM over the same mapped operands
+  // FP64 SIMT or exact-slice tensor-core GEMM over the same mapped operands; `made`
+  // counts the launches of a stage
+  long long made = 0;
   auto mgemm = [&](const MappedGemm &mg) -> cudaError_t {
-    if (c->prec == HOTRG_BF16XS && D > 1) return gemm_xs(mg, c->xs_digits, g.xw, c->err, st);
+    if (c->prec == HOTRG_BF16XS && D > 1) return gemm_xs(mg, c->xs_digits, g.xw, c->err, st, &made);
+    made += 1;
     return gemm_f64(mg, st);
+  };
+  auto count_stage = [&](int stage) {
+    pf.launched(stage, (int)made);
+    made = 0;
   };
   // A tensor-core contraction segment (its launches depend only on the key):
   // run eagerly the first time (the GEMM autotuner times its shapes then),
@@ -638,11 +645,11 @@ hotrg_status step_group(hotrg_ctx *c, Group &g, hotrg_dir dir, int step) {
     }
     pf.begin(HOTRG_ST_ENV);
     if (xs) {
-      CK_CUDA(c, syrk_xs(mp, 4, c->xs_digits, g.xw, c->err, st));
+      CK_CUDA(c, syrk_xs(mp, 4, c->xs_digits, g.xw, c->err, st, &made));
     } else {
       for (const MappedGemm &m : mp) CK_CUDA(c, mgemm(m));
     }
-    pf.launched(HOTRG_ST_ENV, 4);
+    count_stage(HOTRG_ST_ENV);
     pf.end(HOTRG_ST_ENV);
     // G[x1,x2,u1,u2] = sum_{k,k'} A[x1,u1,k,k'] B[x2,u2,k,k']
     pf.begin(HOTRG_ST_GRAM);
@@ -658,12 +665,12 @@ hotrg_status step_group(hotrg_ctx *c, Group &g, hotrg_dir dir, int step) {
     }
     if (xs) {
       gl.batch = 2 * G;                // A_R follows A_L, B_R follows B_L, G_R follows G_L
-      CK_CUDA(c, gemm_xs(gl, c->xs_digits, g.xw, c->err, st));
+      CK_CUDA(c, gemm_xs(gl, c->xs_digits, g.xw, c->err, st, &made));
     } else {
       CK_CUDA(c, mgemm(gl));
       CK_CUDA(c, mgemm(gr));
     }
-    pf.launched(HOTRG_ST_GRAM, 2);
+    count_stage(HOTRG_ST_GRAM);
   }
   // the tensor-core chain closed its own Gram stage (it may run as a graph)
   if (tc) pf.begin(HOTRG_ST_GRAM);
@@ -828,7 +835,7 @@ hotrg_status step_group(hotrg_ctx *c, Group &g, hotrg_dir dir, int step) {
     g5.capC = sPQ * G;
     g5.err = c->err;
     CK_CUDA(c, mgemm(g5));
-    pf.launched(HOTRG_ST_PROJ_P, 1);
+    count_stage(HOTRG_ST_PROJ_P);
     pf.end(HOTRG_ST_PROJ_P);
     // a6: Q[a][y][y'][x1'][x2'] = sum_{x2,k} P[(a,x1',y),(x2,k)] T[x2,x2',k,y']
     pf.begin(HOTRG_ST_PROJ_Q);
@@ -842,7 +849,7 @@ hotrg_status step_group(hotrg_ctx *c, Group &g, hotrg_dir dir, int step) {
     g6.capC = sPQ * G;
     g6.err = c->err;
     CK_CUDA(c, mgemm(g6));
-    pf.launched(HOTRG_ST_PROJ_Q, 1);
+    count_stage(HOTRG_ST_PROJ_Q);
     pf.end(HOTRG_ST_PROJ_Q);
     // a7: T'[(a,y,y'), b] = sum_{x1',x2'} Q[(a,y,y'),(x1',x2')] U[(x1' x2'), b]
     pf.begin(HOTRG_ST_PROJ_T);
@@ -856,7 +863,7 @@ hotrg_status step_group(hotrg_ctx *c, Group &g, hotrg_dir dir, int step) {
     g7.capC = g.sT * G;
     g7.err = c->err;
     CK_CUDA(c, mgemm(g7));
-    pf.launched(HOTRG_ST_PROJ_T, 1);
+    count_stage(HOTRG_ST_PROJ_T);
     pf.end(HOTRG_ST_PROJ_T);
   }
 
@@ -865,7 +872,7 @@ hotrg_status step_group(hotrg_ctx *c, Group &g, hotrg_dir dir, int step) {
   const long long count = (long long)Dn * Dn * E2;
   CK_CUDA(c, maxabs_scale_log(g.Tn, count, g.sT, g.scal + 1, kScal, g.scal, kScal,
                               ldexp(1.0, -(step + 1)), rec + 5, g.sRec, c->err, G, st));
-  pf.launched(HOTRG_ST_RESCALE, 3);
+  pf.launched(HOTRG_ST_RESCALE, 2);
   pf.end(HOTRG_ST_RESCALE);
   std::swap(g.T, g.Tn);
   if (ydir) g.dx = Dn; else g.dy = Dn;

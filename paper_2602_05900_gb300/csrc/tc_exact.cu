@@ -745,7 +745,8 @@ bool syrk_xs_fits(int M, int K, int batch, int S, const XsWork &w) {
   return M > 0 && K > 0 && batch <= kXsMaxBatch && xs_min_split(K) == 1 && xs_fits(M, 0, K, S, batch, w);
 }
 
-cudaError_t syrk_xs(const MappedGemm *g, int count, int S, const XsWork &w, int *err_flag, cudaStream_t s) {
+cudaError_t syrk_xs(const MappedGemm *g, int count, int S, const XsWork &w, int *err_flag, cudaStream_t s,
+                    long long *launches) {
   const int M = g[0].M, K = g[0].K, G = g[0].batch < 1 ? 1 : g[0].batch;
   if (count < 1 || !syrk_xs_fits(M, K, count * G, S, w))
     return cudaErrorInvalidValue;
@@ -760,10 +761,11 @@ cudaError_t syrk_xs(const MappedGemm *g, int count, int S, const XsWork &w, int 
     if ((e = xs_split(pa, q.am, q.ak, a, s))) return e;
   }
   const XsOperand all{w.sa, w.sca, M, K, xs_pitch(K), S, count * G, ea, M};
+  *launches += count + 1;
   return xs_gemm(all, all, M, M, K, g[0].C, g[0].cm, g[0].cn, g[0].bC, 1, 0, err_flag, s);
 }
 
-cudaError_t gemm_xs(const MappedGemm &g, int S, const XsWork &w, int *err_flag, cudaStream_t s) {
+cudaError_t gemm_xs(const MappedGemm &g, int S, const XsWork &w, int *err_flag, cudaStream_t s, long long *launches) {
   if (g.M <= 0 || g.N <= 0) return cudaSuccess;
   const int batch = g.batch < 1 ? 1 : g.batch;
   if (!xs_fits(g.M, g.N, g.K, S, batch, w)) return cudaErrorInvalidValue;
@@ -776,6 +778,7 @@ cudaError_t gemm_xs(const MappedGemm &g, int S, const XsWork &w, int *err_flag, 
   cudaError_t e;
   if ((e = xs_split(pa, g.am, g.ak, a, s)) || (e = xs_split(pb, g.bn, g.bk, b, s))) return e;
   const int ks = xs_min_split(g.K);
+  *launches += ks == 1 ? 3 : 4;
   if (ks == 1) return xs_gemm(a, b, g.M, g.N, g.K, g.C, g.cm, g.cn, g.bC, 1, 0, err_flag, s);
   const long long mn = (long long)g.M * g.N;
   if ((e = xs_gemm(a, b, g.M, g.N, g.K, w.parts, map1(g.N), map1(1), mn, ks, mn * batch,

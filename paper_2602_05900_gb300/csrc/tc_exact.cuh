@@ -110,8 +110,8 @@ void xs_gemm_needs(int M, int N, int K, int S, int batch, long long need[5]);
 // The mapped GEMM of `g` (C(m, n) = sum_k A(m, k) B(n, k) through index maps,
 // batched) as an exact-slice tensor-core GEMM with S digits: the operands are
 // gathered and sliced, K is split into exact parts, the result is written in
-// FP64 through g's output maps.
-cudaError_t gemm_xs(const MappedGemm &g, int S, const XsWork &w, int *err_flag, cudaStream_t s);
+// FP64 through g's output maps.  `launches` is incremented.
+cudaError_t gemm_xs(const MappedGemm &g, int S, const XsWork &w, int *err_flag, cudaStream_t s, long long *launches);
 
 // Whether gemm_xs of that size fits the scratch.
 bool xs_fits(int M, int N, int K, int S, int batch, const XsWork &w);
@@ -121,6 +121,7 @@ bool xs_fits(int M, int N, int K, int S, int batch, const XsWork &w);
 // once and all products are one launch.  The scratch has to fit count * batch
 // instances of A (syrk_xs_fits with that batch; K <= kXsMaxSumK).
 bool syrk_xs_fits(int M, int K, int batch, int S, const XsWork &w);
-cudaError_t syrk_xs(const MappedGemm *g, int count, int S, const XsWork &w, int *err_flag, cudaStream_t s);
+cudaError_t syrk_xs(const MappedGemm *g, int count, int S, const XsWork &w, int *err_flag, cudaStream_t s,
+                    long long *launches);
 
 }  // namespace hotrg
