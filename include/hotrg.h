@@ -198,7 +198,8 @@ hotrg_status hotrg_trace_y(hotrg_ctx *ctx);
  *   uniform, 1/sqrt(D0).  stream: a cudaStream_t (NULL = legacy default).  All
  *   device memory is allocated here (HOTRG_ENOMEM if it does not fit).
  * hotrg_itebd_step: nsteps updates of every chain; synchronises once at the
- *   end; HOTRG_ENONFINITE if a bond's density matrix lost all positive weight.
+ *   end; HOTRG_ENONFINITE if a bond's density matrix lost all positive weight,
+ *   HOTRG_EEIG if its eigensolve did not finish.
  * hotrg_itebd_energy: energy per site of every chain into out_n[n]: the mean
  *   of <theta|h|theta>/<theta|theta> over the two bonds, theta = lam (P Q) and
  *   lam_other (Q P) (the Schmidt values of each bond's left neighbour).
@@ -248,7 +249,8 @@ hotrg_status hotrg_create(const double *T0, int D0, int D_cut, hotrg_prec prec,
  * method, stopped at a residual of 1e-12 relative to the largest eigenvalue.
  * If that bound is not reached within HOTRG_OPT_EIG_MAX_ITERS iterations the
  * step fails with HOTRG_EEIG (latched; the context keeps the state of the last
- * completed step).
+ * completed step).  A whole-matrix diagonalisation that does not finish is reported
+ * as HOTRG_EEIG at the end of its step.
  */
 hotrg_status hotrg_step(hotrg_ctx *ctx, hotrg_dir dir);
 

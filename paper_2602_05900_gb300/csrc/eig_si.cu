@@ -461,7 +461,7 @@ cudaError_t jacobi_full(const SiBatch &b, double *work, cudaStream_t s, long lon
     *launches += 1;
     H = B.C;
   }
-  const SmallEig se{P, m, H, B.Cp, true, b.graded, B.X, n, b.k, B.th, B.flag, B.sweeps, B.flag + 3};
+  const SmallEig se{P, m, H, B.Cp, true, b.graded, B.X, n, b.k, B.th, B.flag, b.err, B.sweeps, B.flag + 3};
   return small_eig(se, s, launches);
 }
 
@@ -706,7 +706,7 @@ cudaError_t si_solve(const SiBatch &b, double *work, double tol, int max_iter, c
       launch_pdl(k_rr_sym, gmm, 256, 0, s, Wn, Tn, Ck, m);                                  // H = W^T X^T Y W
       nl += 2;
       if ((e = cudaGetLastError())) return e;
-      const SmallEig se{P, m, Ck, slot(4), false, false, B.W, m, m, B.th, B.flag, B.sweeps, B.flag + 3};
+      const SmallEig se{P, m, Ck, slot(4), false, false, B.W, m, m, B.th, B.flag, nullptr, B.sweeps, B.flag + 3};
       if ((e = small_eig(se, s, &nl))) return e;                    // H = Z Theta Z^T (Z in B.W)
       launch_pdl(k_rr_mm, gmm, 256, 0, s, Wn, 0, B.W, 1.0, 0.0, Rr, m, always, always);     // R = W Z
       nl += 1;

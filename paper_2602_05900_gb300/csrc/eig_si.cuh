@@ -29,7 +29,8 @@ struct SiBatch {
   bool has_warm;
   int kw;
   bool xs;               // G X on the tensor cores (exact slices) instead of FP64 SIMT
-  int *err;              // device flag set to 2 if a tensor-core wait runs out (xs only)
+  int *err;              // device flag raised to 2 if a tensor-core wait runs out (xs), to kErrEig
+                         // (eig_small.cuh) if jacobi_full does not finish
   PSet trace;            // Tr G of problem z at trace.at(z)[0] (iteration shift)
   bool has_trace;
   double shift_rel;      // initial shift / Tr G

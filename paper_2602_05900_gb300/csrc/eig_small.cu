@@ -39,6 +39,7 @@
 // matrices, m = 16 to 96) leaves residuals and orthonormality at 1e-15 and at
 // most a few rotations for stage 4.
 #include <math.h>
+#include <stdlib.h>
 
 #include <type_traits>
 #include <utility>
@@ -548,12 +549,20 @@ __global__ void __launch_bounds__(256) k_se_mm(MmOp op0, MmOp op1, int P, int m,
 // and always including the largest entry of the matrix -- are rotated at once
 // (Eq. 6), and the accumulated rotation W follows.  Stops when nothing needs
 // rotating; *rounds receives the round count (maximum over problems), flag is
-// set to 2 if kSparseRounds * m rounds do not suffice.  Eigenvalues descending
+// set to 2, and *err (if given) raised to kErrEig, if max_rounds do not suffice.  Eigenvalues descending
 // in theta, Wout columns in the same order.  The search compares FP32
 // magnitudes taken from the bits (an FP64 comparison of every entry would cost
 // more than the rotations: m^2 of them at two per clock).
 constexpr int kSparseRounds = 32;
 constexpr int kSparseThreads = 1024;
+
+// Rounds before a solve is given up: many times what any matrix has been seen to
+// take.  The bounds-checked build lets a test lower them.
+int sparse_rounds(int m) {
+  if constexpr (kChecked)
+    if (const char *v = getenv("HOTRG_TEST_SPARSE_ROUNDS")) return atoi(v);
+  return kSparseRounds * m;
+}
 
 size_t sparse_smem(int m) {
   return (size_t)2 * m * (m + 1) * sizeof(double) + (size_t)m * (sizeof(int) + sizeof(float)) +
@@ -561,7 +570,8 @@ size_t sparse_smem(int m) {
 }
 
 __global__ void __launch_bounds__(kSparseThreads, 1)
-    k_rr_sparse_jacobi(PSet Hin, int m, int floor_exp, PSet Wout, PSet theta, int *flag, int *rounds_out) {
+    k_rr_sparse_jacobi(PSet Hin, int m, int floor_exp, int max_rounds, PSet Wout, PSet theta, int *flag, int *err,
+                       int *rounds_out) {
   pdl_enter();
   extern __shared__ double ssh[];
   const int ld = m + 1, maxsel = m / 2 + 1;
@@ -589,7 +599,7 @@ __global__ void __launch_bounds__(kSparseThreads, 1)
   const float fl = ldexpf(mag32(mx, 0, bias), -floor_exp);
   int round = 0;
   bool done = false;
-  for (; round < kSparseRounds * m; ++round) {
+  for (; round < max_rounds; ++round) {
     for (int p = threadIdx.x; p < m; p += blockDim.x) rt[p] = sqrtf(mag32(H[p * ld + p], bias));
     if (threadIdx.x == 0) nsel = 0;
     __syncthreads();
@@ -659,7 +669,10 @@ __global__ void __launch_bounds__(kSparseThreads, 1)
     __syncthreads();
   }
   if (threadIdx.x == 0) {
-    if (!done) atomicExch(flag, 2);
+    if (!done) {
+      atomicExch(flag, 2);
+      if (err) atomicMax(err, kErrEig);
+    }
     atomicMax(rounds_out, round);
   }
   // sort descending (rank of each diagonal entry, ties by index); best[] now
@@ -804,8 +817,8 @@ cudaError_t small_eig(const SmallEig &a, cudaStream_t s, long long *launches) {
   newton_schulz();
   mm1(op(a.H, 1, X, 1.0, 0.0, Y));
   mm1(sym(X, Y, S));
-  launch_pdl(k_rr_sparse_jacobi, dim3(1, 1, P), kSparseThreads, sparse_smem(m), s, S, m, floor_exp, W, a.theta, a.flag,
-                                                                          a.rounds);
+  launch_pdl(k_rr_sparse_jacobi, dim3(1, 1, P), kSparseThreads, sparse_smem(m), s, S, m, floor_exp, sparse_rounds(m), W,
+             a.theta, a.flag, a.err, a.rounds);
   *launches += 1;
   mm1(MmOp{X, W, W, W, a.out, 0, 0, 0, 1.0, 0.0, a.rows, a.cols});
   return cudaGetLastError();

@@ -10,6 +10,7 @@
 
 namespace hotrg {
 
+constexpr int kErrEig = 4;          // in a context's device error flag: a direct solve did not finish
 constexpr int kSmallEigSlots = 7;   // m x m scratch matrices per problem
 
 struct SmallEig {
@@ -26,6 +27,7 @@ struct SmallEig {
   int rows, cols;        // rows, cols <= m
   PSet theta;            // m eigenvalues, descending
   int *flag;             // set to 2 if the last stage did not finish
+  int *err;              // (optional) raised to kErrEig then
   int *rounds, *sweeps;  // maxima over problems: FP64 rounds, FP32 sweeps
 };
 

@@ -38,6 +38,7 @@
 #include "common.cuh"
 #include "dev_pool.cuh"
 #include "eig_si.cuh"
+#include "eig_small.cuh"
 #include "launch.cuh"
 #include "tc_exact.cuh"
 #include "tc_gemm.cuh"
@@ -338,7 +339,7 @@ void tensor_from_sqrt(int q, const double *W, const double *w, double *T0) {
 
 // Reads the device error flag after a synchronisation: 1 = a max-norm was zero
 // or not finite, 2 = a bounded device wait ran out, 3 = an index outside its
-// buffer (bounds-checked build only).
+// buffer (bounds-checked build only), kErrEig = a direct eigensolve did not finish.
 hotrg_status check_flag(hotrg_ctx *c) {
   int herr = 0;
   if (cudaMemcpy(&herr, c->err, sizeof(int), cudaMemcpyDeviceToHost) != cudaSuccess)
@@ -346,6 +347,7 @@ hotrg_status check_flag(hotrg_ctx *c) {
   if (herr == 1) return fail(c, HOTRG_ENONFINITE, "max-norm of a coarse-grained tensor was zero or not finite");
   if (herr == 3)
     return fail(c, HOTRG_EBOUNDS, "a kernel's mapped index fell outside its buffer (bounds-checked build)");
+  if (herr == kErrEig) return fail(c, HOTRG_EEIG, "a direct eigensolve did not finish within its rounds");
   if (herr) return fail(c, HOTRG_ETIMEOUT, "a tensor-core kernel's bounded wait ran out");
   return HOTRG_OK;
 }
@@ -694,6 +696,7 @@ hotrg_status step_group(hotrg_ctx *c, Group &g, hotrg_dir dir, int step) {
     sb.k = n;
     sb.m = jacobi_block(n);
     sb.G = pset_linear(g.GL, g.sT);
+    sb.err = c->err;
     long long nl = 0;
     CK_CUDA(c, jacobi_full(sb, g.si_work, st, &nl));
     const SiOut o = si_outputs(g.si_work, G, n, sb.m);
@@ -708,6 +711,7 @@ hotrg_status step_group(hotrg_ctx *c, Group &g, hotrg_dir dir, int step) {
     sb.n = n;
     sb.k = k;
     sb.G = pset_pairs(g.GL, g.GR, g.sT);
+    sb.err = c->err;
     long long nl = 0;
     bool ok = false;
     if (n + (n & 1) <= kSiMaxBlock) {
@@ -727,7 +731,6 @@ hotrg_status step_group(hotrg_ctx *c, Group &g, hotrg_dir dir, int step) {
       if (m > n) m = n & ~1;
       sb.m = m;
       sb.xs = c->eig_tc;
-      sb.err = c->err;
       sb.trace = PSet{g.scal + 2, g.scal + 3, kScal};
       sb.has_trace = true;
       sb.shift_rel = 0x1.0p-40;

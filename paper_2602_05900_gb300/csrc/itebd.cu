@@ -32,6 +32,7 @@
 #include "launch.cuh"
 #include "dev_pool.cuh"
 #include "eig_si.cuh"
+#include "eig_small.cuh"
 #include "hotrg.h"
 #include "xxz.cuh"
 
@@ -278,6 +279,7 @@ hotrg_status itebd_update(hotrg_itebd *c) {
   sb.m = jacobi_block(n);
   sb.G = pset_linear(warm ? c->theta : c->rho, c->sM);
   sb.graded = warm;
+  sb.err = c->err;
   long long nl = 0;
   ICK(c, jacobi_full(sb, c->si_work, st, &nl));
   const SiOut o = si_outputs(c->si_work, G, n, sb.m);
@@ -317,6 +319,7 @@ hotrg_status isync(hotrg_itebd *c) {
   ICK(c, cudaStreamSynchronize(c->stream));
   int h = 0;
   ICK(c, cudaMemcpy(&h, c->err, sizeof(int), cudaMemcpyDeviceToHost));
+  if (h == kErrEig) return ifail(c, HOTRG_EEIG, "a bond's eigensolve did not finish within its rounds");
   if (h) return ifail(c, HOTRG_ENONFINITE, "a bond's density matrix has no positive weight");
   return HOTRG_OK;
 }
