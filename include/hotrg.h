@@ -28,7 +28,11 @@
  * Ownership and errors:
  *   - Every host buffer stays owned by the caller; the library copies what it
  *     needs before returning.  A context owns all device memory it uses and
- *     releases it in hotrg_destroy.
+ *     gives it up in hotrg_destroy (hotrg_itebd_destroy): buffers of 1 GiB and more
+ *     to the device, smaller ones to a pool that later contexts and hotrg_dgemm_emu
+ *     take theirs from.  The pool keeps at most 4 GiB of idle memory per device
+ *     until the process ends; other allocations of the process get it when the
+ *     device has no other memory left.
  *   - No C++ exception crosses this interface.  Every call returns a status;
  *     the first error seen by a context is latched: later calls on it return
  *     the same status without doing work, and hotrg_last_error() returns a

@@ -201,9 +201,8 @@ __global__ void __launch_bounds__(1024, 1)
   __syncthreads();
   const double sc = s_scale;
   auto at = [&](int i) { return i < h ? i : HM + i - h; };   // row or column of index i
-  // H is symmetric by definition; its stored copy may not be (a projected
-  // matrix whose basis amplifies rounding), and the two-sided rotations of an
-  // unsymmetric matrix do not settle: read the symmetric part
+  // the symmetric part: two-sided rotations of a matrix whose triangles differ by
+  // rounding (a product's, in a tile on the diagonal) do not settle
   for (int e = tid; e < m * m; e += T) {
     const int a = e / m, b = e % m;
     Abuf[at(a) * ld + at(b)] = to_f32(0.5 * (H[e] + H[(size_t)b * m + a]) * sc);

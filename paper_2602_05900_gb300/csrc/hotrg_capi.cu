@@ -631,9 +631,11 @@ hotrg_status step_group(hotrg_ctx *c, Group &g, hotrg_dir dir, int step) {
         {BR, map2(E, sy, sxp), map2(E, syp, sx)},    // B_R[x2',k,u2',k']: sum over (x2, y')
     };
     // exact slices, where the scratch of one product holds them (it is sized by the
-    // a6 contraction): the four partials as one batch, and both sides' Gram matrices
-    // as one (18 launches for the six products before, 8 now, the same bits: a D = 13
-    // chain pass 6.22 -> 5.74 ms, D = 32 13.27 -> 12.82 ms, a D = 21 run 16.64 -> 16.33 ms)
+    // largest operands of single products at eight digits): the four partials as one
+    // batch, and both sides' Gram matrices as one (18 launches for the six products
+    // before, 8 now, the same bits: a D = 13 chain pass 6.22 -> 5.74 ms, D = 32 13.27 ->
+    // 12.82 ms, a D = 21 run, whose early steps fit, 16.64 -> 16.33 ms).  A chain's time
+    // steps (E = 4) fit; square steps, D = E = D_cut, do at four digits only.
     const bool xs = c->prec == HOTRG_BF16XS && D > 1 && syrk_xs_fits((int)DE, (int)DE, 4 * G, c->xs_digits, g.xw) &&
                     xs_fits((int)D2, (int)D2, (int)E2, c->xs_digits, 2 * G, g.xw);
     MappedGemm mp[4];

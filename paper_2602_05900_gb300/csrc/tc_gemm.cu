@@ -81,7 +81,7 @@ __device__ __forceinline__ void store_out(const TcEpilogue &e, long long off, fl
 }
 
 // Stores 4 consecutive columns (off .. off + 3) of an F32 or F64 output at once
-// (16-byte stores; tc_gemm checked the alignment when it set e.vec4).
+// (16-byte stores; tc_gemm checked the alignment when it set e.vec).
 __device__ __forceinline__ void store_out4(const TcEpilogue &e, long long off, float v0, float v1,
                                            float v2, float v3, long long zoff, int *err) {
   if (!checked_ok(zoff + off, e.cap, err) || !checked_ok(zoff + off + 3, e.cap, err)) return;
